@@ -209,46 +209,51 @@ __device__ __forceinline__ void ld16(const float *src, float (&v)[16])
     }
 }
 
-// four float4 at p, p + 8 ld, p + 16 ld, p + 24 ld (a warp's coalesced 32-row x 16-column block)
-__device__ __forceinline__ void ld_rows4(const float *p, int ld, float4 (&v)[4])
+// 8 bytes from global memory, asking L2 to fetch the whole aligned 256-byte
+// block around them: the four lanes of a row read 32 bytes (16 entries) of
+// each half at a time, and the 256-byte block holds the rest of the row
+// segment, which the next sub-chunks read
+__device__ __forceinline__ uint2 ld8_l2block(const void *p)
 {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        v[i] = *reinterpret_cast<const float4 *>(p + (size_t)(8 * i) * ld);
-}
-
-// 16 bytes from global memory, asking L2 to fetch the whole aligned 256-byte
-// block around them: a phase-2 epilogue thread reads its row's old values 32
-// bytes (16 entries) of each half at a time, and the 256-byte block holds the
-// rest of its row segment, which the next sub-chunks read
-__device__ __forceinline__ uint4 ld16_l2block(const void *p)
-{
-    uint4 v;
-    asm volatile("ld.global.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
+    uint2 v;
+    asm volatile("ld.global.L2::256B.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
     return v;
 }
 
-// For a matrix held as a BF16 split pair: 16 consecutive values hi + lo of one
-// row (the sum is exact in FP32), into v[0..3]
-__device__ __forceinline__ void ld_row16_split(const __nv_bfloat16 *h, const __nv_bfloat16 *l, float4 (&v)[4])
+// Four columns of the rows p, p + 8 ld, p + 16 ld, p + 24 ld of a matrix held
+// as a BF16 split pair (as packed: hi in x, y, lo in z, w) or in FP32
+__device__ __forceinline__ void ld_old_split(const __nv_bfloat16 *h, const __nv_bfloat16 *l, int ld, uint4 (&v)[4])
 {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const uint4 a = ld16_l2block(h + 8 * i), b = ld16_l2block(l + 8 * i);
-        const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-        float f[8];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&av[q]));
-            const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&bv[q]));
-            f[2 * q] = x.x + y.x;
-            f[2 * q + 1] = x.y + y.y;
-        }
-        v[2 * i] = make_float4(f[0], f[1], f[2], f[3]);
-        v[2 * i + 1] = make_float4(f[4], f[5], f[6], f[7]);
+    for (int i = 0; i < 4; ++i) {
+        const uint2 a = ld8_l2block(h + (size_t)(8 * i) * ld), b = ld8_l2block(l + (size_t)(8 * i) * ld);
+        v[i] = make_uint4(a.x, a.y, b.x, b.y);
     }
+}
+__device__ __forceinline__ void ld_old_f32(const float *p, int ld, uint4 (&v)[4])
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        v[i] = *reinterpret_cast<const uint4 *>(p + (size_t)(8 * i) * ld);
+}
+// their values: hi + lo (exact in FP32), or as they are
+__device__ __forceinline__ void unsplit4(const uint4 &p, float (&f)[4])
+{
+    const uint32_t h[2] = {p.x, p.y}, l[2] = {p.z, p.w};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&h[q]));
+        const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&l[q]));
+        f[2 * q] = x.x + y.x;
+        f[2 * q + 1] = x.y + y.y;
+    }
+}
+__device__ __forceinline__ void unpack4(const uint4 &p, float (&f)[4])
+{
+    f[0] = __uint_as_float(p.x);
+    f[1] = __uint_as_float(p.y);
+    f[2] = __uint_as_float(p.z);
+    f[3] = __uint_as_float(p.w);
 }
 
 // 16 BF16 values held as 8 packed pairs: two 16-byte stores, or the masked entries
@@ -1062,12 +1067,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS1, 1) k_tc_ph
 // over this CTA's 128 rows) to slot nb + 2 bm + r.
 // ---------------------------------------------------------------------------
 // Epilogue warps: EPI / 4 per TMEM lane quarter, a template parameter of the
-// phase-2 kernels.  A C' tile has K = T, so its MMAs take about as long as its
-// 256 x 256 outputs take to finish: where the MMAs are the shorter part
-// (T up to about 1300 in BF16X3), twelve epilogue warps with two 64 KB
-// operand stages ran phase 2 5% faster than eight with three at 1000 x 17000;
-// where they are the longer part, the third stage keeps them fed (1600 x
-// 30000: 3.0 ms against 3.7 with two).  p2_epi picks one per launch.
+// phase-2 kernels: eight warps (168 registers) with three 64 KB operand
+// stages, or twelve (128 registers) with two.  The finished tile is taken from
+// TMEM in the fragment layout of the 16x256b load: the four lanes of a row
+// hold 16 consecutive columns after one exchange, so old values come and new
+// ones go straight between registers and memory (32 bytes of each half per
+// row), row sums stay in registers and column sums are reduced by shuffles;
+// only mirrored tiles pass through shared memory.  Against the former layout
+// (one row per lane, every block staged through shared memory; twelve warps)
+// phase 2 at 1000 x 17000 went from 0.776 to 0.734 ms with twelve warps and
+// 0.715 with eight, whose third stage keeps the MMAs fed.  Left in that time:
+// 0.57 ms are the main loop alone (0.53 with half its operand loads: the MMAs),
+// 0.05 the epilogue's arithmetic, 0.09 its loads and stores.
 constexpr int N2 = 256;                    // tile edge
 constexpr uint32_t STAGE2 = 4 * A_BYTES;   // per CTA: A hi, A lo, B hi, B lo (128 rows each)
 
@@ -1339,7 +1350,9 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
         constexpr int PARTS = EPI / 4;
         const int e = warp - 2, wq = warp & 3, third = e >> 2;
         const int c_begin = (16 * third) / PARTS, c_end = (16 * (third + 1)) / PARTS;
-        const int r = wq * 32 + lane;  // row of this CTA's 128-row half
+        const int r = wq * 32 + lane;  // row of this CTA's 128-row half (running sums of K chunks)
+        // a finished tile's fragments (see frag_to_rows): rows er + 8 i, columns ec .. ec + 3 of 16
+        const int er = lane >> 2, ec = 8 * (lane & 1) + 2 * (lane & 2);
         float *blk = blocks + (size_t)e * Cfg::BLK;  // this warp's 32 x 16 staging block, rows of 17
         const int tt = threadIdx.x - 64;  // 0..383
         const uint32_t tempty_even = mapa_shared(smem_u32(&sy.tempty[0]), 0);
@@ -1410,288 +1423,253 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
             // the tile's column norms (shared), this row's norm and its first old values
             if (tt < N2)
                 colnrm[tt] = n0 + tt < nn ? nrm[n0 + tt] : 0.0f;
-            const int k = m0 + r, k0 = m0 + wq * 32;
-            const bool krow = k < nn;  // rows past the network (last block's padding) hold nothing
-            const float nk_ = krow ? nrm[k] : 0.0f;
+            const int k0 = m0 + wq * 32;
+            float nrow[4];  // norms of this lane's rows (those past the network hold nothing)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                nrow[i] = k0 + er + 8 * i < nn ? nrm[k0 + er + 8 * i] : 0.0f;
             // old values (rows past the network are padding inside the array; their values are never
-            // used).  FP32: loaded coalesced (8 rows x 64 B per load), lane l takes columns
-            // 4 (l & 3) .. + 3 of the warp's rows (l >> 2) + 8 i, i = 0..3, and each lane gets its own
-            // row through the staging block.  A split-held C: each lane loads its own row, 32 bytes of
-            // each half per sub-chunk, L2 fetching the row's 256-byte block at the first
-            const size_t xo = sst ? (size_t)k * ld + n0 : (size_t)(k0 + (lane >> 2)) * ld + n0 + 4 * (lane & 3);
-            const float *xblk = sst ? nullptr : X + xo;
-            float4 nxt[4];
+            // used): this lane's rows er, er + 8, er + 16, er + 24 of the warp's 32, four columns of each
+            const size_t xo = (size_t)(k0 + er) * ld + n0 + ec;
+            uint4 nxt[4];
             if (n0 + c_begin * 16 < ld) {
                 if (sst)
-                    ld_row16_split(Xh + xo + c_begin * 16, Xl + xo + c_begin * 16, nxt);
+                    ld_old_split(Xh + xo + c_begin * 16, Xl + xo + c_begin * 16, ld, nxt);
                 else
-                    ld_rows4(xblk + c_begin * 16, ld, nxt);
+                    ld_old_f32(X + xo + c_begin * 16, ld, nxt);
             }
             epi_bar_p2<EPI>();
             // on a timed-out wait every epilogue warp still runs the named barriers below
             const bool live = wait_bounded(&sy.tfull[buf], (uint32_t)(idx >> 1) & 1u, &sy.abort, d.ctl) &&
                               !*(volatile int *)&sy.abort;
             tc_fence_after();
-            float r1 = 0.0f, r2 = 0.0f, rv = 0.0f;
+            float r1[4], r2[4], rv[4];  // this lane's four rows: sums over its columns
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                r1[i] = r2[i] = rv[i] = 0.0f;
             // this warp's row sums of a column group, into its slot (zeros where nothing was summed)
             auto flush = [&](int grp) {
-                rowred[(grp * NS + 0) * 128 + r] = r1;
-                rowred[(grp * NS + 1) * 128 + r] = r2;
-                if (SIM_SIGMA)
-                    rowred[(grp * NS + 2) * 128 + r] = rv;
-                r1 = r2 = rv = 0.0f;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float q1 = r1[i], q2 = r2[i], qv = rv[i];
+#pragma unroll
+                    for (int off = 1; off <= 2; off <<= 1) {  // the four lanes of a row
+                        q1 += __shfl_xor_sync(0xffffffffu, q1, off);
+                        q2 += __shfl_xor_sync(0xffffffffu, q2, off);
+                        if (SIM_SIGMA)
+                            qv += __shfl_xor_sync(0xffffffffu, qv, off);
+                    }
+                    if ((lane & 3) == 0) {
+                        const int row = wq * 32 + er + 8 * i;
+                        rowred[(grp * NS + 0) * 128 + row] = q1;
+                        rowred[(grp * NS + 1) * 128 + row] = q2;
+                        if (SIM_SIGMA)
+                            rowred[(grp * NS + 2) * 128 + row] = qv;
+                    }
+                    r1[i] = r2[i] = rv[i] = 0.0f;
+                }
             };
             for (int grp = p2_group(c_begin); grp <= p2_group(c_end - 1); ++grp)
                 flush(grp);  // (all zero: a timed-out tile leaves no stale sums)
             const uint32_t tbase = sy.tmem + buf * N2 + ((uint32_t)(wq * 32) << 16);
             // accumulator columns one sub-chunk ahead: each sub-chunk's TMEM load is issued once the
-            // previous one's arithmetic is done and lands while that one's stores go out
+            // previous one's values have been taken and lands while that one's arithmetic and stores run
             uint32_t accr[16];
             if (live)
-                tmem_ld16_nowait(tbase + c_begin * 16, accr);
+                tmem_ld_frag16_nowait(tbase + c_begin * 16, accr);
 #pragma unroll 1
             for (int c = c_begin; c < c_end && live; ++c) {  // this warp's 16-column sub-chunks
                 const int cc = c * 16, j0 = n0 + cc;
-                const bool inside = krow && j0 < ld;
                 if (c > c_begin && p2_group(c) != p2_group(c - 1))
                     flush(p2_group(c - 1));
-                float old[16], acc[16];
-                if (sst) {  // this lane's own row
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        old[4 * i] = inside ? nxt[i].x : 0.0f;
-                        old[4 * i + 1] = inside ? nxt[i].y : 0.0f;
-                        old[4 * i + 2] = inside ? nxt[i].z : 0.0f;
-                        old[4 * i + 3] = inside ? nxt[i].w : 0.0f;
-                    }
-                } else {  // to this lane's own row through the staging block
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float *b = blk + ((lane >> 2) + 8 * i) * 17 + 4 * (lane & 3);
-                        b[0] = nxt[i].x; b[1] = nxt[i].y; b[2] = nxt[i].z; b[3] = nxt[i].w;
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        old[q] = inside ? blk[lane * 17 + q] : 0.0f;
-                    __syncwarp();  // the block takes the new values next
-                }
-                if (c + 1 < c_end && j0 + 16 < ld) {  // next sub-chunk's old values, in flight meanwhile
-                    if (sst)
-                        ld_row16_split(Xh + xo + (c + 1) * 16, Xl + xo + (c + 1) * 16, nxt);
-                    else
-                        ld_rows4(xblk + (c + 1) * 16, ld, nxt);
-                }
+                float x[4][4], v[4][4];  // [row][column]: numerators, then the summed values; new entries
                 tmem_wait16(accr);
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    acc[q] = __uint_as_float(accr[q]) * ascale;
-                if (it.nchunks > 1) {  // a P tile's last K chunk: add the running sum of the others
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        acc[q] = __ldcg(scr + (size_t)(cc + q) * 128 + r) + acc[q];  // L2: where the adds landed
-                }
-                if (c + 1 == c_end) {  // this warp is done with the accumulator: tell the even CTA
+                frag_to_rows(accr, x);
+                if (c + 1 < c_end) {
+                    tmem_ld_frag16_nowait(tbase + cc + 16, accr);
+                } else {  // this warp is done with the accumulator: tell the even CTA
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0)
                         mbar_arrive_cluster(tempty_even + buf * (uint32_t)sizeof(uint64_t));
                 }
-                // interior sub-chunks of off-diagonal tiles are entirely valid
-                uint32_t vmask = 0xffffu;
-                if (!(k < j0 && j0 + 15 < nn)) {
-                    vmask = 0;
 #pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        vmask |= (k < j0 + q && j0 + q < nn) ? (1u << q) : 0u;
+                for (int i = 0; i < 4; ++i) {
+                    if (sst)
+                        unsplit4(nxt[i], v[i]);
+                    else
+                        unpack4(nxt[i], v[i]);
                 }
-                if (vmask == 0xffffu) {  // interior: no masking
+                if (c + 1 < c_end && j0 + 16 < ld) {  // next sub-chunk's old values, in flight meanwhile
+                    if (sst)
+                        ld_old_split(Xh + xo + (c + 1) * 16, Xl + xo + (c + 1) * 16, ld, nxt);
+                    else
+                        ld_old_f32(X + xo + (c + 1) * 16, ld, nxt);
+                }
+                if (q8) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float4 n4 = reinterpret_cast<const float4 *>(colnrm + cc)[q];
-                        const float nj[4] = {n4.x, n4.y, n4.z, n4.w};
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            x[i][u] *= ascale;
+                }
+                if (it.nchunks > 1) {  // a P tile's last K chunk: add the running sum of the others
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)  // L2: where the adds landed
+                            x[i][u] = __ldcg(scr + (size_t)(cc + ec + u) * 128 + wq * 32 + er + 8 * i) + x[i][u];
+                }
+                const float4 n4 = *reinterpret_cast<const float4 *>(colnrm + cc + ec);
+                const float nj[4] = {n4.x, n4.y, n4.z, n4.w};
+                const bool inner = k0 + 31 < j0 && j0 + 15 < nn;  // the whole 32 x 16 block counts
+                uint32_t vm = 0xffffu;                            // bit 4 i + u: entry (row i, column u) counts
+                float cs[8], cv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    cs[u] = cs[4 + u] = cv[u] = 0.0f;
+                if (inner) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            const int e2 = 4 * q + u;
-                            const float s = tanimoto_clamped(acc[e2], nk_, nj[u]);
-                            const float v = fmaf(a, s, keep * old[e2]);
-                            const float x = SIM_SIGMA ? s : v;
-                            r1 += x;
-                            r2 = fmaf(x, x, r2);
-                            if (SIM_SIGMA)
-                                rv = fmaf(v, v, rv);
-                            old[e2] = v;
-                            acc[e2] = x;
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        const float s = tanimoto_fast(acc[q], nk_, colnrm[cc + q]);
-                        const bool valid = (vmask >> q) & 1u;
-                        const float v = valid ? fmaf(a, s, keep * old[q]) : old[q];
-                        const float x = valid ? (SIM_SIGMA ? s : v) : 0.0f;
-                        r1 += x;
-                        r2 += x * x;
-                        if (SIM_SIGMA)
-                            rv += valid ? v * v : 0.0f;
-                        old[q] = v;
-                        acc[q] = x;
-                    }
-                }
-                // column sums of s under D2 (from registers; v sums come from the staged block)
-                if (SIM_SIGMA) {
-                    float sq[16];  // old[] holds the new values, staged below; acc is consumed here
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        sq[q] = acc[q] * acc[q];
-                    const float t1 = lane_transpose_sum16(sq);
-                    const float t0 = lane_transpose_sum16(acc);
-                    if (lane < 16) {
-                        colred[(wq * NS + 1) * N2 + cc + lane] = t1;
-                        colred[(wq * NS + 0) * N2 + cc + lane] = t0;
-                    }
-                }
-                if (c + 1 < c_end)
-                    tmem_ld16_nowait(tbase + cc + 16, accr);
-                // stage the new values (0 where nothing is stored) in this warp's block
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    blk[lane * 17 + q] = (vmask >> q & 1u) ? old[q] : 0.0f;
-                __syncwarp();
-                // (a) row-major copies, coalesced.  A split-held C: lane l takes 8 columns of rows
-                // (l >> 1) + 16 i, 16-byte stores of each half
-                if (sst) {
-#pragma unroll
-                    for (int i2 = 0; i2 < 2; ++i2) {
-                        const int rr = (lane >> 1) + 16 * i2, kk = k0 + rr, jj = j0 + 8 * (lane & 1);
-                        float f[8];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            f[q] = blk[rr * 17 + 8 * (lane & 1) + q];
-                        uint32_t h4[4], l4[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            split_pair(f[2 * q], f[2 * q + 1], h4[q], l4[q]);
-                        const size_t ro = (size_t)kk * ld + jj;
-                        if (kk < jj && jj + 7 < nn) {
-                            *reinterpret_cast<uint4 *>(Xh + ro) = make_uint4(h4[0], h4[1], h4[2], h4[3]);
-                            *reinterpret_cast<uint4 *>(Xl + ro) = make_uint4(l4[0], l4[1], l4[2], l4[3]);
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                if (kk < jj + q && jj + q < nn) {
-                                    reinterpret_cast<uint16_t *>(Xh)[ro + q] = (uint16_t)(h4[q >> 1] >> (16 * (q & 1)));
-                                    reinterpret_cast<uint16_t *>(Xl)[ro + q] = (uint16_t)(l4[q >> 1] >> (16 * (q & 1)));
-                                }
-                        }
-                    }
-                }
-#pragma unroll
-                for (int i2 = 0; i2 < (sst ? 0 : 4); ++i2) {
-                    const int rr = (lane >> 2) + 8 * i2, kk = k0 + rr, jj = j0 + 4 * (lane & 3);
-                    float f[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        f[q] = blk[rr * 17 + 4 * (lane & 3) + q];
-                    const size_t ro = (size_t)kk * ld + jj;
-                    if (q8) {
-                        if (kk < jj && jj + 3 < nn) {
-                            *reinterpret_cast<float4 *>(X + ro) = make_float4(f[0], f[1], f[2], f[3]);
-                            *reinterpret_cast<uint32_t *>(d.C8 + ro) =
-                                e4m3x2(f[0], f[1], sC) | e4m3x2(f[2], f[3], sC) << 16;
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                if (kk < jj + q && jj + q < nn) {
-                                    X[ro + q] = f[q];
-                                    d.C8[ro + q] = (uint8_t)e4m3x2(f[q], 0.0f, sC);
-                                }
-                        }
-                        continue;
-                    }
-                    uint32_t h2[2], l2[2];
-                    split_pair(f[0], f[1], h2[0], l2[0]);
-                    split_pair(f[2], f[3], h2[1], l2[1]);
-                    if (kk < jj && jj + 3 < nn) {
-                        if (!sst)
-                            *reinterpret_cast<float4 *>(X + ro) = make_float4(f[0], f[1], f[2], f[3]);
-                        *reinterpret_cast<uint2 *>(Xh + ro) = make_uint2(h2[0], h2[1]);
-                        if (wlo)
-                            *reinterpret_cast<uint2 *>(Xl + ro) = make_uint2(l2[0], l2[1]);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (kk < jj + q && jj + q < nn) {
-                                if (!sst)
-                                    X[ro + q] = f[q];
-                                reinterpret_cast<uint16_t *>(Xh)[ro + q] = (uint16_t)(h2[q >> 1] >> (16 * (q & 1)));
-                                if (wlo)
-                                    reinterpret_cast<uint16_t *>(Xl)[ro + q] =
-                                        (uint16_t)(l2[q >> 1] >> (16 * (q & 1)));
+                            const float s = tanimoto_clamped(x[i][u], nrow[i], nj[u]);
+                            const float w = fmaf(a, s, keep * v[i][u]);
+                            const float y = SIM_SIGMA ? s : w;
+                            r1[i] += y;
+                            r2[i] = fmaf(y, y, r2[i]);
+                            cs[u] += y;
+                            cs[4 + u] = fmaf(y, y, cs[4 + u]);
+                            if (SIM_SIGMA) {
+                                rv[i] = fmaf(w, w, rv[i]);
+                                cv[u] = fmaf(w, w, cv[u]);
                             }
+                            v[i][u] = w;
+                        }
+                } else {
+                    vm = 0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int kk = k0 + er + 8 * i, jj = j0 + ec + u;
+                            const bool valid = kk < jj && jj < nn;
+                            const float s = tanimoto_fast(x[i][u], nrow[i], nj[u]);
+                            const float w = valid ? fmaf(a, s, keep * v[i][u]) : 0.0f;
+                            const float y = valid ? (SIM_SIGMA ? s : w) : 0.0f;
+                            r1[i] += y;
+                            r2[i] = fmaf(y, y, r2[i]);
+                            cs[u] += y;
+                            cs[4 + u] = fmaf(y, y, cs[4 + u]);
+                            if (SIM_SIGMA) {
+                                rv[i] = fmaf(w, w, rv[i]);
+                                cv[u] = fmaf(w, w, cv[u]);
+                            }
+                            v[i][u] = w;
+                            vm |= valid ? 1u << (4 * i + u) : 0u;
+                        }
+                }
+                // (a) the new entries, row-major, from this lane's registers: the four lanes of a row
+                // write 16 consecutive columns (32 bytes of each BF16 half, 64 of FP32)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const size_t ro = xo + (size_t)(8 * i) * ld + cc;
+                    const uint32_t m = vm >> (4 * i) & 15u;
+                    if (!q8) {
+                        uint32_t h2[2], l2[2];
+                        split_pair(v[i][0], v[i][1], h2[0], l2[0]);
+                        split_pair(v[i][2], v[i][3], h2[1], l2[1]);
+                        if (m == 15u) {
+                            *reinterpret_cast<uint2 *>(Xh + ro) = make_uint2(h2[0], h2[1]);
+                            if (wlo)
+                                *reinterpret_cast<uint2 *>(Xl + ro) = make_uint2(l2[0], l2[1]);
+                        } else if (m) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (m >> u & 1u) {
+                                    reinterpret_cast<uint16_t *>(Xh)[ro + u] = (uint16_t)(h2[u >> 1] >> (16 * (u & 1)));
+                                    if (wlo)
+                                        reinterpret_cast<uint16_t *>(Xl)[ro + u] =
+                                            (uint16_t)(l2[u >> 1] >> (16 * (u & 1)));
+                                }
+                        }
+                    } else {
+                        const uint32_t p8 = e4m3x2(v[i][0], v[i][1], sC) | e4m3x2(v[i][2], v[i][3], sC) << 16;
+                        if (m == 15u) {
+                            *reinterpret_cast<uint32_t *>(d.C8 + ro) = p8;
+                        } else if (m) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (m >> u & 1u)
+                                    d.C8[ro + u] = (uint8_t)(p8 >> (8 * u));
+                        }
+                    }
+                    if (!sst) {
+                        if (m == 15u) {
+                            *reinterpret_cast<float4 *>(X + ro) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+                        } else if (m) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (m >> u & 1u)
+                                    X[ro + u] = v[i][u];
+                        }
                     }
                 }
-                // (b) mirrored entries (j, k): lane l takes column (l & 15), rows 16 (l >> 4) + 0..15,
-                //     and the column sums over the warp's 32 rows
+                // (b) the column sums over the warp's 32 rows: this lane's four rows are summed above,
+                // the eight lanes of a column reduce-scatter their eight sums (7 shuffles)
                 {
+                    const float t = lanes8_reduce_scatter8(cs);
+                    const int e2 = (lane >> 2 & 1) + 2 * (lane >> 3 & 1);  // this lane's column of the four
+                    colred[(wq * NS + (lane >> 4)) * N2 + cc + ec + e2] = t;
+                    if (SIM_SIGMA) {
+                        const float tv = lanes8_reduce_scatter4(cv);
+                        if (!(lane & 4))
+                            colred[(wq * NS + 2) * N2 + cc + ec + (lane >> 3 & 1) + 2 * (lane >> 4)] = tv;
+                    }
+                }
+                // (c) mirrored entries (j, k), through this warp's staging block: lane l takes column
+                // (l & 15), rows 16 (l >> 4) + 0..15
+                if (mirror) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            blk[(er + 8 * i) * 17 + ec + u] = v[i][u];
+                    __syncwarp();
                     const int col = lane & 15, h16 = 16 * (lane >> 4);
                     float g[16];
 #pragma unroll
                     for (int m = 0; m < 16; ++m)
                         g[m] = blk[(h16 + m) * 17 + col];
-                    float c1 = 0.0f, c2 = 0.0f;
+                    const int jm = j0 + col, km = k0 + h16;
+                    const uint32_t mmask =
+                        jm >= nn ? 0u : (km + 15 < jm ? 0xffffu : (km >= jm ? 0u : ((1u << (jm - km)) - 1u)));
+                    const size_t mo = (size_t)jm * ld + km;
+                    if (q8 && mmask) {
+                        uint32_t p8[4];
 #pragma unroll
-                    for (int m = 0; m < 16; ++m) {
-                        c1 += g[m];
-                        c2 += g[m] * g[m];
-                    }
-                    c1 += __shfl_xor_sync(0xffffffffu, c1, 16);
-                    c2 += __shfl_xor_sync(0xffffffffu, c2, 16);
-                    if (lane < 16) {
-                        if (SIM_SIGMA) {
-                            colred[(wq * NS + 2) * N2 + cc + lane] = c2;  // sum of v^2
+                        for (int q = 0; q < 4; ++q)
+                            p8[q] = e4m3x2(g[4 * q], g[4 * q + 1], sC) | e4m3x2(g[4 * q + 2], g[4 * q + 3], sC) << 16;
+                        uint8_t *dst = d.C8 + mo;
+                        if (mmask == 0xffffu) {
+                            *reinterpret_cast<uint4 *>(dst) = make_uint4(p8[0], p8[1], p8[2], p8[3]);
                         } else {
-                            colred[(wq * NS + 0) * N2 + cc + lane] = c1;
-                            colred[(wq * NS + 1) * N2 + cc + lane] = c2;
-                        }
-                    }
-                    if (mirror && q8) {
-                        const int jm = j0 + col, km = k0 + h16;
-                        const uint32_t mmask =
-                            jm >= nn ? 0u : (km + 15 < jm ? 0xffffu : (km >= jm ? 0u : ((1u << (jm - km)) - 1u)));
-                        if (mmask) {
-                            uint32_t p8[4];
 #pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                p8[q] = e4m3x2(g[4 * q], g[4 * q + 1], sC) | e4m3x2(g[4 * q + 2], g[4 * q + 3], sC) << 16;
-                            uint8_t *dst = d.C8 + (size_t)jm * ld + km;
-                            if (mmask == 0xffffu) {
-                                *reinterpret_cast<uint4 *>(dst) = make_uint4(p8[0], p8[1], p8[2], p8[3]);
-                            } else {
-#pragma unroll
-                                for (int q = 0; q < 16; ++q)
-                                    if (mmask >> q & 1u)
-                                        dst[q] = (uint8_t)(p8[q >> 2] >> (8 * (q & 3)));
-                            }
+                            for (int q = 0; q < 16; ++q)
+                                if (mmask >> q & 1u)
+                                    dst[q] = (uint8_t)(p8[q >> 2] >> (8 * (q & 3)));
                         }
-                    } else if (mirror) {
+                    } else if (mmask) {
                         uint32_t hv[8], lv[8];
 #pragma unroll
                         for (int q = 0; q < 8; ++q)
                             split_pair(g[2 * q], g[2 * q + 1], hv[q], lv[q]);
-                        const int jm = j0 + col, km = k0 + h16;
-                        const uint32_t mmask =
-                            jm >= nn ? 0u : (km + 15 < jm ? 0xffffu : (km >= jm ? 0u : ((1u << (jm - km)) - 1u)));
-                        if (mmask) {
-                            const size_t mo = (size_t)jm * ld + km;
-                            st16_packed(Xh + mo, hv, mmask);
-                            if (wlo)
-                                st16_packed(Xl + mo, lv, mmask);
-                        }
+                        st16_packed(Xh + mo, hv, mmask);
+                        if (wlo)
+                            st16_packed(Xl + mo, lv, mmask);
                     }
+                    __syncwarp();  // the block is rewritten by the next sub-chunk
                 }
-                __syncwarp();  // the block is rewritten by the next sub-chunk
             }
             if (live)
                 flush(p2_group(c_end - 1));
@@ -1890,20 +1868,15 @@ struct P2Spec {
 const P2Spec TC_P2_SPEC[TC_P2_CANDS] = {{0, 192, 0, 0}, {1, 48, 0, 0},  {1, 192, 0, 0},
                                         {1, 192, 1, 0}, {1, 768, 0, 0}, {1, 192, 0, 1}};
 
-int p2_epi(long long mma_slots);
-
-// One phase-2 schedule of every network's upper-triangle P and C tiles (only
-// the networks whose phase-2 kernel configuration p2_epi is epi, if epi > 0).
+// One phase-2 schedule of every network's upper-triangle P and C tiles.
 // A P tile is one unit of the LPT assignment (its whole K) and is listed as
 // its K chunks, consecutively, on the pair it is assigned to (see P2Item).
 void build_p2(const std::vector<const Dev *> &ds, int pairs, const P2Spec &sp, std::vector<int> &off,
-              std::vector<int> &tiles, std::vector<int> &nets, int epi = 0)
+              std::vector<int> &tiles, std::vector<int> &nets)
 {
     std::vector<std::pair<long long, std::pair<int, int>>> all;
     for (int k = 0; k < (int)ds.size(); ++k) {
         const Dev &d = *ds[k];
-        if (epi > 0 && p2_epi(tile_cost(d, false, 0)) != epi)
-            continue;
         for (int isP = 1; isP >= 0; --isP) {
             const int nb = ceil_div(isP ? d.Tp : d.Gp, N2);
             long long c = tile_cost(d, isP != 0, 0);
@@ -2031,11 +2004,13 @@ cudaError_t phase2_smem_limits()
 }
 
 // Epilogue warps of phase 2 for networks whose C' tiles take mma_slots MMA
-// issue slots each (the largest over a set): 12 (two operand stages) while
-// the MMAs are shorter than the epilogue, about 290 slots of the dense peak
-// at 1000 x 17000 (1000 x 17000 under BF16X3: 192 slots), else 8 (three
-// stages; 1600 x 30000: 336 slots)
-int p2_epi(long long mma_slots) { return mma_slots > 256 ? 8 : 12; }
+// issue slots each (the largest over a set): twelve (two operand stages) only
+// where a tile is almost all epilogue, eight (three stages) otherwise.
+// Measured, twelve against eight: FP8MIX at 1000 x 17000 (32 slots) 0.633 and
+// 0.675 ms; BF16X3 at 250 x 2100 (48) even; at 600 x 6000 (120) 131 and 134 us,
+// at 1000 x 17000 (192) 0.734 and 0.715 ms, a set of twelve networks (48 to
+// 192) 1.12 and 0.97 ms; 1600 x 30000 (336) 3.7 and 2.9 ms.
+int p2_epi(long long mma_slots) { return mma_slots > 64 ? 8 : 12; }
 
 // One phase-2 launch of EPI epilogue warps
 template <int EPI, class... Args>
@@ -2282,15 +2257,12 @@ struct TcSet {
         int *off = nullptr;
     };
     struct P2 {               // a phase-2 schedule: per pair, a list of packed tiles and their networks
-        // one launch per phase-2 kernel configuration (p2_epi) among the networks, each network in
-        // the configuration of its own single runs (the autotuner's last candidate swaps them; the
-        // two give the same bits: see p2_group)
-        struct Part {
-            int epi2 = 12, pairs = 0;
-            int *off = nullptr, *tiles = nullptr, *nets = nullptr;
-        };
-        Part part[2];
-        int nparts = 0;
+        // one launch over every network, in the configuration p2_epi picks for the longest C' tile
+        // of the set (the autotuner's last candidate takes the other; the two give the same bits: see
+        // p2_group).  One launch per configuration among the networks was slower: the twelve-network
+        // set's phase 2 took 1.02 ms in two launches against 0.97.
+        int epi2 = 8, pairs = 0;
+        int *off = nullptr, *tiles = nullptr, *nets = nullptr;
     };
     std::vector<P1> p1;
     std::vector<P2> p2;
@@ -2353,23 +2325,17 @@ cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out)
                 e = upload(&c.off, off);
             t->p1.push_back(c);
         }
-        bool has[2] = {false, false};  // networks whose phase 2 runs 12 / 8 epilogue warps
+        long long slots = 0;  // the longest C' tile decides the set's phase-2 configuration
         for (const Dev *d : ds)
-            has[p2_epi(tile_cost(*d, false, 0)) == 8] = true;
+            slots = std::max(slots, (long long)tile_cost(*d, false, 0));
         for (int q = 0; q < TC_P2_CANDS && !e; ++q) {
             TcSet::P2 c;
-            for (int g = 0; g < 2 && !e; ++g) {
-                if (!has[g])
-                    continue;
-                std::vector<int> off, tiles, nets;
-                TcSet::P2::Part &pt = c.part[c.nparts++];
-                // the networks whose single runs use configuration g; the candidate may run the other
-                build_p2(ds, t->pairs, TC_P2_SPEC[q], off, tiles, nets, g ? 8 : 12);
-                pt.epi2 = (g != 0) != (TC_P2_SPEC[q].other != 0) ? 8 : 12;
-                pt.pairs = (int)off.size() - 1;
-                if (!(e = upload(&pt.off, off)) && !(e = upload(&pt.tiles, tiles)))
-                    e = upload(&pt.nets, nets);
-            }
+            std::vector<int> off, tiles, nets;
+            build_p2(ds, t->pairs, TC_P2_SPEC[q], off, tiles, nets);
+            c.epi2 = (p2_epi(slots) == 8) != (TC_P2_SPEC[q].other != 0) ? 8 : 12;
+            c.pairs = (int)off.size() - 1;
+            if (!(e = upload(&c.off, off)) && !(e = upload(&c.tiles, tiles)))
+                e = upload(&c.nets, nets);
             t->p2.push_back(c);
         }
     }
@@ -2400,16 +2366,13 @@ cudaError_t tc_set_launch(TcSet *t, int p1, int p2, cudaStream_t s, cudaEvent_t 
         return e;
     if (ev1)
         cudaEventRecord(ev1, s);
-    for (int g = 0; g < c.nparts; ++g) {
-        const TcSet::P2::Part &pt = c.part[g];
-        a.sched_off = pt.off;
-        a.sched = pt.tiles;
-        a.sched_net = pt.nets;
-        if (pt.epi2 == 8)
-            launch_p2_set<8>(t->diag == 2, 2 * pt.pairs, s, a);
-        else
-            launch_p2_set<12>(t->diag == 2, 2 * pt.pairs, s, a);
-    }
+    a.sched_off = c.off;
+    a.sched = c.tiles;
+    a.sched_net = c.nets;
+    if (c.epi2 == 8)
+        launch_p2_set<8>(t->diag == 2, 2 * c.pairs, s, a);
+    else
+        launch_p2_set<12>(t->diag == 2, 2 * c.pairs, s, a);
     if (ev2)
         cudaEventRecord(ev2, s);
     return launch_fin_tail_set(t->devs, t->blocks, t->nblocks, t->n, s);
@@ -2436,12 +2399,11 @@ void tc_set_destroy(TcSet *t)
         cudaFree(c.items);
         cudaFree(c.off);
     }
-    for (auto &c : t->p2)
-        for (auto &q : c.part) {
-            cudaFree(q.off);
-            cudaFree(q.tiles);
-            cudaFree(q.nets);
-        }
+    for (auto &c : t->p2) {
+        cudaFree(c.off);
+        cudaFree(c.tiles);
+        cudaFree(c.nets);
+    }
     delete t;
 }
 

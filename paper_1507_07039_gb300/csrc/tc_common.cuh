@@ -353,6 +353,70 @@ __device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16])
                  : "memory");
 }
 
+// 32 rows x 16 columns of an accumulator in the fragment layout of the
+// 16x256b load, without waiting: r[0..7] from the warp's TMEM lanes 0-15,
+// r[8..15] from its lanes 16-31; in each half of eight, registers 4 c + {0, 1}
+// are row lane / 4, columns 8 c + 2 (lane & 3) + {0, 1}, and 4 c + {2, 3} the
+// same columns of row lane / 4 + 8.
+__device__ __forceinline__ void tmem_ld_frag16_nowait(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                   "=r"(r[15])
+                 : "r"(taddr + (16u << 16)));
+}
+// That fragment with four consecutive columns per lane: x[i][u] is row
+// lane / 4 + 8 i, column 8 (lane & 1) + 4 ((lane >> 1) & 1) + u of the 16 (the
+// lanes of a pair swap one of their two column pairs: 8 shuffles for 16 values).
+__device__ __forceinline__ void frag_to_rows(const uint32_t (&r)[16], float (&x)[4][4])
+{
+    const bool odd = threadIdx.x & 1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int b = 8 * (i >> 1) + 2 * (i & 1);  // columns 0-7 of this row; columns 8-15 at b + 4
+        const uint32_t s0 = odd ? r[b] : r[b + 4], s1 = odd ? r[b + 1] : r[b + 5];
+        const uint32_t t0 = __shfl_xor_sync(0xffffffffu, s0, 1), t1 = __shfl_xor_sync(0xffffffffu, s1, 1);
+        x[i][0] = __uint_as_float(odd ? t0 : r[b]);
+        x[i][1] = __uint_as_float(odd ? t1 : r[b + 1]);
+        x[i][2] = __uint_as_float(odd ? r[b + 4] : t0);
+        x[i][3] = __uint_as_float(odd ? r[b + 5] : t1);
+    }
+}
+// Sums of v[0..7] over the eight lanes with the same lane & 3; lane l returns
+// the total of entry 4 (l >> 4) + 2 (l >> 3 & 1) + (l >> 2 & 1).  Fixed order.
+__device__ __forceinline__ float lanes8_reduce_scatter8(const float (&v)[8])
+{
+    const int lane = threadIdx.x & 31;
+    float a[4], b[2];
+    bool up = lane & 16;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        a[k] = (up ? v[4 + k] : v[k]) + __shfl_xor_sync(0xffffffffu, up ? v[k] : v[4 + k], 16);
+    up = lane & 8;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        b[k] = (up ? a[2 + k] : a[k]) + __shfl_xor_sync(0xffffffffu, up ? a[k] : a[2 + k], 8);
+    up = lane & 4;
+    return (up ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, up ? b[0] : b[1], 4);
+}
+// As above for four entries: lanes l and l ^ 4 both return the total of entry
+// 2 (l >> 4) + (l >> 3 & 1).
+__device__ __forceinline__ float lanes8_reduce_scatter4(const float (&v)[4])
+{
+    const int lane = threadIdx.x & 31;
+    float a[2];
+    bool up = lane & 16;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        a[k] = (up ? v[2 + k] : v[k]) + __shfl_xor_sync(0xffffffffu, up ? v[k] : v[2 + k], 16);
+    up = lane & 8;
+    const float b = (up ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, up ? a[0] : a[1], 8);
+    return b + __shfl_xor_sync(0xffffffffu, b, 4);
+}
+
 // ---- the pipeline ------------------------------------------------------------------
 template <int STAGES>
 struct Sync {
@@ -427,24 +491,6 @@ __device__ __forceinline__ void drain(Sync<STAGES> &sy, Ctl *ctl)
 {
     for (int kb = sy.consumed; kb < sy.issued; ++kb)
         wait_bounded(&sy.full[kb % STAGES], (uint32_t)(kb / STAGES) & 1u, &sy.abort, ctl, true);
-}
-
-// Sum v[q] (16 values) over the 32 lanes so that lanes l and l ^ 16 both end
-// with the total for q = l & 15 (16 shuffles; fixed order, so deterministic).
-__device__ __forceinline__ float lane_transpose_sum16(float (&v)[16])
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int k = 0; k < off; ++k) {
-            const float send = up ? v[k] : v[k + off];
-            const float keep = up ? v[k + off] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-    }
-    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
 // named barrier among the 256 threads of eight epilogue warps
