@@ -39,7 +39,6 @@ METRIC = "PANDA iterations/s + TFLOP/s, BF16-split vs FP32, at max|ΔW|≤1e-4 v
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0, "sm_max_mhz": 2070.0}
-SMS, FP32_LANES = 152, 128
 ALPHA = 0.1
 GRAPH_ITERS = 8  # iterations per captured graph launch (the library's default)
 
@@ -147,15 +146,9 @@ def algorithmic_flops(T: int, G: int) -> float:
 
 def kernel_algorithmic_work(name: str, T: int, G: int) -> tuple[float, str]:
     """Algorithmic flops one launch of a kernel does, and the unit."""
-    if name in ("k_phase1",):            # W . C_off product + fused update
-        return 2.0 * T * G * G, "flop"
-    if name in ("k_rn",):
-        return 2.0 * T * T * G, "flop"
-    if name in ("k_phase2",):            # symmetric halves of both similarity products
-        return 1.0 * T * G * G + 1.0 * T * T * G, "flop"
-    if name in ("k_tc_phase1",):         # both products of phase 1 in one launch
+    if name in ("k_tc_phase1", "k_f32_phase1"):  # both products of phase 1 in one launch
         return 2.0 * T * G * G + 2.0 * T * T * G, "flop"
-    if name in ("k_tc_phase2",):
+    if name in ("k_tc_phase2", "k_f32_phase2"):  # symmetric halves of both similarity products
         return 1.0 * T * G * G + 1.0 * T * T * G, "flop"
     return 0.0, "flop"
 
@@ -163,9 +156,9 @@ def kernel_algorithmic_work(name: str, T: int, G: int) -> tuple[float, str]:
 def kernel_split_work(name: str, T: int, G: int) -> tuple[float, float]:
     """A tensor-core launch's algorithmic flops split into the gene-sized
     products (W.C, W^T.W) and the TF-sized ones (P.W, W.W^T)."""
-    if name == "k_tc_phase1":
+    if name in ("k_tc_phase1", "k_f32_phase1"):
         return 2.0 * T * G * G, 2.0 * T * T * G
-    if name == "k_tc_phase2":
+    if name in ("k_tc_phase2", "k_f32_phase2"):
         return 1.0 * T * G * G, 1.0 * T * T * G
     return 0.0, 0.0
 
@@ -214,37 +207,27 @@ def tensor_peak(peaks: dict, peak_src: str, ck: dict | None, timed_ms: float) ->
 
 def kernel_flops(panda, prec: int, name: str, T: int, G: int) -> tuple[float, float, float]:
     """(useful flops, issued tensor flops, issued flops in BF16-MMA time
-    units) of one launch of a tensor-core kernel: BF16X3 issues three MMAs per
-    product, BF16X2 two; FP8MIX runs the gene-sized products as one E4M3 MMA,
+    units) of one launch of a tensor-core kernel: FP32 issues six MMAs per
+    product (its operands' exact three-way BF16 splits), BF16X3 three, BF16X2
+    two; FP8MIX runs the gene-sized products as one E4M3 MMA,
     which takes half the time of a BF16 one, and the TF-sized ones as BF16X3."""
     useful = kernel_algorithmic_work(name, T, G)[0]
     big, small = kernel_split_work(name, T, G)
     if prec == panda.PANDA_FP8MIX:
         return useful, big + 3.0 * small, 0.5 * big + 3.0 * small
-    terms = 3.0 if prec == panda.PANDA_BF16X3 else 2.0
+    terms = {panda.PANDA_FP32: 6.0, panda.PANDA_BF16X3: 3.0}.get(prec, 2.0)
     return useful, terms * useful, terms * useful
 
 
 def roofline(panda, prec, kstats, T, G, wl_name, peaks, peak_src, ck, timed_ms, ffma, iters_per_s):
     """The bench line's roofline object: the dominant kernel against the peak
-    of its pipe, every product kernel beside it, and the whole iteration."""
+    of its pipe, every product kernel beside it, and the whole iteration.
+    ffma: the measured FP32 FMA rate, reported beside the FP32 mode's figures
+    (whose products run on the tensor cores)."""
     top = max(kstats, key=lambda k: k[1])
     work, _ = kernel_algorithmic_work(top[0], T, G)
     avg_s = top[1] / top[2] / 1000.0
     hbm = peaks.get("hbm_gbs", FALLBACK["hbm_gbs"])
-    if prec == panda.PANDA_FP32:
-        if ffma:
-            peak, src = ffma, "FP32 FFMA loop on every SM, timed by CUDA events on this GPU (measured)"
-        else:
-            peak = SMS * FP32_LANES * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-            src = (f"FP32 FFMA: 152 SMs x 128 lanes x 2 flop x {peaks.get('sm_max_mhz', 2070.0):.0f} MHz "
-                   f"(nominal, {peak_src} max clock)")
-        roof = {"bound": "alu", "achieved": work / avg_s / 1e12, "peak": peak, "unit": "TFLOP/s",
-                "peak_source": src}
-        roof["frac"] = roof["achieved"] / roof["peak"]
-        roof["kernel"] = top[0]
-        roof["traffic"] = traffic_for(top[0], wl_name)
-        return roof
     bf16, src = tensor_peak(peaks, peak_src, ck, timed_ms)
     fp8 = prec == panda.PANDA_FP8MIX
     peak = 2.0 * bf16 if fp8 else bf16
@@ -280,6 +263,8 @@ def roofline(panda, prec, kstats, T, G, wl_name, peaks, peak_src, ck, timed_ms, 
         "issued_frac": issued_units_iter * iters_per_s / 1e12 / bf16,
         "note": "useful = 3TG^2 + 3T^2G flop per iteration; issued counts every MMA the split issues"}
     roof["hbm_peak_gbs"] = hbm
+    if prec == panda.PANDA_FP32:
+        roof["ffma_peak_tflops"] = ffma
     return roof
 
 

@@ -57,7 +57,8 @@ extern "C" {
  * carry 16 significant bits instead of 24; panda_get and panda_get_state
  * return hi + lo (exact in FP32) with the diagonal from its FP64 vector. */
 typedef enum {
-    PANDA_FP32 = 0,   /* FP32 FFMA products (SIMT) */
+    PANDA_FP32 = 0,   /* FP32 products on the tensor cores: x = h + m + l in BF16 exactly, the six part
+                         products down to 2^-16, summed in FP32 registers every 64 terms */
     PANDA_BF16X3 = 1, /* tensor cores: x = hi + lo in BF16, hi*hi + hi*lo + lo*hi, FP32 accumulation */
     PANDA_BF16X2 = 2, /* tensor cores: A operands split hi + lo, B operands BF16 hi only: hi*hi + lo*hi
                          (about 2^-9 relative error on each B entry; 2/3 of BF16X3's tensor work) */

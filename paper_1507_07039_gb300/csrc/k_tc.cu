@@ -1751,9 +1751,11 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
+}  // namespace
+
 // Row-major BF16 matrix rows x cols (cols = K, contiguous), box 64 x box_rows,
 // 128-byte swizzle.
-cudaError_t make_map(CUtensorMap *m, const void *base, int rows, int cols, int box_rows)
+cudaError_t tc_make_map(CUtensorMap *m, const void *base, int rows, int cols, int box_rows)
 {
     // box: 64 columns (128 B, the swizzle span) by box_rows rows
     auto fn = encode_fn();
@@ -1768,6 +1770,8 @@ cudaError_t make_map(CUtensorMap *m, const void *base, int rows, int cols, int b
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
+
+namespace {
 
 // 8-bit [rows][cols] array (E4M3 bytes), boxes of 128 bytes by box_rows rows
 cudaError_t make_map8(CUtensorMap *m, const void *base, int rows, int cols, int box_rows)
@@ -2159,7 +2163,7 @@ cudaError_t tc_prepare(Dev &d, cudaStream_t s, bool fresh_scales)
         TcMaps *m = &h->maps;
         std::memset(m, 0, sizeof *m);
         d.tc_host = h;
-        if ((e = make_map(&m->Ph, d.Ph, d.Tp, d.Tp, 128)) || (e = make_map(&m->Pl, d.Pl, d.Tp, d.Tp, 128)))
+        if ((e = tc_make_map(&m->Ph, d.Ph, d.Tp, d.Tp, 128)) || (e = tc_make_map(&m->Pl, d.Pl, d.Tp, d.Tp, 128)))
             return e;
         if (d.fp8) {
             if ((e = make_map8(&m->C8, d.C8, d.Gp, d.Gp, 128)))
@@ -2169,17 +2173,17 @@ cudaError_t tc_prepare(Dev &d, cudaStream_t s, bool fresh_scales)
                     (e = make_map8(&m->Wt8[b], d.Wt8[b], d.Gp, d.Tp, 128)))
                     return e;
         } else {
-            if ((e = make_map(&m->Ch, d.Ch, d.Gp, d.Gp, 128)) || (e = make_map(&m->Chm, d.Ch, d.Gp, d.Gp, 64)))
+            if ((e = tc_make_map(&m->Ch, d.Ch, d.Gp, d.Gp, 128)) || (e = tc_make_map(&m->Chm, d.Ch, d.Gp, d.Gp, 64)))
                 return e;
             if (d.split_b &&
-                ((e = make_map(&m->Cl, d.Cl, d.Gp, d.Gp, 128)) || (e = make_map(&m->Clm, d.Cl, d.Gp, d.Gp, 64))))
+                ((e = tc_make_map(&m->Cl, d.Cl, d.Gp, d.Gp, 128)) || (e = tc_make_map(&m->Clm, d.Cl, d.Gp, d.Gp, 64))))
                 return e;
         }
         for (int b = 0; b < 2; ++b)
-            if ((e = make_map(&m->Wh[b], d.Wh[b], d.Tp, d.Gp, 128)) ||
-                (e = make_map(&m->Wl[b], d.Wl[b], d.Tp, d.Gp, 128)) ||
-                (e = make_map(&m->Whm[b], d.Wh[b], d.Tp, d.Gp, 64)) ||
-                (e = make_map(&m->Wlm[b], d.Wl[b], d.Tp, d.Gp, 64)))
+            if ((e = tc_make_map(&m->Wh[b], d.Wh[b], d.Tp, d.Gp, 128)) ||
+                (e = tc_make_map(&m->Wl[b], d.Wl[b], d.Tp, d.Gp, 128)) ||
+                (e = tc_make_map(&m->Whm[b], d.Wh[b], d.Tp, d.Gp, 64)) ||
+                (e = tc_make_map(&m->Wlm[b], d.Wl[b], d.Tp, d.Gp, 64)))
                 return e;
         int dev = 0, nsm = 0;
         if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)))
@@ -2414,8 +2418,8 @@ cudaError_t tc_gram(const __nv_bfloat16 *Zh, const __nv_bfloat16 *Zl, int Gp, in
     if (e)
         return e;
     GemmMaps maps;
-    if ((e = make_map(&maps.Ah, Zh, Gp, Kp, 128)) || (e = make_map(&maps.Al, Zl, Gp, Kp, 128)) ||
-        (e = make_map(&maps.Bh, Zh, Gp, Kp, 128)) || (e = make_map(&maps.Bl, Zl, Gp, Kp, 128)))
+    if ((e = tc_make_map(&maps.Ah, Zh, Gp, Kp, 128)) || (e = tc_make_map(&maps.Al, Zl, Gp, Kp, 128)) ||
+        (e = tc_make_map(&maps.Bh, Zh, Gp, Kp, 128)) || (e = tc_make_map(&maps.Bl, Zl, Gp, Kp, 128)))
         return e;
     k_tc_gemm_pair<<<dim3(Gp / 128, Gp / PAIR_N), THREADS, pair_smem(), s>>>(maps, Kp, Gp, C, ctl, 0, 0);
     return cudaGetLastError();
@@ -2500,18 +2504,18 @@ cudaError_t tc_selftest_gemm(int M, int N, int K, const float *A, const float *B
         TRY(cudaMemset(Bl, 0, (size_t)Np * Kp * 2));
     }
     if (mn & 2) {
-        TRY(make_map(&maps.Ah, Ah, Kp, Mp, 64));
-        TRY(make_map(&maps.Al, Al, Kp, Mp, 64));
+        TRY(tc_make_map(&maps.Ah, Ah, Kp, Mp, 64));
+        TRY(tc_make_map(&maps.Al, Al, Kp, Mp, 64));
     } else {
-        TRY(make_map(&maps.Ah, Ah, Mp, Kp, 128));
-        TRY(make_map(&maps.Al, Al, Mp, Kp, 128));
+        TRY(tc_make_map(&maps.Ah, Ah, Mp, Kp, 128));
+        TRY(tc_make_map(&maps.Al, Al, Mp, Kp, 128));
     }
     if (mn & 1) {
-        TRY(make_map(&maps.Bh, Bh, Kp, Np, 64));
-        TRY(make_map(&maps.Bl, Bl, Kp, Np, 64));
+        TRY(tc_make_map(&maps.Bh, Bh, Kp, Np, 64));
+        TRY(tc_make_map(&maps.Bl, Bl, Kp, Np, 64));
     } else {
-        TRY(make_map(&maps.Bh, Bh, Np, Kp, 128));
-        TRY(make_map(&maps.Bl, Bl, Np, Kp, 128));
+        TRY(tc_make_map(&maps.Bh, Bh, Np, Kp, 128));
+        TRY(tc_make_map(&maps.Bl, Bl, Np, Kp, 128));
     }
     constexpr size_t st_smem = 1024 + 3 * (4 * A_BYTES) + sizeof(Sync<3>) + 16;
     if (pair)

@@ -135,7 +135,7 @@ int plan_memory(panda_ctx *c)
     d.c_split = (c->prec == PANDA_BF16X3 || c->prec == PANDA_BF16X2) ? 1 : 0;
     for (int b = 0; b < 2; ++b) {
         DALLOC(d.W[b], Tp * Gp);
-        if (!d.c_split)  // the FP32 path's operand, FP8MIX's source of its E4M3 transposes
+        if (d.fp8)  // the source of the E4M3 transposes
             DALLOC(d.Wt[b], Gp * Tp);
     }
     DALLOC(d.Poff, Tp * Tp);
@@ -149,17 +149,21 @@ int plan_memory(panda_ctx *c)
     DALLOC(d.csqC, Gp);
     DALLOC(d.rsqW, Tp);
     DALLOC(d.csqW, Gp);
-    if (c->prec == PANDA_FP32)
-        DALLOC(d.Rn, Tp * Gp);
     DALLOC(d.wrow_part, (size_t)c->nbG * Tp);
     DALLOC(d.wcol_part, (size_t)c->nbT * Gp);
     DALLOC(d.hpart, (size_t)c->nbT * c->nbG);
-    // partial-sum slots: one per 128-row block (FP32 path); on the tensor-core
-    // path one per 256-column block for the row role plus one per 128-row half
-    // for the column role (see k_tc.cu)
-    d.nsP = tensor_prec(c->prec) ? 3 * ceil_div(c->Tp, 256) : c->nbT;
-    d.nsC = tensor_prec(c->prec) ? 3 * ceil_div(c->Gp, 256) : c->nbG;
-    d.tri_slots = tensor_prec(c->prec) ? 1 : 0;
+    // partial-sum slots: one per 128-row block where tiles are 128 x 128 (FP32 networks too
+    // small for CTA pairs); with 256 x 256 tiles one per 256-column block for the row role plus
+    // one per 128-row half for the column role (see k_tc.cu)
+    int nsm = 0;
+    CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+    size_t f32_slots = 0, f32_fix = 0;
+    bool pair_tiles = true;
+    if (c->prec == PANDA_FP32)
+        f32_plan(d, nsm, &f32_slots, &f32_fix, &d.p1_cuts, &pair_tiles);
+    d.nsP = pair_tiles ? 3 * ceil_div(c->Tp, 256) : c->nbT;
+    d.nsC = pair_tiles ? 3 * ceil_div(c->Gp, 256) : c->nbG;
+    d.tri_slots = pair_tiles ? 1 : 0;
     DALLOC(d.ps_sum, (size_t)d.nsP * Tp);
     DALLOC(d.ps_sq, (size_t)d.nsP * Tp);
     DALLOC(d.ps_vsq, (size_t)d.nsP * Tp);
@@ -172,17 +176,28 @@ int plan_memory(panda_ctx *c)
     DALLOC(c->d_flags, 4);
     DALLOC(c->d_stats, 4);
     DALLOC(c->d_partials, 1024);
-    if (tensor_prec(c->prec)) {
-        for (int b = 0; b < 2; ++b) {
-            DALLOC(d.Wh[b], Tp * Gp);
-            DALLOC(d.Wl[b], Tp * Gp);
+    for (int b = 0; b < 2; ++b) {
+        DALLOC(d.Wh[b], Tp * Gp);
+        DALLOC(d.Wl[b], Tp * Gp);
+    }
+    DALLOC(d.Ph, Tp * Tp);
+    DALLOC(d.Pl, Tp * Tp);
+    if (c->prec == PANDA_FP32) {  // three-way splits, tile sums and the cut tiles' slots and counters
+        for (int b = 0; b < 2; ++b)
+            DALLOC(d.Wm[b], Tp * Gp);
+        DALLOC(d.Pm, Tp * Tp);
+        DALLOC(d.Ch, Gp * Gp);
+        DALLOC(d.Cm, Gp * Gp);
+        DALLOC(d.Cl, Gp * Gp);
+        DALLOC(d.p1_acc, f32_slots);
+        if (d.p1_cuts > 0) {
+            DALLOC(d.p1_fix, f32_fix);
+            DALLOC(d.p1_flag, (size_t)d.p1_cuts * 2);
         }
-        DALLOC(d.Ph, Tp * Tp);
-        DALLOC(d.Pl, Tp * Tp);
+    }
+    if (tensor_prec(c->prec)) {
         // running sums of the long products' K chunks: one 128 x 256 slot per CTA of the
         // persistent phase-1 and phase-2 launches (at most one CTA per SM)
-        int nsm = 0;
-        CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
         DALLOC(d.p1_acc, (size_t)nsm * 128 * 256);
         d.p1_cuts = tc_phase1_cuts(d);  // tiles cut between two pairs: a slot and a flag per CTA rank
         if (d.p1_cuts < 0)
@@ -320,6 +335,8 @@ int derive_state(panda_ctx *c, bool split_diag)
     CU(launch_row_norms(d.Coff, c->G, c->G, c->Gp, d.cd, d.csqC, c->stream));
     if (tensor_prec(c->prec))
         CU(tc_prepare(d, c->stream));
+    else
+        CU(f32_prepare(d, c->cur, c->stream));
     return 0;
 }
 
@@ -332,11 +349,11 @@ void drop_graphs(panda_ctx *c)
         }
 }
 
-int n_kernels(const panda_ctx *c) { return tensor_prec(c->prec) ? TC_KERNELS : SIMT_KERNELS; }
+int n_kernels(const panda_ctx *c) { return tensor_prec(c->prec) ? TC_KERNELS : F32_KERNELS; }
 
 const char *kernel_name(const panda_ctx *c, int i)
 {
-    return tensor_prec(c->prec) ? TC_KERNEL_NAMES[i] : SIMT_KERNEL_NAMES[i];
+    return tensor_prec(c->prec) ? TC_KERNEL_NAMES[i] : F32_KERNEL_NAMES[i];
 }
 
 // slot: which iteration of a graph (or chunk) this is, for the timing events
@@ -344,7 +361,7 @@ int launch_iteration(panda_ctx *c, int cur, int slot)
 {
     KernelEvents ke{c->prof ? c->ev.data() + (size_t)slot * (n_kernels(c) + 1) : nullptr, 0};
     cudaError_t e = tensor_prec(c->prec) ? launch_iteration_tc(c->d, cur, c->stream, ke)
-                                            : launch_iteration_simt(c->d, cur, c->stream, ke);
+                                            : launch_iteration_f32(c->d, cur, c->stream, ke);
     if (e != cudaSuccess)
         return set_err(c, PANDA_ECUDA, std::string("iteration launch: ") + cudaGetErrorString(e));
     return 0;
@@ -509,6 +526,7 @@ void free_all(panda_ctx *c)
     if (c->stream)
         cudaStreamSynchronize(c->stream);
     tc_release(c->d);
+    f32_release(c->d);
     if (c->c_stage)
         cudaFree(c->c_stage);
     c->c_stage = nullptr;
@@ -776,14 +794,12 @@ int panda_run(panda_ctx *c, float alpha, double tol, int max_iter, int *iters_ou
     return c->h_ctl->converged ? PANDA_OK : PANDA_NOT_CONVERGED;
 }
 
-// The tensor-core path keeps only the upper triangle of FP32 P and C current.
+// The iteration keeps only the upper triangle of FP32 P and C current.
 static int full_matrices(panda_ctx *c)
 {
-    if (tensor_prec(c->prec)) {
-        CU(launch_symmetrize(c->d.Poff, c->T, c->Tp, c->stream));
-        if (!c->d.c_split)
-            CU(launch_symmetrize(c->d.Coff, c->G, c->Gp, c->stream));
-    }
+    CU(launch_symmetrize(c->d.Poff, c->T, c->Tp, c->stream));
+    if (!c->d.c_split)
+        CU(launch_symmetrize(c->d.Coff, c->G, c->Gp, c->stream));
     return 0;
 }
 
@@ -1006,6 +1022,8 @@ int panda_load(panda_ctx *c, const void *buf, long long bytes)
     CU(launch_diag_to_float(d.cd, d.cdf, c->G, c->stream));
     if (tensor_prec(c->prec))
         CU(tc_prepare(d, c->stream, false));  // keep the saved E4M3 scales
+    else
+        CU(f32_prepare(d, c->cur, c->stream));
     c->h_ctl->iters = h.iters;
     c->h_ctl->active = 0;
     c->h_ctl->status = 0;

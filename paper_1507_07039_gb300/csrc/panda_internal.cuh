@@ -19,6 +19,7 @@
 // plus per-tile partial sums (scratch) and a small control block.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <cmath>
 #include <vector>
@@ -71,6 +72,9 @@ struct Dev {
     // BF16 split copies (tensor-core path only; NULL otherwise)
     __nv_bfloat16 *Wh[2], *Wl[2];  // W^T operands are read from these MN-major
     __nv_bfloat16 *Ph, *Pl, *Ch, *Cl;
+    // FP32 path: the middle parts of the three-way splits (h, m, l) of W, P_off and C_off
+    __nv_bfloat16 *Wm[2], *Pm, *Cm;
+    void *f32_host;              // host-side tensor maps and work lists (FP32 path)
     // 1: C is held only as its split pair Ch + Cl (BF16X3, BF16X2): its upper
     // triangle and diagonal 256-blocks are the state, Coff is NULL between
     // calls (a staging buffer while a create or set_state derives the state)
@@ -249,6 +253,22 @@ cudaError_t launch_iteration_tc(const Dev &d, int cur, cudaStream_t s, KernelEve
 // timed-out wait sets ST_TIMEOUT in ctl (device memory).
 cudaError_t tc_gram(const __nv_bfloat16 *Zh, const __nv_bfloat16 *Zl, int Gp, int Kp, float *C, Ctl *ctl,
                     cudaStream_t s);
+
+// Row-major BF16 matrix rows x cols as a tensor map: boxes of 64 columns (128
+// bytes, the swizzle span) by box_rows rows; what lies outside reads as zero.
+cudaError_t tc_make_map(CUtensorMap *m, const void *base, int rows, int cols, int box_rows);
+
+// ---- FP32 path (k_f32.cu) ----------------------------------------------------
+constexpr int F32_KERNELS = 5;
+extern const char *const F32_KERNEL_NAMES[F32_KERNELS];
+// The work lists of a network (Dev needs its sizes), kept in d.f32_host, and the
+// scratch they need: floats of the per-CTA slots and of the cut tiles' slots,
+// cut tiles (two counters each), the tile shape.
+void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fixes, bool *pair);
+// Split copies of the state in W[cur], Poff, Coff; tensor maps and device lists at the first call.
+cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s);
+void f32_release(Dev &d);
+cudaError_t launch_iteration_f32(const Dev &d, int cur, cudaStream_t s, KernelEvents &ke);
 
 struct TcSet;
 // Schedule candidates of the set engine's autotuner: phase 1 (the order of each
