@@ -185,9 +185,11 @@ int panda_info(const panda_ctx *ctx, int *T, int *G, int *prec, int *t);
 long long panda_device_bytes(const panda_ctx *ctx);
 
 /* The most device memory the context has held at once: under PANDA_BF16X3
- * and PANDA_BF16X2 a create or panda_set_state also stages C in FP32 (4 G^2
- * bytes, padded) while it derives the split state, and frees it before it
- * returns.  PANDA_ALLOC_LIMIT_BYTES caps this peak. */
+ * and PANDA_BF16X2 a create or panda_set_state from a host C also stages it in
+ * FP32 (4 G^2 bytes, padded) while it derives the split state, and frees it
+ * before it returns (a C in device memory is read where it lies, but a cap
+ * without room for the stage is refused all the same).
+ * PANDA_ALLOC_LIMIT_BYTES caps this peak. */
 long long panda_device_bytes_peak(const panda_ctx *ctx);
 
 /* Measurement support (the paper has no counterpart: it times the whole loop

@@ -1306,14 +1306,18 @@ void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fix
     *pair = p.pair;
 }
 
-cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s)
+int f32_diag_block(const Dev &d) { return static_cast<const F32Host *>(d.f32_host)->plan.pair ? 256 : 128; }
+
+cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
 {
     auto split = [&](const float *X, size_t n, __nv_bfloat16 *h, __nv_bfloat16 *m, __nv_bfloat16 *l) {
         k_split3<<<(int)std::min<size_t>(2432, (n / 4 + 255) / 256), 256, 0, s>>>(X, n / 4, h, m, l);
     };
-    split(d.W[cur], (size_t)d.Tp * d.Gp, d.Wh[cur], d.Wm[cur], d.Wl[cur]);
-    split(d.Poff, (size_t)d.Tp * d.Tp, d.Ph, d.Pm, d.Pl);
-    split(d.Coff, (size_t)d.Gp * d.Gp, d.Ch, d.Cm, d.Cl);
+    if (restored) {
+        split(d.W[cur], (size_t)d.Tp * d.Gp, d.Wh[cur], d.Wm[cur], d.Wl[cur]);
+        split(d.Poff, (size_t)d.Tp * d.Tp, d.Ph, d.Pm, d.Pl);
+        split(d.Coff, (size_t)d.Gp * d.Gp, d.Ch, d.Cm, d.Cl);
+    }
     cudaError_t e = cudaGetLastError();
     F32Host *h = static_cast<F32Host *>(d.f32_host);
     if (e || h->ready)

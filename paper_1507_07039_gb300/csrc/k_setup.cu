@@ -135,9 +135,19 @@ __device__ __forceinline__ void stats_term(float x, float mh, float ml, float &a
 // mean from stats (the difference kept as an FP32 pair, its square from
 // two_prod).  About as accurate as FP64 sums of the FP32 entries, on the FP32
 // pipe.
+// Rows that are not 16-byte aligned (a caller's array, read where it lies) are
+// read as scalars in the same groups and order: the same sums to the bit.
+__device__ __forceinline__ float4 load4(const float *x, int c4, bool aligned)
+{
+    if (aligned)
+        return __ldcs(reinterpret_cast<const float4 *>(x) + c4);
+    const float *p = x + 4 * (size_t)c4;
+    return make_float4(__ldcs(p), __ldcs(p + 1), __ldcs(p + 2), __ldcs(p + 3));
+}
+
 template <int MODE>
-__global__ void k_stats_partial(const float *__restrict__ X, int rows, int cols, int ld, const double *stats,
-                                double *partials)
+__global__ void k_stats_partial(const float *__restrict__ X, int rows, int cols, int ld, bool aligned,
+                                const double *stats, double *partials)
 {
     __shared__ double sh[RED_THREADS];
     float mh = 0.0f, ml = 0.0f;
@@ -150,11 +160,10 @@ __global__ void k_stats_partial(const float *__restrict__ X, int rows, int cols,
     double tot = 0.0;
     for (int r = blockIdx.x; r < rows; r += gridDim.x) {
         const float *x = X + (size_t)r * ld;
-        const float4 *x4 = reinterpret_cast<const float4 *>(x);
         float acc = 0.0f, cmp = 0.0f;
 #pragma unroll 2
         for (int c = threadIdx.x; c < c4n; c += RED_THREADS) {
-            const float4 v = __ldcs(x4 + c);
+            const float4 v = load4(x, c, aligned);
             stats_term<MODE>(v.x, mh, ml, acc, cmp);
             stats_term<MODE>(v.y, mh, ml, acc, cmp);
             stats_term<MODE>(v.z, mh, ml, acc, cmp);
@@ -210,28 +219,170 @@ __device__ __forceinline__ float zscore_one(float x, float4 q)
     return __fadd_rn(p, __fmaf_rn(t, q.z, __fmaf_rn(s, q.w, pe)));
 }
 
-// Block b takes rows b, b + gridDim.x, ...; 4-wide column groups, then the
-// ragged columns.
-__global__ void k_apply_zscore(float *X, int rows, int cols, int ld, const double *stats)
+// ---- a state from its networks ------------------------------------------------
+// One pass over each network where it lies (the caller's device array, or the
+// buffer it was copied into): entries checked, Z-scored on the way when `stats`
+// is given, and written in every form the iteration reads.  The former
+// sequence (copy into a padded FP32 matrix, check, Z-score in place, strip the
+// diagonal, split) passed over C six to ten times and staged it in a matrix of
+// its own: panda_set_state at 1000 x 17000 took 3.5 ms under BF16X3.
+
+// BF16 parts of four values (N = 2: hi, lo; 3: h, m, l), each the nearest to
+// what the ones before leave
+template <int N>
+__device__ __forceinline__ void parts4(const float (&v)[4], uint2 (&p)[N])
 {
-    if (!(stats[1] > 0.0))
-        return;
-    const float4 q = stats_pairs(stats);
-    const int c4n = cols >> 2;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        float *x = X + (size_t)r * ld;
-        float4 *x4 = reinterpret_cast<float4 *>(x);
-#pragma unroll 2
-        for (int c = threadIdx.x; c < c4n; c += blockDim.x) {
-            float4 v = x4[c];
-            v.x = zscore_one(v.x, q);
-            v.y = zscore_one(v.y, q);
-            v.z = zscore_one(v.z, q);
-            v.w = zscore_one(v.w, q);
-            x4[c] = v;
+    float x[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        uint32_t w[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            asm("cvt.rn.satfinite.bf16x2.f32 %0, %2, %1;" : "=r"(w[h]) : "f"(x[2 * h]), "f"(x[2 * h + 1]));
+            x[2 * h] -= __uint_as_float(w[h] << 16);
+            x[2 * h + 1] -= __uint_as_float(w[h] & 0xffff0000u);
         }
-        for (int c = (c4n << 2) + threadIdx.x; c < cols; c += blockDim.x)
-            x[c] = zscore_one(x[c], q);
+        p[q] = make_uint2(w[0], w[1]);
+    }
+}
+// four entries' parts at element offset o (a multiple of 4) of the parts that are held
+__device__ __forceinline__ void put_parts(const Parts &t, size_t o, const float (&v)[4])
+{
+    if (!t.h)
+        return;
+    if (t.m) {
+        uint2 p[3];
+        parts4<3>(v, p);
+        *reinterpret_cast<uint2 *>(t.h + o) = p[0];
+        *reinterpret_cast<uint2 *>(t.m + o) = p[1];
+        *reinterpret_cast<uint2 *>(t.l + o) = p[2];
+    } else {
+        uint2 p[2];
+        parts4<2>(v, p);
+        *reinterpret_cast<uint2 *>(t.h + o) = p[0];
+        *reinterpret_cast<uint2 *>(t.l + o) = p[1];
+    }
+}
+
+// W (rows x cols, row stride ldi) into out (row stride ldo, a multiple of 4) and
+// its parts; block y takes a row, 1024 columns per block.  X may be out itself.
+__global__ void k_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo, Parts parts,
+                         int *flags)
+{
+    const int r = blockIdx.y, c = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    int bad = 0;
+    if (c < cols) {
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u] = c + u < cols ? X[(size_t)r * ldi + c + u] : 0.0f;
+            bad |= !isfinite(v[u]);
+            if (stats && c + u < cols)
+                v[u] = zscore_one(v[u], stats_pairs(stats));
+        }
+        const size_t o = (size_t)r * ldo + c;
+        *reinterpret_cast<float4 *>(out + o) = make_float4(v[0], v[1], v[2], v[3]);
+        put_parts(parts, o, v);
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0)
+        atomicOr(&flags[0], 1);
+}
+
+// A symmetric n x n network (row stride ldi) as 64 x 64 blocks: each pair of
+// mirror blocks (bi, bj), (bj, bi), bi <= bj, is read once, along rows, into
+// shared memory.  flags as in k_check_finite_sym.  Written: block (bi, bj) of
+// out.F and of the parts, block (bj, bi) too where the form holds it; the
+// diagonal goes to out.d and out.df and reads as zero in F and the parts.  X
+// may be out.F itself (each block pair is one block's alone).  256 threads.
+constexpr int LB = 64;
+__global__ void __launch_bounds__(256) k_load_sym(const float *X, int n, int ldi, int npairs, const double *stats, SymOut out,
+                                                  int *flags)
+{
+    __shared__ float a[LB][LB + 1], b[LB][LB + 1];
+    const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // loads: 4 rows of 64
+    const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // stores: 16 rows of 16 x 4
+    int bad = 0, asym = 0;
+    for (int t = blockIdx.x; t < npairs; t += gridDim.x) {
+        // pairs are numbered column by column of the upper triangle; 8t + 1 < 2^24 for n <= 46000, so the
+        // FP32 square root is close; the loops correct it
+        int bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+        while (bj > 0 && bj * (bj + 1) / 2 > t)
+            --bj;
+        while ((bj + 1) * (bj + 2) / 2 <= t)
+            ++bj;
+        const int bi = t - bj * (bj + 1) / 2, i0 = bi * LB, j0 = bj * LB;
+        const bool diag = bi == bj;
+#pragma unroll
+        for (int k = 0; k < LB; k += 4) {
+            const int ra = i0 + k + ty, ca = j0 + tx;
+            a[k + ty][tx] = (ra < n && ca < n) ? X[(size_t)ra * ldi + ca] : 0.0f;
+        }
+        if (!diag) {
+#pragma unroll
+            for (int k = 0; k < LB; k += 4) {
+                const int rb = j0 + k + ty, cb = i0 + tx;
+                b[k + ty][tx] = (rb < n && cb < n) ? X[(size_t)rb * ldi + cb] : 0.0f;
+            }
+        }
+        __syncthreads();
+        const float(*m)[LB + 1] = diag ? a : b;
+        // rows of the upper block
+#pragma unroll
+        for (int k = 0; k < LB; k += 16) {
+            const int r = k + tr, gi = i0 + r;
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int gj = j0 + c4 + u;
+                v[u] = a[r][c4 + u];
+                bad |= !isfinite(v[u]) | !isfinite(m[r][c4 + u]);
+                asym |= v[u] != m[c4 + u][r];
+                if (stats && gi < n && gj < n)
+                    v[u] = zscore_one(v[u], stats_pairs(stats));
+                if (gi == gj && gi < n) {
+                    out.d[gi] = (double)v[u];
+                    out.df[gi] = v[u];
+                    v[u] = 0.0f;
+                }
+            }
+            if (gi < n && j0 + c4 < n) {
+                const size_t o = (size_t)gi * out.ld + j0 + c4;
+                if (out.F)
+                    *reinterpret_cast<float4 *>(out.F + o) = make_float4(v[0], v[1], v[2], v[3]);
+                put_parts(out.parts, o, v);
+            }
+        }
+        // rows of the lower block, from the upper one's columns
+        const bool lf = out.F && out.f_full, lp = out.parts.h && (out.p_full || i0 / out.p_block == j0 / out.p_block);
+        if (!diag && (lf || lp)) {
+#pragma unroll
+            for (int k = 0; k < LB; k += 16) {
+                const int r = k + tr, gj = j0 + r;
+                float v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    v[u] = a[c4 + u][r];
+                    if (stats && gj < n && i0 + c4 + u < n)
+                        v[u] = zscore_one(v[u], stats_pairs(stats));
+                }
+                if (gj < n && i0 + c4 < n) {
+                    const size_t o = (size_t)gj * out.ld + i0 + c4;
+                    if (lf)
+                        *reinterpret_cast<float4 *>(out.F + o) = make_float4(v[0], v[1], v[2], v[3]);
+                    if (lp)
+                        put_parts(out.parts, o, v);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    bad = __syncthreads_or(bad);
+    asym = __syncthreads_or(asym);
+    if (threadIdx.x == 0) {
+        if (bad)
+            atomicOr(&flags[0], 1);
+        if (asym)
+            atomicOr(&flags[1], 1);
     }
 }
 
@@ -276,11 +427,12 @@ __device__ __forceinline__ void sq_add(float x, float &acc, float &cmp)
     cmp = __fadd_rn(cmp, pe);
 }
 
-// out[i] = sum_j X[i][j]^2 (+ diag[i]^2): one warp per row, lane l taking the
-// 4-wide column groups l, l + 32, ... (rows start 16-byte aligned), then the
+// out[i] = sum_j X[i][j]^2, X Z-scored on the way when `stats` is given; with
+// `diag` the entry on the diagonal is left out and diag[i]^2 added: one warp
+// per row, lane l taking the 4-wide column groups l, l + 32, ..., then the
 // ragged columns.  Compensated FP32 pairs folded into an FP64 total every 16
 // groups, FP64 across the warp: a fixed order.
-__global__ void k_row_norms(const float *__restrict__ X, int rows, int cols, int ld,
+__global__ void k_row_norms(const float *__restrict__ X, int rows, int cols, int ld, bool aligned, const double *stats,
                             const double *diag, float *out)
 {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -288,26 +440,31 @@ __global__ void k_row_norms(const float *__restrict__ X, int rows, int cols, int
     if (warp >= rows)
         return;
     const float *x = X + (size_t)warp * ld;
-    const float4 *x4 = reinterpret_cast<const float4 *>(x);
-    const int c4n = cols >> 2;
+    const int c4n = cols >> 2, skip = diag ? warp : -1;
+    const float4 q = stats ? stats_pairs(stats) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    auto term = [&](float v, int c, float &acc, float &cmp) {
+        if (stats)
+            v = zscore_one(v, q);
+        sq_add(c == skip ? 0.0f : v, acc, cmp);
+    };
     double tot = 0.0;
     for (int c0 = 0; c0 < c4n; c0 += 16 * 32) {
         float acc = 0.0f, cmp = 0.0f;
         const int ce = min(c4n, c0 + 16 * 32);
 #pragma unroll 4
         for (int c = c0 + lane; c < ce; c += 32) {
-            const float4 v = x4[c];
-            sq_add(v.x, acc, cmp);
-            sq_add(v.y, acc, cmp);
-            sq_add(v.z, acc, cmp);
-            sq_add(v.w, acc, cmp);
+            const float4 v = load4(x, c, aligned);
+            term(v.x, 4 * c, acc, cmp);
+            term(v.y, 4 * c + 1, acc, cmp);
+            term(v.z, 4 * c + 2, acc, cmp);
+            term(v.w, 4 * c + 3, acc, cmp);
         }
         tot += (double)acc + (double)cmp;
     }
     {
         float acc = 0.0f, cmp = 0.0f;
         for (int c = (c4n << 2) + lane; c < cols; c += 32)
-            sq_add(x[c], acc, cmp);
+            term(x[c], c, acc, cmp);
         tot += (double)acc + (double)cmp;
     }
     for (int o = 16; o > 0; o >>= 1)
@@ -320,35 +477,31 @@ __global__ void k_row_norms(const float *__restrict__ X, int rows, int cols, int
 }
 
 // out[j] = sum_i X[i][j]^2 over the first `rows` rows: the squared column
-// norms of a row-major matrix without its transpose.  Thread j walks column
-// j down the rows (a warp's loads are 32 consecutive columns of one row),
-// compensated FP32 pairs folded into an FP64 total every 256 rows.
-__global__ void k_col_norms(const float *__restrict__ X, int rows, int cols, int ld, float *out)
+// norms of a row-major matrix without its transpose.  A block takes 32
+// columns, its eight warps every eighth row (compensated FP32 pairs folded
+// into FP64 every 32 of them), FP64 across the warps in a fixed order.
+__global__ void __launch_bounds__(256) k_col_norms(const float *__restrict__ X, int rows, int cols, int ld, float *out)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols)
-        return;
+    __shared__ double sh[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
     double tot = 0.0;
-    for (int r0 = 0; r0 < rows; r0 += 256) {
-        float acc = 0.0f, cmp = 0.0f;
-        const int re = min(rows, r0 + 256);
-#pragma unroll 4
-        for (int r = r0; r < re; ++r)
-            sq_add(X[(size_t)r * ld + j], acc, cmp);
-        tot += (double)acc + (double)cmp;
+    if (j < cols)
+        for (int r0 = w; r0 < rows; r0 += 256) {
+            float acc = 0.0f, cmp = 0.0f;
+            const int re = min(rows, r0 + 256);
+#pragma unroll 8
+            for (int r = r0; r < re; r += 8)
+                sq_add(X[(size_t)r * ld + j], acc, cmp);
+            tot += (double)acc + (double)cmp;
+        }
+    sh[w][lane] = tot;
+    __syncthreads();
+    if (w == 0 && j < cols) {
+        double t = 0.0;
+        for (int q = 0; q < 8; ++q)
+            t += sh[q][lane];
+        out[j] = (float)t;
     }
-    out[j] = (float)tot;
-}
-
-__global__ void k_scan_nonfinite(const float *__restrict__ X, long long n, int *flag)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    long long stride = (long long)gridDim.x * blockDim.x;
-    int bad = 0;
-    for (; i < n; i += stride)
-        bad |= !isfinite(X[i]);
-    if (__syncthreads_or(bad) && threadIdx.x == 0)
-        atomicOr(flag, 1);
 }
 
 // Lower triangle from the upper one: X[r][c] = X[c][r] for r > c (32 x 32
@@ -420,16 +573,59 @@ __global__ void k_standardize_rows(const float *__restrict__ X, int G, int N, __
     }
 }
 
-// out[r][c] = hi[r][c] + lo[r][c] for r <= c < n: the upper triangle of a
-// matrix held as a BF16 split pair (the sum is exact in FP32: lo's last bit is
-// no finer than the last bit of the FP32 value the pair was split from).
-__global__ void k_unsplit_upper(const __nv_bfloat16 *__restrict__ H, const __nv_bfloat16 *__restrict__ L, int n,
-                                int ldi, float *__restrict__ out, int ldo)
+// The full symmetric n x n matrix (row stride ldo, any alignment) from its
+// strict upper triangle, FP32 in X or a BF16 split pair H + L (exact in FP32;
+// row stride ldi, a multiple of 4), and its FP64 diagonal, in 64 x 64 blocks:
+// each block above the diagonal is read once and written twice, the second
+// time turned through shared memory.  256 threads.
+__global__ void __launch_bounds__(256) k_store_sym(const float *__restrict__ X, const __nv_bfloat16 *__restrict__ H,
+                                                   const __nv_bfloat16 *__restrict__ L, int n, int ldi, int npairs,
+                                                   const double *__restrict__ diag, float *__restrict__ out, int ldo)
 {
-    const int r = blockIdx.y;
-    for (int c = r + blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-        const size_t i = (size_t)r * ldi + c;
-        out[(size_t)r * ldo + c] = __bfloat162float(H[i]) + __bfloat162float(L[i]);
+    __shared__ float a[LB][LB + 1];
+    const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // stores: 4 rows of 64
+    const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // loads: 16 rows of 16 x 4
+    for (int t = blockIdx.x; t < npairs; t += gridDim.x) {
+        int bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);  // as in k_load_sym
+        while (bj > 0 && bj * (bj + 1) / 2 > t)
+            --bj;
+        while ((bj + 1) * (bj + 2) / 2 <= t)
+            ++bj;
+        const int bi = t - bj * (bj + 1) / 2, i0 = bi * LB, j0 = bj * LB;
+#pragma unroll
+        for (int k = 0; k < LB; k += 16) {
+            const int r = k + tr, gi = i0 + r, gj = j0 + c4;
+            float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            if (gi < n && gj < n) {  // (the padding up to the row stride is readable)
+                const size_t o = (size_t)gi * ldi + gj;
+                if (X) {
+                    const float4 f = *reinterpret_cast<const float4 *>(X + o);
+                    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+                } else {
+                    const uint2 h = *reinterpret_cast<const uint2 *>(H + o), l = *reinterpret_cast<const uint2 *>(L + o);
+                    v[0] = __uint_as_float(h.x << 16) + __uint_as_float(l.x << 16);
+                    v[1] = __uint_as_float(h.x & 0xffff0000u) + __uint_as_float(l.x & 0xffff0000u);
+                    v[2] = __uint_as_float(h.y << 16) + __uint_as_float(l.y << 16);
+                    v[3] = __uint_as_float(h.y & 0xffff0000u) + __uint_as_float(l.y & 0xffff0000u);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                a[r][c4 + u] = v[u];
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < LB; k += 4) {
+            const int r = k + ty;
+            if (i0 + r < n && j0 + tx < n) {
+                const bool up = bi < bj || r < tx;
+                out[(size_t)(i0 + r) * ldo + j0 + tx] =
+                    bi == bj && r == tx ? (float)diag[i0 + r] : (up ? a[r][tx] : a[tx][r]);
+            }
+            if (bi < bj && j0 + r < n && i0 + tx < n)
+                out[(size_t)(j0 + r) * ldo + i0 + tx] = a[tx][r];
+        }
+        __syncthreads();
     }
 }
 
@@ -456,14 +652,12 @@ cudaError_t launch_unit_diag(float *X, int n, int ld, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_unsplit_sym(const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi, float *out, int ldo,
-                              cudaStream_t s)
+cudaError_t launch_store_sym(const float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi,
+                             const double *diag, float *out, int ldo, cudaStream_t s)
 {
-    if (n <= 0)
-        return cudaSuccess;
-    k_unsplit_upper<<<dim3(ceil_div(n, 1024) < 8 ? ceil_div(n, 1024) : 8, n), 256, 0, s>>>(H, L, n, ldi, out, ldo);
-    cudaError_t e = cudaGetLastError();
-    return e ? e : launch_symmetrize(out, n, ldo, s);
+    const int nb = ceil_div(n, LB), npairs = nb * (nb + 1) / 2;
+    k_store_sym<<<npairs < 152 * 12 ? npairs : 152 * 12, 256, 0, s>>>(X, H, L, n, ldi, npairs, diag, out, ldo);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_symmetrize(float *X, int n, int ld, cudaStream_t s)
@@ -494,17 +688,30 @@ cudaError_t launch_check_finite_sym(const float *X, int rows, int cols, int ld, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_zscore(float *X, int rows, int cols, int ld, double *stats, double *partials,
-                          cudaStream_t s)
+cudaError_t launch_stats(const float *X, int rows, int cols, int ld, double *stats, double *partials, cudaStream_t s)
 {
-    if (!rows_aligned(X, ld) || ((uintptr_t)stats & 15))
+    if ((uintptr_t)stats & 15)
         return cudaErrorInvalidValue;
+    const bool al = rows_aligned(X, ld);
     double count = (double)rows * (double)cols;
-    k_stats_partial<0><<<RED_BLOCKS, RED_THREADS, 0, s>>>(X, rows, cols, ld, stats, partials);
+    k_stats_partial<0><<<RED_BLOCKS, RED_THREADS, 0, s>>>(X, rows, cols, ld, al, stats, partials);
     k_stats_final<<<1, RED_THREADS, 0, s>>>(partials, RED_BLOCKS, count, 0, stats);
-    k_stats_partial<1><<<RED_BLOCKS, RED_THREADS, 0, s>>>(X, rows, cols, ld, stats, partials);
+    k_stats_partial<1><<<RED_BLOCKS, RED_THREADS, 0, s>>>(X, rows, cols, ld, al, stats, partials);
     k_stats_final<<<1, RED_THREADS, 0, s>>>(partials, RED_BLOCKS, count, 1, stats);
-    k_apply_zscore<<<rows < 152 * 8 ? rows : 152 * 8, 256, 0, s>>>(X, rows, cols, ld, stats);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo,
+                          const Parts &parts, int *flags, cudaStream_t s)
+{
+    k_load_w<<<dim3(ceil_div(cols, 1024), rows), 256, 0, s>>>(X, rows, cols, ldi, stats, out, ldo, parts, flags);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags, cudaStream_t s)
+{
+    const int nb = ceil_div(n, LB), npairs = nb * (nb + 1) / 2;
+    k_load_sym<<<npairs < 152 * 6 ? npairs : 152 * 6, 256, 0, s>>>(X, n, ldi, npairs, stats, out, flags);
     return cudaGetLastError();
 }
 
@@ -527,24 +734,16 @@ cudaError_t launch_transpose(const float *X, int rows_p, int cols_p, float *Y, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_row_norms(const float *X, int rows, int cols, int ld, const double *diag,
+cudaError_t launch_row_norms(const float *X, int rows, int cols, int ld, const double *stats, const double *diag,
                              float *out, cudaStream_t s)
 {
-    if (!rows_aligned(X, ld))
-        return cudaErrorInvalidValue;
-    k_row_norms<<<ceil_div(rows * 32, 256), 256, 0, s>>>(X, rows, cols, ld, diag, out);
+    k_row_norms<<<ceil_div(rows * 32, 256), 256, 0, s>>>(X, rows, cols, ld, rows_aligned(X, ld), stats, diag, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_col_norms(const float *X, int rows, int cols, int ld, float *out, cudaStream_t s)
 {
-    k_col_norms<<<ceil_div(cols, 256), 256, 0, s>>>(X, rows, cols, ld, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_scan_nonfinite(const float *X, long long n, int *flag, cudaStream_t s)
-{
-    k_scan_nonfinite<<<1024, 256, 0, s>>>(X, n, flag);
+    k_col_norms<<<ceil_div(cols, 32), 256, 0, s>>>(X, rows, cols, ld, out);
     return cudaGetLastError();
 }
 

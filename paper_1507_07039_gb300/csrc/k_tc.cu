@@ -2135,26 +2135,22 @@ bool tc_supported()
     return major == 10 && minor == 3 && encode_fn() != nullptr;
 }
 
-cudaError_t tc_prepare(Dev &d, cudaStream_t s, bool fresh_scales)
+cudaError_t tc_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
 {
     cudaError_t e = set_smem_limits();
     if (e)
         return e;
     const size_t TG = (size_t)d.Tp * d.Gp;
-    // split copies of the current state (both W buffers get their maps; buffer 0 holds W now)
-    for (int b = 0; b < 2; ++b)
-        k_split<<<1024, 256, 0, s>>>(d.W[b], TG, d.Wh[b], d.Wl[b]);
-    k_split<<<1024, 256, 0, s>>>(d.Poff, (size_t)d.Tp * d.Tp, d.Ph, d.Pl);
+    if (restored) {  // (C's split pair is in the checkpoint)
+        k_split<<<1024, 256, 0, s>>>(d.W[cur], TG, d.Wh[cur], d.Wl[cur]);
+        k_split<<<1024, 256, 0, s>>>(d.Poff, (size_t)d.Tp * d.Tp, d.Ph, d.Pl);
+    }
     if (d.fp8) {  // scales from the state's norms (or as restored), then the E4M3 copies
-        if (fresh_scales)
+        if (!restored)
             k_fp8_init<<<1, 1024, 0, s>>>(d);
-        for (int b = 0; b < 2; ++b) {
-            k_to_e4m3<<<1024, 256, 0, s>>>(d.W[b], TG, d.W8[b], d.f8 + b);
-            k_to_e4m3<<<1024, 256, 0, s>>>(d.Wt[b], TG, d.Wt8[b], d.f8 + b);
-        }
+        k_to_e4m3<<<1024, 256, 0, s>>>(d.W[cur], TG, d.W8[cur], d.f8 + cur);
+        k_to_e4m3<<<1024, 256, 0, s>>>(d.Wt[cur], TG, d.Wt8[cur], d.f8 + cur);
         k_to_e4m3<<<2048, 256, 0, s>>>(d.Coff, (size_t)d.Gp * d.Gp, d.C8, d.f8 + 2);
-    } else if (d.Coff) {  // C's split pair from the FP32 C being derived (a restored pair is kept)
-        k_split<<<2048, 256, 0, s>>>(d.Coff, (size_t)d.Gp * d.Gp, d.Ch, (d.split_b || d.c_split) ? d.Cl : nullptr);
     }
     if ((e = cudaGetLastError()))
         return e;

@@ -174,7 +174,7 @@ int plan_memory(panda_ctx *c)
     DALLOC(d.hist, HIST_CAP);
     DALLOC(d.e2tab, HIST_CAP + 1);
     DALLOC(c->d_flags, 4);
-    DALLOC(c->d_stats, 4);
+    DALLOC(c->d_stats, 12);
     DALLOC(c->d_partials, 1024);
     for (int b = 0; b < 2; ++b) {
         DALLOC(d.Wh[b], Tp * Gp);
@@ -276,67 +276,94 @@ int download(panda_ctx *c, float *dst, const float *src, int ld, int rows, int c
     return 0;
 }
 
-// Validate the freshly uploaded networks: finite entries, exact symmetry.
-int validate(panda_ctx *c)
+// Whether p is device (or managed) memory.
+bool device_pointer(const void *p)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// The state in W[c->cur], P and C from the three networks (each host or device
+// memory; C's row stride ldc, 0: G): validated, Z-scored if `normalize`, every
+// derived vector and copy made.  A device network is read where it lies; a
+// host one is first copied to where its FP32 matrix lives (or, for a C held as
+// its split pair, into a staging buffer).  One wait at the end tells what the
+// checks found.
+int load_state(panda_ctx *c, const float *W, const float *P, const float *C, int ldc, bool normalize)
 {
     Dev &d = c->d;
-    int flags[4];
+    const int T = c->T, G = c->G;
+    int rc;
+    struct { const float *src; int ld; } w{W, G}, p{P, T}, x{C, ldc > 0 ? ldc : G};
+    if (!device_pointer(W)) {
+        if ((rc = upload(c, d.W[c->cur], c->Gp, W, T, G)))
+            return rc;
+        w = {d.W[c->cur], c->Gp};
+    }
+    if (!device_pointer(P)) {
+        if ((rc = upload(c, d.Poff, c->Tp, P, T, T)))
+            return rc;
+        p = {d.Poff, c->Tp};
+    }
+    if (!device_pointer(C)) {
+        if ((rc = stage_c(c)) || (rc = upload(c, d.Coff, c->Gp, C, G, G, x.ld)))
+            return rc;
+        x = {d.Coff, c->Gp};
+    } else if (d.c_split && c->limit >= 0 && c->bytes + 4LL * c->Gp * c->Gp > c->limit) {
+        // (a cap that leaves no room for staging C is refused whether or not this call stages it)
+        return set_err(c, PANDA_ENOMEM, "device memory plan exceeds PANDA_ALLOC_LIMIT_BYTES");
+    }
+    const double *st[3] = {nullptr, nullptr, nullptr};
+    if (normalize) {
+        for (int q = 0; q < 3; ++q)
+            st[q] = c->d_stats + 4 * q;
+        CU(launch_stats(w.src, T, G, w.ld, c->d_stats, c->d_partials, c->stream));
+        CU(launch_stats(p.src, T, T, p.ld, c->d_stats + 4, c->d_partials, c->stream));
+        CU(launch_stats(x.src, G, G, x.ld, c->d_stats + 8, c->d_partials, c->stream));
+    }
+    const bool f32 = c->prec == PANDA_FP32;
     CU(cudaMemsetAsync(c->d_flags, 0, 4 * sizeof(int), c->stream));
-    CU(launch_check_finite_sym(d.W[c->cur], c->T, c->G, c->Gp, false, c->d_flags, c->stream));
-    CU(launch_check_finite_sym(d.Poff, c->T, c->T, c->Tp, true, c->d_flags, c->stream));
-    CU(launch_check_finite_sym(d.Coff, c->G, c->G, c->Gp, true, c->d_flags, c->stream));
-    CU(cudaMemcpyAsync(flags, c->d_flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CU(launch_load_w(w.src, T, G, w.ld, st[0], d.W[c->cur], c->Gp, Parts{d.Wh[c->cur], d.Wm[c->cur], d.Wl[c->cur]},
+                     c->d_flags, c->stream));
+    // a network loaded in place keeps both triangles, for the norms below; FP8MIX's E4M3 copy of C is made from both
+    const SymOut po{d.Poff, p.src == d.Poff, Parts{d.Ph, d.Pm, d.Pl}, 1, 256, c->Tp, d.pd, d.pdf};
+    const SymOut xo{d.c_split ? nullptr : d.Coff, d.fp8 || x.src == d.Coff,
+                    Parts{d.Ch, d.Cm, d.Cl}, 0, f32 ? f32_diag_block(d) : 256, c->Gp, d.cd, d.cdf};
+    CU(launch_load_sym(p.src, T, p.ld, st[1], po, c->d_flags, c->stream));
+    CU(launch_load_sym(x.src, G, x.ld, st[2], xo, c->d_flags, c->stream));
+    CU(launch_row_norms(d.W[c->cur], T, G, c->Gp, nullptr, nullptr, d.rsqW, c->stream));
+    if (d.Wt[c->cur])
+        CU(launch_transpose(d.W[c->cur], c->Tp, c->Gp, d.Wt[c->cur], c->stream));
+    CU(launch_col_norms(d.W[c->cur], T, G, c->Gp, d.csqW, c->stream));
+    // from the same entries as loaded: in place they are Z-scored by now
+    CU(launch_row_norms(p.src, T, T, p.ld, p.src == d.Poff ? nullptr : st[1], d.pd, d.rsqP, c->stream));
+    CU(launch_row_norms(x.src, G, G, x.ld, xo.F && x.src == xo.F ? nullptr : st[2], d.cd, d.csqC, c->stream));
+    if (tensor_prec(c->prec))
+        CU(tc_prepare(d, c->cur, c->stream, false));
+    else
+        CU(f32_prepare(d, c->cur, c->stream, false));
+    int flags[4];
+    double stats[12];
+    CU(cudaMemcpyAsync(flags, c->d_flags, sizeof flags, cudaMemcpyDeviceToHost, c->stream));
+    if (normalize)
+        CU(cudaMemcpyAsync(stats, c->d_stats, sizeof stats, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
     if (flags[0])
         return set_err(c, PANDA_ENONFINITE, "an input network has a non-finite entry");
     if (flags[1])
         return set_err(c, PANDA_EASYM, "P0 or C0 is not exactly symmetric");
-    return 0;
-}
-
-int zscore_all(panda_ctx *c)
-{
-    Dev &d = c->d;
-    struct { float *X; int rows, cols, ld; const char *name; } nets[3] = {
-        {d.W[c->cur], c->T, c->G, c->Gp, "W0"},
-        {d.Poff, c->T, c->T, c->Tp, "P0"},
-        {d.Coff, c->G, c->G, c->Gp, "C0"}};
-    for (auto &n : nets) {
-        double st[2];
-        CU(launch_zscore(n.X, n.rows, n.cols, n.ld, c->d_stats, c->d_partials, c->stream));
-        CU(cudaMemcpyAsync(st, c->d_stats, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        CU(cudaStreamSynchronize(c->stream));
-        if (!(st[1] > 0.0))
+    const char *names[3] = {"W0", "P0", "C0"};
+    for (int q = 0; normalize && q < 3; ++q) {
+        if (!(stats[4 * q + 1] > 0.0))
             return set_err(c, PANDA_EDEGENERATE,
-                           std::string(n.name) + " has zero standard deviation; its Z-score is undefined");
-        if (!std::isfinite(st[0]) || !std::isfinite(st[1]))
-            return set_err(c, PANDA_ENONFINITE, std::string(n.name) + " statistics are not finite");
+                           std::string(names[q]) + " has zero standard deviation; its Z-score is undefined");
+        if (!std::isfinite(stats[4 * q]) || !std::isfinite(stats[4 * q + 1]))
+            return set_err(c, PANDA_ENONFINITE, std::string(names[q]) + " statistics are not finite");
     }
-    return 0;
-}
-
-// From full W (in W[cur]), P and C (diagonals in place): strip diagonals,
-// transposed W, squared norms, split copies.
-int derive_state(panda_ctx *c, bool split_diag)
-{
-    Dev &d = c->d;
-    if (split_diag) {
-        CU(launch_split_diag(d.Poff, c->T, c->Tp, d.pd, d.pdf, c->stream));
-        CU(launch_split_diag(d.Coff, c->G, c->Gp, d.cd, d.cdf, c->stream));
-    }
-    CU(launch_row_norms(d.W[c->cur], c->T, c->G, c->Gp, nullptr, d.rsqW, c->stream));
-    if (d.Wt[c->cur]) {
-        CU(launch_transpose(d.W[c->cur], c->Tp, c->Gp, d.Wt[c->cur], c->stream));
-        CU(launch_row_norms(d.Wt[c->cur], c->G, c->T, c->Tp, nullptr, d.csqW, c->stream));  // columns of W
-    } else {
-        CU(launch_col_norms(d.W[c->cur], c->T, c->G, c->Gp, d.csqW, c->stream));
-    }
-    CU(launch_row_norms(d.Poff, c->T, c->T, c->Tp, d.pd, d.rsqP, c->stream));
-    CU(launch_row_norms(d.Coff, c->G, c->G, c->Gp, d.cd, d.csqC, c->stream));
-    if (tensor_prec(c->prec))
-        CU(tc_prepare(d, c->stream));
-    else
-        CU(f32_prepare(d, c->cur, c->stream));
     return 0;
 }
 
@@ -612,16 +639,8 @@ int create_common(panda_ctx **out, int T, int G, const float *W0, const float *P
             c->err = std::string("cudaEventCreate: ") + cudaGetErrorString(e);
             return fail(PANDA_ECUDA);
         }
-    if ((rc = plan_memory(c)) || (rc = stage_c(c)))
-        return fail(rc);
-    if ((rc = upload(c, c->d.W[0], c->Gp, W0, T, G)) || (rc = upload(c, c->d.Poff, c->Tp, P0, T, T)) ||
-        (rc = upload(c, c->d.Coff, c->Gp, C0, G, G, ldc)))
-        return fail(rc);
-    if ((rc = validate(c)))
-        return fail(rc);
-    if (c->normalize && (rc = zscore_all(c)))
-        return fail(rc);
-    if ((rc = derive_state(c, true)) || (rc = push_ctl(c)) || (rc = unstage_c(c)))
+    if ((rc = plan_memory(c)) || (rc = load_state(c, W0, P0, C0, ldc, c->normalize != 0)) || (rc = push_ctl(c)) ||
+        (rc = unstage_c(c)))
         return fail(rc);
     e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -803,36 +822,37 @@ static int full_matrices(panda_ctx *c)
     return 0;
 }
 
-// Whether p is device (or managed) memory of the current device.
-static bool device_pointer(const void *p)
+// Network X (P or C) into dst (n x n, dense).  Device memory: one kernel mirrors
+// the upper triangle, puts the diagonal in and writes dst.  Host memory: a C held
+// as its split pair the same way through a temporary device buffer; an FP32
+// matrix is mirrored where it is and copied, its diagonal put in on the host.
+static int get_sym(panda_ctx *c, float *dst, float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, const double *diag,
+                   int n, int ld)
 {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
-}
-
-// C (G x G, dense, host or device) from its split pair: straight into device
-// memory, through a temporary device buffer into host memory.
-static int get_split_c(panda_ctx *c, float *C)
-{
-    Dev &d = c->d;
-    const int G = c->G;
-    if (device_pointer(C)) {
-        CU(launch_unsplit_sym(d.Ch, d.Cl, G, c->Gp, C, G, c->stream));
+    if (device_pointer(dst)) {
+        CU(launch_store_sym(X, H, L, n, ld, diag, dst, n, c->stream));
         return 0;
     }
-    float *tmp = nullptr;
-    CU(cudaMalloc(&tmp, sizeof(float) * (size_t)G * G));
-    cudaError_t e = launch_unsplit_sym(d.Ch, d.Cl, G, c->Gp, tmp, G, c->stream);
-    if (!e)
-        e = cudaMemcpyAsync(C, tmp, sizeof(float) * (size_t)G * G, cudaMemcpyDeviceToHost, c->stream);
-    if (!e)
-        e = cudaStreamSynchronize(c->stream);
-    cudaFree(tmp);
-    CU(e);
+    if (!X) {
+        float *tmp = nullptr;
+        CU(cudaMalloc(&tmp, sizeof(float) * (size_t)n * n));
+        cudaError_t e = launch_store_sym(X, H, L, n, ld, diag, tmp, n, c->stream);
+        if (!e)
+            e = cudaMemcpyAsync(dst, tmp, sizeof(float) * (size_t)n * n, cudaMemcpyDeviceToHost, c->stream);
+        if (!e)
+            e = cudaStreamSynchronize(c->stream);
+        cudaFree(tmp);
+        CU(e);
+        return 0;
+    }
+    CU(launch_symmetrize(X, n, ld, c->stream));
+    if (int rc = download(c, dst, X, ld, n, n))
+        return rc;
+    std::vector<double> dg(n);
+    CU(cudaMemcpyAsync(dg.data(), diag, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaStreamSynchronize(c->stream));
+    for (int i = 0; i < n; ++i)
+        dst[(size_t)i * (n + 1)] = (float)dg[i];
     return 0;
 }
 
@@ -841,32 +861,13 @@ static int get_impl(panda_ctx *c, float *W, float *P, float *C)
     if (int rc = check_state(c))
         return rc;
     Dev &d = c->d;
-    if ((P || C) && full_matrices(c))
-        return PANDA_ECUDA;
-    if (W) {
-        int rc = download(c, W, d.W[c->cur], c->Gp, c->T, c->G);
-        if (rc)
-            return rc;
-    }
-    struct { float *dst; const float *src; const double *diag; int n, ld; } nets[2] = {
-        {P, d.Poff, d.pd, c->T, c->Tp}, {C, d.Coff, d.cd, c->G, c->Gp}};
-    for (auto &n : nets) {
-        if (!n.dst)
-            continue;
-        int rc = (n.dst == C && d.c_split) ? get_split_c(c, C) : download(c, n.dst, n.src, n.ld, n.n, n.n);
-        if (rc)
-            return rc;
-        // diagonal entries, rounded from the FP64 diagonal
-        std::vector<double> dg(n.n);
-        CU(cudaMemcpyAsync(dg.data(), n.diag, n.n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        CU(cudaStreamSynchronize(c->stream));
-        std::vector<float> f(n.n);
-        for (int i = 0; i < n.n; ++i)
-            f[i] = (float)dg[i];
-        CU(cudaMemcpy2DAsync(n.dst, (size_t)(n.n + 1) * sizeof(float), f.data(), sizeof(float),
-                             sizeof(float), n.n, cudaMemcpyDefault, c->stream));
-        CU(cudaStreamSynchronize(c->stream));  // f is released at the end of this scope
-    }
+    int rc = 0;
+    if (W && (rc = download(c, W, d.W[c->cur], c->Gp, c->T, c->G)))
+        return rc;
+    if (P && (rc = get_sym(c, P, d.Poff, nullptr, nullptr, d.pd, c->T, c->Tp)))
+        return rc;
+    if (C && (rc = get_sym(c, C, d.c_split ? nullptr : d.Coff, d.Ch, d.Cl, d.cd, c->G, c->Gp)))
+        return rc;
     CU(cudaStreamSynchronize(c->stream));
     return 0;
 }
@@ -903,14 +904,10 @@ int panda_set_state(panda_ctx *c, const float *W, const float *P, const float *C
     if (!W || !P || !C || t < 0 || t >= HIST_CAP)
         return set_err(c, PANDA_EINVAL, "W, P, C must be non-NULL and 0 <= t < 65536");
     drop_graphs(c);
-    Dev &d = c->d;
     c->cur = 0;
     c->state_ok = false;  // until the new networks are in, validated and their vectors derived
     int rc;
-    if ((rc = stage_c(c)))
-        return rc;
-    if ((rc = upload(c, d.W[0], c->Gp, W, c->T, c->G)) || (rc = upload(c, d.Poff, c->Tp, P, c->T, c->T)) ||
-        (rc = upload(c, d.Coff, c->Gp, C, c->G, c->G)) || (rc = validate(c)) || (rc = derive_state(c, true))) {
+    if ((rc = load_state(c, W, P, C, 0, false))) {
         unstage_c(c);
         return rc;
     }
@@ -1021,9 +1018,9 @@ int panda_load(panda_ctx *c, const void *buf, long long bytes)
     CU(launch_diag_to_float(d.pd, d.pdf, c->T, c->stream));
     CU(launch_diag_to_float(d.cd, d.cdf, c->G, c->stream));
     if (tensor_prec(c->prec))
-        CU(tc_prepare(d, c->stream, false));  // keep the saved E4M3 scales
+        CU(tc_prepare(d, c->cur, c->stream, true));  // keep the saved E4M3 scales
     else
-        CU(f32_prepare(d, c->cur, c->stream));
+        CU(f32_prepare(d, c->cur, c->stream, true));
     c->h_ctl->iters = h.iters;
     c->h_ctl->active = 0;
     c->h_ctl->status = 0;

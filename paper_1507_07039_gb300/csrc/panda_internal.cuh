@@ -171,23 +171,46 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e)
 // ---- launchers (k_setup.cu) ------------------------------------------------
 cudaError_t launch_check_finite_sym(const float *X, int rows, int cols, int ld, bool sym,
                                     int *flags, cudaStream_t s);
-cudaError_t launch_zscore(float *X, int rows, int cols, int ld, double *stats, double *partials,
-                          cudaStream_t s);
+// Z-score statistics of X (read only): stats[0] = mean, stats[1] = population std, then the
+// FP32 pairs that the loads below apply; 4 doubles, 16-byte aligned
+cudaError_t launch_stats(const float *X, int rows, int cols, int ld, double *stats, double *partials, cudaStream_t s);
+// BF16 parts of a matrix: h, l (two-way split) or h, m, l (three-way, exact); h NULL: none
+struct Parts {
+    __nv_bfloat16 *h, *m, *l;
+};
+// What a symmetric network becomes: its FP32 matrix F (NULL: not held) with a zero diagonal,
+// both triangles if f_full, else the upper one and the diagonal 64-blocks; its parts, both
+// triangles if p_full, else the upper one and the diagonal blocks of p_block; its diagonal.
+struct SymOut {
+    float *F;
+    int f_full;
+    Parts parts;
+    int p_full, p_block;
+    int ld;  // row stride of F and the parts
+    double *d;
+    float *df;
+};
+// X (device memory, any alignment, row stride ldi) checked (flags[0] |= 1: a non-finite entry,
+// flags[1] |= 1: not symmetric), Z-scored when stats is not NULL, and written in those forms
+cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo,
+                          const Parts &parts, int *flags, cudaStream_t s);
+cudaError_t launch_load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags,
+                            cudaStream_t s);
 cudaError_t launch_split_diag(float *X, int n, int ld, double *d, float *df, cudaStream_t s);
 cudaError_t launch_transpose(const float *X, int rows_p, int cols_p, float *Y, cudaStream_t s);
 // out[j] = sum over the first `rows` rows of X[i][j]^2 (squared column norms, no transpose)
 cudaError_t launch_col_norms(const float *X, int rows, int cols, int ld, float *out, cudaStream_t s);
-cudaError_t launch_row_norms(const float *X, int rows, int cols, int ld, const double *diag,
+// out[i] = sum_j X[i][j]^2, X Z-scored by stats (NULL: as it is); with diag (not NULL) the
+// diagonal entry left out and diag[i]^2 added
+cudaError_t launch_row_norms(const float *X, int rows, int cols, int ld, const double *stats, const double *diag,
                              float *out, cudaStream_t s);
 cudaError_t launch_diag_to_float(const double *d, float *df, int n, cudaStream_t s);
-cudaError_t launch_scan_nonfinite(const float *X, long long n, int *flag, cudaStream_t s);
 // X[r][c] = X[c][r] for r > c: the full matrix from its upper triangle
 cudaError_t launch_symmetrize(float *X, int n, int ld, cudaStream_t s);
-// out (n x n, row stride ldo) = the symmetric matrix whose upper triangle is
-// held as the BF16 split pair H + L (row stride ldi); diagonal entries are
-// H + L too (callers put the FP64 diagonal in place afterwards)
-cudaError_t launch_unsplit_sym(const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi, float *out, int ldo,
-                              cudaStream_t s);
+// out (n x n, row stride ldo) = the symmetric matrix with this strict upper triangle (FP32 X, or
+// X NULL and the BF16 split pair H + L; row stride ldi) and this diagonal
+cudaError_t launch_store_sym(const float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi,
+                             const double *diag, float *out, int ldo, cudaStream_t s);
 // Pearson initialisation (Sec. II-A): unit-norm centred rows of X (G x N) as a
 // BF16 split [G][Kp]; flags[0] |= 1 (non-finite) / 2 (zero variance)
 cudaError_t launch_standardize_rows(const float *X, int G, int N, __nv_bfloat16 *Zh, __nv_bfloat16 *Zl, int Kp,
@@ -227,8 +250,10 @@ cudaError_t measure_ffma_peak(double *tflops);
 constexpr int TC_KERNELS = 5;
 extern const char *const TC_KERNEL_NAMES[TC_KERNELS];
 bool tc_supported();
-// fresh_scales: derive the FP8MIX scales from the state's norms (false: keep those restored)
-cudaError_t tc_prepare(Dev &d, cudaStream_t s, bool fresh_scales = true);  // split copies of the state, tensor maps
+// Tensor maps and schedules (at the first call) and FP8MIX's E4M3 copies of the state in W[cur],
+// Coff.  restored: the state came back from a checkpoint, so its BF16 split copies are made here
+// too and the FP8MIX scales are kept; else the scales are derived from the state's norms.
+cudaError_t tc_prepare(Dev &d, int cur, cudaStream_t s, bool restored);
 void tc_release(Dev &d);
 // Tiles of one network's phase 1 cut between two CTA pairs (each needs a
 // running-sum slot per CTA rank and a flag per rank); -1 on a CUDA error.
@@ -265,8 +290,10 @@ extern const char *const F32_KERNEL_NAMES[F32_KERNELS];
 // scratch they need: floats of the per-CTA slots and of the cut tiles' slots,
 // cut tiles (two counters each), the tile shape.
 void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fixes, bool *pair);
-// Split copies of the state in W[cur], Poff, Coff; tensor maps and device lists at the first call.
-cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s);
+// Tensor maps and device lists at the first call; restored: also the split copies of W[cur], Poff, Coff.
+cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s, bool restored);
+// Edge of the diagonal blocks inside which phase 2 keeps both triangles of C's split copy.
+int f32_diag_block(const Dev &d);
 void f32_release(Dev &d);
 cudaError_t launch_iteration_f32(const Dev &d, int cur, cudaStream_t s, KernelEvents &ke);
 
