@@ -1294,11 +1294,13 @@ const char *const F32_KERNEL_NAMES[F32_KERNELS] = {"k_f32_phase1", "k_reduce_wno
 
 void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fixes, bool *pair)
 {
-    F32Host *h = new F32Host;
-    d.f32_host = h;
-    h->plan = f32_plan_for(d, nsm);
+    F32Host *h = static_cast<F32Host *>(d.f32_host);
+    if (!h) {
+        d.f32_host = h = new F32Host;
+        h->plan = f32_plan_for(d, nsm);
+        h->workers = h->plan.pair ? nsm / 2 : nsm;
+    }
     const F32Plan &p = h->plan;
-    h->workers = p.pair ? nsm / 2 : nsm;
     const size_t slot = p.pair ? Tile<true>::SLOT : Tile<false>::SLOT, ranks = p.pair ? 2 : 1;
     *slot_floats = slot * ranks * (size_t)h->workers;
     *fix_floats = slot * ranks * (size_t)std::max(p.p1.slots, p.p2.slots);

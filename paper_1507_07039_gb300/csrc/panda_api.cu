@@ -30,11 +30,15 @@ struct panda_ctx {
     bool state_ok = true;
     Dev d{};
     Ctl *h_ctl = nullptr;  // pinned mirror of the device control block
-    std::vector<void *> allocs;
+    // one allocation for everything the context holds: sized by a first pass over the memory plan
+    // (arena NULL), carved by a second
+    char *arena = nullptr;
+    size_t arena_used = 0;
     long long bytes = 0;       // device memory held between calls
     long long peak = 0;        // the most held at once (staging buffers included)
     long long limit = -1;
     float *c_stage = nullptr;  // FP32 C while a create or set_state derives a split-held state
+    int e2_filled = 0;       // entries of d.e2tab that hold e^{2 alpha t} for e2_alpha
     float e2_alpha = -1.0f;  // alpha for which d.e2tab is filled
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     int *d_flags = nullptr;
@@ -99,19 +103,10 @@ int dalloc(panda_ctx *c, T **p, size_t count)
         *p = nullptr;
         return set_err(c, PANDA_ENOMEM, "device memory plan exceeds PANDA_ALLOC_LIMIT_BYTES");
     }
-    void *q = nullptr;
-    cudaError_t e = cudaMalloc(&q, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        *p = nullptr;
-        return set_err(c, PANDA_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    }
-    c->allocs.push_back(q);
     c->bytes += (long long)bytes;
     c->peak = c->bytes > c->peak ? c->bytes : c->peak;
-    e = cudaMemsetAsync(q, 0, bytes, c->stream);
-    if (e != cudaSuccess)
-        return set_err(c, PANDA_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+    void *q = c->arena ? c->arena + c->arena_used : nullptr;
+    c->arena_used += (bytes + 511) & ~size_t(511);
     *p = static_cast<T *>(q);
     return 0;
 }
@@ -123,6 +118,8 @@ int dalloc(panda_ctx *c, T **p, size_t count)
             return r_;                     \
     } while (0)
 
+// The context's device arrays.  Called twice by alloc_plan: first without an
+// arena, to add up the sizes (and check them against the cap), then to carve it.
 int plan_memory(panda_ctx *c)
 {
     Dev &d = c->d;
@@ -160,7 +157,7 @@ int plan_memory(panda_ctx *c)
     size_t f32_slots = 0, f32_fix = 0;
     bool pair_tiles = true;
     if (c->prec == PANDA_FP32)
-        f32_plan(d, nsm, &f32_slots, &f32_fix, &d.p1_cuts, &pair_tiles);
+        f32_plan(d, nsm, &f32_slots, &f32_fix, &d.p1_cuts, &pair_tiles);  // (computed at the first call)
     d.nsP = pair_tiles ? 3 * ceil_div(c->Tp, 256) : c->nbT;
     d.nsC = pair_tiles ? 3 * ceil_div(c->Gp, 256) : c->nbG;
     d.tri_slots = pair_tiles ? 1 : 0;
@@ -222,10 +219,30 @@ int plan_memory(panda_ctx *c)
     return 0;
 }
 
-// A split-held C (d.c_split) is derived from an FP32 copy: stage_c gives Coff
-// a zeroed Gp x Gp FP32 buffer for that (within PANDA_ALLOC_LIMIT_BYTES,
-// counted in the peak, not in the memory held between calls), unstage_c frees
-// it once the split pair is written.
+// One cudaMalloc and one memset: each of the forty or so arrays on its own
+// cost a create and its destroy milliseconds (cudaFree waits for the device).
+int alloc_plan(panda_ctx *c)
+{
+    int rc = plan_memory(c);
+    if (rc)
+        return rc;
+    void *q = nullptr;
+    cudaError_t e = cudaMalloc(&q, c->arena_used);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return set_err(c, PANDA_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
+    c->arena = static_cast<char *>(q);
+    CU(cudaMemsetAsync(q, 0, c->arena_used, c->stream));
+    c->arena_used = 0;
+    c->bytes = 0;
+    return plan_memory(c);
+}
+
+// A host C that is to be held as its split pair is first copied to a staging
+// buffer: stage_c gives Coff a Gp x Gp FP32 buffer for that (within
+// PANDA_ALLOC_LIMIT_BYTES, counted in the peak, not in the memory held between
+// calls), unstage_c frees it once the split pair is written.
 int stage_c(panda_ctx *c)
 {
     Dev &d = c->d;
@@ -237,7 +254,6 @@ int stage_c(panda_ctx *c)
     CU(cudaMalloc(&c->c_stage, bytes));
     const long long held = c->bytes + (long long)bytes;
     c->peak = held > c->peak ? held : c->peak;
-    CU(cudaMemsetAsync(c->c_stage, 0, bytes, c->stream));
     d.Coff = c->c_stage;
     return 0;
 }
@@ -420,17 +436,23 @@ int ensure_graph(panda_ctx *c, int cur)
     return 0;
 }
 
-int fill_e2(panda_ctx *c, float alpha)
+// e^{2 alpha t} of Eq. 6 for t = 0 .. upto (FP64, computed on the host; 256
+// entries at least, then doubling: all 65537 took a first run 0.8 ms)
+int fill_e2(panda_ctx *c, float alpha, int upto)
 {
-    if (c->e2_alpha == alpha)
-        return 0;
-    std::vector<double> tab(HIST_CAP + 1);
-    for (int t = 0; t <= HIST_CAP; ++t)
-        tab[t] = std::exp(2.0 * (double)alpha * (double)t);  // e^{2 alpha t} of Eq. 6
-    CU(cudaMemcpyAsync(c->d.e2tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice,
-                       c->stream));
-    CU(cudaStreamSynchronize(c->stream));
+    if (c->e2_alpha != alpha)
+        c->e2_filled = 0;
     c->e2_alpha = alpha;
+    if (c->e2_filled > upto)
+        return 0;
+    const int t0 = c->e2_filled, t1 = std::min(HIST_CAP + 1, std::max({256, 2 * t0, upto + 1}));
+    std::vector<double> tab(t1 - t0);
+    for (int t = t0; t < t1; ++t)
+        tab[t - t0] = std::exp(2.0 * (double)alpha * (double)t);
+    c->e2_filled = 0;  // until the copy is queued
+    CU(cudaMemcpyAsync(c->d.e2tab + t0, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    CU(cudaStreamSynchronize(c->stream));
+    c->e2_filled = t1;
     return 0;
 }
 
@@ -447,14 +469,13 @@ struct DriveState {
 
 int drive_begin(panda_ctx *c, float alpha, double tol, int max_iter, bool use_graph, DriveState &ds)
 {
-    int rc = fill_e2(c, alpha);
-    if (rc)
-        return rc;
     Ctl &h = *c->h_ctl;
     ds.start = ds.before = h.iters;
     ds.use_graph = use_graph && c->graph_iters > 0 && c->stream != nullptr;  // the legacy NULL stream cannot be captured
     if ((long long)ds.start + max_iter > (long long)HIST_CAP)
         return set_err(c, PANDA_EINVAL, "iteration count would exceed the supported maximum (65536)");
+    if (int rc = fill_e2(c, alpha, ds.start + max_iter))
+        return rc;
     h.active = max_iter > 0;
     h.stop_at = ds.start + max_iter;
     if (c->d.p1_flag)  // a run that gave up (a bounded wait ran out) may have left a cut tile's flag raised
@@ -557,9 +578,8 @@ void free_all(panda_ctx *c)
     if (c->c_stage)
         cudaFree(c->c_stage);
     c->c_stage = nullptr;
-    for (void *p : c->allocs)
-        cudaFree(p);
-    c->allocs.clear();
+    cudaFree(c->arena);
+    c->arena = nullptr;
     if (c->h_ctl)
         cudaFreeHost(c->h_ctl);
     for (auto &ev : c->ev)
@@ -633,13 +653,7 @@ int create_common(panda_ctx **out, int T, int G, const float *W0, const float *P
     }
     std::memset(c->h_ctl, 0, sizeof(Ctl));
     c->h_ctl->iters = opts.t0;
-    c->ev.resize((size_t)(c->graph_iters > 0 ? c->graph_iters : 1) * 17, nullptr);
-    for (auto &ev : c->ev)
-        if ((e = cudaEventCreate(&ev)) != cudaSuccess) {
-            c->err = std::string("cudaEventCreate: ") + cudaGetErrorString(e);
-            return fail(PANDA_ECUDA);
-        }
-    if ((rc = plan_memory(c)) || (rc = load_state(c, W0, P0, C0, ldc, c->normalize != 0)) || (rc = push_ctl(c)) ||
+    if ((rc = alloc_plan(c)) || (rc = load_state(c, W0, P0, C0, ldc, c->normalize != 0)) || (rc = push_ctl(c)) ||
         (rc = unstage_c(c)))
         return fail(rc);
     e = cudaStreamSynchronize(c->stream);
@@ -903,7 +917,7 @@ int panda_set_state(panda_ctx *c, const float *W, const float *P, const float *C
         return PANDA_EINVAL;
     if (!W || !P || !C || t < 0 || t >= HIST_CAP)
         return set_err(c, PANDA_EINVAL, "W, P, C must be non-NULL and 0 <= t < 65536");
-    drop_graphs(c);
+    // (captured graphs stay: they hold the context's own buffers, whose addresses do not change)
     c->cur = 0;
     c->state_ok = false;  // until the new networks are in, validated and their vectors derived
     int rc;
@@ -1068,6 +1082,19 @@ int panda_set_profiling(panda_ctx *c, int on)
 {
     if (check_ctx(c))
         return PANDA_EINVAL;
+    if (on && c->ev.empty()) {  // the timing events, made when they are first asked for
+        c->ev.resize((size_t)(c->graph_iters > 0 ? c->graph_iters : 1) * 17, nullptr);
+        for (auto &ev : c->ev) {
+            const cudaError_t e = cudaEventCreate(&ev);
+            if (e != cudaSuccess) {
+                for (auto &x : c->ev)
+                    if (x)
+                        cudaEventDestroy(x);
+                c->ev.clear();
+                return set_err(c, PANDA_ECUDA, std::string("cudaEventCreate: ") + cudaGetErrorString(e));
+            }
+        }
+    }
     if (c->prof != (on != 0))
         drop_graphs(c);  // graphs are captured with or without the timing events
     c->prof = on != 0;
