@@ -30,11 +30,15 @@
 // two thirds of BF16X3's bytes per MMA.
 //
 // Two tile shapes, the same code: 256 x 256 on a CTA pair (cta_group::2), and
-// 128 x 128 on one CTA for networks with too few tiles to fill the chip
-// (operand bytes per flop double).  Tiles that would leave workers idle are
-// cut along K (f32_plan): every part but the last to arrive leaves its sums in
-// slots in L2; the last one adds all parts in part order, so the result does
-// not depend on who that is, and nobody waits.
+// 128 x 64 on one CTA for networks with too few tiles to fill the chip with
+// pairs (operand bytes per flop are three times a pair's, but more SMs work, a
+// tile's epilogue is a quarter as long, and a third operand stage fits).
+// Against 128 x 128 on one CTA the narrow tile took phases 1 + 2 from 94 to
+// 85 us at 1000 x 1000, 97 to 78 us at 250 x 2100 and 44 to 38 us at 125 x 125
+// (with the timing events' own 5 us each).  Tiles that would leave workers idle are cut along K (f32_plan):
+// every part but the last to arrive leaves its sums in slots in L2; the last
+// one adds all parts in part order, so the result does not depend on who that
+// is, and nobody waits.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -54,8 +58,6 @@ using namespace tc;
 
 constexpr int EPI = 8;                         // epilogue warps: two per TMEM lane quarter
 constexpr int NTHREADS = 128 + 32 * EPI;       // warpgroup 0: TMA, MMA (two warps idle); then the epilogue
-constexpr int ST = 2;                          // operand stages
-constexpr uint32_t STAGE = 6 * A_BYTES;        // per CTA: A h, m, l and B h, m, l (128 rows x 64 each)
 
 struct F32Maps {
     CUtensorMap P[3];       // P_off parts [Tp][Tp], boxes of 64 x 128
@@ -66,9 +68,9 @@ struct F32Maps {
 };
 
 // A work item: part `part` of `nparts` of a tile, stages [s0, s1) of its K.
-// Phase 1: a = mt | nt << 16, and stages run over R-num (TFs) first, then
-// A-num (genes); part 0 holds all of R-num.  Phase 2: a = bm | bn << 15, bit 31
-// set for a P tile.  fix (cut tiles): its arrival counter, slot: its first slot.
+// Phase 1: a = mt | nt << 16 (row and column tile), and stages run over R-num
+// (TFs) first, then A-num (genes); part 0 holds all of R-num.  Phase 2: a =
+// bm | bn << 15 (row and column tile), bit 31 set for a P tile.  fix (cut tiles): its arrival counter, slot: its first slot.
 struct __align__(16) Item {
     uint32_t a;
     uint16_t s0, s1;
@@ -79,32 +81,49 @@ static_assert(sizeof(Item) == 16, "one 16-byte load");
 
 template <bool PAIR>
 struct Tile {
-    static constexpr int N = PAIR ? 256 : 128;     // tile columns
+    static constexpr int M = PAIR ? 256 : 128, N = PAIR ? 256 : 64;  // tile rows and columns
+    static constexpr int BROWS = PAIR ? 128 : 64;                    // B rows that one CTA loads
+    static constexpr uint32_t B_PART = BROWS * BK * 2;
+    static constexpr uint32_t STAGE = 3 * A_BYTES + 3 * B_PART;      // per CTA: A h, m, l and B h, m, l
     static constexpr int NCH = N / 32;             // 16-column chunks of one epilogue warp
     static constexpr int SLOT = 128 * N;           // floats of one CTA's tile sums
     static constexpr uint32_t COLS = 512;          // TMEM columns held
 };
 
+constexpr int MAX_ST = 3;
 struct Sync {
-    uint64_t full[ST], empty[ST];
+    uint64_t full[MAX_ST], empty[MAX_ST];
     uint64_t done[2], free_[2];  // a stage's accumulator is complete / drained
     uint64_t fin;                // every MMA of this CTA (pair) is complete
     uint32_t tmem;
     int abort, issued, consumed, last;
 };
+constexpr size_t sync_bytes() { return (sizeof(Sync) + 15) & ~size_t(15); }
 
-constexpr size_t f32_smem(int N, int NS)
-{
-    // stages, barriers, column vectors (3 N), column sums (4 NS N), row sums (2 NS 128), staging blocks, h
-    return 1024 + (size_t)ST * STAGE + ((sizeof(Sync) + 15) & ~size_t(15)) +
-           (size_t)(N + 4 * NS * N + 2 * NS * 128 + EPI * 32 * 17) * sizeof(float) + 64;
-}
-// phase 1 needs three column vectors and one sum, phase 2 one vector and two (D2: three) sums
-template <bool PAIR>
-constexpr size_t p1_smem() { return f32_smem(Tile<PAIR>::N, 2); }
+// Operand stages, and the rows that a warp stages at a time for its mirrored
+// stores: what fits beside the sums (three under D2)
 template <bool PAIR, bool SIM>
-constexpr size_t p2_smem() { return f32_smem(Tile<PAIR>::N, SIM ? 3 : 2); }
-static_assert(p2_smem<true, true>() <= 232448, "fits in the shared memory of a CTA");
+constexpr int stages_of() { return PAIR || SIM ? 2 : 3; }
+template <bool PAIR, bool SIM>
+constexpr int mirror_rows() { return PAIR && !SIM ? 16 : 8; }
+// stages, barriers; c_j, |W_.j|^2, |C_.j|^2 of the columns, the column sums [quarter], row sums [half], h
+template <bool PAIR>
+constexpr size_t p1_smem()
+{
+    return 1024 + (size_t)stages_of<PAIR, false>() * Tile<PAIR>::STAGE + sync_bytes() +
+           (7 * Tile<PAIR>::N + 2 * 128) * sizeof(float) + EPI * sizeof(double);
+}
+// stages, barriers; the column norms, column sums [quarter][sum], row sums [half][sum], staging blocks
+template <bool PAIR, bool SIM>
+constexpr size_t p2_smem()
+{
+    constexpr int N = Tile<PAIR>::N, NS = SIM ? 3 : 2;
+    return 1024 + (size_t)stages_of<PAIR, SIM>() * Tile<PAIR>::STAGE + sync_bytes() +
+           (N + 4 * NS * N + 2 * NS * 128 + EPI * mirror_rows<PAIR, SIM>() * 17) * sizeof(float);
+}
+static_assert(p1_smem<true>() <= 232448 && p2_smem<true, false>() <= 232448 && p2_smem<true, true>() <= 232448 &&
+                  p1_smem<false>() <= 232448 && p2_smem<false, false>() <= 232448 && p2_smem<false, true>() <= 232448,
+              "fits in the shared memory of a CTA");
 
 __device__ __forceinline__ uint8_t *align1024(uint8_t *p)
 {
@@ -179,7 +198,7 @@ __device__ __forceinline__ void group_sync()  // the CTA, or both of the pair
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 2, %0;" ::"n"(32 * EPI) : "memory"); }
 
 // Barriers and TMEM, once per CTA.
-template <bool PAIR>
+template <bool PAIR, int ST>
 __device__ __forceinline__ void setup(Sync &sy)
 {
     if (threadIdx.x == 0) {
@@ -206,7 +225,7 @@ __device__ __forceinline__ void setup(Sync &sy)
     group_sync<PAIR>();  // both CTAs' barriers exist before any cross-CTA signal
     tc_fence_after();
 }
-template <bool PAIR>
+template <bool PAIR, int ST>
 __device__ __forceinline__ void teardown(Sync &sy, Ctl *ctl, bool even)
 {
     tc_fence_before();
@@ -228,10 +247,11 @@ __device__ __forceinline__ void teardown(Sync &sy, Ctl *ctl, bool even)
 }
 
 // The TMA producer: for every stage of every item, issue(item, stage, k, buffer, barrier).
-template <bool PAIR, class Load>
+template <bool PAIR, int ST, class Load>
 __device__ __forceinline__ void producer(Sync &sy, uint8_t *stages, const Item *items, int first, int last,
                                          uint32_t rank, Ctl *ctl, Load load)
 {
+    constexpr uint32_t STAGE = Tile<PAIR>::STAGE;
     int g = 0;
     for (int n = first; n < last; ++n) {
         const Item it = items[n];
@@ -251,11 +271,11 @@ __device__ __forceinline__ void producer(Sync &sy, uint8_t *stages, const Item *
 
 // The MMA issuer: every stage into a fresh accumulator, buffer g & 1.  mn(item,
 // stage) gives which operands are MN-major (bit 0: B, bit 1: A).
-template <bool PAIR, class Mn>
+template <bool PAIR, int ST, class Mn>
 __device__ __forceinline__ void issuer(Sync &sy, uint8_t *stages, const Item *items, int first, int last, Ctl *ctl,
                                        Mn mn)
 {
-    constexpr uint32_t idesc = idesc_bf16_f32(PAIR ? 256 : 128, Tile<PAIR>::N);
+    constexpr uint32_t idesc = idesc_bf16_f32(Tile<PAIR>::M, Tile<PAIR>::N), STAGE = Tile<PAIR>::STAGE;
     int g = 0;
     bool ok = true;
     for (int n = first; n < last && ok; ++n) {
@@ -272,19 +292,19 @@ __device__ __forceinline__ void issuer(Sync &sy, uint8_t *stages, const Item *it
             const uint32_t dacc = sy.tmem + (uint32_t)buf * Tile<PAIR>::N;
             const int m = mn(it, s);
             const uint32_t id = idesc | ((m & 1) ? IDESC_B_MN : 0u) | ((m & 2) ? IDESC_A_MN : 0u);
-            // descriptors of part 0 at K slice 0; a part adds A_BYTES, a slice 32 B (K-major) or 2 KB (MN-major)
+            // descriptors of part 0 at K slice 0; a part adds its bytes, a slice 32 B (K-major) or 2 KB (MN-major)
             const uint64_t a0 = (m & 2) ? sdesc_mn_sw128(base, A_BYTES / 2) : sdesc_k_sw128(base);
             const uint64_t b0 = (m & 1) ? sdesc_mn_sw128(base + 3 * A_BYTES, A_BYTES / 2)
                                         : sdesc_k_sw128(base + 3 * A_BYTES);
             const uint64_t as = (m & 2) ? 2048 >> 4 : 32 >> 4, bs = (m & 1) ? 2048 >> 4 : 32 >> 4;
-            constexpr uint64_t PART = A_BYTES >> 4;
+            constexpr uint64_t APART = A_BYTES >> 4, BPART = Tile<PAIR>::B_PART >> 4;
             // smallest products first: m.m, h.l, l.h, then h.m, m.h, then h.h
             constexpr int pa[6] = {1, 0, 2, 0, 1, 0}, pb[6] = {1, 2, 0, 1, 0, 0};
 #pragma unroll
             for (int t = 0; t < 6; ++t)
 #pragma unroll
                 for (int kk = 0; kk < BK / 16; ++kk)
-                    mma<PAIR>(dacc, a0 + pa[t] * PART + kk * as, b0 + pb[t] * PART + kk * bs, id,
+                    mma<PAIR>(dacc, a0 + pa[t] * APART + kk * as, b0 + pb[t] * BPART + kk * bs, id,
                               (t == 0 && kk == 0) ? 0u : 1u);
             commit<PAIR>(&sy.empty[st]);
             commit<PAIR>(&sy.done[buf]);
@@ -443,7 +463,8 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
     k_f32_phase1(const __grid_constant__ F32Maps maps, const __grid_constant__ Dev d, int cur,
                  const int *__restrict__ off, const Item *__restrict__ items)
 {
-    constexpr int N = Tile<PAIR>::N, NCH = Tile<PAIR>::NCH, SLOT = Tile<PAIR>::SLOT;
+    constexpr int N = Tile<PAIR>::N, NCH = Tile<PAIR>::NCH, SLOT = Tile<PAIR>::SLOT, ST = stages_of<PAIR, false>();
+    constexpr uint32_t STAGE = Tile<PAIR>::STAGE, B_PART = Tile<PAIR>::B_PART;
     Ctl *ctl = d.ctl;
     if (!ctl->active)  // every CTA sees the same value
         return;
@@ -459,21 +480,21 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
     const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x;
     const int first = off[worker], last = off[worker + 1];
     const int nR = ceil_div(d.Tp, BK);
-    setup<PAIR>(sy);
+    setup<PAIR, ST>(sy);
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (warp == 0 && lane == 0) {
-            producer<PAIR>(sy, stages, items, first, last, rank, ctl,
+            producer<PAIR, ST>(sy, stages, items, first, last, rank, ctl,
                            [&](const Item &it, int s, uint8_t *b, uint64_t *bar) {
-                               const int m0 = (int)(it.a & 0xffffu) * (PAIR ? 256 : 128) + 128 * (int)rank;
+                               const int m0 = (int)(it.a & 0xffffu) * Tile<PAIR>::M + 128 * (int)rank;
                                const int n0 = (int)(it.a >> 16) * N, nb0 = n0 + 128 * (int)rank;
                                if (s < nR) {  // P_off rows x W columns, K over TFs
                                    const int k = s * BK;
                                    for (int p = 0; p < 3; ++p) {
                                        load_box<PAIR>(b + p * A_BYTES, &maps.P[p], bar, k, m0);
-                                       for (int h = 0; h < 2; ++h)
-                                           load_box<PAIR>(b + (3 + p) * A_BYTES + h * (A_BYTES / 2),
+                                       for (int h = 0; h < Tile<PAIR>::BROWS / 64; ++h)
+                                           load_box<PAIR>(b + 3 * A_BYTES + p * B_PART + h * (A_BYTES / 2),
                                                           &maps.Wm[cur][p], bar, nb0 + 64 * h, k);
                                    }
                                    return;
@@ -481,17 +502,17 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                                const int k = (s - nR) * BK;
                                for (int p = 0; p < 3; ++p) {
                                    load_box<PAIR>(b + p * A_BYTES, &maps.W[cur][p], bar, k, m0);
+                                   uint8_t *bb = b + 3 * A_BYTES + p * B_PART;
                                    if (k >= n0) {  // C_off[j][k] at or past the tile's diagonal block: stored rows
-                                       load_box<PAIR>(b + (3 + p) * A_BYTES, &maps.C[p], bar, k, nb0);
+                                       load_box<PAIR>(bb, PAIR ? &maps.C[p] : &maps.Cm[p], bar, k, nb0);
                                    } else {        // C_off[k][j], rows k of the upper triangle
-                                       for (int h = 0; h < 2; ++h)
-                                           load_box<PAIR>(b + (3 + p) * A_BYTES + h * (A_BYTES / 2), &maps.Cm[p], bar,
-                                                          nb0 + 64 * h, k);
+                                       for (int h = 0; h < Tile<PAIR>::BROWS / 64; ++h)
+                                           load_box<PAIR>(bb + h * (A_BYTES / 2), &maps.Cm[p], bar, nb0 + 64 * h, k);
                                    }
                                }
                            });
         } else if (warp == 1 && lane == 0 && rank == 0) {
-            issuer<PAIR>(sy, stages, items, first, last, ctl, [&](const Item &it, int s) {
+            issuer<PAIR, ST>(sy, stages, items, first, last, ctl, [&](const Item &it, int s) {
                 return (s < nR || (s - nR) * BK < (int)(it.a >> 16) * N) ? 1 : 0;
             });
         }
@@ -509,7 +530,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
         for (int n = first; n < last; ++n) {
             const Item it = items[n];
             const bool cut = it.nparts > 1;
-            const int nt = (int)(it.a >> 16), m0 = (int)(it.a & 0xffffu) * (PAIR ? 256 : 128) + 128 * (int)rank;
+            const int nt = (int)(it.a >> 16), m0 = (int)(it.a & 0xffffu) * Tile<PAIR>::M + 128 * (int)rank;
             const int n0 = nt * N;
             // slots: this CTA's own for an uncut tile's R-num; a cut tile's R-num and parts
             float *rslot = d.p1_acc + (size_t)blockIdx.x * SLOT;
@@ -689,7 +710,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
             }
         }
     }
-    teardown<PAIR>(sy, ctl, !PAIR || rank == 0);
+    teardown<PAIR, ST>(sy, ctl, !PAIR || rank == 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -701,6 +722,8 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                  const int *__restrict__ off, const Item *__restrict__ items)
 {
     constexpr int N = Tile<PAIR>::N, NCH = Tile<PAIR>::NCH, SLOT = Tile<PAIR>::SLOT, NS = SIM ? 3 : 2;
+    constexpr int ST = stages_of<PAIR, SIM>(), MR = mirror_rows<PAIR, SIM>();
+    constexpr uint32_t STAGE = Tile<PAIR>::STAGE, B_PART = Tile<PAIR>::B_PART;
     Ctl *ctl = d.ctl;
     if (!ctl->active)
         return;
@@ -710,36 +733,37 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
     float *colnrm = reinterpret_cast<float *>(stages + ST * STAGE + ((sizeof(Sync) + 15) & ~size_t(15)));
     float *colred = colnrm + N;             // [quarter][sum][column]
     float *rowred = colred + 4 * NS * N;    // [half][sum][row]
-    float *blocks = rowred + 2 * NS * 128;  // per epilogue warp: 32 x 16 staging block, rows of 17
+    float *blocks = rowred + 2 * NS * 128;  // per epilogue warp: MR x 16 staging block, rows of 17
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0;
     const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x;
     const int first = off[worker], last = off[worker + 1];
-    setup<PAIR>(sy);
+    setup<PAIR, ST>(sy);
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (warp == 0 && lane == 0) {
-            producer<PAIR>(sy, stages, items, first, last, rank, ctl,
+            producer<PAIR, ST>(sy, stages, items, first, last, rank, ctl,
                            [&](const Item &it, int s, uint8_t *b, uint64_t *bar) {
-                               const int m0 = (int)(it.a & 0x7fffu) * N + 128 * (int)rank;
+                               const int m0 = (int)(it.a & 0x7fffu) * Tile<PAIR>::M + 128 * (int)rank;
                                const int n0 = (int)(it.a >> 15 & 0x7fffu) * N + 128 * (int)rank, k = s * BK;
                                for (int p = 0; p < 3; ++p) {
+                                   uint8_t *bb = b + 3 * A_BYTES + p * B_PART;
                                    if (it.a >> 31) {  // P: rows of W', K over genes
                                        load_box<PAIR>(b + p * A_BYTES, &maps.W[cur][p], bar, k, m0);
-                                       load_box<PAIR>(b + (3 + p) * A_BYTES, &maps.W[cur][p], bar, k, n0);
+                                       load_box<PAIR>(bb, PAIR ? &maps.W[cur][p] : &maps.Wm[cur][p], bar, k, n0);
                                        continue;
                                    }
-                                   for (int h = 0; h < 2; ++h) {  // C: columns of W', K over TFs, MN-major
+                                   // C: columns of W', K over TFs, MN-major
+                                   for (int h = 0; h < 2; ++h)
                                        load_box<PAIR>(b + p * A_BYTES + h * (A_BYTES / 2), &maps.Wm[cur][p], bar,
                                                       m0 + 64 * h, k);
-                                       load_box<PAIR>(b + (3 + p) * A_BYTES + h * (A_BYTES / 2), &maps.Wm[cur][p], bar,
-                                                      n0 + 64 * h, k);
-                                   }
+                                   for (int h = 0; h < Tile<PAIR>::BROWS / 64; ++h)
+                                       load_box<PAIR>(bb + h * (A_BYTES / 2), &maps.Wm[cur][p], bar, n0 + 64 * h, k);
                                }
                            });
         } else if (warp == 1 && lane == 0 && rank == 0) {
-            issuer<PAIR>(sy, stages, items, first, last, ctl,
+            issuer<PAIR, ST>(sy, stages, items, first, last, ctl,
                          [](const Item &it, int) { return it.a >> 31 ? 0 : 3; });
         }
     } else {
@@ -748,7 +772,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
         const int er = lane >> 2, ec = 8 * (lane & 1) + 2 * (lane & 2);
         const uint32_t free_even = PAIR ? mapa_shared(smem_u32(&sy.free_[0]), 0) : 0;
         const uint32_t tq = sy.tmem + ((uint32_t)(wq * 32) << 16) + half * (N / 2);
-        float *blk = blocks + (size_t)e * (32 * 17);
+        float *blk = blocks + (size_t)e * (MR * 17);
         int g = 0;
         for (int n = first; n < last; ++n) {
             const Item it = items[n];
@@ -781,12 +805,12 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                     put_slot<NCH>(fix, tt, acc);
             }
             const int nn = isP ? d.T : d.G, ld = isP ? d.Tp : d.Gp;
-            const int m0 = bm * N + 128 * (int)rank, n0 = bn * N;
+            const int m0 = bm * Tile<PAIR>::M + 128 * (int)rank, n0 = bn * N;
             const float *nrm = isP ? d.rsqW : d.csqW;
             float *X = isP ? d.Poff : d.Coff;
             __nv_bfloat16 *Xs[3] = {isP ? d.Ph : d.Ch, isP ? d.Pm : d.Cm, isP ? d.Pl : d.Cl};
             // split copies of the lower triangle: all of P, of C only inside diagonal tiles
-            const bool mirror = isP || bm == bn;
+            const bool mirror = isP || (PAIR ? bm == bn : bm == bn >> 1);
             const bool rows_in = m0 < ld;
             const float a = ctl->alpha;
             epi_bar();  // colnrm, colred and rowred of the item before are no longer read
@@ -903,46 +927,55 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                                 }
                         }
                     }
-                    // mirrored entries (j, k) through this warp's staging block: lane l takes column
-                    // (l & 15), rows 16 (l >> 4) + 0..15
+                    // mirrored entries (j, k) through this warp's staging block, MR rows at a time: lane l
+                    // takes column (l & 15), rows (MR / 2) (l >> 4) + 0 .. MR / 2 - 1
                     if (mirror) {
+                        constexpr int H = MR / 2;
+                        const int col = lane & 15, jm = j0 + col;
+#pragma unroll 1
+                        for (int r0 = 0; r0 < 32; r0 += MR) {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
+                            for (int i = 0; i < 4; ++i)
+                                if (8 * i >= r0 && 8 * i < r0 + MR)
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                blk[(er + 8 * i) * 17 + ec + u] = v[i][u];
-                        __syncwarp();
-                        const int col = lane & 15, h16 = 16 * (lane >> 4), jm = j0 + col, km = k0 + h16;
-                        const uint32_t mm =
-                            jm >= nn ? 0u : (km + 15 < jm ? 0xffffu : (km >= jm ? 0u : ((1u << (jm - km)) - 1u)));
-                        if (mm) {
-                            uint32_t q3[3][8];
+                                    for (int u = 0; u < 4; ++u)
+                                        blk[(er + 8 * i - r0) * 17 + ec + u] = v[i][u];
+                            __syncwarp();
+                            const int km = k0 + r0 + H * (lane >> 4);
+                            constexpr uint32_t all = (1u << H) - 1u;
+                            const uint32_t mm =
+                                jm >= nn ? 0u : (km + H - 1 < jm ? all : (km >= jm ? 0u : ((1u << (jm - km)) - 1u)));
+                            if (mm) {
+                                uint32_t q3[3][H / 2];
 #pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                uint32_t p[3];
-                                split3(blk[(h16 + 2 * q) * 17 + col], blk[(h16 + 2 * q + 1) * 17 + col], p);
-                                q3[0][q] = p[0];
-                                q3[1][q] = p[1];
-                                q3[2][q] = p[2];
-                            }
-                            const size_t mo = (size_t)jm * ld + km;
+                                for (int q = 0; q < H / 2; ++q) {
+                                    const float *b = blk + (H * (lane >> 4) + 2 * q) * 17 + col;
+                                    uint32_t p[3];
+                                    split3(b[0], b[17], p);
+                                    q3[0][q] = p[0];
+                                    q3[1][q] = p[1];
+                                    q3[2][q] = p[2];
+                                }
+                                const size_t mo = (size_t)jm * ld + km;
 #pragma unroll
-                            for (int p = 0; p < 3; ++p) {
-                                if (mm == 0xffffu) {
-                                    reinterpret_cast<uint4 *>(Xs[p] + mo)[0] =
-                                        make_uint4(q3[p][0], q3[p][1], q3[p][2], q3[p][3]);
-                                    reinterpret_cast<uint4 *>(Xs[p] + mo)[1] =
-                                        make_uint4(q3[p][4], q3[p][5], q3[p][6], q3[p][7]);
-                                } else {
+                                for (int p = 0; p < 3; ++p) {
+                                    if (mm == all) {
+                                        if (H == 8)
+                                            *reinterpret_cast<uint4 *>(Xs[p] + mo) =
+                                                make_uint4(q3[p][0], q3[p][1], q3[p][H / 2 - 2], q3[p][H / 2 - 1]);
+                                        else
+                                            *reinterpret_cast<uint2 *>(Xs[p] + mo) = make_uint2(q3[p][0], q3[p][1]);
+                                    } else {
 #pragma unroll
-                                    for (int q = 0; q < 16; ++q)
-                                        if (mm >> q & 1u)
-                                            reinterpret_cast<uint16_t *>(Xs[p])[mo + q] =
-                                                (uint16_t)(q3[p][q >> 1] >> (16 * (q & 1)));
+                                        for (int q = 0; q < H; ++q)
+                                            if (mm >> q & 1u)
+                                                reinterpret_cast<uint16_t *>(Xs[p])[mo + q] =
+                                                    (uint16_t)(q3[p][q >> 1] >> (16 * (q & 1)));
+                                    }
                                 }
                             }
+                            __syncwarp();  // the block is rewritten
                         }
-                        __syncwarp();  // the block is rewritten by the next chunk
                     }
                 }
                 const float t = lanes8_reduce_scatter8(cs);
@@ -996,17 +1029,17 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                                 S[(size_t)(nb + 2 * bm + (int)rank) * ld + n0 + j] = colsum(j);
                         if (tt < 128)
                             S[(size_t)bn * ld + m0 + tt] = rowsum(tt);
-                    } else if (tt < 128) {  // one slot per 128-block; a diagonal tile's two roles share it
-                        const float rs = rowsum(tt), cs1 = colsum(tt);
-                        S[(size_t)bn * ld + m0 + tt] = bm == bn ? rs + cs1 : rs;
-                        if (bm != bn)
-                            S[(size_t)bm * ld + n0 + tt] = cs1;
+                    } else {  // row role in slot bn, column role in slot nb + bm
+                        if (tt < N)
+                            S[(size_t)(nb + bm) * ld + n0 + tt] = colsum(tt);
+                        if (tt < 128)
+                            S[(size_t)bn * ld + m0 + tt] = rowsum(tt);
                     }
                 }
             }
         }
     }
-    teardown<PAIR>(sy, ctl, !PAIR || rank == 0);
+    teardown<PAIR, ST>(sy, ctl, !PAIR || rank == 0);
 }
 
 // h, m, l of a whole array (padding stays zero): four values per thread
@@ -1061,12 +1094,14 @@ void finish(const std::vector<std::vector<Item>> &list, Phase &ph)
     }
 }
 
-// Costs in stages of K = 64 (measured: 1.9 us on a pair, 1.3 us on one CTA): a
+// Costs in stages of K = 64 (measured: 1.9 us on a pair, 0.8 us on one CTA): a
 // finished tile's epilogue, and what a cut costs each part (its sums to L2, the
 // counter, a pipeline that starts empty) and the part that finishes.
-constexpr double EPILOGUE[2] = {7.0, 10.0}, CUT = 3.0, CUT_LAST = 3.0;  // [one CTA], [pair]
-constexpr double STAGE_US[2] = {1.3, 1.9};
+constexpr double EPILOGUE[2] = {6.0, 10.0}, CUT[2] = {4.0, 3.0}, CUT_LAST[2] = {4.0, 3.0};  // [one CTA], [pair]
+constexpr double STAGE_US[2] = {0.8, 1.9};
 constexpr int MIN_PART = 4;
+constexpr int tile_m(bool pair) { return pair ? Tile<true>::M : Tile<false>::M; }
+constexpr int tile_n(bool pair) { return pair ? Tile<true>::N : Tile<false>::N; }
 
 // Phase 1 with the tiles from `whole` on cut in one of two ways, the ones
 // before whole, in rounds: np > 0, every tile in np equal parts (the first
@@ -1075,7 +1110,7 @@ constexpr int MIN_PART = 4;
 // ends (never inside R-num, and no part under MIN_PART stages).
 Phase plan_phase1_cut(const Dev &d, int workers, bool pair, int whole, int np)
 {
-    const int N = pair ? 256 : 128, nmt = ceil_div(d.Tp, N), ntile = nmt * ceil_div(d.Gp, N);
+    const int nmt = ceil_div(d.Tp, tile_m(pair)), ntile = nmt * ceil_div(d.Gp, tile_n(pair));
     const int nR = ceil_div(d.Tp, BK), K = nR + ceil_div(d.Gp, BK), rest = ntile - whole;
     const double E = EPILOGUE[pair];
     Phase ph;
@@ -1124,7 +1159,8 @@ Phase plan_phase1_cut(const Dev &d, int workers, bool pair, int whole, int np)
                 it.fix = (uint16_t)ph.fixes;
                 it.slot = (uint16_t)ph.slots;
             }
-            const double c = it.s1 - it.s0 + (n > 1 ? CUT : 0.0) + (p == n - 1 ? E + (n > 1 ? CUT_LAST : 0.0) : 0.0);
+            const double c = it.s1 - it.s0 + (n > 1 ? CUT[pair] : 0.0) +
+                             (p == n - 1 ? E + (n > 1 ? CUT_LAST[pair] : 0.0) : 0.0);
             if (np > 0) {
                 parts.push_back({c, it});
             } else {
@@ -1152,7 +1188,7 @@ Phase plan_phase1_cut(const Dev &d, int workers, bool pair, int whole, int np)
 // whichever way leaves the busiest worker the least.
 Phase plan_phase1(const Dev &d, int workers, bool pair)
 {
-    const int N = pair ? 256 : 128, ntile = ceil_div(d.Tp, N) * ceil_div(d.Gp, N);
+    const int ntile = ceil_div(d.Tp, tile_m(pair)) * ceil_div(d.Gp, tile_n(pair));
     const int nR = ceil_div(d.Tp, BK), K = nR + ceil_div(d.Gp, BK);
     Phase best = plan_phase1_cut(d, workers, pair, ntile, 1);
     if ((double)ceil_div(ntile, workers) * workers <= 1.05 * ntile)
@@ -1172,15 +1208,15 @@ Phase plan_phase1(const Dev &d, int workers, bool pair)
 // longest first to the least loaded worker.
 Phase plan_phase2_cap(const Dev &d, int workers, bool pair, int cap)
 {
-    const int N = pair ? 256 : 128;
+    const int M = tile_m(pair), N = tile_n(pair);
     const double E = EPILOGUE[pair];
     Phase ph;
     std::vector<std::pair<double, Item>> all;
     for (int isP = 1; isP >= 0; --isP) {
-        const int nb = ceil_div(isP ? d.Tp : d.Gp, N), K = ceil_div(isP ? d.Gp : d.Tp, BK);
+        const int ld = isP ? d.Tp : d.Gp, nbm = ceil_div(ld, M), nbn = ceil_div(ld, N), K = ceil_div(isP ? d.Gp : d.Tp, BK);
         const int np = std::min(ceil_div(K, cap), 64);
-        for (int bm = 0; bm < nb; ++bm)
-            for (int bn = bm; bn < nb; ++bn) {
+        for (int bm = 0; bm < nbm; ++bm)
+            for (int bn = bm * (M / N); bn < nbn; ++bn) {
                 for (int p = 0; p < np; ++p) {
                     Item it{};
                     it.a = (uint32_t)bm | (uint32_t)bn << 15 | (isP ? 0x80000000u : 0u);
@@ -1190,8 +1226,10 @@ Phase plan_phase2_cap(const Dev &d, int workers, bool pair, int cap)
                         it.fix = (uint16_t)ph.fixes;
                         it.slot = (uint16_t)ph.slots;
                     }
-                    all.push_back({it.s1 - it.s0 + (np > 1 ? CUT : 0.0) +
-                                       (p == np - 1 ? E + (np > 1 ? CUT_LAST : 0.0) : 0.0),
+                    // (a mirrored tile's epilogue takes almost twice as long)
+                    const double e = isP || bn < (bm + 1) * (M / N) ? 1.8 * E : E;
+                    all.push_back({it.s1 - it.s0 + (np > 1 ? CUT[pair] : 0.0) +
+                                       (p == np - 1 ? e + (np > 1 ? CUT_LAST[pair] : 0.0) : 0.0),
                                    it});
                 }
                 if (np > 1) {
@@ -1208,11 +1246,11 @@ Phase plan_phase2_cap(const Dev &d, int workers, bool pair, int cap)
 
 Phase plan_phase2(const Dev &d, int workers, bool pair)
 {
-    const int N = pair ? 256 : 128, nP = ceil_div(d.Tp, N), nC = ceil_div(d.Gp, N);
+    auto tiles = [&](int ld) { return (long long)ceil_div(ld, tile_m(pair)) * (ceil_div(ld, tile_n(pair)) + 2) / 2; };
     Phase best;
     for (int cap : {1 << 20, 256, 64, 32, 16, 8, 5}) {
-        const long long parts = (long long)nP * (nP + 1) / 2 * ceil_div(ceil_div(d.Gp, BK), cap) +
-                                (long long)nC * (nC + 1) / 2 * ceil_div(ceil_div(d.Tp, BK), cap);
+        const long long parts = tiles(d.Tp) * ceil_div(ceil_div(d.Gp, BK), cap) +
+                                tiles(d.Gp) * ceil_div(ceil_div(d.Tp, BK), cap);
         if (cap < (1 << 20) && parts > 8LL * workers)  // enough items to balance without cutting more
             break;
         Phase ph = plan_phase2_cap(d, workers, pair, cap);
@@ -1308,7 +1346,7 @@ void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fix
     *pair = p.pair;
 }
 
-int f32_diag_block(const Dev &d) { return static_cast<const F32Host *>(d.f32_host)->plan.pair ? 256 : 128; }
+int f32_diag_block(const Dev &d) { return static_cast<const F32Host *>(d.f32_host)->plan.pair ? 256 : 64; }
 
 cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
 {

@@ -303,7 +303,7 @@ __device__ __forceinline__ void reduce_wnorms_block(const Dev &d, int b)
     const bool ok = x < (rows ? d.T : d.G);
     const float *const src[1] = {rows ? d.wrow_part : d.wcol_part};
     double out[1];
-    slot_sums<1>(src, 0, rows ? d.nbG : d.nbT, 0, 0, rows ? d.Tp : d.Gp, x, ok, out, sh);
+    slot_sums<1>(src, 0, rows ? d.nwr : d.nbT, 0, 0, rows ? d.Tp : d.Gp, x, ok, out, sh);
     if (threadIdx.x >= RS_ROWS)
         return;
     if (ok)
@@ -468,7 +468,12 @@ __device__ __forceinline__ void fin_block(const Dev &d, int b)
     const int ld = isP ? d.Tp : d.Gp;
     const float *const src[3] = {isP ? d.ps_sum : d.cs_sum, isP ? d.ps_sq : d.cs_sq, isP ? d.ps_vsq : d.cs_vsq};
     double sums[3];
-    if (d.tri_slots) {
+    if (d.tri_slots == 2) {
+        // 128 x 64 tiles: a row of 64-block b has row-role partials in slots [2 (b / 2), nb) and
+        // column-role partials in [nb, nb + b / 2 + 1)
+        const int nb = ceil_div(ld, 64), b64 = ((isP ? b : b - bT) * RS_ROWS) >> 6;
+        slot_sums<3>(src, b64 & ~1, nb, nb, nb + b64 / 2 + 1, ld, i, ok, sums, sh);
+    } else if (d.tri_slots) {
         // a row of 256-block b has row-role partials in slots [b, nb) (tiles (b, bn >= b)) and
         // column-role partials in [nb, nb + 2 b + 2) (tiles (bm <= b, b), one per CTA of the pair)
         const int nb = ceil_div(ld, 256), b256 = ((isP ? b : b - bT) * RS_ROWS) >> 8;
@@ -525,7 +530,7 @@ __device__ __forceinline__ void tail_block(const Dev &d)
     if (!ctl->active)
         return;
     __shared__ double sh[256];
-    const int n = d.nbT * d.nbG;
+    const int n = d.nbT * d.nwr;
     double s = 0.0;
     for (int q = threadIdx.x; q < n; q += blockDim.x)
         s += d.hpart[q];

@@ -146,21 +146,21 @@ int plan_memory(panda_ctx *c)
     DALLOC(d.csqC, Gp);
     DALLOC(d.rsqW, Tp);
     DALLOC(d.csqW, Gp);
-    DALLOC(d.wrow_part, (size_t)c->nbG * Tp);
-    DALLOC(d.wcol_part, (size_t)c->nbT * Gp);
-    DALLOC(d.hpart, (size_t)c->nbT * c->nbG);
-    // partial-sum slots: one per 128-row block where tiles are 128 x 128 (FP32 networks too
-    // small for CTA pairs); with 256 x 256 tiles one per 256-column block for the row role plus
-    // one per 128-row half for the column role (see k_tc.cu)
+    // partial-sum slots: one per column tile (256 columns on a CTA pair; 64 in FP32 networks too
+    // small for pairs) for the row role, plus one per 128 rows for the column role
     int nsm = 0;
     CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
     size_t f32_slots = 0, f32_fix = 0;
     bool pair_tiles = true;
     if (c->prec == PANDA_FP32)
         f32_plan(d, nsm, &f32_slots, &f32_fix, &d.p1_cuts, &pair_tiles);  // (computed at the first call)
-    d.nsP = pair_tiles ? 3 * ceil_div(c->Tp, 256) : c->nbT;
-    d.nsC = pair_tiles ? 3 * ceil_div(c->Gp, 256) : c->nbG;
-    d.tri_slots = pair_tiles ? 1 : 0;
+    d.nsP = pair_tiles ? 3 * ceil_div(c->Tp, 256) : 3 * c->nbT;
+    d.nsC = pair_tiles ? 3 * ceil_div(c->Gp, 256) : 3 * c->nbG;
+    d.tri_slots = pair_tiles ? 1 : 2;
+    d.nwr = pair_tiles ? ceil_div(c->Gp, 256) : 2 * c->nbG;
+    DALLOC(d.wrow_part, (size_t)d.nwr * Tp);
+    DALLOC(d.wcol_part, (size_t)c->nbT * Gp);
+    DALLOC(d.hpart, (size_t)c->nbT * d.nwr);
     DALLOC(d.ps_sum, (size_t)d.nsP * Tp);
     DALLOC(d.ps_sq, (size_t)d.nsP * Tp);
     DALLOC(d.ps_vsq, (size_t)d.nsP * Tp);

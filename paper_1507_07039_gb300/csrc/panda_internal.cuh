@@ -57,15 +57,16 @@ struct Dev {
     float *rsqP, *csqC, *rsqW, *csqW;
     // scratch
     float *Rn;                   // Tp x Gp  P_off . W  (SIMT path)
-    float *wrow_part;            // nbG x Tp
+    int nwr;                     // phase 1's column tiles: slots of the next two arrays
+    float *wrow_part;            // nwr x Tp
     float *wcol_part;            // nbT x Gp
-    double *hpart;               // nbT * nbG
+    double *hpart;               // nwr x nbT
     float *ps_sum, *ps_sq, *ps_vsq;  // nsP x Tp  row partials of P'
     float *cs_sum, *cs_sq, *cs_vsq;  // nsC x Gp  row partials of C'
     int nsP, nsC;                    // partial-sum slots per row (0: one per 128-row block)
-    int tri_slots;                   // 1: the tensor-core layout of those slots (row roles in
-                                     // [0, nb), column roles from nb, nb = 256-blocks); 0: one
-                                     // slot per 128-block, every slot written
+    int tri_slots;                   // layout of those slots (rows of tiles as row roles first, then
+                                     // column roles): 1: 256-column tiles of CTA pairs; 2: 64-column
+                                     // tiles; 0: one slot per 128-block, every slot written
     Ctl *ctl;
     double *hist;                // HIST_CAP
     double *e2tab;               // HIST_CAP + 1: e^{2 alpha t}, computed on the host

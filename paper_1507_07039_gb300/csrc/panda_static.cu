@@ -119,6 +119,7 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     d.T = T; d.G = G;
     d.Tp = round_up(T, TILE); d.Gp = round_up(G, TILE);
     d.nbT = d.Tp / TILE; d.nbG = d.Gp / TILE;
+    d.nwr = d.nbG;
     d.diag = diag;
     unsigned char *p = base;
     auto take = [&p](size_t bytes) { unsigned char *q = p; p += bytes; return q; };
