@@ -355,7 +355,7 @@ void panda_batch_destroy(panda_batch *b);
  * stream) and blocks until the iteration is done.  When it returns an error
  * (PANDA_ENONFINITE included) dW, dP and dC hold what they held before.
  *
- * Working memory is one file-scope device array of about 7.4 MB, sized for
+ * Working memory is one file-scope device array of about 11.5 MB, sized for
  * T, G <= PANDA_STATIC_MAX_NODES; larger shapes are rejected with
  * PANDA_EINVAL before any GPU work.  Every GPU that loads the library's
  * device code holds the array until the process exits; with CUDA's lazy
@@ -363,8 +363,7 @@ void panda_batch_destroy(panda_batch *b);
  * device, so a caller with a fixed memory budget makes that call at
  * start-up.  The first call on each device also looks up the array's device
  * address (with that device current); make that first call before any
- * stream capture.  All calls share the array and clear it at
- * their start, so calls that overlap on the GPU (for example on two streams)
+ * stream capture.  All calls share the array, so calls that overlap on the GPU (for example on two streams)
  * race and must be serialised by the caller.  Errors are reported by the
  * return code and panda_last_error(NULL). */
 #define PANDA_STATIC_MAX_NODES 512

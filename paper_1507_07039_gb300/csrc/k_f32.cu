@@ -1290,7 +1290,7 @@ struct F32Host {
     F32Maps maps;
     F32Plan plan;  // its lists are on the device once `ready`
     bool ready = false;
-    int workers = 0;
+    int grid[2] = {0, 0};  // CTAs of the two phases
     int *off[2] = {nullptr, nullptr};
     Item *items[2] = {nullptr, nullptr};
 };
@@ -1305,6 +1305,66 @@ cudaError_t smem_limits(K1 p1, K2 p2, K3 p2s)
     return cudaFuncSetAttribute(p2s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p2_smem<PAIR, true>());
 }
 
+cudaError_t all_smem_limits()
+{
+    cudaError_t e = smem_limits<true>(k_f32_phase1<true>, k_f32_phase2<true, false>, k_f32_phase2<true, true>);
+    return e ? e : smem_limits<false>(k_f32_phase1<false>, k_f32_phase2<false, false>, k_f32_phase2<false, true>);
+}
+
+cudaError_t make_maps(const Dev &d, F32Maps &m)
+{
+    std::memset(&m, 0, sizeof m);
+    __nv_bfloat16 *P[3] = {d.Ph, d.Pm, d.Pl}, *C[3] = {d.Ch, d.Cm, d.Cl};
+    cudaError_t e;
+    for (int p = 0; p < 3; ++p) {
+        if ((e = tc_make_map(&m.P[p], P[p], d.Tp, d.Tp, 128)) || (e = tc_make_map(&m.C[p], C[p], d.Gp, d.Gp, 128)) ||
+            (e = tc_make_map(&m.Cm[p], C[p], d.Gp, d.Gp, 64)))
+            return e;
+        for (int b = 0; b < 2; ++b) {
+            __nv_bfloat16 *W[3] = {d.Wh[b], d.Wm[b], d.Wl[b]};
+            if ((e = tc_make_map(&m.W[b][p], W[p], d.Tp, d.Gp, 128)) ||
+                (e = tc_make_map(&m.Wm[b][p], W[p], d.Tp, d.Gp, 64)))
+                return e;
+        }
+    }
+    return cudaSuccess;
+}
+
+// panda_step_static's work lists and control block, by value in one launch
+struct StaticArgs {
+    Item items[2][F32_STATIC_ITEMS];
+    int n[2];
+    float alpha;
+    double e2;
+};
+constexpr size_t STATIC_LIST = F32_STATIC_LIST_BYTES / 2;  // one phase: its offsets (256 bytes), then its items
+static_assert((F32_STATIC_ITEMS + 1) * sizeof(int) <= 256, "the offsets fit");
+
+__global__ void k_f32_static_lists(const __grid_constant__ StaticArgs a, uint8_t *lists, Ctl *ctl, double *e2tab, int *flags)
+{
+    const int t = threadIdx.x;
+    for (int ph = 0; ph < 2; ++ph) {
+        int *off = reinterpret_cast<int *>(lists + ph * STATIC_LIST);
+        Item *it = reinterpret_cast<Item *>(lists + ph * STATIC_LIST + 256);
+        if (t <= a.n[ph])
+            off[t] = t;  // CTA t: item t
+        if (t < a.n[ph])
+            it[t] = a.items[ph][t];
+    }
+    if (t < 4)
+        flags[t] = 0;
+    if (t == 0) {
+        Ctl c{};
+        c.active = 1;
+        c.stop_at = 1;
+        c.alpha = a.alpha;
+        c.tol = -1.0;
+        *ctl = c;
+        e2tab[0] = 1.0;
+        e2tab[1] = a.e2;
+    }
+}
+
 template <class T>
 cudaError_t to_device(T **dst, const std::vector<T> &v)
 {
@@ -1317,7 +1377,7 @@ cudaError_t to_device(T **dst, const std::vector<T> &v)
 template <bool PAIR>
 void launch(const F32Host &h, const Dev &d, int cur, cudaStream_t s, int phase)
 {
-    const int grid = (PAIR ? 2 : 1) * h.workers;
+    const int grid = h.grid[phase - 1];
     if (phase == 1)
         k_f32_phase1<PAIR><<<grid, NTHREADS, p1_smem<PAIR>(), s>>>(h.maps, d, cur, h.off[0], h.items[0]);
     else if (d.diag == 2)
@@ -1336,11 +1396,11 @@ void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fix
     if (!h) {
         d.f32_host = h = new F32Host;
         h->plan = f32_plan_for(d, nsm);
-        h->workers = h->plan.pair ? nsm / 2 : nsm;
+        h->grid[0] = h->grid[1] = h->plan.pair ? nsm & ~1 : nsm;
     }
     const F32Plan &p = h->plan;
     const size_t slot = p.pair ? Tile<true>::SLOT : Tile<false>::SLOT, ranks = p.pair ? 2 : 1;
-    *slot_floats = slot * ranks * (size_t)h->workers;
+    *slot_floats = slot * (size_t)h->grid[0];
     *fix_floats = slot * ranks * (size_t)std::max(p.p1.slots, p.p2.slots);
     *fixes = std::max(p.p1.fixes, p.p2.fixes);
     *pair = p.pair;
@@ -1362,22 +1422,7 @@ cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
     F32Host *h = static_cast<F32Host *>(d.f32_host);
     if (e || h->ready)
         return e;
-    std::memset(&h->maps, 0, sizeof h->maps);
-    F32Maps &m = h->maps;
-    __nv_bfloat16 *P[3] = {d.Ph, d.Pm, d.Pl}, *C[3] = {d.Ch, d.Cm, d.Cl};
-    for (int p = 0; p < 3; ++p) {
-        if ((e = tc_make_map(&m.P[p], P[p], d.Tp, d.Tp, 128)) || (e = tc_make_map(&m.C[p], C[p], d.Gp, d.Gp, 128)) ||
-            (e = tc_make_map(&m.Cm[p], C[p], d.Gp, d.Gp, 64)))
-            return e;
-        for (int b = 0; b < 2; ++b) {
-            __nv_bfloat16 *W[3] = {d.Wh[b], d.Wm[b], d.Wl[b]};
-            if ((e = tc_make_map(&m.W[b][p], W[p], d.Tp, d.Gp, 128)) ||
-                (e = tc_make_map(&m.Wm[b][p], W[p], d.Tp, d.Gp, 64)))
-                return e;
-        }
-    }
-    if ((e = smem_limits<true>(k_f32_phase1<true>, k_f32_phase2<true, false>, k_f32_phase2<true, true>)) ||
-        (e = smem_limits<false>(k_f32_phase1<false>, k_f32_phase2<false, false>, k_f32_phase2<false, true>)))
+    if ((e = make_maps(d, h->maps)) || (e = all_smem_limits()))
         return e;
     const F32Plan &p = h->plan;
     if ((e = to_device(&h->off[0], p.p1.off)) || (e = to_device(&h->items[0], p.p1.items)) ||
@@ -1419,6 +1464,55 @@ cudaError_t launch_iteration_f32(const Dev &d, int cur, cudaStream_t s, KernelEv
         launch<false>(h, d, cur ^ 1, s, 2);
     ke.mark(s);
     return launch_fin_tail(d, s, ke);
+}
+
+cudaError_t f32_static_host(const Dev &d, void *lists, void **host)
+{
+    F32Host *h = new F32Host;
+    cudaError_t e;
+    if ((e = make_maps(d, h->maps)) || (e = all_smem_limits())) {
+        delete h;
+        return e;
+    }
+    h->plan.pair = false;
+    h->ready = true;
+    for (int ph = 0; ph < 2; ++ph) {
+        h->off[ph] = reinterpret_cast<int *>(static_cast<uint8_t *>(lists) + ph * STATIC_LIST);
+        h->items[ph] = reinterpret_cast<Item *>(static_cast<uint8_t *>(lists) + ph * STATIC_LIST + 256);
+    }
+    const int nt = d.Gp / 64, mt = d.Tp / 128;
+    h->grid[0] = nt * mt;
+    for (int ld : {d.Tp, d.Gp})
+        for (int bm = 0; bm < ld / 128; ++bm)
+            h->grid[1] += ld / 64 - 2 * bm;
+    *host = h;
+    return cudaSuccess;
+}
+
+cudaError_t f32_static_lists(const Dev &d, float alpha, double e2, void *lists, int *flags, cudaStream_t s)
+{
+    StaticArgs a{};
+    a.alpha = alpha;
+    a.e2 = e2;
+    auto add = [&](int ph, uint32_t code, int stages) {
+        Item it{};
+        it.a = code;
+        it.s1 = (uint16_t)stages;
+        it.nparts = 1;
+        a.items[ph][a.n[ph]++] = it;
+    };
+    const int nR = d.Tp / BK, nA = d.Gp / BK;
+    for (int nt = 0; nt < d.Gp / 64; ++nt)
+        for (int mt = 0; mt < d.Tp / 128; ++mt)
+            add(0, (uint32_t)mt | (uint32_t)nt << 16, nR + nA);
+    for (int isP = 1; isP >= 0; --isP) {
+        const int ld = isP ? d.Tp : d.Gp;
+        for (int bm = 0; bm < ld / 128; ++bm)
+            for (int bn = 2 * bm; bn < ld / 64; ++bn)
+                add(1, (uint32_t)bm | (uint32_t)bn << 15 | (isP ? 0x80000000u : 0u), isP ? nA : nR);
+    }
+    k_f32_static_lists<<<1, 64, 0, s>>>(a, static_cast<uint8_t *>(lists), d.ctl, d.e2tab, flags);
+    return cudaGetLastError();
 }
 
 }  // namespace panda

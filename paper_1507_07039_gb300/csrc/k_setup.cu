@@ -1,7 +1,7 @@
-// One-time kernels of panda_create / panda_set_state: input validation, the
-// Z-score of each network (Section II-A, NormalizeNetwork) with FP64
-// statistics, stripping the diagonals of P and C into FP64 vectors, the
-// transposed copy of W and the initial squared norms.
+// State in and out: input validation, the Z-score of each network (Section
+// II-A, NormalizeNetwork) with FP64 statistics, the diagonals of P and C into
+// FP64 vectors, every copy that the iteration reads, the initial squared
+// norms; and the networks back into dense arrays.
 //
 // Every reduction here runs with a fixed grid and a fixed summation order, so
 // results are identical from run to run.
@@ -13,69 +13,6 @@ namespace {
 
 constexpr int RED_BLOCKS = 1024;
 constexpr int RED_THREADS = 256;
-
-// flags[0] |= 1 on a non-finite entry (rows x cols, row stride ld): block b
-// reads rows b, b + gridDim.x, ... along the row.
-__global__ void k_check_finite(const float *__restrict__ X, int rows, int cols, int ld, int *flags)
-{
-    int bad = 0;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x)
-        for (int c = threadIdx.x; c < cols; c += blockDim.x)
-            bad |= !isfinite(X[(size_t)r * ld + c]);
-    if (__syncthreads_or(bad) && threadIdx.x == 0)
-        atomicOr(&flags[0], 1);
-}
-
-// A square n x n matrix as 32 x 32 blocks: each pair of mirror blocks (bi, bj)
-// and (bj, bi), bi <= bj, is read once, along rows, into shared memory, so the
-// whole matrix is read once and coalesced.  flags[0] |= 1 on a non-finite
-// entry, flags[1] |= 1 when X[i][j] != X[j][i].  Pairs are numbered column by
-// column of the upper triangle: pair t has bj = the largest j with
-// j(j+1)/2 <= t and bi = t - bj(bj+1)/2.  256 threads.
-__global__ void k_check_finite_sym(const float *__restrict__ X, int n, int ld, int npairs, int *flags)
-{
-    __shared__ float a[32][33], b[32][33];
-    __shared__ int pij[2];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    int bad = 0, asym = 0;
-    for (int t = blockIdx.x; t < npairs; t += gridDim.x) {
-        if (threadIdx.x == 0) {
-            // 8t + 1 < 2^24 for n <= 46000, so the FP32 square root is close; the loops correct it
-            int j = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-            while (j > 0 && (long long)j * (j + 1) / 2 > t)
-                --j;
-            while ((long long)(j + 1) * (j + 2) / 2 <= t)
-                ++j;
-            pij[0] = t - (int)((long long)j * (j + 1) / 2);
-            pij[1] = j;
-        }
-        __syncthreads();
-        const int i0 = pij[0] * 32, j0 = pij[1] * 32;
-#pragma unroll
-        for (int k = ty; k < 32; k += 8) {
-            const int ra = i0 + k, ca = j0 + tx, rb = j0 + k, cb = i0 + tx;
-            a[k][tx] = (ra < n && ca < n) ? X[(size_t)ra * ld + ca] : 0.0f;
-            b[k][tx] = (rb < n && cb < n) ? X[(size_t)rb * ld + cb] : 0.0f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = ty; k < 32; k += 8) {
-            // a[k][tx] = X[i0 + k][j0 + tx], its mirror X[j0 + tx][i0 + k] = b[tx][k]
-            const float v = a[k][tx];
-            bad |= !isfinite(v) | !isfinite(b[k][tx]);
-            asym |= (i0 + k < n && j0 + tx < n && v != b[tx][k]);
-        }
-        __syncthreads();
-    }
-    bad = __syncthreads_or(bad);
-    asym = __syncthreads_or(asym);
-    if (threadIdx.x == 0) {
-        if (bad)
-            atomicOr(&flags[0], 1);
-        if (asym)
-            atomicOr(&flags[1], 1);
-    }
-}
 
 __device__ double block_sum_fixed(double v, double *sh)
 {
@@ -265,19 +202,21 @@ __device__ __forceinline__ void put_parts(const Parts &t, size_t o, const float 
 }
 
 // W (rows x cols, row stride ldi) into out (row stride ldo, a multiple of 4) and
-// its parts; block y takes a row, 1024 columns per block.  X may be out itself.
+// its parts, zeros in the padding (row gridDim.y - 1, column ldo - 1 the last);
+// block y takes a row, 1024 columns per block.  X may be out itself.
 __global__ void k_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo, Parts parts,
                          int *flags)
 {
     const int r = blockIdx.y, c = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     int bad = 0;
-    if (c < cols) {
+    if (c < ldo) {
         float v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            v[u] = c + u < cols ? X[(size_t)r * ldi + c + u] : 0.0f;
+            const bool in = r < rows && c + u < cols;
+            v[u] = in ? X[(size_t)r * ldi + c + u] : 0.0f;
             bad |= !isfinite(v[u]);
-            if (stats && c + u < cols)
+            if (stats && in)
                 v[u] = zscore_one(v[u], stats_pairs(stats));
         }
         const size_t o = (size_t)r * ldo + c;
@@ -290,7 +229,8 @@ __global__ void k_load_w(const float *X, int rows, int cols, int ldi, const doub
 
 // A symmetric n x n network (row stride ldi) as 64 x 64 blocks: each pair of
 // mirror blocks (bi, bj), (bj, bi), bi <= bj, is read once, along rows, into
-// shared memory.  flags as in k_check_finite_sym.  Written: block (bi, bj) of
+// shared memory.  flags[0] |= 1 on a non-finite entry, flags[1] |= 1 when
+// X[i][j] != X[j][i].  Written, padding (to out.ld) included: block (bi, bj) of
 // out.F and of the parts, block (bj, bi) too where the form holds it; the
 // diagonal goes to out.d and out.df and reads as zero in F and the parts.  X
 // may be out.F itself (each block pair is one block's alone).  256 threads.
@@ -345,7 +285,7 @@ __global__ void __launch_bounds__(256) k_load_sym(const float *X, int n, int ldi
                     v[u] = 0.0f;
                 }
             }
-            if (gi < n && j0 + c4 < n) {
+            if (gi < out.ld && j0 + c4 < out.ld) {
                 const size_t o = (size_t)gi * out.ld + j0 + c4;
                 if (out.F)
                     *reinterpret_cast<float4 *>(out.F + o) = make_float4(v[0], v[1], v[2], v[3]);
@@ -365,7 +305,7 @@ __global__ void __launch_bounds__(256) k_load_sym(const float *X, int n, int ldi
                     if (stats && gj < n && i0 + c4 + u < n)
                         v[u] = zscore_one(v[u], stats_pairs(stats));
                 }
-                if (gj < n && i0 + c4 < n) {
+                if (gj < out.ld && i0 + c4 < out.ld) {
                     const size_t o = (size_t)gj * out.ld + i0 + c4;
                     if (lf)
                         *reinterpret_cast<float4 *>(out.F + o) = make_float4(v[0], v[1], v[2], v[3]);
@@ -384,18 +324,6 @@ __global__ void __launch_bounds__(256) k_load_sym(const float *X, int n, int ldi
         if (asym)
             atomicOr(&flags[1], 1);
     }
-}
-
-__global__ void k_split_diag(float *X, int n, int ld, double *d, float *df)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n)
-        return;
-    size_t o = (size_t)i * ld + i;
-    double v = (double)X[o];
-    d[i] = v;
-    df[i] = (float)v;
-    X[o] = 0.0f;
 }
 
 __global__ void k_diag_to_float(const double *d, float *df, int n)
@@ -573,6 +501,19 @@ __global__ void k_standardize_rows(const float *__restrict__ X, int G, int N, __
     }
 }
 
+__device__ __forceinline__ bool faulted(const Guard &g)
+{
+    return g.flags && (g.flags[0] | g.flags[1] | g.ctl->status);
+}
+
+__global__ void k_store_w(const float *__restrict__ X, int cols, int ldi, float *__restrict__ out, Guard g)
+{
+    if (faulted(g))
+        return;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x)
+        out[(size_t)blockIdx.y * cols + c] = X[(size_t)blockIdx.y * ldi + c];
+}
+
 // The full symmetric n x n matrix (row stride ldo, any alignment) from its
 // strict upper triangle, FP32 in X or a BF16 split pair H + L (exact in FP32;
 // row stride ldi, a multiple of 4), and its FP64 diagonal, in 64 x 64 blocks:
@@ -580,8 +521,11 @@ __global__ void k_standardize_rows(const float *__restrict__ X, int G, int N, __
 // time turned through shared memory.  256 threads.
 __global__ void __launch_bounds__(256) k_store_sym(const float *__restrict__ X, const __nv_bfloat16 *__restrict__ H,
                                                    const __nv_bfloat16 *__restrict__ L, int n, int ldi, int npairs,
-                                                   const double *__restrict__ diag, float *__restrict__ out, int ldo)
+                                                   const double *__restrict__ diag, float *__restrict__ out, int ldo,
+                                                   Guard g)
 {
+    if (faulted(g))
+        return;
     __shared__ float a[LB][LB + 1];
     const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // stores: 4 rows of 64
     const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // loads: 16 rows of 16 x 4
@@ -653,10 +597,16 @@ cudaError_t launch_unit_diag(float *X, int n, int ld, cudaStream_t s)
 }
 
 cudaError_t launch_store_sym(const float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi,
-                             const double *diag, float *out, int ldo, cudaStream_t s)
+                             const double *diag, float *out, int ldo, Guard g, cudaStream_t s)
 {
     const int nb = ceil_div(n, LB), npairs = nb * (nb + 1) / 2;
-    k_store_sym<<<npairs < 152 * 12 ? npairs : 152 * 12, 256, 0, s>>>(X, H, L, n, ldi, npairs, diag, out, ldo);
+    k_store_sym<<<npairs < 152 * 12 ? npairs : 152 * 12, 256, 0, s>>>(X, H, L, n, ldi, npairs, diag, out, ldo, g);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_store_w(const float *X, int rows, int cols, int ldi, float *out, Guard g, cudaStream_t s)
+{
+    k_store_w<<<dim3(ceil_div(cols, 1024), rows), 256, 0, s>>>(X, cols, ldi, out, g);
     return cudaGetLastError();
 }
 
@@ -671,23 +621,6 @@ cudaError_t launch_symmetrize(float *X, int n, int ld, cudaStream_t s)
 // keep every row 16-byte aligned.
 static bool rows_aligned(const void *X, int ld) { return (ld & 3) == 0 && ((uintptr_t)X & 15) == 0; }
 
-cudaError_t launch_check_finite_sym(const float *X, int rows, int cols, int ld, bool sym,
-                                    int *flags, cudaStream_t s)
-{
-    if (rows <= 0 || cols <= 0)
-        return cudaSuccess;
-    if (sym) {
-        if (rows != cols)
-            return cudaErrorInvalidValue;
-        const int nb = ceil_div(rows, 32);
-        const int npairs = (int)((long long)nb * (nb + 1) / 2);
-        k_check_finite_sym<<<npairs < 152 * 8 ? npairs : 152 * 8, 256, 0, s>>>(X, rows, ld, npairs, flags);
-    } else {
-        k_check_finite<<<rows < RED_BLOCKS ? rows : RED_BLOCKS, 256, 0, s>>>(X, rows, cols, ld, flags);
-    }
-    return cudaGetLastError();
-}
-
 cudaError_t launch_stats(const float *X, int rows, int cols, int ld, double *stats, double *partials, cudaStream_t s)
 {
     if ((uintptr_t)stats & 15)
@@ -701,23 +634,17 @@ cudaError_t launch_stats(const float *X, int rows, int cols, int ld, double *sta
     return cudaGetLastError();
 }
 
-cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo,
+cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int rows_p, int ldo,
                           const Parts &parts, int *flags, cudaStream_t s)
 {
-    k_load_w<<<dim3(ceil_div(cols, 1024), rows), 256, 0, s>>>(X, rows, cols, ldi, stats, out, ldo, parts, flags);
+    k_load_w<<<dim3(ceil_div(ldo, 1024), rows_p), 256, 0, s>>>(X, rows, cols, ldi, stats, out, ldo, parts, flags);
     return cudaGetLastError();
 }
 
 cudaError_t launch_load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags, cudaStream_t s)
 {
-    const int nb = ceil_div(n, LB), npairs = nb * (nb + 1) / 2;
+    const int nb = ceil_div(out.ld, LB), npairs = nb * (nb + 1) / 2;
     k_load_sym<<<npairs < 152 * 6 ? npairs : 152 * 6, 256, 0, s>>>(X, n, ldi, npairs, stats, out, flags);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_split_diag(float *X, int n, int ld, double *d, float *df, cudaStream_t s)
-{
-    k_split_diag<<<ceil_div(n, 256), 256, 0, s>>>(X, n, ld, d, df);
     return cudaGetLastError();
 }
 

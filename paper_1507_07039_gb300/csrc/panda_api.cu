@@ -154,19 +154,19 @@ int plan_memory(panda_ctx *c)
     bool pair_tiles = true;
     if (c->prec == PANDA_FP32)
         f32_plan(d, nsm, &f32_slots, &f32_fix, &d.p1_cuts, &pair_tiles);  // (computed at the first call)
-    d.nsP = pair_tiles ? 3 * ceil_div(c->Tp, 256) : 3 * c->nbT;
-    d.nsC = pair_tiles ? 3 * ceil_div(c->Gp, 256) : 3 * c->nbG;
-    d.tri_slots = pair_tiles ? 1 : 2;
+    const int nsP = pair_tiles ? 3 * ceil_div(c->Tp, 256) : 3 * c->nbT;
+    const int nsC = pair_tiles ? 3 * ceil_div(c->Gp, 256) : 3 * c->nbG;
+    d.narrow = pair_tiles ? 0 : 1;
     d.nwr = pair_tiles ? ceil_div(c->Gp, 256) : 2 * c->nbG;
     DALLOC(d.wrow_part, (size_t)d.nwr * Tp);
     DALLOC(d.wcol_part, (size_t)c->nbT * Gp);
     DALLOC(d.hpart, (size_t)c->nbT * d.nwr);
-    DALLOC(d.ps_sum, (size_t)d.nsP * Tp);
-    DALLOC(d.ps_sq, (size_t)d.nsP * Tp);
-    DALLOC(d.ps_vsq, (size_t)d.nsP * Tp);
-    DALLOC(d.cs_sum, (size_t)d.nsC * Gp);
-    DALLOC(d.cs_sq, (size_t)d.nsC * Gp);
-    DALLOC(d.cs_vsq, (size_t)d.nsC * Gp);
+    DALLOC(d.ps_sum, (size_t)nsP * Tp);
+    DALLOC(d.ps_sq, (size_t)nsP * Tp);
+    DALLOC(d.ps_vsq, (size_t)nsP * Tp);
+    DALLOC(d.cs_sum, (size_t)nsC * Gp);
+    DALLOC(d.cs_sq, (size_t)nsC * Gp);
+    DALLOC(d.cs_vsq, (size_t)nsC * Gp);
     DALLOC(d.ctl, 1);
     DALLOC(d.hist, HIST_CAP);
     DALLOC(d.e2tab, HIST_CAP + 1);
@@ -343,7 +343,7 @@ int load_state(panda_ctx *c, const float *W, const float *P, const float *C, int
     }
     const bool f32 = c->prec == PANDA_FP32;
     CU(cudaMemsetAsync(c->d_flags, 0, 4 * sizeof(int), c->stream));
-    CU(launch_load_w(w.src, T, G, w.ld, st[0], d.W[c->cur], c->Gp, Parts{d.Wh[c->cur], d.Wm[c->cur], d.Wl[c->cur]},
+    CU(launch_load_w(w.src, T, G, w.ld, st[0], d.W[c->cur], c->Tp, c->Gp, Parts{d.Wh[c->cur], d.Wm[c->cur], d.Wl[c->cur]},
                      c->d_flags, c->stream));
     // a network loaded in place keeps both triangles, for the norms below; FP8MIX's E4M3 copy of C is made from both
     const SymOut po{d.Poff, p.src == d.Poff, Parts{d.Ph, d.Pm, d.Pl}, 1, 256, c->Tp, d.pd, d.pdf};
@@ -844,13 +844,13 @@ static int get_sym(panda_ctx *c, float *dst, float *X, const __nv_bfloat16 *H, c
                    int n, int ld)
 {
     if (device_pointer(dst)) {
-        CU(launch_store_sym(X, H, L, n, ld, diag, dst, n, c->stream));
+        CU(launch_store_sym(X, H, L, n, ld, diag, dst, n, Guard{}, c->stream));
         return 0;
     }
     if (!X) {
         float *tmp = nullptr;
         CU(cudaMalloc(&tmp, sizeof(float) * (size_t)n * n));
-        cudaError_t e = launch_store_sym(X, H, L, n, ld, diag, tmp, n, c->stream);
+        cudaError_t e = launch_store_sym(X, H, L, n, ld, diag, tmp, n, Guard{}, c->stream);
         if (!e)
             e = cudaMemcpyAsync(dst, tmp, sizeof(float) * (size_t)n * n, cudaMemcpyDeviceToHost, c->stream);
         if (!e)

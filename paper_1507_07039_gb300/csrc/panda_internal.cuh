@@ -28,7 +28,7 @@
 
 namespace panda {
 
-constexpr int TILE = 128;          // padding granule and SIMT tile edge
+constexpr int TILE = 128;          // padding granule
 constexpr int HIST_CAP = 1 << 16;  // iterations whose h is kept on the device
 
 // Device control block, read by every kernel of an iteration.
@@ -56,17 +56,14 @@ struct Dev {
     float *pdf, *cdf;            // FP32 copies of the diagonals for epilogues
     float *rsqP, *csqC, *rsqW, *csqW;
     // scratch
-    float *Rn;                   // Tp x Gp  P_off . W  (SIMT path)
     int nwr;                     // phase 1's column tiles: slots of the next two arrays
     float *wrow_part;            // nwr x Tp
     float *wcol_part;            // nbT x Gp
     double *hpart;               // nwr x nbT
-    float *ps_sum, *ps_sq, *ps_vsq;  // nsP x Tp  row partials of P'
-    float *cs_sum, *cs_sq, *cs_vsq;  // nsC x Gp  row partials of C'
-    int nsP, nsC;                    // partial-sum slots per row (0: one per 128-row block)
-    int tri_slots;                   // layout of those slots (rows of tiles as row roles first, then
-                                     // column roles): 1: 256-column tiles of CTA pairs; 2: 64-column
-                                     // tiles; 0: one slot per 128-block, every slot written
+    float *ps_sum, *ps_sq, *ps_vsq;  // slots x Tp  row partials of P'
+    float *cs_sum, *cs_sq, *cs_vsq;  // slots x Gp  row partials of C'
+    int narrow;                      // layout of those slots, row roles first, then column roles:
+                                     // 0: 256-column tiles of CTA pairs; 1: FP32's 64-column tiles
     Ctl *ctl;
     double *hist;                // HIST_CAP
     double *e2tab;               // HIST_CAP + 1: e^{2 alpha t}, computed on the host
@@ -170,8 +167,6 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e)
 }
 
 // ---- launchers (k_setup.cu) ------------------------------------------------
-cudaError_t launch_check_finite_sym(const float *X, int rows, int cols, int ld, bool sym,
-                                    int *flags, cudaStream_t s);
 // Z-score statistics of X (read only): stats[0] = mean, stats[1] = population std, then the
 // FP32 pairs that the loads below apply; 4 doubles, 16-byte aligned
 cudaError_t launch_stats(const float *X, int rows, int cols, int ld, double *stats, double *partials, cudaStream_t s);
@@ -192,12 +187,12 @@ struct SymOut {
     float *df;
 };
 // X (device memory, any alignment, row stride ldi) checked (flags[0] |= 1: a non-finite entry,
-// flags[1] |= 1: not symmetric), Z-scored when stats is not NULL, and written in those forms
-cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo,
+// flags[1] |= 1: not symmetric), Z-scored when stats is not NULL, and written in those forms, the
+// padding up to rows_p x ldo (W) or ld x ld as zeros
+cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int rows_p, int ldo,
                           const Parts &parts, int *flags, cudaStream_t s);
 cudaError_t launch_load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags,
                             cudaStream_t s);
-cudaError_t launch_split_diag(float *X, int n, int ld, double *d, float *df, cudaStream_t s);
 cudaError_t launch_transpose(const float *X, int rows_p, int cols_p, float *Y, cudaStream_t s);
 // out[j] = sum over the first `rows` rows of X[i][j]^2 (squared column norms, no transpose)
 cudaError_t launch_col_norms(const float *X, int rows, int cols, int ld, float *out, cudaStream_t s);
@@ -210,8 +205,15 @@ cudaError_t launch_diag_to_float(const double *d, float *df, int n, cudaStream_t
 cudaError_t launch_symmetrize(float *X, int n, int ld, cudaStream_t s);
 // out (n x n, row stride ldo) = the symmetric matrix with this strict upper triangle (FP32 X, or
 // X NULL and the BF16 split pair H + L; row stride ldi) and this diagonal
+// (guard, when given: nothing is written if the checks or the iteration found a fault)
+struct Guard {
+    const int *flags;
+    const Ctl *ctl;
+};
 cudaError_t launch_store_sym(const float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi,
-                             const double *diag, float *out, int ldo, cudaStream_t s);
+                             const double *diag, float *out, int ldo, Guard g, cudaStream_t s);
+// out (rows x cols, dense) = X (row stride ldi)
+cudaError_t launch_store_w(const float *X, int rows, int cols, int ldi, float *out, Guard g, cudaStream_t s);
 // Pearson initialisation (Sec. II-A): unit-norm centred rows of X (G x N) as a
 // BF16 split [G][Kp]; flags[0] |= 1 (non-finite) / 2 (zero variance)
 cudaError_t launch_standardize_rows(const float *X, int G, int N, __nv_bfloat16 *Zh, __nv_bfloat16 *Zl, int Kp,
@@ -230,10 +232,7 @@ struct KernelEvents {
     }
 };
 
-// ---- one iteration, FP32 SIMT path (k_simt.cu) -----------------------------
-constexpr int SIMT_KERNELS = 6;
-extern const char *const SIMT_KERNEL_NAMES[SIMT_KERNELS];
-cudaError_t launch_iteration_simt(const Dev &d, int cur, cudaStream_t s, KernelEvents &ke);
+// ---- after the products (k_norms.cu) ----------------------------------------
 // shared tail of every path: diagonals, norms of P and C, h, stop test
 cudaError_t launch_fin_tail(const Dev &d, cudaStream_t s, KernelEvents &ke);
 // FP64 sums of the per-tile norm partials of W' (shared by both paths)
@@ -297,6 +296,16 @@ cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s, bool restored);
 int f32_diag_block(const Dev &d);
 void f32_release(Dev &d);
 cudaError_t launch_iteration_f32(const Dev &d, int cur, cudaStream_t s, KernelEvents &ke);
+// panda_step_static's single iteration: whole tiles, one per CTA, so at most F32_STATIC_ITEMS of
+// them a phase for 512 x 512.  f32_static_lists writes both phases' lists to `lists` (device,
+// F32_STATIC_LIST_BYTES), arms *d.ctl for one iteration at growth factors e2[0], e2[1], and clears
+// flags[0..3]; f32_static_host returns the tensor maps of a Dev whose arrays lie at `d` (kept per
+// device and padded shape by the caller).
+constexpr int F32_STATIC_ITEMS = 40;
+constexpr size_t F32_STATIC_LIST_BYTES = 2 * (F32_STATIC_ITEMS * 16 + 256);
+constexpr size_t F32_STATIC_SLOT_BYTES = (size_t)F32_STATIC_ITEMS * 128 * 64 * sizeof(float);
+cudaError_t f32_static_host(const Dev &d, void *lists, void **host);
+cudaError_t f32_static_lists(const Dev &d, float alpha, double e2, void *lists, int *flags, cudaStream_t s);
 
 struct TcSet;
 // Schedule candidates of the set engine's autotuner: phase 1 (the order of each

@@ -8,20 +8,26 @@
 // synchronisation) is not acceptable.  For them this entry point takes its
 // working memory from one file-scope device array of fixed size instead.
 //
-// The array is `g_scratch` below: STATIC_BYTES bytes (about 7.4 MB), sized
+// The array is `g_scratch` below: STATIC_BYTES bytes (about 11.5 MB), sized
 // for networks of at most PANDA_STATIC_MAX_NODES TFs and genes.  Every GPU
 // that loads the library's device code holds it until the process exits (with
 // CUDA's lazy module loading that happens at the first call on the device, so
 // a caller with a fixed budget makes that call at start-up).  In host code its
 // name only stands for the device array; the device address is looked up once
 // per device with cudaGetSymbolAddress, with that device current, on the
-// first call made on it.  All calls share the array and each call clears it
-// first, so two calls that overlap on the GPU (for example on two streams)
-// race with each other.
+// first call made on it.  All calls share the array, so two calls that overlap
+// on the GPU (for example on two streams) race with each other.
 //
-// The iteration itself is the FP32 SIMT path of panda_step (the same kernels,
-// so the same results), run on a copy of the caller's networks laid out in
-// the array.
+// The iteration itself is the FP32 path of panda_step (the same kernels, whole
+// tiles), run on a copy of the caller's networks laid out in the array.
+//
+// One call is bound by its launches and its wait for the device.  Everything is
+// queued at once and waited for once: the kernels that read the networks check
+// them and zero the padding on the way, the iteration runs whatever the checks
+// find, and the kernels that write the results back look at the findings
+// themselves.  At 64 x 256 a call took 282 us with the array cleared, the
+// networks copied, checked, waited for and stripped in passes of their own
+// and FFMA products.
 #include "panda.h"
 #include "panda_internal.cuh"
 
@@ -42,19 +48,23 @@ constexpr size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 constexpr size_t SQ = al256(sizeof(float) * SMAX * SMAX);  // one padded square matrix
 constexpr size_t VF = al256(sizeof(float) * SMAX);
 constexpr size_t VD = al256(sizeof(double) * SMAX);
-constexpr size_t PART = al256(sizeof(float) * SNB * SMAX);
-constexpr size_t STATIC_BYTES = 7 * SQ                  // W[2], Wt[2], Poff, Coff, Rn
+constexpr size_t PART = al256(sizeof(float) * 3 * SNB * SMAX);  // partial-sum slots
+constexpr size_t BF = al256(sizeof(__nv_bfloat16) * SMAX * SMAX);  // one part of a padded square matrix
+constexpr size_t STATIC_BYTES = 4 * SQ                  // W[2], Poff, Coff
+                                + 12 * BF               // three parts of W[2], P, C
                                 + 2 * VD + 6 * VF       // pd, cd; pdf, cdf, rsqP, csqC, rsqW, csqW
                                 + 8 * PART              // wrow, wcol, ps_sum/sq/vsq, cs_sum/sq/vsq
-                                + al256(sizeof(double) * SNB * SNB)  // hpart
+                                + al256(sizeof(double) * 2 * SNB * SNB)  // hpart
                                 + al256(sizeof(Ctl)) + 2 * al256(2 * sizeof(double))  // ctl, hist, e2tab
-                                + al256(4 * sizeof(int));            // validation flags
+                                + al256(4 * sizeof(int))             // validation flags
+                                + al256(F32_STATIC_SLOT_BYTES) + al256(F32_STATIC_LIST_BYTES);
 
 __device__ __align__(256) unsigned char g_scratch[STATIC_BYTES];
 
 constexpr int MAX_DEVICES = 64;
 std::mutex g_mu;
 unsigned char *g_addr[MAX_DEVICES] = {};
+void *g_host[MAX_DEVICES][SNB][SNB] = {};  // tensor maps over the array, per padded shape
 
 // Device address of g_scratch on the current device (looked up once).
 cudaError_t scratch_address(int dev, unsigned char **out)
@@ -69,13 +79,6 @@ cudaError_t scratch_address(int dev, unsigned char **out)
     }
     *out = g_addr[dev];
     return cudaSuccess;
-}
-
-__global__ void k_put_diag(float *X, int n, int ld, const double *d)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n)
-        X[(size_t)i * ld + i] = (float)d[i];
 }
 
 int fail(int code, const std::string &msg)
@@ -119,17 +122,20 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     d.T = T; d.G = G;
     d.Tp = round_up(T, TILE); d.Gp = round_up(G, TILE);
     d.nbT = d.Tp / TILE; d.nbG = d.Gp / TILE;
-    d.nwr = d.nbG;
+    d.nwr = 2 * d.nbG;
+    d.narrow = 1;
     d.diag = diag;
     unsigned char *p = base;
     auto take = [&p](size_t bytes) { unsigned char *q = p; p += bytes; return q; };
+    auto part = [&take]() { return (__nv_bfloat16 *)take(BF); };
     for (int b = 0; b < 2; ++b) {
         d.W[b] = (float *)take(SQ);
-        d.Wt[b] = (float *)take(SQ);
+        d.Wh[b] = part(); d.Wm[b] = part(); d.Wl[b] = part();
     }
     d.Poff = (float *)take(SQ);
     d.Coff = (float *)take(SQ);
-    d.Rn = (float *)take(SQ);
+    d.Ph = part(); d.Pm = part(); d.Pl = part();
+    d.Ch = part(); d.Cm = part(); d.Cl = part();
     d.pd = (double *)take(VD);
     d.cd = (double *)take(VD);
     d.pdf = (float *)take(VF);
@@ -146,69 +152,55 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     d.cs_sum = (float *)take(PART);
     d.cs_sq = (float *)take(PART);
     d.cs_vsq = (float *)take(PART);
-    d.hpart = (double *)take(al256(sizeof(double) * SNB * SNB));
+    d.hpart = (double *)take(al256(sizeof(double) * 2 * SNB * SNB));
     d.ctl = (Ctl *)take(al256(sizeof(Ctl)));
     d.hist = (double *)take(al256(2 * sizeof(double)));
     d.e2tab = (double *)take(al256(2 * sizeof(double)));
     int *flags = (int *)take(al256(4 * sizeof(int)));
 
-    // zero everything: padding, partial sums, flags
-    SCU(cudaMemsetAsync(base, 0, STATIC_BYTES, s));
-    SCU(cudaMemcpy2DAsync(d.W[0], (size_t)d.Gp * 4, dW, (size_t)G * 4, (size_t)G * 4, T,
-                          cudaMemcpyDeviceToDevice, s));
-    SCU(cudaMemcpy2DAsync(d.Poff, (size_t)d.Tp * 4, dP, (size_t)T * 4, (size_t)T * 4, T,
-                          cudaMemcpyDeviceToDevice, s));
-    SCU(cudaMemcpy2DAsync(d.Coff, (size_t)d.Gp * 4, dC, (size_t)G * 4, (size_t)G * 4, G,
-                          cudaMemcpyDeviceToDevice, s));
-    SCU(launch_check_finite_sym(d.W[0], T, G, d.Gp, false, flags, s));
-    SCU(launch_check_finite_sym(d.Poff, T, T, d.Tp, true, flags, s));
-    SCU(launch_check_finite_sym(d.Coff, G, G, d.Gp, true, flags, s));
+    d.p1_acc = (float *)take(al256(F32_STATIC_SLOT_BYTES));
+    void *lists = take(al256(F32_STATIC_LIST_BYTES));
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        void *&host = g_host[dev][d.nbT - 1][d.nbG - 1];
+        if (!host)
+            SCU(f32_static_host(d, lists, &host));
+        d.f32_host = host;
+    }
+
+    // one iteration at index t: counter 0, growth factor e^{2 alpha t} in slot 1
+    SCU(f32_static_lists(d, alpha, std::exp(2.0 * (double)alpha * (double)t), lists, flags, s));
+    // the state, exactly as a context builds it
+    const SymOut po{d.Poff, 0, Parts{d.Ph, d.Pm, d.Pl}, 1, 64, d.Tp, d.pd, d.pdf};
+    const SymOut xo{d.Coff, 0, Parts{d.Ch, d.Cm, d.Cl}, 0, 64, d.Gp, d.cd, d.cdf};
+    SCU(launch_load_w(dW, T, G, G, nullptr, d.W[0], d.Tp, d.Gp, Parts{d.Wh[0], d.Wm[0], d.Wl[0]}, flags, s));
+    SCU(launch_load_sym(dP, T, T, nullptr, po, flags, s));
+    SCU(launch_load_sym(dC, G, G, nullptr, xo, flags, s));
+    SCU(launch_row_norms(d.W[0], T, G, d.Gp, nullptr, nullptr, d.rsqW, s));
+    SCU(launch_col_norms(d.W[0], T, G, d.Gp, d.csqW, s));
+    SCU(launch_row_norms(dP, T, T, T, nullptr, d.pd, d.rsqP, s));
+    SCU(launch_row_norms(dC, G, G, G, nullptr, d.cd, d.csqC, s));
+    KernelEvents ke{nullptr, 0};
+    SCU(launch_iteration_f32(d, 0, s, ke));
+    // results back into the caller's buffers, diagonals from the FP64 vectors; a failed call leaves
+    // the caller's networks as they were
+    const Guard g{flags, d.ctl};
+    SCU(launch_store_w(d.W[1], T, G, d.Gp, dW, g, s));
+    SCU(launch_store_sym(d.Poff, nullptr, nullptr, T, d.Tp, d.pd, dP, T, g, s));
+    SCU(launch_store_sym(d.Coff, nullptr, nullptr, G, d.Gp, d.cd, dC, G, g, s));
+    Ctl hc{};
     int hflags[4] = {0, 0, 0, 0};
+    SCU(cudaMemcpyAsync(&hc, d.ctl, sizeof hc, cudaMemcpyDeviceToHost, s));
     SCU(cudaMemcpyAsync(hflags, flags, sizeof hflags, cudaMemcpyDeviceToHost, s));
     SCU(cudaStreamSynchronize(s));
     if (hflags[0])
         return fail(PANDA_ENONFINITE, "panda_step_static: a network has a non-finite entry");
     if (hflags[1])
         return fail(PANDA_EASYM, "panda_step_static: P or C is not exactly symmetric");
-
-    // derived state, exactly as a context builds it
-    SCU(launch_split_diag(d.Poff, T, d.Tp, d.pd, d.pdf, s));
-    SCU(launch_split_diag(d.Coff, G, d.Gp, d.cd, d.cdf, s));
-    SCU(launch_transpose(d.W[0], d.Tp, d.Gp, d.Wt[0], s));
-    SCU(launch_row_norms(d.W[0], T, G, d.Gp, nullptr, nullptr, d.rsqW, s));
-    SCU(launch_row_norms(d.Wt[0], G, T, d.Tp, nullptr, nullptr, d.csqW, s));  // columns of W
-    SCU(launch_row_norms(d.Poff, T, T, d.Tp, nullptr, d.pd, d.rsqP, s));
-    SCU(launch_row_norms(d.Coff, G, G, d.Gp, nullptr, d.cd, d.csqC, s));
-
-    // one iteration at index t: counter 0, growth factor e^{2 alpha t} in slot 1
-    Ctl hc{};
-    hc.active = 1;
-    hc.iters = 0;
-    hc.stop_at = 1;
-    hc.alpha = alpha;
-    hc.tol = -1.0;
-    const double e2[2] = {1.0, std::exp(2.0 * (double)alpha * (double)t)};
-    SCU(cudaMemcpyAsync(d.ctl, &hc, sizeof hc, cudaMemcpyHostToDevice, s));
-    SCU(cudaMemcpyAsync(d.e2tab, e2, sizeof e2, cudaMemcpyHostToDevice, s));
-    KernelEvents ke{nullptr, 0};
-    SCU(launch_iteration_simt(d, 0, s, ke));
-    SCU(cudaMemcpyAsync(&hc, d.ctl, sizeof hc, cudaMemcpyDeviceToHost, s));
-    SCU(cudaStreamSynchronize(s));
-    // a failed iteration leaves the caller's networks as they were
+    if (hc.status & ST_TIMEOUT)
+        return fail(PANDA_ETIMEOUT, "panda_step_static: a bounded device wait expired");
     if (hc.status & ST_NONFINITE)
         return fail(PANDA_ENONFINITE, "panda_step_static: the networks became non-finite (left unchanged)");
-
-    // results back into the caller's buffers, diagonals from the FP64 vectors
-    SCU(cudaMemcpy2DAsync(dW, (size_t)G * 4, d.W[1], (size_t)d.Gp * 4, (size_t)G * 4, T,
-                          cudaMemcpyDeviceToDevice, s));
-    SCU(cudaMemcpy2DAsync(dP, (size_t)T * 4, d.Poff, (size_t)d.Tp * 4, (size_t)T * 4, T,
-                          cudaMemcpyDeviceToDevice, s));
-    SCU(cudaMemcpy2DAsync(dC, (size_t)G * 4, d.Coff, (size_t)d.Gp * 4, (size_t)G * 4, G,
-                          cudaMemcpyDeviceToDevice, s));
-    k_put_diag<<<ceil_div(T, 256), 256, 0, s>>>(dP, T, T, d.pd);
-    k_put_diag<<<ceil_div(G, 256), 256, 0, s>>>(dC, G, G, d.cd);
-    SCU(cudaGetLastError());
-    SCU(cudaStreamSynchronize(s));
     if (h_out)
         *h_out = hc.h_last;
     return PANDA_OK;
