@@ -7,7 +7,7 @@
 //   k_f32_phase2  upper-triangle tiles of W'.W'^T (P, K = genes) and
 //                 W'^T.W' (C, K = TFs) with the damped update of Eq. 5, the
 //                 FP32 upper triangle, split copies, partial sums for Eq. 6
-//   k_fin, k_tail (k_norms.cu)
+//   k_fin (k_norms.cu): diagonals, norms, h, stop test
 //
 // Every FP32 operand is held beside its value as three BF16 parts, h = bf16(x),
 // m = bf16(x - h), l = x - h - m: 3 x 8 significant bits, so h + m + l = x
@@ -466,8 +466,6 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
     constexpr int N = Tile<PAIR>::N, NCH = Tile<PAIR>::NCH, SLOT = Tile<PAIR>::SLOT, ST = stages_of<PAIR, false>();
     constexpr uint32_t STAGE = Tile<PAIR>::STAGE, B_PART = Tile<PAIR>::B_PART;
     Ctl *ctl = d.ctl;
-    if (!ctl->active)  // every CTA sees the same value
-        return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *stages = align1024(smem_raw);
     Sync &sy = *reinterpret_cast<Sync *>(stages + ST * STAGE);
@@ -478,9 +476,10 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0;
     const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x;
-    const int first = off[worker], last = off[worker + 1];
     const int nR = ceil_div(d.Tp, BK);
     setup<PAIR, ST>(sy);
+    const bool active = ctl->active;  // every CTA sees the same value
+    const int first = off[worker], last = active ? off[worker + 1] : first;
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
@@ -725,8 +724,6 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
     constexpr int ST = stages_of<PAIR, SIM>(), MR = mirror_rows<PAIR, SIM>();
     constexpr uint32_t STAGE = Tile<PAIR>::STAGE, B_PART = Tile<PAIR>::B_PART;
     Ctl *ctl = d.ctl;
-    if (!ctl->active)
-        return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *stages = align1024(smem_raw);
     Sync &sy = *reinterpret_cast<Sync *>(stages + ST * STAGE);
@@ -737,8 +734,9 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0;
     const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x;
-    const int first = off[worker], last = off[worker + 1];
     setup<PAIR, ST>(sy);
+    const bool active = ctl->active;
+    const int first = off[worker], last = active ? off[worker + 1] : first;
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
@@ -1375,20 +1373,21 @@ cudaError_t to_device(T **dst, const std::vector<T> &v)
 }
 
 template <bool PAIR>
-void launch(const F32Host &h, const Dev &d, int cur, cudaStream_t s, int phase)
+cudaError_t launch_phase(const F32Host &h, const Dev &d, int cur, cudaStream_t s, int phase)
 {
     const int grid = h.grid[phase - 1];
     if (phase == 1)
-        k_f32_phase1<PAIR><<<grid, NTHREADS, p1_smem<PAIR>(), s>>>(h.maps, d, cur, h.off[0], h.items[0]);
-    else if (d.diag == 2)
-        k_f32_phase2<PAIR, true><<<grid, NTHREADS, p2_smem<PAIR, true>(), s>>>(h.maps, d, cur, h.off[1], h.items[1]);
-    else
-        k_f32_phase2<PAIR, false><<<grid, NTHREADS, p2_smem<PAIR, false>(), s>>>(h.maps, d, cur, h.off[1], h.items[1]);
+        return launch(k_f32_phase1<PAIR>, grid, NTHREADS, p1_smem<PAIR>(), s, h.maps, d, cur, h.off[0], h.items[0]);
+    if (d.diag == 2)
+        return launch(k_f32_phase2<PAIR, true>, grid, NTHREADS, p2_smem<PAIR, true>(), s, h.maps, d, cur, h.off[1],
+                            h.items[1]);
+    return launch(k_f32_phase2<PAIR, false>, grid, NTHREADS, p2_smem<PAIR, false>(), s, h.maps, d, cur, h.off[1],
+                        h.items[1]);
 }
 
 }  // namespace
 
-const char *const F32_KERNEL_NAMES[F32_KERNELS] = {"k_f32_phase1", "k_reduce_wnorms", "k_f32_phase2", "k_fin", "k_tail"};
+const char *const F32_KERNEL_NAMES[F32_KERNELS] = {"k_f32_phase1", "k_reduce_wnorms", "k_f32_phase2", "k_fin"};
 
 void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fixes, bool *pair)
 {
@@ -1448,22 +1447,18 @@ void f32_release(Dev &d)
 cudaError_t launch_iteration_f32(const Dev &d, int cur, cudaStream_t s, KernelEvents &ke)
 {
     const F32Host &h = *static_cast<const F32Host *>(d.f32_host);
+    cudaError_t e;
     ke.mark(s);
-    if (h.plan.pair)
-        launch<true>(h, d, cur, s, 1);
-    else
-        launch<false>(h, d, cur, s, 1);
-    ke.mark(s);
-    cudaError_t e = launch_reduce_wnorms(d, s);
-    if (e)
+    if ((e = h.plan.pair ? launch_phase<true>(h, d, cur, s, 1) : launch_phase<false>(h, d, cur, s, 1)))
         return e;
     ke.mark(s);
-    if (h.plan.pair)
-        launch<true>(h, d, cur ^ 1, s, 2);
-    else
-        launch<false>(h, d, cur ^ 1, s, 2);
+    if ((e = launch_reduce_wnorms(d, s)))
+        return e;
     ke.mark(s);
-    return launch_fin_tail(d, s, ke);
+    if ((e = h.plan.pair ? launch_phase<true>(h, d, cur ^ 1, s, 2) : launch_phase<false>(h, d, cur ^ 1, s, 2)))
+        return e;
+    ke.mark(s);
+    return launch_fin(d, s, ke);
 }
 
 cudaError_t f32_static_host(const Dev &d, void *lists, void **host)

@@ -1,6 +1,6 @@
 // What every path's iteration shares after its products: the norms of W'
-// (k_reduce_wnorms), the diagonals of Eq. 6 and the norms of P' and C' (k_fin),
-// h, the counter and the stop test (k_tail), for one network or a set.  Every
+// (k_reduce_wnorms), then the diagonals of Eq. 6, the norms of P' and C', h, the
+// counter and the stop test (k_fin), for one network or a set.  Every
 // reduction has a fixed order, so an iteration is deterministic.  Also the
 // FP32 FMA rate of the device (measurement support).
 #include "panda_internal.cuh"
@@ -121,85 +121,11 @@ __global__ void __launch_bounds__(RS_ROWS * RS_GROUPS) k_reduce_wnorms_set(const
     reduce_wnorms_block(devs[w.x], w.y);
 }
 
-// ---------------------------------------------------------------------------
-// Eq. 6 diagonals and the squared norms of P' and C' (32 rows per block, the
-// row partial sums added by 8 threads per row).  Blocks [0, ceil(T/32)) take
-// rows of P, the rest rows of C.
-// ---------------------------------------------------------------------------
-// block b of one network's launch: b < ceil(T/32) rows of P, the rest rows of C
-__device__ __forceinline__ void fin_block(const Dev &d, int b)
-{
-    const Ctl *ctl = d.ctl;
-    if (!ctl->active)
-        return;
-    __shared__ double sh[3][RS_GROUPS][RS_ROWS];
-    const int bT = ceil_div(d.T, RS_ROWS);
-    const bool isP = b < bT;
-    const int i = ((isP ? b : b - bT) * RS_ROWS) + (threadIdx.x & (RS_ROWS - 1));
-    const int n = isP ? d.T : d.G;       // network size
-    const bool ok = i < n;
-    const int ld = isP ? d.Tp : d.Gp;
-    const float *const src[3] = {isP ? d.ps_sum : d.cs_sum, isP ? d.ps_sq : d.cs_sq, isP ? d.ps_vsq : d.cs_vsq};
-    double sums[3];
-    if (d.narrow) {
-        // 128 x 64 tiles: a row of 64-block b has row-role partials in slots [2 (b / 2), nb) and
-        // column-role partials in [nb, nb + b / 2 + 1)
-        const int nb = ceil_div(ld, 64), b64 = ((isP ? b : b - bT) * RS_ROWS) >> 6;
-        slot_sums<3>(src, b64 & ~1, nb, nb, nb + b64 / 2 + 1, ld, i, ok, sums, sh);
-    } else {
-        // 256 x 256 tiles: a row of 256-block b has row-role partials in slots [b, nb) (tiles
-        // (b, bn >= b)) and column-role partials in [nb, nb + 2 b + 2) (tiles (bm <= b, b), one per
-        // CTA of the pair)
-        const int nb = ceil_div(ld, 256), b256 = ((isP ? b : b - bT) * RS_ROWS) >> 8;
-        slot_sums<3>(src, b256, nb, nb, nb + 2 * b256 + 2, ld, i, ok, sums, sh);
-    }
-    if (threadIdx.x >= RS_ROWS)
-        return;
-    float nrm = 0.0f;  // the row's new squared norm (0 past the network)
-    if (ok) {
-        const double s1 = sums[0], s2 = sums[1], sv = sums[2];
-        const double alpha = (double)ctl->alpha;
-        const int t = ctl->iters + 1;
-        const double growth = d.e2tab[t < HIST_CAP ? t : HIST_CAP];
-        double sigma = 0.0;  // population std of the n - 1 off-diagonal entries (0 for one entry)
-        if (n > 2) {
-            const double m = s1 / (double)(n - 1);
-            const double var = s2 / (double)(n - 1) - m * m;
-            sigma = var > 0.0 ? sqrt(var) : 0.0;
-        }
-        const double gain = d.diag == 1 ? 1.0 : alpha;  // PANDA_DIAG_D0_LITERAL has no alpha
-        const double mult = isP ? (double)d.G : (double)d.T;  // N_a with P, N_e with C
-        double *dg = isP ? d.pd : d.cd;
-        const double nd = (1.0 - alpha) * dg[i] + gain * mult * sigma * growth;
-        dg[i] = nd;
-        const float ndf = (float)nd;
-        nrm = (float)(sv + nd * nd);
-        (isP ? d.pdf : d.cdf)[i] = ndf;
-        (isP ? d.rsqP : d.csqC)[i] = nrm;
-        if (!isfinite(ndf) || !isfinite(nrm))
-            atomicOr(&d.ctl->status, ST_NONFINITE);
-    }
-    if (d.fp8)  // the whole first warp, past the network too
-        fp8_norm_max(&d.f8n[isP ? 0 : 1], nrm);
-}
-
-__global__ void __launch_bounds__(RS_ROWS * RS_GROUPS) k_fin(const __grid_constant__ Dev d)
-{
-    fin_block(d, blockIdx.x);
-}
-
-__global__ void __launch_bounds__(RS_ROWS * RS_GROUPS) k_fin_set(const Dev *devs, const int2 *blocks)
-{
-    const int2 w = blocks[blockIdx.x];
-    fin_block(devs[w.x], w.y);
-}
-
-// h (Eq. 7), the counter and the stop test: one block per network.
+// h (Eq. 7), the counter and the stop test, by the last block of a network's k_fin to finish (a
+// kernel of its own cost every iteration about 3 us at the smallest networks).
 __device__ __forceinline__ void tail_block(const Dev &d)
 {
     Ctl *ctl = d.ctl;
-    if (!ctl->active)
-        return;
     __shared__ double sh[256];
     const int n = d.nbT * d.nwr;
     double s = 0.0;
@@ -222,53 +148,127 @@ __device__ __forceinline__ void tail_block(const Dev &d)
         ctl->converged = h < ctl->tol;
         if (d.fp8) {  // the new state's norm maxima, and the scale of the next W' (Eq. 2)
             for (int q = 0; q < 4; ++q) {
-                d.f8n[4 + q] = d.f8n[q];
+                d.f8n[4 + q] = *(volatile unsigned *)&d.f8n[q];
                 d.f8n[q] = 0u;
             }
             d.f8[3] = e4m3_scale(fp8_bound_w(__uint_as_float(d.f8n[4]), __uint_as_float(d.f8n[5]),
                                              __uint_as_float(d.f8n[6]), __uint_as_float(d.f8n[7])));
         }
+        ctl->fin_blocks = 0;
+        int status = *(volatile int *)&ctl->status;  // the other blocks' findings
         if (!isfinite(h))
-            ctl->status |= ST_NONFINITE;
-        if (ctl->converged || t >= ctl->stop_at || ctl->status)
+            ctl->status = status |= ST_NONFINITE;
+        if (ctl->converged || t >= ctl->stop_at || status)
             ctl->active = 0;
     }
 }
 
-__global__ void k_tail(const __grid_constant__ Dev d) { tail_block(d); }
+// ---------------------------------------------------------------------------
+// Eq. 6 diagonals and the squared norms of P' and C' (32 rows per block, the
+// row partial sums added by 8 threads per row).  Blocks [0, ceil(T/32)) take
+// rows of P, the rest rows of C.
+// ---------------------------------------------------------------------------
+// block b of one network's launch: b < ceil(T/32) rows of P, the rest rows of C
+__device__ __forceinline__ void fin_block(const Dev &d, int b)
+{
+    const Ctl *ctl = d.ctl;
+    if (!ctl->active)  // (the network's last block clears it once every other block has passed here)
+        return;
+    __shared__ int last;
+    __shared__ double sh[3][RS_GROUPS][RS_ROWS];
+    const int bT = ceil_div(d.T, RS_ROWS);
+    const bool isP = b < bT;
+    const int i = ((isP ? b : b - bT) * RS_ROWS) + (threadIdx.x & (RS_ROWS - 1));
+    const int n = isP ? d.T : d.G;       // network size
+    const bool ok = i < n;
+    const int ld = isP ? d.Tp : d.Gp;
+    const float *const src[3] = {isP ? d.ps_sum : d.cs_sum, isP ? d.ps_sq : d.cs_sq, isP ? d.ps_vsq : d.cs_vsq};
+    double sums[3];
+    if (d.narrow) {
+        // 128 x 64 tiles: a row of 64-block b has row-role partials in slots [2 (b / 2), nb) and
+        // column-role partials in [nb, nb + b / 2 + 1)
+        const int nb = ceil_div(ld, 64), b64 = ((isP ? b : b - bT) * RS_ROWS) >> 6;
+        slot_sums<3>(src, b64 & ~1, nb, nb, nb + b64 / 2 + 1, ld, i, ok, sums, sh);
+    } else {
+        // 256 x 256 tiles: a row of 256-block b has row-role partials in slots [b, nb) (tiles
+        // (b, bn >= b)) and column-role partials in [nb, nb + 2 b + 2) (tiles (bm <= b, b), one per
+        // CTA of the pair)
+        const int nb = ceil_div(ld, 256), b256 = ((isP ? b : b - bT) * RS_ROWS) >> 8;
+        slot_sums<3>(src, b256, nb, nb, nb + 2 * b256 + 2, ld, i, ok, sums, sh);
+    }
+    float nrm = 0.0f;  // the row's new squared norm (0 past the network)
+    if (threadIdx.x < RS_ROWS && ok) {
+        const double s1 = sums[0], s2 = sums[1], sv = sums[2];
+        const double alpha = (double)ctl->alpha;
+        const int t = ctl->iters + 1;
+        const double growth = d.e2tab[t < HIST_CAP ? t : HIST_CAP];
+        double sigma = 0.0;  // population std of the n - 1 off-diagonal entries (0 for one entry)
+        if (n > 2) {
+            const double m = s1 / (double)(n - 1);
+            const double var = s2 / (double)(n - 1) - m * m;
+            sigma = var > 0.0 ? sqrt(var) : 0.0;
+        }
+        const double gain = d.diag == 1 ? 1.0 : alpha;  // PANDA_DIAG_D0_LITERAL has no alpha
+        const double mult = isP ? (double)d.G : (double)d.T;  // N_a with P, N_e with C
+        double *dg = isP ? d.pd : d.cd;
+        const double nd = (1.0 - alpha) * dg[i] + gain * mult * sigma * growth;
+        dg[i] = nd;
+        const float ndf = (float)nd;
+        nrm = (float)(sv + nd * nd);
+        (isP ? d.pdf : d.cdf)[i] = ndf;
+        (isP ? d.rsqP : d.csqC)[i] = nrm;
+        if (!isfinite(ndf) || !isfinite(nrm))
+            atomicOr(&d.ctl->status, ST_NONFINITE);
+    }
+    if (d.fp8 && threadIdx.x < RS_ROWS)  // the whole first warp, past the network too
+        fp8_norm_max(&d.f8n[isP ? 0 : 1], nrm);
+    if (threadIdx.x < RS_ROWS)
+        __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0)
+        last = atomicAdd(&d.ctl->fin_blocks, 1u) + 1u == (unsigned)(bT + ceil_div(d.G, RS_ROWS));
+    __syncthreads();
+    if (last) {
+        __threadfence();
+        tail_block(d);
+    }
+}
 
-__global__ void k_tail_set(const Dev *devs) { tail_block(devs[blockIdx.x]); }
+__global__ void __launch_bounds__(RS_ROWS * RS_GROUPS) k_fin(const __grid_constant__ Dev d)
+{
+    fin_block(d, blockIdx.x);
+}
+
+__global__ void __launch_bounds__(RS_ROWS * RS_GROUPS) k_fin_set(const Dev *devs, const int2 *blocks)
+{
+    const int2 w = blocks[blockIdx.x];
+    fin_block(devs[w.x], w.y);
+}
 
 }  // namespace
 
 cudaError_t launch_reduce_wnorms(const Dev &d, cudaStream_t s)
 {
-    k_reduce_wnorms<<<ceil_div(d.T, RS_ROWS) + ceil_div(d.G, RS_ROWS), RS_ROWS * RS_GROUPS, 0, s>>>(d);
-    return cudaGetLastError();
+    return launch(k_reduce_wnorms, set_norm_blocks(d.T, d.G), RS_ROWS * RS_GROUPS, 0, s, d);
 }
 
 cudaError_t launch_reduce_wnorms_set(const Dev *devs, const int2 *blocks, int nblocks, cudaStream_t s)
 {
-    k_reduce_wnorms_set<<<nblocks, RS_ROWS * RS_GROUPS, 0, s>>>(devs, blocks);
-    return cudaGetLastError();
+    return launch(k_reduce_wnorms_set, nblocks, RS_ROWS * RS_GROUPS, 0, s, devs, blocks);
 }
 
-cudaError_t launch_fin_tail_set(const Dev *devs, const int2 *blocks, int nblocks, int nnets, cudaStream_t s)
+cudaError_t launch_fin_set(const Dev *devs, const int2 *blocks, int nblocks, cudaStream_t s)
 {
-    k_fin_set<<<nblocks, RS_ROWS * RS_GROUPS, 0, s>>>(devs, blocks);
-    k_tail_set<<<nnets, 256, 0, s>>>(devs);
-    return cudaGetLastError();
+    return launch(k_fin_set, nblocks, RS_ROWS * RS_GROUPS, 0, s, devs, blocks);
 }
 
 int set_norm_blocks(int T, int G) { return ceil_div(T, RS_ROWS) + ceil_div(G, RS_ROWS); }
 
-cudaError_t launch_fin_tail(const Dev &d, cudaStream_t s, KernelEvents &ke)
+cudaError_t launch_fin(const Dev &d, cudaStream_t s, KernelEvents &ke)
 {
-    k_fin<<<ceil_div(d.T, RS_ROWS) + ceil_div(d.G, RS_ROWS), RS_ROWS * RS_GROUPS, 0, s>>>(d);
+    cudaError_t e = launch(k_fin, set_norm_blocks(d.T, d.G), RS_ROWS * RS_GROUPS, 0, s, d);
     ke.mark(s);
-    k_tail<<<1, 256, 0, s>>>(d);
-    ke.mark(s);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace panda

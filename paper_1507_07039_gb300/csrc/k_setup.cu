@@ -5,6 +5,8 @@
 //
 // Every reduction here runs with a fixed grid and a fixed summation order, so
 // results are identical from run to run.
+#include <algorithm>
+
 #include "panda_internal.cuh"
 
 namespace panda {
@@ -202,12 +204,12 @@ __device__ __forceinline__ void put_parts(const Parts &t, size_t o, const float 
 }
 
 // W (rows x cols, row stride ldi) into out (row stride ldo, a multiple of 4) and
-// its parts, zeros in the padding (row gridDim.y - 1, column ldo - 1 the last);
-// block y takes a row, 1024 columns per block.  X may be out itself.
-__global__ void k_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo, Parts parts,
-                         int *flags)
+// its parts, zeros in the padding (column ldo - 1 the last);
+// block (x, y) takes 1024 columns of row y.  X may be out itself.
+__device__ __forceinline__ void load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int ldo,
+                                       const Parts &parts, int *flags, int x, int r)
 {
-    const int r = blockIdx.y, c = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int c = 4 * (x * blockDim.x + threadIdx.x);
     int bad = 0;
     if (c < ldo) {
         float v[4];
@@ -235,14 +237,16 @@ __global__ void k_load_w(const float *X, int rows, int cols, int ldi, const doub
 // diagonal goes to out.d and out.df and reads as zero in F and the parts.  X
 // may be out.F itself (each block pair is one block's alone).  256 threads.
 constexpr int LB = 64;
-__global__ void __launch_bounds__(256) k_load_sym(const float *X, int n, int ldi, int npairs, const double *stats, SymOut out,
-                                                  int *flags)
+__host__ __device__ inline int block_pairs(int ld) { return ceil_div(ld, LB) * (ceil_div(ld, LB) + 1) / 2; }
+__device__ __forceinline__ void load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags,
+                                         int first, int step)
 {
+    const int npairs = block_pairs(out.ld);
     __shared__ float a[LB][LB + 1], b[LB][LB + 1];
     const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // loads: 4 rows of 64
     const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // stores: 16 rows of 16 x 4
     int bad = 0, asym = 0;
-    for (int t = blockIdx.x; t < npairs; t += gridDim.x) {
+    for (int t = first; t < npairs; t += step) {
         // pairs are numbered column by column of the upper triangle; 8t + 1 < 2^24 for n <= 46000, so the
         // FP32 square root is close; the loops correct it
         int bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
@@ -326,6 +330,22 @@ __global__ void __launch_bounds__(256) k_load_sym(const float *X, int n, int ldi
     }
 }
 
+// One launch: blocks [0, nc) C, [nc, nc + np) P, the rest W.
+__global__ void __launch_bounds__(256) k_load(const __grid_constant__ StateIn in, float *W, Parts wparts, int Gp,
+                                              const __grid_constant__ SymOut P, const __grid_constant__ SymOut C, int nc,
+                                              int np, int *flags)
+{
+    const int b = blockIdx.x;
+    if (b < nc) {
+        load_sym(in.C, in.G, in.ldc, in.sc, C, flags, b, nc);
+    } else if (b < nc + np) {
+        load_sym(in.P, in.T, in.ldp, in.sp, P, flags, b - nc, np);
+    } else {
+        const int q = b - nc - np, xb = ceil_div(Gp, 1024);
+        load_w(in.W, in.T, in.G, in.ldw, in.sw, W, Gp, wparts, flags, q % xb, q / xb);
+    }
+}
+
 __global__ void k_diag_to_float(const double *d, float *df, int n)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -360,13 +380,14 @@ __device__ __forceinline__ void sq_add(float x, float &acc, float &cmp)
 // per row, lane l taking the 4-wide column groups l, l + 32, ..., then the
 // ragged columns.  Compensated FP32 pairs folded into an FP64 total every 16
 // groups, FP64 across the warp: a fixed order.
-__global__ void k_row_norms(const float *__restrict__ X, int rows, int cols, int ld, bool aligned, const double *stats,
-                            const double *diag, float *out)
+__device__ __forceinline__ void row_norms(const float *__restrict__ X, int rows, int cols, int ld, const double *stats,
+                                          const double *diag, float *out, int block)
 {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int warp = block * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (warp >= rows)
         return;
+    const bool aligned = (ld & 3) == 0 && ((uintptr_t)X & 15) == 0;
     const float *x = X + (size_t)warp * ld;
     const int c4n = cols >> 2, skip = diag ? warp : -1;
     const float4 q = stats ? stats_pairs(stats) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -408,10 +429,10 @@ __global__ void k_row_norms(const float *__restrict__ X, int rows, int cols, int
 // norms of a row-major matrix without its transpose.  A block takes 32
 // columns, its eight warps every eighth row (compensated FP32 pairs folded
 // into FP64 every 32 of them), FP64 across the warps in a fixed order.
-__global__ void __launch_bounds__(256) k_col_norms(const float *__restrict__ X, int rows, int cols, int ld, float *out)
+__device__ __forceinline__ void col_norms(const float *__restrict__ X, int rows, int cols, int ld, float *out, int block)
 {
     __shared__ double sh[8][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = block * 32 + lane;
     double tot = 0.0;
     if (j < cols)
         for (int r0 = w; r0 < rows; r0 += 256) {
@@ -430,6 +451,21 @@ __global__ void __launch_bounds__(256) k_col_norms(const float *__restrict__ X, 
             t += sh[q][lane];
         out[j] = (float)t;
     }
+}
+
+// One launch: blocks of 8 rows of C, then of P, then of W, then of 32 columns of W.
+__global__ void __launch_bounds__(256) k_norms(const __grid_constant__ StateNorms n)
+{
+    const StateIn &in = n.in;
+    const int bG = ceil_div(in.G, 8), bT = ceil_div(in.T, 8), b = blockIdx.x;
+    if (b < bG)
+        row_norms(in.C, in.G, in.G, in.ldc, in.sc, n.cd, n.csqC, b);
+    else if (b < bG + bT)
+        row_norms(in.P, in.T, in.T, in.ldp, in.sp, n.pd, n.rsqP, b - bG);
+    else if (b < bG + 2 * bT)
+        row_norms(in.W, in.T, in.G, in.ldw, nullptr, nullptr, n.rsqW, b - bG - bT);
+    else
+        col_norms(in.W, in.T, in.G, in.ldw, n.csqW, b - bG - 2 * bT);
 }
 
 // Lower triangle from the upper one: X[r][c] = X[c][r] for r > c (32 x 32
@@ -501,35 +537,20 @@ __global__ void k_standardize_rows(const float *__restrict__ X, int G, int N, __
     }
 }
 
-__device__ __forceinline__ bool faulted(const Guard &g)
-{
-    return g.flags && (g.flags[0] | g.flags[1] | g.ctl->status);
-}
-
-__global__ void k_store_w(const float *__restrict__ X, int cols, int ldi, float *__restrict__ out, Guard g)
-{
-    if (faulted(g))
-        return;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x)
-        out[(size_t)blockIdx.y * cols + c] = X[(size_t)blockIdx.y * ldi + c];
-}
-
-// The full symmetric n x n matrix (row stride ldo, any alignment) from its
+// The full symmetric n x n matrix (dense, any alignment) from its
 // strict upper triangle, FP32 in X or a BF16 split pair H + L (exact in FP32;
 // row stride ldi, a multiple of 4), and its FP64 diagonal, in 64 x 64 blocks:
 // each block above the diagonal is read once and written twice, the second
 // time turned through shared memory.  256 threads.
-__global__ void __launch_bounds__(256) k_store_sym(const float *__restrict__ X, const __nv_bfloat16 *__restrict__ H,
-                                                   const __nv_bfloat16 *__restrict__ L, int n, int ldi, int npairs,
-                                                   const double *__restrict__ diag, float *__restrict__ out, int ldo,
-                                                   Guard g)
+__device__ __forceinline__ void store_sym(const float *__restrict__ X, const __nv_bfloat16 *__restrict__ H,
+                                          const __nv_bfloat16 *__restrict__ L, int n, int ldi,
+                                          const double *__restrict__ diag, float *__restrict__ out, int first, int step)
 {
-    if (faulted(g))
-        return;
+    const int npairs = block_pairs(n), ldo = n;
     __shared__ float a[LB][LB + 1];
     const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // stores: 4 rows of 64
     const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // loads: 16 rows of 16 x 4
-    for (int t = blockIdx.x; t < npairs; t += gridDim.x) {
+    for (int t = first; t < npairs; t += step) {
         int bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);  // as in k_load_sym
         while (bj > 0 && bj * (bj + 1) / 2 > t)
             --bj;
@@ -573,6 +594,24 @@ __global__ void __launch_bounds__(256) k_store_sym(const float *__restrict__ X, 
     }
 }
 
+// One launch: blocks [0, nc) C, [nc, nc + np) P, the rest rows of W.
+__global__ void __launch_bounds__(256) k_store(const __grid_constant__ StateOut o, int nc, int np)
+{
+    if (o.flags && (o.flags[0] | o.flags[1] | o.ctl->status))
+        return;
+    const int b = blockIdx.x;
+    if (b < nc) {
+        store_sym(o.C, o.Ch, o.Cl, o.G, o.Gp, o.cd, o.oC, b, nc);
+    } else if (b < nc + np) {
+        store_sym(o.P, nullptr, nullptr, o.T, o.Tp, o.pd, o.oP, b - nc, np);
+    } else {
+        const int r = b - nc - np;
+#pragma unroll 4
+        for (int c = threadIdx.x; c < o.G; c += 256)
+            o.oW[(size_t)r * o.G + c] = o.W[(size_t)r * o.Gp + c];
+    }
+}
+
 // X_ii = 1 for i < n (a correlation matrix's diagonal)
 __global__ void k_unit_diag(float *X, int n, int ld)
 {
@@ -596,17 +635,13 @@ cudaError_t launch_unit_diag(float *X, int n, int ld, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_store_sym(const float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi,
-                             const double *diag, float *out, int ldo, Guard g, cudaStream_t s)
+cudaError_t launch_store(const StateOut &o, cudaStream_t s)
 {
-    const int nb = ceil_div(n, LB), npairs = nb * (nb + 1) / 2;
-    k_store_sym<<<npairs < 152 * 12 ? npairs : 152 * 12, 256, 0, s>>>(X, H, L, n, ldi, npairs, diag, out, ldo, g);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_store_w(const float *X, int rows, int cols, int ldi, float *out, Guard g, cudaStream_t s)
-{
-    k_store_w<<<dim3(ceil_div(cols, 1024), rows), 256, 0, s>>>(X, cols, ldi, out, g);
+    const int nc = o.oC ? std::min(block_pairs(o.G), 152 * 12) : 0, np = o.oP ? std::min(block_pairs(o.T), 152 * 4) : 0;
+    const int n = nc + np + (o.oW ? o.T : 0);
+    if (n == 0)
+        return cudaSuccess;
+    k_store<<<n, 256, 0, s>>>(o, nc, np);
     return cudaGetLastError();
 }
 
@@ -634,17 +669,17 @@ cudaError_t launch_stats(const float *X, int rows, int cols, int ld, double *sta
     return cudaGetLastError();
 }
 
-cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int rows_p, int ldo,
-                          const Parts &parts, int *flags, cudaStream_t s)
+cudaError_t launch_load(const StateIn &in, float *W, const Parts &wparts, int Tp, int Gp, const SymOut &P, const SymOut &C,
+                        int *flags, cudaStream_t s)
 {
-    k_load_w<<<dim3(ceil_div(ldo, 1024), rows_p), 256, 0, s>>>(X, rows, cols, ldi, stats, out, ldo, parts, flags);
+    const int nc = std::min(block_pairs(C.ld), 152 * 6), np = std::min(block_pairs(P.ld), 152 * 2);
+    k_load<<<nc + np + Tp * ceil_div(Gp, 1024), 256, 0, s>>>(in, W, wparts, Gp, P, C, nc, np, flags);
     return cudaGetLastError();
 }
 
-cudaError_t launch_load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags, cudaStream_t s)
+cudaError_t launch_norms(const StateNorms &n, cudaStream_t s)
 {
-    const int nb = ceil_div(out.ld, LB), npairs = nb * (nb + 1) / 2;
-    k_load_sym<<<npairs < 152 * 6 ? npairs : 152 * 6, 256, 0, s>>>(X, n, ldi, npairs, stats, out, flags);
+    k_norms<<<ceil_div(n.in.G, 8) + 2 * ceil_div(n.in.T, 8) + ceil_div(n.in.G, 32), 256, 0, s>>>(n);
     return cudaGetLastError();
 }
 
@@ -658,19 +693,6 @@ cudaError_t launch_transpose(const float *X, int rows_p, int cols_p, float *Y, c
 {
     dim3 grid(cols_p / 32, rows_p / 32), block(32, 8);
     k_transpose<<<grid, block, 0, s>>>(X, rows_p, cols_p, Y);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_row_norms(const float *X, int rows, int cols, int ld, const double *stats, const double *diag,
-                             float *out, cudaStream_t s)
-{
-    k_row_norms<<<ceil_div(rows * 32, 256), 256, 0, s>>>(X, rows, cols, ld, rows_aligned(X, ld), stats, diag, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_col_norms(const float *X, int rows, int cols, int ld, float *out, cudaStream_t s)
-{
-    k_col_norms<<<ceil_div(cols, 32), 256, 0, s>>>(X, rows, cols, ld, out);
     return cudaGetLastError();
 }
 

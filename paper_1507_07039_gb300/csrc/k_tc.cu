@@ -18,7 +18,7 @@
 //                 C: both only inside diagonal 256-blocks), row partial sums
 //                 for Eq. 6.  (Only the upper triangle of FP32 P and C is ever
 //                 read here; panda_get and panda_save mirror it first.)
-//   k_fin, k_tail (shared): Eq. 6 diagonals, norms, h, stop test.
+//   k_fin (shared): Eq. 6 diagonals, norms, h, stop test.
 //
 // P and C are symmetric.  "P_off rows" are read K-major from the full split
 // copy.  For "C_off rows" j against genes k, the availability product reads
@@ -45,7 +45,7 @@
 namespace panda {
 
 const char *const TC_KERNEL_NAMES[TC_KERNELS] = {"k_tc_phase1", "k_reduce_wnorms", "k_tc_phase2",
-                                                 "k_fin", "k_tail"};
+                                                 "k_fin"};
 
 namespace {
 
@@ -1020,12 +1020,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS1, 1)
     k_tc_phase1(const __grid_constant__ TcMaps maps, const __grid_constant__ Dev d, int cur, const int4 *items,
                 const int *off)
 {
-    if (!d.ctl->active)  // both CTAs of a pair see the same value and leave together
-        return;
     phase1_tmem_alloc();
     int g = 0, tile = 0, u[2] = {0, 0};
     const int pair = blockIdx.x >> 1, rank = (int)cluster_ctarank();
-    for (int q = off[pair]; q < off[pair + 1]; ++q) {
+    const bool active = d.ctl->active;  // both CTAs of a pair see the same value
+    for (int q = off[pair]; active && q < off[pair + 1]; ++q) {
         const int4 w = items[q];
         const bool cut = w.w >= 0;
         float *scr = cut ? d.p1_fix + (size_t)(2 * w.w + rank) * P1_SLOT : d.p1_acc + (size_t)blockIdx.x * P1_SLOT;
@@ -1171,7 +1170,8 @@ struct P2One {
     __device__ const Dev &dev(int) const { return d; }
     __device__ const TcMaps &maps(int) const { return m; }
     __device__ int cur(int) const { return c; }  // the W' buffer (the launch passes it)
-    __device__ bool active(int) const { return true; }  // the kernel left at once otherwise
+    __device__ bool active(int) const { return true; }  // no tile runs otherwise
+    __device__ bool any() const { return d.ctl->active != 0; }
 };
 struct P2Set {
     const SetArgs &a;
@@ -1183,6 +1183,7 @@ struct P2Set {
     // phase 2 works on W' (the other buffer: the count moves on only in k_tail)
     __device__ int cur(int k) const { return set_cur(a, k) ^ 1; }
     __device__ bool active(int k) const { return a.devs[k].ctl->active != 0; }
+    __device__ bool any() const { return true; }
 };
 
 // The body of phase 2 for one CTA pair's scheduled tiles.  A stopped network's
@@ -1206,7 +1207,6 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int pair = blockIdx.x >> 1;
-    const int first = src.off[pair], last = src.off[pair + 1];
 
     if (threadIdx.x == 0) {
         for (int q = 0; q < ST2; ++q) {
@@ -1227,6 +1227,7 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
     tc_fence_before();
     cluster_sync();  // both CTAs' barriers exist before any cross-CTA signal
     tc_fence_after();
+    const int first = src.off[pair], last = src.any() ? src.off[pair + 1] : first;
 
     if (warp == 0) {
         if (lane == 0) {  // ---- TMA producer (both CTAs; completion counted on the even CTA) ----
@@ -1715,8 +1716,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EPI, 1)
     k_tc_phase2(const __grid_constant__ TcMaps maps, const __grid_constant__ Dev d, int cur,
                 const int *__restrict__ sched_off, const int *__restrict__ sched)
 {
-    if (!d.ctl->active)  // both CTAs of a pair see the same value and leave together
-        return;
     phase2_pair<SIM_SIGMA, EPI>(P2One{maps, d, cur, sched_off, sched}, d.ctl);
 }
 
@@ -2017,21 +2016,22 @@ cudaError_t phase2_smem_limits()
 int p2_epi(long long mma_slots) { return mma_slots > 64 ? 8 : 12; }
 
 // One phase-2 launch of EPI epilogue warps
-template <int EPI, class... Args>
-void launch_p2_one(bool sim, int grid, cudaStream_t s, const Args &...args)
+template <int EPI>
+cudaError_t launch_p2_one(bool sim, int grid, cudaStream_t s, const TcMaps &m, const Dev &d, int cur, const int *off,
+                          const int *tiles)
 {
     if (sim)
-        k_tc_phase2<true, EPI><<<grid, P2Cfg<true, EPI>::THREADS, phase2_smem<true, EPI>(), s>>>(args...);
-    else
-        k_tc_phase2<false, EPI><<<grid, P2Cfg<false, EPI>::THREADS, phase2_smem<false, EPI>(), s>>>(args...);
+        return launch(k_tc_phase2<true, EPI>, grid, P2Cfg<true, EPI>::THREADS, phase2_smem<true, EPI>(), s, m, d, cur,
+                            off, tiles);
+    return launch(k_tc_phase2<false, EPI>, grid, P2Cfg<false, EPI>::THREADS, phase2_smem<false, EPI>(), s, m, d, cur,
+                        off, tiles);
 }
 template <int EPI>
-void launch_p2_set(bool sim, int grid, cudaStream_t s, const SetArgs &a)
+cudaError_t launch_p2_set(bool sim, int grid, cudaStream_t s, const SetArgs &a)
 {
     if (sim)
-        k_tc_phase2_set<true, EPI><<<grid, P2Cfg<true, EPI>::THREADS, phase2_smem<true, EPI>(), s>>>(a);
-    else
-        k_tc_phase2_set<false, EPI><<<grid, P2Cfg<false, EPI>::THREADS, phase2_smem<false, EPI>(), s>>>(a);
+        return launch(k_tc_phase2_set<true, EPI>, grid, P2Cfg<true, EPI>::THREADS, phase2_smem<true, EPI>(), s, a);
+    return launch(k_tc_phase2_set<false, EPI>, grid, P2Cfg<false, EPI>::THREADS, phase2_smem<false, EPI>(), s, a);
 }
 
 cudaError_t set_smem_limits()
@@ -2227,19 +2227,19 @@ cudaError_t launch_iteration_tc(const Dev &d, int cur, cudaStream_t s, KernelEve
 {
     const TcHost &h = *static_cast<const TcHost *>(d.tc_host);
     const TcMaps &m = h.maps;
+    cudaError_t e;
     ke.mark(s);
-    k_tc_phase1<<<h.grid1, THREADS1, phase1_smem(), s>>>(m, d, cur, h.p1_items, h.p1_off);
-    ke.mark(s);
-    cudaError_t e = launch_reduce_wnorms(d, s);
-    if (e)
+    if ((e = launch(k_tc_phase1, h.grid1, THREADS1, phase1_smem(), s, m, d, cur, h.p1_items, h.p1_off)))
         return e;
     ke.mark(s);
-    if (h.epi2 == 8)
-        launch_p2_one<8>(d.diag == 2, h.grid2, s, m, d, cur ^ 1, h.sched_off, h.sched);
-    else
-        launch_p2_one<12>(d.diag == 2, h.grid2, s, m, d, cur ^ 1, h.sched_off, h.sched);
+    if ((e = launch_reduce_wnorms(d, s)))
+        return e;
     ke.mark(s);
-    return launch_fin_tail(d, s, ke);
+    if ((e = h.epi2 == 8 ? launch_p2_one<8>(d.diag == 2, h.grid2, s, m, d, cur ^ 1, h.sched_off, h.sched)
+                         : launch_p2_one<12>(d.diag == 2, h.grid2, s, m, d, cur ^ 1, h.sched_off, h.sched)))
+        return e;
+    ke.mark(s);
+    return launch_fin(d, s, ke);
 }
 
 // ---- sets of networks: one launch per phase over all networks' tiles ---------------
@@ -2360,22 +2360,21 @@ cudaError_t tc_set_launch(TcSet *t, int p1, int p2, cudaStream_t s, cudaEvent_t 
     SetArgs a{t->devs, t->maps, t->parity, a1.items, a1.off, t->acc, nullptr, nullptr, nullptr};
     if (ev0)
         cudaEventRecord(ev0, s);
-    k_tc_phase1_set<<<2 * t->pairs, THREADS1, phase1_smem(), s>>>(a);
-    cudaError_t e = launch_reduce_wnorms_set(t->devs, t->blocks, t->nblocks, s);
-    if (e)
+    cudaError_t e;
+    if ((e = launch(k_tc_phase1_set, 2 * t->pairs, THREADS1, phase1_smem(), s, a)) ||
+        (e = launch_reduce_wnorms_set(t->devs, t->blocks, t->nblocks, s)))
         return e;
     if (ev1)
         cudaEventRecord(ev1, s);
     a.sched_off = c.off;
     a.sched = c.tiles;
     a.sched_net = c.nets;
-    if (c.epi2 == 8)
-        launch_p2_set<8>(t->diag == 2, 2 * c.pairs, s, a);
-    else
-        launch_p2_set<12>(t->diag == 2, 2 * c.pairs, s, a);
+    if ((e = c.epi2 == 8 ? launch_p2_set<8>(t->diag == 2, 2 * c.pairs, s, a)
+                         : launch_p2_set<12>(t->diag == 2, 2 * c.pairs, s, a)))
+        return e;
     if (ev2)
         cudaEventRecord(ev2, s);
-    return launch_fin_tail_set(t->devs, t->blocks, t->nblocks, t->n, s);
+    return launch_fin_set(t->devs, t->blocks, t->nblocks, s);
 }
 
 cudaError_t tc_set_gather(TcSet *t, Ctl *host, cudaStream_t s)

@@ -343,21 +343,21 @@ int load_state(panda_ctx *c, const float *W, const float *P, const float *C, int
     }
     const bool f32 = c->prec == PANDA_FP32;
     CU(cudaMemsetAsync(c->d_flags, 0, 4 * sizeof(int), c->stream));
-    CU(launch_load_w(w.src, T, G, w.ld, st[0], d.W[c->cur], c->Tp, c->Gp, Parts{d.Wh[c->cur], d.Wm[c->cur], d.Wl[c->cur]},
-                     c->d_flags, c->stream));
     // a network loaded in place keeps both triangles, for the norms below; FP8MIX's E4M3 copy of C is made from both
     const SymOut po{d.Poff, p.src == d.Poff, Parts{d.Ph, d.Pm, d.Pl}, 1, 256, c->Tp, d.pd, d.pdf};
     const SymOut xo{d.c_split ? nullptr : d.Coff, d.fp8 || x.src == d.Coff,
                     Parts{d.Ch, d.Cm, d.Cl}, 0, f32 ? f32_diag_block(d) : 256, c->Gp, d.cd, d.cdf};
-    CU(launch_load_sym(p.src, T, p.ld, st[1], po, c->d_flags, c->stream));
-    CU(launch_load_sym(x.src, G, x.ld, st[2], xo, c->d_flags, c->stream));
-    CU(launch_row_norms(d.W[c->cur], T, G, c->Gp, nullptr, nullptr, d.rsqW, c->stream));
+    StateIn in{w.src, p.src, x.src, T, G, w.ld, p.ld, x.ld, st[0], st[1], st[2]};
+    CU(launch_load(in, d.W[c->cur], Parts{d.Wh[c->cur], d.Wm[c->cur], d.Wl[c->cur]}, c->Tp, c->Gp, po, xo, c->d_flags,
+                   c->stream));
     if (d.Wt[c->cur])
         CU(launch_transpose(d.W[c->cur], c->Tp, c->Gp, d.Wt[c->cur], c->stream));
-    CU(launch_col_norms(d.W[c->cur], T, G, c->Gp, d.csqW, c->stream));
-    // from the same entries as loaded: in place they are Z-scored by now
-    CU(launch_row_norms(p.src, T, T, p.ld, p.src == d.Poff ? nullptr : st[1], d.pd, d.rsqP, c->stream));
-    CU(launch_row_norms(x.src, G, G, x.ld, xo.F && x.src == xo.F ? nullptr : st[2], d.cd, d.csqC, c->stream));
+    // norms of the same entries as loaded: those loaded in place are Z-scored by now
+    in.W = d.W[c->cur];
+    in.ldw = c->Gp;
+    in.sp = p.src == d.Poff ? nullptr : st[1];
+    in.sc = xo.F && x.src == xo.F ? nullptr : st[2];
+    CU(launch_norms(StateNorms{in, d.pd, d.cd, d.rsqW, d.csqW, d.rsqP, d.csqC}, c->stream));
     if (tensor_prec(c->prec))
         CU(tc_prepare(d, c->cur, c->stream, false));
     else
@@ -400,9 +400,9 @@ const char *kernel_name(const panda_ctx *c, int i)
 }
 
 // slot: which iteration of a graph (or chunk) this is, for the timing events
-int launch_iteration(panda_ctx *c, int cur, int slot)
+int launch_iteration(panda_ctx *c, int cur, int slot, bool capturing = false)
 {
-    KernelEvents ke{c->prof ? c->ev.data() + (size_t)slot * (n_kernels(c) + 1) : nullptr, 0};
+    KernelEvents ke{c->prof ? c->ev.data() + (size_t)slot * (n_kernels(c) + 1) : nullptr, 0, capturing};
     cudaError_t e = tensor_prec(c->prec) ? launch_iteration_tc(c->d, cur, c->stream, ke)
                                             : launch_iteration_f32(c->d, cur, c->stream, ke);
     if (e != cudaSuccess)
@@ -418,7 +418,7 @@ int ensure_graph(panda_ctx *c, int cur)
     CU(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     int rc = 0;
     for (int k = 0; k < c->graph_iters && !rc; ++k)
-        rc = launch_iteration(c, cur ^ (k & 1), k);
+        rc = launch_iteration(c, cur ^ (k & 1), k, true);
     cudaError_t e = cudaStreamEndCapture(c->stream, &g);
     if (rc) {
         if (g)
@@ -493,7 +493,9 @@ int drive_launch(panda_ctx *c, DriveState &ds)
     ds.before = h.iters;
     const int cur = c->cur ^ ((ds.before - ds.start) & 1);
     int rc;
-    if (ds.use_graph) {
+    // (a graph runs graph_iters iterations; fewer than that left are launched one by one: the rest of
+    // a graph would be kernels that find nothing to do, 1.5 us each)
+    if (ds.use_graph && h.stop_at - ds.before >= c->graph_iters) {
         if ((rc = ensure_graph(c, cur)))
             return rc;
         CU(cudaGraphLaunch(c->gexec[cur], c->stream));
@@ -836,54 +838,60 @@ static int full_matrices(panda_ctx *c)
     return 0;
 }
 
-// Network X (P or C) into dst (n x n, dense).  Device memory: one kernel mirrors
-// the upper triangle, puts the diagonal in and writes dst.  Host memory: a C held
-// as its split pair the same way through a temporary device buffer; an FP32
-// matrix is mirrored where it is and copied, its diagonal put in on the host.
-static int get_sym(panda_ctx *c, float *dst, float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, const double *diag,
-                   int n, int ld)
-{
-    if (device_pointer(dst)) {
-        CU(launch_store_sym(X, H, L, n, ld, diag, dst, n, Guard{}, c->stream));
-        return 0;
-    }
-    if (!X) {
-        float *tmp = nullptr;
-        CU(cudaMalloc(&tmp, sizeof(float) * (size_t)n * n));
-        cudaError_t e = launch_store_sym(X, H, L, n, ld, diag, tmp, n, Guard{}, c->stream);
-        if (!e)
-            e = cudaMemcpyAsync(dst, tmp, sizeof(float) * (size_t)n * n, cudaMemcpyDeviceToHost, c->stream);
-        if (!e)
-            e = cudaStreamSynchronize(c->stream);
-        cudaFree(tmp);
-        CU(e);
-        return 0;
-    }
-    CU(launch_symmetrize(X, n, ld, c->stream));
-    if (int rc = download(c, dst, X, ld, n, n))
-        return rc;
-    std::vector<double> dg(n);
-    CU(cudaMemcpyAsync(dg.data(), diag, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaStreamSynchronize(c->stream));
-    for (int i = 0; i < n; ++i)
-        dst[(size_t)i * (n + 1)] = (float)dg[i];
-    return 0;
-}
-
+// The networks into dense arrays (each may be NULL).  Those in device memory: one
+// launch mirrors the upper triangles, puts the diagonals in and writes them all.
+// Host memory: W is copied; a C held as its split pair is written so into a
+// temporary device buffer and copied; an FP32 matrix is mirrored where it is
+// and copied, its diagonal put in on the host.
 static int get_impl(panda_ctx *c, float *W, float *P, float *C)
 {
     if (int rc = check_state(c))
         return rc;
     Dev &d = c->d;
-    int rc = 0;
-    if (W && (rc = download(c, W, d.W[c->cur], c->Gp, c->T, c->G)))
-        return rc;
-    if (P && (rc = get_sym(c, P, d.Poff, nullptr, nullptr, d.pd, c->T, c->Tp)))
-        return rc;
-    if (C && (rc = get_sym(c, C, d.c_split ? nullptr : d.Coff, d.Ch, d.Cl, d.cd, c->G, c->Gp)))
-        return rc;
-    CU(cudaStreamSynchronize(c->stream));
-    return 0;
+    StateOut o{c->T, c->G, c->Tp, c->Gp, d.W[c->cur], d.Poff, d.c_split ? nullptr : d.Coff, d.Ch, d.Cl, d.pd, d.cd,
+               nullptr, nullptr, nullptr, nullptr, nullptr};
+    if (W && device_pointer(W))
+        o.oW = W, W = nullptr;
+    if (P && device_pointer(P))
+        o.oP = P, P = nullptr;
+    float *tmp = nullptr;
+    if (C && device_pointer(C)) {
+        o.oC = C, C = nullptr;
+    } else if (C && d.c_split) {
+        CU(cudaMalloc(&tmp, sizeof(float) * (size_t)c->G * c->G));
+        o.oC = tmp;
+    }
+    std::vector<double> dg[2];
+    auto rest = [&]() -> int {
+        CU(launch_store(o, c->stream));
+        if (W)
+            if (int rc = download(c, W, d.W[c->cur], c->Gp, c->T, c->G))
+                return rc;
+        if (tmp)
+            CU(cudaMemcpyAsync(C, tmp, sizeof(float) * (size_t)c->G * c->G, cudaMemcpyDeviceToHost, c->stream));
+        struct { float *dst, *X; const double *diag; int n, ld; } sym[2] = {{P, d.Poff, d.pd, c->T, c->Tp},
+                                                                             {tmp ? nullptr : C, d.Coff, d.cd, c->G, c->Gp}};
+        for (int q = 0; q < 2; ++q) {
+            if (!sym[q].dst)
+                continue;
+            CU(launch_symmetrize(sym[q].X, sym[q].n, sym[q].ld, c->stream));
+            if (int rc = download(c, sym[q].dst, sym[q].X, sym[q].ld, sym[q].n, sym[q].n))
+                return rc;
+            dg[q].resize(sym[q].n);
+            CU(cudaMemcpyAsync(dg[q].data(), sym[q].diag, sym[q].n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        }
+        CU(cudaStreamSynchronize(c->stream));
+        for (int q = 0; q < 2; ++q)
+            for (size_t i = 0; i < dg[q].size(); ++i)
+                sym[q].dst[i * (sym[q].n + 1)] = (float)dg[q][i];
+        return 0;
+    };
+    const int rc = rest();
+    if (tmp) {
+        cudaStreamSynchronize(c->stream);
+        cudaFree(tmp);
+    }
+    return rc;
 }
 
 int panda_get(panda_ctx *c, float *W, float *P, float *C)
@@ -1265,7 +1273,8 @@ float median3(const float (&v)[panda_batch::TUNE_REPS])
 // candidate with the default phase 2, the fastest by median kept, then of each
 // phase-2 candidate); afterwards the captured graph with the chosen pair.
 // Every schedule gives the same results.  Then all control blocks are read back.
-int batch_chunk(panda_batch *b)
+// left: the most iterations any network may still run; fewer than a graph's are launched one by one.
+int batch_chunk(panda_batch *b, int left)
 {
     cudaError_t e;
     constexpr int R = panda_batch::TUNE_REPS;
@@ -1281,6 +1290,10 @@ int batch_chunk(panda_batch *b)
         }
         if ((e = tc_set_launch(b->set, p1, p2, b->stream, b->ev[0], b->ev[1], b->ev[2])))
             return b->err = std::string("set launch: ") + cudaGetErrorString(e), PANDA_ECUDA;
+    } else if (left < b->graph_iters) {
+        for (int k = 0; k < left; ++k)
+            if ((e = tc_set_launch(b->set, b->p1, b->p2, b->stream, nullptr, nullptr, nullptr)))
+                return b->err = std::string("set launch: ") + cudaGetErrorString(e), PANDA_ECUDA;
     } else {
         int rc = batch_graph(b);
         if (rc)
@@ -1333,13 +1346,17 @@ int batch_run_set(panda_batch *b, float alpha, double tol, int max_iter, int *it
     if (e)
         return b->err = std::string("set parity: ") + cudaGetErrorString(e), PANDA_ECUDA;
     bool any = max_iter > 0;
-    int rc = 0;
+    int rc = 0, left = max_iter;
     while (any && !rc) {
-        if ((rc = batch_chunk(b)))
+        if ((rc = batch_chunk(b, left)))
             break;
         any = false;
+        left = 0;
         for (size_t k = 0; k < n; ++k)
-            any = any || b->h_ctls[k].active;
+            if (b->h_ctls[k].active) {
+                any = true;
+                left = std::max(left, b->h_ctls[k].stop_at - b->h_ctls[k].iters);
+            }
     }
     if (rc) {
         cudaStreamSynchronize(b->stream);

@@ -39,7 +39,7 @@ struct Ctl {
     int status;     // bit 0: non-finite state; bit 1: device wait timed out
     int converged;  // 1 when the last iteration gave h < tol
     float alpha;
-    float pad0;
+    unsigned fin_blocks;  // k_fin: blocks done in this iteration (the last one runs the tail)
     double tol;
     double h_last;
 };
@@ -124,6 +124,14 @@ __host__ __device__ inline float fp8_bound_c(float mcC, float mcW)
     return 1.001f * fmaxf(sqrtf(mcC), 1.25f * sqrtf(mcW));
 }
 
+// A kernel launch that returns its error.
+template <class... P, class... A>
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args)
+{
+    kernel<<<grid, block, smem, s>>>(static_cast<P>(args)...);
+    return cudaGetLastError();
+}
+
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline int round_up(int a, int b) { return ceil_div(a, b) * b; }
 
@@ -186,34 +194,42 @@ struct SymOut {
     double *d;
     float *df;
 };
-// X (device memory, any alignment, row stride ldi) checked (flags[0] |= 1: a non-finite entry,
-// flags[1] |= 1: not symmetric), Z-scored when stats is not NULL, and written in those forms, the
-// padding up to rows_p x ldo (W) or ld x ld as zeros
-cudaError_t launch_load_w(const float *X, int rows, int cols, int ldi, const double *stats, float *out, int rows_p, int ldo,
-                          const Parts &parts, int *flags, cudaStream_t s);
-cudaError_t launch_load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags,
-                            cudaStream_t s);
+// The networks of a state where they lie (device memory, any alignment, row strides ld*), each
+// Z-scored by its stats (NULL: as it is)
+struct StateIn {
+    const float *W, *P, *C;
+    int T, G, ldw, ldp, ldc;
+    const double *sw, *sp, *sc;
+};
+// Checked (flags[0] |= 1: a non-finite entry, flags[1] |= 1: P or C not symmetric) and written in
+// those forms, the padding up to Tp x Gp, Tp x Tp and Gp x Gp as zeros
+cudaError_t launch_load(const StateIn &in, float *W, const Parts &wparts, int Tp, int Gp, const SymOut &P, const SymOut &C,
+                        int *flags, cudaStream_t s);
 cudaError_t launch_transpose(const float *X, int rows_p, int cols_p, float *Y, cudaStream_t s);
-// out[j] = sum over the first `rows` rows of X[i][j]^2 (squared column norms, no transpose)
-cudaError_t launch_col_norms(const float *X, int rows, int cols, int ld, float *out, cudaStream_t s);
-// out[i] = sum_j X[i][j]^2, X Z-scored by stats (NULL: as it is); with diag (not NULL) the
-// diagonal entry left out and diag[i]^2 added
-cudaError_t launch_row_norms(const float *X, int rows, int cols, int ld, const double *stats, const double *diag,
-                             float *out, cudaStream_t s);
+// Squared norms: rows and columns of W (as loaded, row stride Gp), rows of P and C from where
+// they lie, the diagonal entry left out and pd, cd added; P and C Z-scored by their stats
+struct StateNorms {
+    StateIn in;       // (in.W, in.ldw: W as loaded; in.sw unused)
+    const double *pd, *cd;
+    float *rsqW, *csqW, *rsqP, *csqC;
+};
+cudaError_t launch_norms(const StateNorms &n, cudaStream_t s);
 cudaError_t launch_diag_to_float(const double *d, float *df, int n, cudaStream_t s);
 // X[r][c] = X[c][r] for r > c: the full matrix from its upper triangle
 cudaError_t launch_symmetrize(float *X, int n, int ld, cudaStream_t s);
-// out (n x n, row stride ldo) = the symmetric matrix with this strict upper triangle (FP32 X, or
-// X NULL and the BF16 split pair H + L; row stride ldi) and this diagonal
-// (guard, when given: nothing is written if the checks or the iteration found a fault)
-struct Guard {
+// The state back into dense device arrays (each may be NULL): W (row stride Gp) and the symmetric
+// matrices with these strict upper triangles (FP32 X, or X NULL and the BF16 split pair H + L)
+// and diagonals.  With guard.flags: nothing is written if the checks or the iteration found a fault.
+struct StateOut {
+    int T, G, Tp, Gp;
+    const float *W, *P, *C;
+    const __nv_bfloat16 *Ch, *Cl;
+    const double *pd, *cd;
+    float *oW, *oP, *oC;
     const int *flags;
     const Ctl *ctl;
 };
-cudaError_t launch_store_sym(const float *X, const __nv_bfloat16 *H, const __nv_bfloat16 *L, int n, int ldi,
-                             const double *diag, float *out, int ldo, Guard g, cudaStream_t s);
-// out (rows x cols, dense) = X (row stride ldi)
-cudaError_t launch_store_w(const float *X, int rows, int cols, int ldi, float *out, Guard g, cudaStream_t s);
+cudaError_t launch_store(const StateOut &o, cudaStream_t s);
 // Pearson initialisation (Sec. II-A): unit-norm centred rows of X (G x N) as a
 // BF16 split [G][Kp]; flags[0] |= 1 (non-finite) / 2 (zero variance)
 cudaError_t launch_standardize_rows(const float *X, int G, int N, __nv_bfloat16 *Zh, __nv_bfloat16 *Zl, int Kp,
@@ -225,29 +241,30 @@ cudaError_t launch_unit_diag(float *X, int n, int ld, cudaStream_t s);
 struct KernelEvents {
     cudaEvent_t *ev;
     int n;  // events recorded so far
+    bool capturing;  // a graph is being captured: the record becomes an event-record node
     void mark(cudaStream_t s)
     {
-        if (ev)  // external: inside a graph capture this becomes an event-record node
-            cudaEventRecordWithFlags(ev[n++], s, cudaEventRecordExternal);
+        if (ev)
+            cudaEventRecordWithFlags(ev[n++], s, capturing ? cudaEventRecordExternal : cudaEventRecordDefault);
     }
 };
 
 // ---- after the products (k_norms.cu) ----------------------------------------
-// shared tail of every path: diagonals, norms of P and C, h, stop test
-cudaError_t launch_fin_tail(const Dev &d, cudaStream_t s, KernelEvents &ke);
-// FP64 sums of the per-tile norm partials of W' (shared by both paths)
+// Diagonals, norms of P and C, h, counter, stop test
+cudaError_t launch_fin(const Dev &d, cudaStream_t s, KernelEvents &ke);
+// FP64 sums of the per-tile norm partials of W'
 cudaError_t launch_reduce_wnorms(const Dev &d, cudaStream_t s);
 // The same kernels over a set of networks (device arrays): blocks[b] = (network,
-// that network's block), set_norm_blocks(T, G) blocks per network; one k_tail block per network.
+// that network's block), set_norm_blocks(T, G) blocks per network.
 cudaError_t launch_reduce_wnorms_set(const Dev *devs, const int2 *blocks, int nblocks, cudaStream_t s);
-cudaError_t launch_fin_tail_set(const Dev *devs, const int2 *blocks, int nblocks, int nnets, cudaStream_t s);
+cudaError_t launch_fin_set(const Dev *devs, const int2 *blocks, int nblocks, cudaStream_t s);
 int set_norm_blocks(int T, int G);
 // FP32 FFMA throughput of the current device in TFLOP/s (best of several
 // timed launches of a loop of independent FMAs on every SM)
 cudaError_t measure_ffma_peak(double *tflops);
 
 // ---- tensor-core path (k_tc.cu) --------------------------------------------
-constexpr int TC_KERNELS = 5;
+constexpr int TC_KERNELS = 4;
 extern const char *const TC_KERNEL_NAMES[TC_KERNELS];
 bool tc_supported();
 // Tensor maps and schedules (at the first call) and FP8MIX's E4M3 copies of the state in W[cur],
@@ -284,7 +301,7 @@ cudaError_t tc_gram(const __nv_bfloat16 *Zh, const __nv_bfloat16 *Zl, int Gp, in
 cudaError_t tc_make_map(CUtensorMap *m, const void *base, int rows, int cols, int box_rows);
 
 // ---- FP32 path (k_f32.cu) ----------------------------------------------------
-constexpr int F32_KERNELS = 5;
+constexpr int F32_KERNELS = 4;
 extern const char *const F32_KERNEL_NAMES[F32_KERNELS];
 // The work lists of a network (Dev needs its sizes), kept in d.f32_host, and the
 // scratch they need: floats of the per-CTA slots and of the cut tiles' slots,

@@ -173,21 +173,18 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     // the state, exactly as a context builds it
     const SymOut po{d.Poff, 0, Parts{d.Ph, d.Pm, d.Pl}, 1, 64, d.Tp, d.pd, d.pdf};
     const SymOut xo{d.Coff, 0, Parts{d.Ch, d.Cm, d.Cl}, 0, 64, d.Gp, d.cd, d.cdf};
-    SCU(launch_load_w(dW, T, G, G, nullptr, d.W[0], d.Tp, d.Gp, Parts{d.Wh[0], d.Wm[0], d.Wl[0]}, flags, s));
-    SCU(launch_load_sym(dP, T, T, nullptr, po, flags, s));
-    SCU(launch_load_sym(dC, G, G, nullptr, xo, flags, s));
-    SCU(launch_row_norms(d.W[0], T, G, d.Gp, nullptr, nullptr, d.rsqW, s));
-    SCU(launch_col_norms(d.W[0], T, G, d.Gp, d.csqW, s));
-    SCU(launch_row_norms(dP, T, T, T, nullptr, d.pd, d.rsqP, s));
-    SCU(launch_row_norms(dC, G, G, G, nullptr, d.cd, d.csqC, s));
-    KernelEvents ke{nullptr, 0};
+    StateIn in{dW, dP, dC, T, G, G, T, G, nullptr, nullptr, nullptr};
+    SCU(launch_load(in, d.W[0], Parts{d.Wh[0], d.Wm[0], d.Wl[0]}, d.Tp, d.Gp, po, xo, flags, s));
+    in.W = d.W[0];
+    in.ldw = d.Gp;
+    SCU(launch_norms(StateNorms{in, d.pd, d.cd, d.rsqW, d.csqW, d.rsqP, d.csqC}, s));
+    KernelEvents ke{nullptr, 0, false};
     SCU(launch_iteration_f32(d, 0, s, ke));
     // results back into the caller's buffers, diagonals from the FP64 vectors; a failed call leaves
     // the caller's networks as they were
-    const Guard g{flags, d.ctl};
-    SCU(launch_store_w(d.W[1], T, G, d.Gp, dW, g, s));
-    SCU(launch_store_sym(d.Poff, nullptr, nullptr, T, d.Tp, d.pd, dP, T, g, s));
-    SCU(launch_store_sym(d.Coff, nullptr, nullptr, G, d.Gp, d.cd, dC, G, g, s));
+    SCU(launch_store(StateOut{T, G, d.Tp, d.Gp, d.W[1], d.Poff, d.Coff, nullptr, nullptr, d.pd, d.cd, dW, dP, dC, flags,
+                              d.ctl},
+                     s));
     Ctl hc{};
     int hflags[4] = {0, 0, 0, 0};
     SCU(cudaMemcpyAsync(&hc, d.ctl, sizeof hc, cudaMemcpyDeviceToHost, s));
