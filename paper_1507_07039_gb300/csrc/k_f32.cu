@@ -85,6 +85,9 @@ struct Tile {
     static constexpr int BROWS = PAIR ? 128 : 64;                    // B rows that one CTA loads
     static constexpr uint32_t B_PART = BROWS * BK * 2;
     static constexpr uint32_t STAGE = 3 * A_BYTES + 3 * B_PART;      // per CTA: A h, m, l and B h, m, l
+    // accumulators per stage: a narrow MMA is over before the one before it on the same
+    // accumulator has written back, so one CTA's K slices alternate between two
+    static constexpr int NACC = PAIR ? 1 : 2;
     static constexpr int NCH = N / 32;             // 16-column chunks of one epilogue warp
     static constexpr int SLOT = 128 * N;           // floats of one CTA's tile sums
     static constexpr uint32_t COLS = 512;          // TMEM columns held
@@ -172,22 +175,6 @@ __device__ __forceinline__ void load_box(void *dst, const CUtensorMap *map, uint
         tma_load_2d(dst, map, bar, x, y);
 }
 template <bool PAIR>
-__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc)
-{
-    if (PAIR)
-        mma_bf16_pair(d, a, b, id, acc);
-    else
-        mma_bf16(d, a, b, id, acc);
-}
-template <bool PAIR>
-__device__ __forceinline__ void commit(uint64_t *bar)
-{
-    if (PAIR)
-        mma_commit_pair(bar);
-    else
-        mma_commit(bar);
-}
-template <bool PAIR>
 __device__ __forceinline__ void group_sync()  // the CTA, or both of the pair
 {
     if (PAIR)
@@ -269,50 +256,60 @@ __device__ __forceinline__ void producer(Sync &sy, uint8_t *stages, const Item *
     sy.issued = g;
 }
 
-// The MMA issuer: every stage into a fresh accumulator, buffer g & 1.  mn(item,
+// The MMA issuer (a whole warp): every stage into a fresh accumulator, buffer g & 1.  mn(item,
 // stage) gives which operands are MN-major (bit 0: B, bit 1: A).
 template <bool PAIR, int ST, class Mn>
 __device__ __forceinline__ void issuer(Sync &sy, uint8_t *stages, const Item *items, int first, int last, Ctl *ctl,
                                        Mn mn)
 {
     constexpr uint32_t idesc = idesc_bf16_f32(Tile<PAIR>::M, Tile<PAIR>::N), STAGE = Tile<PAIR>::STAGE;
-    int g = 0;
+    const uint32_t leader = elect_one();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, sy.tmem, 0);
+    int g = 0, st = 0;
+    uint32_t ph = 0;  // stage st and its phase
     bool ok = true;
     for (int n = first; n < last && ok; ++n) {
         const Item it = items[n];
-        for (int s = it.s0; s < it.s1; ++s, ++g) {
-            const int st = g % ST, buf = g & 1;
-            if (!wait_bounded(&sy.free_[buf], ((uint32_t)(g >> 1) & 1u) ^ 1u, &sy.abort, ctl) ||
-                !wait_bounded(&sy.full[st], (uint32_t)(g / ST) & 1u, &sy.abort, ctl)) {
-                ok = false;
+        const int s0 = __shfl_sync(0xffffffffu, (int)it.s0, 0), s1 = __shfl_sync(0xffffffffu, (int)it.s1, 0);
+        for (int s = s0; s < s1; ++s, ++g) {
+            const int buf = g & 1;
+            ok = wait_bounded(&sy.free_[buf], ((uint32_t)(g >> 1) & 1u) ^ 1u, &sy.abort, ctl) &&
+                 wait_bounded(&sy.full[st], ph, &sy.abort, ctl);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok)
                 break;
-            }
             tc_fence_after();
             const uint32_t base = smem_u32(stages + (size_t)st * STAGE);
-            const uint32_t dacc = sy.tmem + (uint32_t)buf * Tile<PAIR>::N;
-            const int m = mn(it, s);
+            const uint32_t dacc = tmem + (uint32_t)buf * (Tile<PAIR>::NACC * Tile<PAIR>::N);
+            const int m = __shfl_sync(0xffffffffu, mn(it, s), 0);
             const uint32_t id = idesc | ((m & 1) ? IDESC_B_MN : 0u) | ((m & 2) ? IDESC_A_MN : 0u);
             // descriptors of part 0 at K slice 0; a part adds its bytes, a slice 32 B (K-major) or 2 KB (MN-major)
             const uint64_t a0 = (m & 2) ? sdesc_mn_sw128(base, A_BYTES / 2) : sdesc_k_sw128(base);
             const uint64_t b0 = (m & 1) ? sdesc_mn_sw128(base + 3 * A_BYTES, A_BYTES / 2)
                                         : sdesc_k_sw128(base + 3 * A_BYTES);
-            const uint64_t as = (m & 2) ? 2048 >> 4 : 32 >> 4, bs = (m & 1) ? 2048 >> 4 : 32 >> 4;
-            constexpr uint64_t APART = A_BYTES >> 4, BPART = Tile<PAIR>::B_PART >> 4;
+            const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32), b_lo = (uint32_t)b0, b_hi = (uint32_t)(b0 >> 32);
+            const uint32_t as = (m & 2) ? 2048 >> 4 : 32 >> 4, bs = (m & 1) ? 2048 >> 4 : 32 >> 4;
+            constexpr uint32_t APART = A_BYTES >> 4, BPART = Tile<PAIR>::B_PART >> 4;
             // smallest products first: m.m, h.l, l.h, then h.m, m.h, then h.h
             constexpr int pa[6] = {1, 0, 2, 0, 1, 0}, pb[6] = {1, 2, 0, 1, 0, 0};
 #pragma unroll
             for (int t = 0; t < 6; ++t)
 #pragma unroll
                 for (int kk = 0; kk < BK / 16; ++kk)
-                    mma<PAIR>(dacc, a0 + pa[t] * APART + kk * as, b0 + pb[t] * BPART + kk * bs, id,
-                              (t == 0 && kk == 0) ? 0u : 1u);
-            commit<PAIR>(&sy.empty[st]);
-            commit<PAIR>(&sy.done[buf]);
+                    mma_bf16_warp<PAIR>(leader, dacc + (kk % Tile<PAIR>::NACC) * Tile<PAIR>::N,
+                                        a_lo + pa[t] * APART + kk * as, a_hi, b_lo + pb[t] * BPART + kk * bs, b_hi, id,
+                                        !(t == 0 && kk < Tile<PAIR>::NACC));
+            mma_commit_warp<PAIR>(leader, &sy.empty[st]);
+            mma_commit_warp<PAIR>(leader, &sy.done[buf]);
+            if (++st == ST) {
+                st = 0;
+                ph ^= 1u;
+            }
         }
     }
     sy.consumed = g;
     // an mbarrier that both CTAs of a pair are told of; only the even one waits on it
-    commit<PAIR>(&sy.fin);
+    mma_commit_warp<PAIR>(leader, &sy.fin);
 }
 
 // ---- the epilogue's side of the main loop ---------------------------------------------
@@ -440,7 +437,9 @@ __device__ __forceinline__ bool sum_stages(Sync &sy, const Item &it, int nR, int
         if (!live)
             continue;
         tc_fence_after();
-        drain<Tile<PAIR>::NCH>(tq + (uint32_t)buf * Tile<PAIR>::N, acc);
+#pragma unroll
+        for (int q = 0; q < Tile<PAIR>::NACC; ++q)
+            drain<Tile<PAIR>::NCH>(tq + (uint32_t)(buf * Tile<PAIR>::NACC + q) * Tile<PAIR>::N, acc);
         if (!(keep && s + 1 == it.s1)) {
             tc_fence_before();
             __syncwarp();
@@ -510,7 +509,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                                    }
                                }
                            });
-        } else if (warp == 1 && lane == 0 && rank == 0) {
+        } else if (warp == 1 && rank == 0) {
             issuer<PAIR, ST>(sy, stages, items, first, last, ctl, [&](const Item &it, int s) {
                 return (s < nR || (s - nR) * BK < (int)(it.a >> 16) * N) ? 1 : 0;
             });
@@ -563,7 +562,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
             // the sums in TMEM: the last stage's buffer of an uncut tile on a pair (kept until the
             // epilogue is done), else columns that no stage uses (one CTA), else wait-free reuse of the
             // slot of part 0 (a pair's cut tile)
-            const uint32_t tsum = PAIR ? tq + (uint32_t)lastbuf * N : tq + 2 * N;
+            const uint32_t tsum = PAIR ? tq + (uint32_t)lastbuf * N : tq + 4 * N;
             const bool in_tmem = !(PAIR && cut);
             float *aslot = fix + FS;
             if (live) {
@@ -760,7 +759,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                                        load_box<PAIR>(bb + h * (A_BYTES / 2), &maps.Wm[cur][p], bar, n0 + 64 * h, k);
                                }
                            });
-        } else if (warp == 1 && lane == 0 && rank == 0) {
+        } else if (warp == 1 && rank == 0) {
             issuer<PAIR, ST>(sy, stages, items, first, last, ctl,
                          [](const Item &it, int) { return it.a >> 31 ? 0 : 3; });
         }
@@ -794,7 +793,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
             }
             if (!mine)
                 continue;
-            const uint32_t tsum = PAIR ? tq + (uint32_t)lastbuf * N : tq + 2 * N;
+            const uint32_t tsum = PAIR ? tq + (uint32_t)lastbuf * N : tq + 4 * N;
             const bool in_tmem = !(PAIR && cut);
             if (live) {
                 if (in_tmem)

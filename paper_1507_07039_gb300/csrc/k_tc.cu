@@ -757,60 +757,64 @@ __device__ __forceinline__ void phase1_tile(const TcMaps &maps, const Dev &d, in
             sy.issued = s;
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {  // ---- MMA issuer of the pair ----
+        if (rank == 0) {  // ---- MMA issuer of the pair (a whole warp, see mma_bf16_warp) ----
             constexpr uint32_t idesc = idesc_bf16_f32(256, 256);
-            int s = 0;
+            const uint32_t leader = elect_one(), tmem = __shfl_sync(0xffffffffu, sy.tmem, 0);
+            const bool fp8 = __shfl_sync(0xffffffffu, d.fp8, 0) != 0, split_b = __shfl_sync(0xffffffffu, d.split_b, 0) != 0;
+            int s = 0, st = g0 % ST1;
+            uint32_t ph = (uint32_t)(g0 / ST1) & 1u;
             for (; s < nk; ++s) {
-                const int kb = kb_of(s), st = (g0 + s) % ST1;
+                const int kb = kb_of(s);
                 // this k-block's accumulator: A-num chunk c in buffer c & 1, R-num in buffer bR; a buffer
                 // is written again only once the epilogue has drained the chunk it held two chunks before
                 const int a = kb - nR, c = a / P1_CHUNK;
                 const int buf = kb >= nR ? (c & 1) : bR;
                 const bool fresh = kb >= nR ? a % P1_CHUNK == 0 : kb == 0;
                 const int prev = kb >= nR ? c - 2 : nc - 2;  // chunk that last used buf (< c0: none here)
-                if (fresh && prev >= c0 &&
-                    !wait_bounded(&sy.buf_free[buf], (uint32_t)(u0[buf] + ((prev - c0) >> 1)) & 1u, &sy.abort,
-                                  ctl))
-                    break;
-                if (!wait_bounded(&sy.full[st], (uint32_t)((g0 + s) / ST1) & 1u, &sy.abort, ctl))
+                bool ok = true;
+                if (fresh && prev >= c0)
+                    ok = wait_bounded(&sy.buf_free[buf], (uint32_t)(u0[buf] + ((prev - c0) >> 1)) & 1u, &sy.abort, ctl);
+                ok = ok && wait_bounded(&sy.full[st], ph, &sy.abort, ctl);
+                if (!__all_sync(0xffffffffu, ok))
                     break;
                 tc_fence_after();
                 const uint32_t base = smem_u32(stages + (size_t)st * STAGE1);
-                const uint32_t dacc = sy.tmem + (uint32_t)buf * 256u;
+                const uint32_t dacc = tmem + (uint32_t)buf * 256u;
                 // a chunk other than the last ends: the epilogue drains it into the running sum
                 const bool chunk_end = kb >= nR && c < nc - 1 && (a % P1_CHUNK == P1_CHUNK - 1);
-                if (kb >= nR && d.fp8) {
+                const bool e4 = kb >= nR && fp8;
+                const bool bmn = !e4 && (kb < nR || (kb - nR) * BK < n0);  // B block loaded MN-major
+                const uint64_t a0 = sdesc_k_sw128(base);
+                const uint64_t b0 = bmn ? sdesc_mn_sw128(base + 2 * A_BYTES, A_BYTES / 2) : sdesc_k_sw128(base + 2 * A_BYTES);
+                const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32), b_lo = (uint32_t)b0,
+                               b_hi = (uint32_t)(b0 >> 32);
+                const uint32_t bs = bmn ? 2048 >> 4 : 32 >> 4, id = bmn ? (idesc | IDESC_B_MN) : idesc;
+                constexpr uint32_t PART = A_BYTES >> 4;
+                if (e4) {  // one E4M3 tile of A, then one of B; K = 32 per MMA
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)  // K = 32 per MMA
-                        mma_e4m3_pair(dacc, sdesc_k_sw128(base + kk * 32), sdesc_k_sw128(base + A_BYTES + kk * 32),
-                                      idesc_e4m3_f32(256, 256), (fresh && kk == 0) ? 0u : 1u);
-                    mma_commit_pair(&sy.empty[st]);
-                    if (chunk_end)
-                        mma_commit_pair(&sy.chunk_done[buf]);
-                    continue;
-                }
-                const bool bmn = kb < nR || (kb - nR) * BK < n0;  // B block loaded MN-major
-                const uint32_t id = bmn ? (idesc | IDESC_B_MN) : idesc;
+                    for (int kk = 0; kk < 4; ++kk)
+                        mma_e4m3_warp(leader, dacc, a_lo + kk * 2, a_hi, a_lo + PART + kk * 2, a_hi,
+                                      idesc_e4m3_f32(256, 256), !(fresh && kk == 0));
+                } else {
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk) {
-                    const uint32_t off = kk * 32;
-                    const uint64_t ah = sdesc_k_sw128(base + off);
-                    const uint64_t al = sdesc_k_sw128(base + A_BYTES + off);
-                    const uint64_t bh = bmn ? sdesc_mn_sw128(base + 2 * A_BYTES + kk * 2048, A_BYTES / 2)
-                                            : sdesc_k_sw128(base + 2 * A_BYTES + off);
-                    const uint64_t bl = bmn ? sdesc_mn_sw128(base + 3 * A_BYTES + kk * 2048, A_BYTES / 2)
-                                            : sdesc_k_sw128(base + 3 * A_BYTES + off);
-                    mma_bf16_pair(dacc, ah, bh, id, (fresh && kk == 0) ? 0u : 1u);
-                    if (d.split_b)
-                        mma_bf16_pair(dacc, ah, bl, id, 1u);
-                    mma_bf16_pair(dacc, al, bh, id, 1u);
+                    for (int kk = 0; kk < BK / 16; ++kk) {
+                        const uint32_t ah = a_lo + kk * 2, bh = b_lo + kk * bs;
+                        mma_bf16_warp<true>(leader, dacc, ah, a_hi, bh, b_hi, id, !(fresh && kk == 0));
+                        if (split_b)
+                            mma_bf16_warp<true>(leader, dacc, ah, a_hi, bh + PART, b_hi, id, true);
+                        mma_bf16_warp<true>(leader, dacc, ah + PART, a_hi, bh, b_hi, id, true);
+                    }
                 }
-                mma_commit_pair(&sy.empty[st]);
+                mma_commit_warp<true>(leader, &sy.empty[st]);
                 if (chunk_end)
-                    mma_commit_pair(&sy.chunk_done[buf]);
+                    mma_commit_warp<true>(leader, &sy.chunk_done[buf]);
+                if (++st == ST1) {
+                    st = 0;
+                    ph ^= 1u;
+                }
             }
             sy.consumed = s;
-            mma_commit_pair(&sy.accum);  // also on abort, so the epilogues can drain
+            mma_commit_warp<true>(leader, &sy.accum);  // also on abort, so the epilogues can drain
         }
     } else {  // ---- epilogue: warps 2..9 of both CTAs ----
         const int e = warp - 2, wq = warp & 3, half = e >> 2;
@@ -1284,9 +1288,11 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
             sy.issued = g;
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {  // ---- MMA issuer of the pair ----
+        if (rank == 0) {  // ---- MMA issuer of the pair (a whole warp, see mma_bf16_warp) ----
             constexpr uint32_t idesc = idesc_bf16_f32(256, N2);
-            int g = 0;
+            const uint32_t leader = elect_one(), tmem = __shfl_sync(0xffffffffu, sy.tmem, 0);
+            int g = 0, st = 0;
+            uint32_t ph = 0;
             bool ok = true;
             for (int n = first, idx = -1; n < last && ok; ++n) {
                 const int net = src.net(n);
@@ -1294,55 +1300,55 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
                     continue;
                 ++idx;
                 const Dev &d = src.dev(net);
-                const int tile = src.tiles[n];
+                const int tile = __shfl_sync(0xffffffffu, src.tiles[n], 0);
                 const P2Item it = p2_item(tile, d);
-                const bool q8 = d.fp8 && tile >= 0;
+                const bool mn = tile >= 0;  // C tiles: both operands MN-major
+                const bool q8 = __shfl_sync(0xffffffffu, d.fp8, 0) != 0 && mn;
+                const bool split_b = __shfl_sync(0xffffffffu, d.split_b, 0) != 0;
+                const int nkb = __shfl_sync(0xffffffffu, it.kb1 - it.kb0, 0);
                 const int buf = idx & 1;
-                if (!wait_bounded(&sy.tempty[buf], ((uint32_t)(idx >> 1) & 1u) ^ 1u, &sy.abort, d.ctl))
+                ok = wait_bounded(&sy.tempty[buf], ((uint32_t)(idx >> 1) & 1u) ^ 1u, &sy.abort, d.ctl);
+                if (!(ok = __all_sync(0xffffffffu, ok)))
                     break;
                 tc_fence_after();
-                const uint32_t dacc = sy.tmem + buf * N2;
-                for (int kb = it.kb0; kb < it.kb1; ++kb, ++g) {
-                    const bool first = kb == it.kb0;  // a fresh accumulator for every item
-                    const int st = g % ST2;
-                    if (!wait_bounded(&sy.full[st], (uint32_t)(g / ST2) & 1u, &sy.abort, d.ctl)) {
-                        ok = false;
+                const uint32_t dacc = tmem + buf * N2;
+                for (int k = 0; k < nkb; ++k, ++g) {  // a fresh accumulator for every item
+                    ok = wait_bounded(&sy.full[st], ph, &sy.abort, d.ctl);
+                    if (!(ok = __all_sync(0xffffffffu, ok)))
                         break;
-                    }
                     tc_fence_after();
                     const uint32_t base = smem_u32(stages + (size_t)st * STAGE2);
+                    const bool kmn = mn && !q8;
+                    const uint64_t a0 = kmn ? sdesc_mn_sw128(base, A_BYTES / 2) : sdesc_k_sw128(base);
+                    const uint32_t a_lo = (uint32_t)a0, hi = (uint32_t)(a0 >> 32), step = kmn ? 2048 >> 4 : 32 >> 4;
+                    constexpr uint32_t PART = A_BYTES >> 4;
+                    const uint32_t id = kmn ? (idesc | IDESC_A_MN | IDESC_B_MN) : idesc;
                     if (q8) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)  // K = 32 per MMA
-                            mma_e4m3_pair(dacc, sdesc_k_sw128(base + kk * 32),
-                                          sdesc_k_sw128(base + A_BYTES + kk * 32), idesc_e4m3_f32(256, N2),
-                                          (first && kk == 0) ? 0u : 1u);
-                        mma_commit_pair(&sy.empty[st]);
-                        continue;
-                    }
-                    const bool mn = tile >= 0;  // C tiles: both operands MN-major
-                    const uint32_t id = mn ? (idesc | IDESC_A_MN | IDESC_B_MN) : idesc;
+                            mma_e4m3_warp(leader, dacc, a_lo + kk * 2, hi, a_lo + PART + kk * 2, hi,
+                                          idesc_e4m3_f32(256, N2), !(k == 0 && kk == 0));
+                    } else {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        const uint32_t off = kk * 32, moff = kk * 2048;
-                        const uint64_t ah = mn ? sdesc_mn_sw128(base + moff, A_BYTES / 2) : sdesc_k_sw128(base + off);
-                        const uint64_t al = mn ? sdesc_mn_sw128(base + A_BYTES + moff, A_BYTES / 2)
-                                               : sdesc_k_sw128(base + A_BYTES + off);
-                        const uint64_t bh = mn ? sdesc_mn_sw128(base + 2 * A_BYTES + moff, A_BYTES / 2)
-                                               : sdesc_k_sw128(base + 2 * A_BYTES + off);
-                        const uint64_t bl = mn ? sdesc_mn_sw128(base + 3 * A_BYTES + moff, A_BYTES / 2)
-                                               : sdesc_k_sw128(base + 3 * A_BYTES + off);
-                        if (d.split_b) {  // hi(A) once from shared memory for hi.hi and hi.lo
-                            mma_bf16_pair_fill_a(dacc, ah, bh, id, (first && kk == 0) ? 0u : 1u);
-                            mma_bf16_pair_lastuse_a(dacc, ah, bl, id, 1u);
-                        } else {
-                            mma_bf16_pair(dacc, ah, bh, id, (first && kk == 0) ? 0u : 1u);
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            const uint32_t ah = a_lo + kk * step, al = ah + PART, bh = al + PART, bl = bh + PART;
+                            const bool acc = !(k == 0 && kk == 0);
+                            if (split_b) {  // hi(A) once from shared memory for hi.hi and hi.lo
+                                mma_bf16_warp<true, KeepA::FILL>(leader, dacc, ah, hi, bh, hi, id, acc);
+                                mma_bf16_warp<true, KeepA::LAST>(leader, dacc, ah, hi, bl, hi, id, true);
+                            } else {
+                                mma_bf16_warp<true>(leader, dacc, ah, hi, bh, hi, id, acc);
+                            }
+                            mma_bf16_warp<true>(leader, dacc, al, hi, bh, hi, id, true);
                         }
-                        mma_bf16_pair(dacc, al, bh, id, 1u);
                     }
-                    mma_commit_pair(&sy.empty[st]);
+                    mma_commit_warp<true>(leader, &sy.empty[st]);
+                    if (++st == ST2) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
                 }
-                mma_commit_pair(&sy.tfull[buf]);
+                mma_commit_warp<true>(leader, &sy.tfull[buf]);
             }
             sy.consumed = g;
         }

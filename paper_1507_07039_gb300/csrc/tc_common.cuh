@@ -273,28 +273,64 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, 
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// As mma_bf16_pair, keeping A in the tensor core's collector buffer for the
-// next MMA (fill) or reading it from there and releasing it (lastuse): the
-// second MMA does not read A from shared memory again.  a_desc is the same.
-__device__ __forceinline__ void mma_bf16_pair_fill_a(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                                     uint32_t idesc, uint32_t accumulate)
+// One lane of the (converged) warp: 1 there, 0 elsewhere.
+__device__ __forceinline__ uint32_t elect_one()
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+    return r;
 }
-__device__ __forceinline__ void mma_bf16_pair_lastuse_a(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                                        uint32_t idesc, uint32_t accumulate)
+// The same MMAs and commits executed by a whole converged warp, taking effect
+// on its elected lane (leader) only.  A warp-uniform issue loop keeps
+// descriptors and addresses in uniform registers; a loop under `lane == 0`
+// moves them there one by one before every MMA (about 85 cycles an issue,
+// measured, more than an MMA of 64 columns takes).
+// Descriptors as halves: only the low word (the address) changes between MMAs.
+// KeepA: A left in the tensor core's collector buffer for the next MMA (FILL),
+// or read from there and released (LAST) instead of from shared memory.
+enum class KeepA { NONE, FILL, LAST };
+#define PANDA_MMA_WARP(GROUP, KIND, KEEP)                                                                           \
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"   \
+                 "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"                                               \
+                 "@q tcgen05.mma.cta_group::" GROUP ".kind::" KIND KEEP " [%0], a, b, %5, p;\n\t}\n" ::"r"(d),     \
+                 "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(id), "r"((uint32_t)accumulate), "r"(leader)        \
+                 : "memory")
+template <bool PAIR, KeepA K = KeepA::NONE>
+__device__ __forceinline__ void mma_bf16_warp(uint32_t leader, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                              uint32_t b_hi, uint32_t id, bool accumulate)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    static_assert(PAIR || K == KeepA::NONE, "only pairs keep A");
+    if (!PAIR)
+        PANDA_MMA_WARP("1", "f16", "");
+    else if (K == KeepA::NONE)
+        PANDA_MMA_WARP("2", "f16", "");
+    else if (K == KeepA::FILL)
+        PANDA_MMA_WARP("2", "f16", ".collector::a::fill");
+    else
+        PANDA_MMA_WARP("2", "f16", ".collector::a::lastuse");
+}
+// E4M3 on a CTA pair, K = 32 per MMA
+__device__ __forceinline__ void mma_e4m3_warp(uint32_t leader, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                              uint32_t b_hi, uint32_t id, bool accumulate)
+{
+    PANDA_MMA_WARP("2", "f8f6f4", "");
+}
+#undef PANDA_MMA_WARP
+template <bool PAIR>
+__device__ __forceinline__ void mma_commit_warp(uint32_t leader, uint64_t *bar)
+{
+    if (PAIR)
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+                     "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], "
+                     "%1;\n\t}\n" ::"r"(smem_u32(bar)),
+                     "h"((uint16_t)0x3), "r"(leader)
+                     : "memory");
+    else
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                     "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(
+                         smem_u32(bar)),
+                     "r"(leader)
+                     : "memory");
 }
 
 // Instruction descriptor of kind::f8f6f4 with E4M3 A and B (format 0 in bits
