@@ -200,15 +200,6 @@ __global__ void k_fp8_init(Dev d)
     }
 }
 
-__device__ __forceinline__ void ld16(const float *src, float (&v)[16])
-{
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 x = reinterpret_cast<const float4 *>(src)[q];
-        v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
-    }
-}
-
 // 8 bytes from global memory, asking L2 to fetch the whole aligned 256-byte
 // block around them: the four lanes of a row read 32 bytes (16 entries) of
 // each half at a time, and the 256-byte block holds the rest of the row
@@ -525,6 +516,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // epilogue (two per TMEM lane quarter, each taking 128 of the 256 columns in
 // 16-column sub-chunks).
 // ---------------------------------------------------------------------------
+// The finished tile is taken as TMEM fragments, like phase 2's: values move
+// straight between registers and memory (8 x 64 bytes per row group), sums in
+// registers and by shuffles, everything a 16-column sub-chunk ahead; only
+// FP8MIX's transposed copy passes through shared memory.  The epilogue is not
+// overlapped with MMAs: 2.6 us per sub-chunk and 21 us per tile when each row
+// belonged to a lane and every block was staged.  Phase 1 at 250 x 2100 (one
+// tile per pair) 67 -> 58.5 us, 600 x 6000 130 -> 123.5 us, FP8MIX at 1000 x
+// 17000 421 -> 401 us, BF16X3 there 1.07 -> 1.06 ms (bound by its MMAs: 12 of
+// 128 cycles a stage of 1530 cycles, at the clock the power limit leaves).
 constexpr int ST1 = 3;
 constexpr uint32_t STAGE1 = 4 * A_BYTES;   // per CTA: A hi, A lo, B hi, B lo (128 rows each)
 constexpr int EPI1 = 8, THREADS1 = 64 + 32 * EPI1;
@@ -552,6 +552,12 @@ constexpr int P2_CHUNK = 64;
 __device__ __forceinline__ void red_add(float *p, float v)
 {
     asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+// four neighbouring entries in one instruction
+__device__ __forceinline__ void red_add4(float *p, float v0, float v1, float v2, float v3)
+{
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v0), "f"(v1), "f"(v2), "f"(v3)
+                 : "memory");
 }
 constexpr size_t P1_SLOT = 128 * 256;  // floats of one CTA's running-sum slot
 
@@ -818,8 +824,10 @@ __device__ __forceinline__ void phase1_tile(const TcMaps &maps, const Dev &d, in
         }
     } else {  // ---- epilogue: warps 2..9 of both CTAs ----
         const int e = warp - 2, wq = warp & 3, half = e >> 2;
-        const int r = wq * 32 + lane, i = m0 + r, k0 = m0 + wq * 32;
         const int tt = threadIdx.x - 64;  // 0..255
+        // finished columns are taken as fragments (see frag_to_rows): rows er + 8 i of the warp's 32, columns
+        // ec .. ec + 3 of 16
+        const int k0 = m0 + wq * 32, er = lane >> 2, ec = 8 * (lane & 1) + 2 * (lane & 2);
         float *blk = blocks + (size_t)e * P1_BLK;
         const int nx = cur ^ 1;
         const float *W = d.W[cur];
@@ -838,15 +846,22 @@ __device__ __forceinline__ void phase1_tile(const TcMaps &maps, const Dev &d, in
             colvec[256 + tt] = cj ? d.csqW[j] : 0.0f;
             colvec[512 + tt] = cj ? d.csqC[j] : 0.0f;
         }
-        const bool ri = i < d.T;
-        const float pdi = ri ? d.pdf[i] : 0.0f, rsp = ri ? d.rsqP[i] : 0.0f, rsw = ri ? d.rsqW[i] : 0.0f;
-        const float *wrow = W + (size_t)i * d.Gp + n0 + half * 128;
-        float nxt[16];
-        ld16(wrow, nxt);
+        float pdi[4], rsp[4], rsw[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = k0 + er + 8 * i;
+            const bool ri = r < d.T;
+            pdi[i] = ri ? d.pdf[r] : 0.0f;
+            rsp[i] = ri ? d.rsqP[r] : 0.0f;
+            rsw[i] = ri ? d.rsqW[r] : 0.0f;
+        }
+        const size_t wo = (size_t)(k0 + er) * d.Gp + n0 + half * 128 + ec;
+        uint4 wnx[4];
+        ld_old_f32(W + wo, d.Gp, wnx);
         epi_bar2();
-        const uint32_t trow = sy.tmem + ((uint32_t)(wq * 32) << 16);
+        const uint32_t trow = sy.tmem + ((uint32_t)(wq * 32) << 16) + half * 128;  // this warp's lanes and columns
         // while the MMAs run on: add each finished A-num chunk but the last into the running sum
-        // (this thread's row r, its 128 columns; [column][row] so a warp's accesses are contiguous)
+        // (fragment registers in fours at [4 chunk-of-16 + q][thread]: 16 bytes each, coalesced)
         bool live = true;
         if (c0 > 0) {  // the tile's head was added into scr by another pair: wait for its flag
             if (threadIdx.x == 64 && !flag_wait_bounded(flag, &sy.abort, ctl))
@@ -862,19 +877,25 @@ __device__ __forceinline__ void phase1_tile(const TcMaps &maps, const Dev &d, in
             tc_fence_after();
             if (!live)
                 break;
+            float4 *sp = reinterpret_cast<float4 *>(scr) + tt;
+            uint32_t v[16];
+            tmem_ld_frag16_nowait(trow + (uint32_t)b * 256u, v);
 #pragma unroll 1
             for (int j = 0; j < 8; ++j) {
-                float v[16];
-                tmem_ld16(trow + (uint32_t)b * 256u + half * 128 + j * 16, v);
-                float *sp = scr + (size_t)(half * 128 + j * 16) * 128 + r;
-                if (c == 0) {
+                tmem_wait16(v);
+                float f[16];
 #pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        sp[q * 128] = v[q];
-                } else {
+                for (int q = 0; q < 16; ++q)
+                    f[q] = __uint_as_float(v[q]);
+                if (j < 7)
+                    tmem_ld_frag16_nowait(trow + (uint32_t)b * 256u + (j + 1) * 16, v);
 #pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        red_add(sp + q * 128, v[q]);
+                for (int q = 0; q < 4; ++q) {
+                    float4 *p = sp + (4 * j + q) * 256;
+                    if (c == 0)
+                        *p = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+                    else
+                        red_add4(&p->x, f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
                 }
             }
             tc_fence_before();
@@ -889,100 +910,119 @@ __device__ __forceinline__ void phase1_tile(const TcMaps &maps, const Dev &d, in
                 flag_raise(flag);
         } else {
         // the running sum's first sub-chunk, from L2 (where the adds landed), in flight while the
-        // last chunk and R-num finish; each later one is fetched a sub-chunk ahead
-        const float *srow = scr + (size_t)(half * 128) * 128 + r;
-        float snxt[16];
+        // last chunk and R-num finish; each later one, the next W and the accumulators are fetched a
+        // sub-chunk ahead
+        const float4 *sp = reinterpret_cast<const float4 *>(scr) + tt;
+        float4 snx[4];
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
-            snxt[q] = (live && nc > 1) ? __ldcg(srow + (size_t)q * 128) : 0.0f;
+        for (int q = 0; q < 4; ++q)
+            snx[q] = (live && nc > 1) ? __ldcg(sp + q * 256) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         live = live && wait_bounded(&sy.accum, tpar, &sy.abort, ctl) && !*(volatile int *)&sy.abort;
         tc_fence_after();
         const float a = ctl->alpha, keep = 1.0f - a, halfa = 0.5f * a;
-        float rowsq = 0.0f, hsum = 0.0f;
+        float rowsq[4] = {0.0f, 0.0f, 0.0f, 0.0f}, hsum = 0.0f;
+        const uint32_t tR = trow + (uint32_t)bR * 256u, tA = trow + (uint32_t)(bR ^ 1) * 256u;  // A: the last chunk
+        uint32_t fr[16], fa[16];
+        if (live) {
+            tmem_ld_frag16_nowait(tR, fr);
+            tmem_ld_frag16_nowait(tA, fa);
+        }
 #pragma unroll 1
         for (int c = 0; c < 8 && live; ++c) {
             const int cc = half * 128 + c * 16, j0 = n0 + cc;
-            float w[16], rr[16], aa[16], wn[16], sa[16];
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                w[q] = nxt[q];
-                sa[q] = snxt[q];
-            }
-            if (c < 7) {
-                ld16(wrow + (c + 1) * 16, nxt);  // next sub-chunk's W and running sum, in flight meanwhile
-                if (nc > 1) {
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        snxt[q] = __ldcg(srow + (size_t)((c + 1) * 16 + q) * 128);
-                }
-            }
-            tmem_ld16(trow + (uint32_t)bR * 256u + cc, rr);
-            tmem_ld16(trow + (uint32_t)(bR ^ 1) * 256u + cc, aa);  // the last A-num chunk
+            float x[4][4], y[4][4], w[4][4];
+            tmem_wait16(fr);
+            tmem_wait16(fa);
             if (nc > 1) {
+                const float sv[16] = {snx[0].x, snx[0].y, snx[0].z, snx[0].w, snx[1].x, snx[1].y, snx[1].z, snx[1].w,
+                                      snx[2].x, snx[2].y, snx[2].z, snx[2].w, snx[3].x, snx[3].y, snx[3].z, snx[3].w};
 #pragma unroll
                 for (int q = 0; q < 16; ++q)
-                    aa[q] = sa[q] + aa[q];
+                    fa[q] = __float_as_uint(sv[q] + __uint_as_float(fa[q]));
             }
+            frag_to_rows(fr, x);
+            frag_to_rows(fa, y);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                wn[q] = 0.0f;
-                if (ri && j0 + q < d.G) {
-                    const float rnum = rr[q] + pdi * w[q];               // P_i. . W_.j
-                    const float anum = fmaf(aa[q], ainv, w[q] * colvec[cc + q]);  // W_i. . C_.j
-                    const float R = tanimoto_fast(rnum, rsp, colvec[256 + cc + q]);
-                    const float A = tanimoto_fast(anum, rsw, colvec[512 + cc + q]);
-                    wn[q] = keep * w[q] + halfa * (A + R);
-                    hsum += fabsf(wn[q] - w[q]);
-                    rowsq += wn[q] * wn[q];
+            for (int i = 0; i < 4; ++i)
+                unpack4(wnx[i], w[i]);
+            if (c < 7) {
+                tmem_ld_frag16_nowait(tR + (c + 1) * 16, fr);
+                tmem_ld_frag16_nowait(tA + (c + 1) * 16, fa);
+                ld_old_f32(W + wo + (c + 1) * 16, d.Gp, wnx);
+                if (nc > 1) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        snx[q] = __ldcg(sp + (4 * (c + 1) + q) * 256);
                 }
-                blk[lane * 17 + q] = wn[q];
             }
-            __syncwarp();
-            // (a) W' and its split copies, row-major and coalesced: lane l takes 4 columns of rows (l >> 2) + 8 i
+            const float4 c4 = *reinterpret_cast<const float4 *>(colvec + cc + ec);
+            const float4 w4 = *reinterpret_cast<const float4 *>(colvec + 256 + cc + ec);
+            const float4 q4 = *reinterpret_cast<const float4 *>(colvec + 512 + cc + ec);
+            const float cdj[4] = {c4.x, c4.y, c4.z, c4.w}, nwj[4] = {w4.x, w4.y, w4.z, w4.w},
+                        ncj[4] = {q4.x, q4.y, q4.z, q4.w};
+            const bool inner = k0 + 31 < d.T && j0 + 15 < d.G;
+            float cs[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            // (a) W' and its split copies, row-major from this lane's registers
 #pragma unroll
-            for (int i2 = 0; i2 < 4; ++i2) {
-                const int rr2 = (lane >> 2) + 8 * i2, jj = j0 + 4 * (lane & 3);
-                float f[4];
+            for (int i = 0; i < 4; ++i) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    f[q] = blk[rr2 * 17 + 4 * (lane & 3) + q];
+                for (int u = 0; u < 4; ++u) {
+                    const float wv = w[i][u];
+                    const float rnum = x[i][u] + pdi[i] * wv;                // P_i. . W_.j
+                    const float anum = fmaf(y[i][u], ainv, wv * cdj[u]);     // W_i. . C_.j
+                    const float R = tanimoto_clamped(rnum, rsp[i], nwj[u]);
+                    const float A = tanimoto_clamped(anum, rsw[i], ncj[u]);
+                    float wn = fmaf(keep, wv, halfa * (A + R));
+                    if (!inner)  // padding stays zero
+                        wn = k0 + er + 8 * i < d.T && j0 + ec + u < d.G ? wn : 0.0f;
+                    hsum += fabsf(wn - wv);
+                    rowsq[i] = fmaf(wn, wn, rowsq[i]);
+                    cs[u] = fmaf(wn, wn, cs[u]);
+                    w[i][u] = wn;
+                }
+                const size_t ro = wo + (size_t)(8 * i) * d.Gp + c * 16;
                 uint32_t h2[2], l2[2];
-                split_pair(f[0], f[1], h2[0], l2[0]);
-                split_pair(f[2], f[3], h2[1], l2[1]);
-                const size_t ro = (size_t)(k0 + rr2) * d.Gp + jj;
-                *reinterpret_cast<float4 *>(Wn + ro) = make_float4(f[0], f[1], f[2], f[3]);
+                split_pair(w[i][0], w[i][1], h2[0], l2[0]);
+                split_pair(w[i][2], w[i][3], h2[1], l2[1]);
+                *reinterpret_cast<float4 *>(Wn + ro) = make_float4(w[i][0], w[i][1], w[i][2], w[i][3]);
                 *reinterpret_cast<uint2 *>(Wh + ro) = make_uint2(h2[0], h2[1]);
                 *reinterpret_cast<uint2 *>(Wl + ro) = make_uint2(l2[0], l2[1]);
                 if (q8)
-                    *reinterpret_cast<uint32_t *>(d.W8[nx] + ro) = e4m3x2(f[0], f[1], s8) | e4m3x2(f[2], f[3], s8) << 16;
+                    *reinterpret_cast<uint32_t *>(d.W8[nx] + ro) = e4m3x2(w[i][0], w[i][1], s8) | e4m3x2(w[i][2], w[i][3], s8) << 16;
             }
-            // (b) the column sums of W'^2 over the warp's 32 rows (lane l: column (l & 15), rows
-            //     16 (l >> 4) + 0..15) and, under FP8MIX, the transposed E4M3 copy
-            {
+            // (b) the column sums of W'^2 over the warp's 32 rows
+            const float t = lanes8_reduce_scatter4(cs);
+            if (!(lane & 4))
+                colred[wq * 256 + cc + ec + (lane >> 3 & 1) + 2 * (lane >> 4)] = t;
+            // (c) under FP8MIX the transposed E4M3 copy, through this warp's staging block: lane l takes
+            //     column (l & 15), rows 16 (l >> 4) + 0..15
+            if (q8) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        blk[(er + 8 * i) * 17 + ec + u] = w[i][u];
+                __syncwarp();
                 const int col = lane & 15, h16 = 16 * (lane >> 4);
-                float g[16];
+                const size_t to = (size_t)(j0 + col) * d.Tp + k0 + h16;
+                uint32_t p8[4];
 #pragma unroll
-                for (int m = 0; m < 16; ++m)
-                    g[m] = blk[(h16 + m) * 17 + col];
-                float c2 = 0.0f;
-#pragma unroll
-                for (int m = 0; m < 16; ++m)
-                    c2 += g[m] * g[m];
-                c2 += __shfl_xor_sync(0xffffffffu, c2, 16);
-                if (lane < 16)
-                    colred[wq * 256 + cc + lane] = c2;
-                if (q8) {
-                    const size_t to = (size_t)(j0 + col) * d.Tp + k0 + h16;
-                    uint32_t p8[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        p8[q] = e4m3x2(g[4 * q], g[4 * q + 1], s8) | e4m3x2(g[4 * q + 2], g[4 * q + 3], s8) << 16;
-                    *reinterpret_cast<uint4 *>(d.Wt8[nx] + to) = make_uint4(p8[0], p8[1], p8[2], p8[3]);
+                for (int q = 0; q < 4; ++q) {
+                    const float *b = blk + (h16 + 4 * q) * 17 + col;
+                    p8[q] = e4m3x2(b[0], b[17], s8) | e4m3x2(b[34], b[51], s8) << 16;
                 }
+                *reinterpret_cast<uint4 *>(d.Wt8[nx] + to) = make_uint4(p8[0], p8[1], p8[2], p8[3]);
+                __syncwarp();
             }
-            __syncwarp();
         }
-        rowred[half * 128 + r] = rowsq;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float rs = rowsq[i];
+            rs += __shfl_xor_sync(0xffffffffu, rs, 1);
+            rs += __shfl_xor_sync(0xffffffffu, rs, 2);
+            if ((lane & 3) == 0)
+                rowred[half * 128 + wq * 32 + er + 8 * i] = rs;
+        }
         double hv = (double)hsum;
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1)
