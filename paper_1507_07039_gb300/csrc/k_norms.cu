@@ -1,5 +1,5 @@
 // What every path's iteration shares after its products: the norms of W'
-// (k_reduce_wnorms), then the diagonals of Eq. 6, the norms of P' and C', h, the
+// and h (k_reduce_wnorms), then the diagonals of Eq. 6, the norms of P' and C', the
 // counter and the stop test (k_fin), for one network or a set.  Every
 // reduction has a fixed order, so an iteration is deterministic.  Also the
 // FP32 FMA rate of the device (measurement support).
@@ -88,13 +88,38 @@ __device__ __forceinline__ void fp8_norm_max(unsigned *slot, float v)
 
 // rsqW[i] = sum_b wrow_part[b][i], csqW[j] = sum_b wcol_part[b][j] (FP64).
 // Blocks [0, ceil(T/32)) take rows of W, the rest its columns.
-// block b of one network's launch: b < ceil(T/32) rows of W, the rest its columns
+// h (Eq. 7) of the iteration under way from phase 1's partial sums, in FP64 in a fixed order.
+__device__ __forceinline__ void sum_h(const Dev &d)
+{
+    __shared__ double sh[8];
+    const int n = d.nbT * d.nwr;
+    double s = 0.0;
+    for (int q = threadIdx.x; q < n; q += RS_ROWS * RS_GROUPS)
+        s += d.hpart[q];
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1)
+        s += __shfl_xor_sync(0xffffffffu, s, off);
+    if ((threadIdx.x & 31) == 0)
+        sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 8; ++q)
+            s += sh[q];
+        d.ctl->h_next = s / ((double)d.T * (double)d.G);
+    }
+}
+
+// block b of one network's launch: b < ceil(T/32) rows of W, then its columns, the last one h
 __device__ __forceinline__ void reduce_wnorms_block(const Dev &d, int b)
 {
     if (!d.ctl->active)
         return;
     __shared__ double sh[1][RS_GROUPS][RS_ROWS];
     const int bT = ceil_div(d.T, RS_ROWS);
+    if (b == bT + ceil_div(d.G, RS_ROWS)) {
+        sum_h(d);
+        return;
+    }
     const bool rows = b < bT;
     const int x = ((rows ? b : b - bT) * RS_ROWS) + (threadIdx.x & (RS_ROWS - 1));
     const bool ok = x < (rows ? d.T : d.G);
@@ -121,46 +146,32 @@ __global__ void __launch_bounds__(RS_ROWS * RS_GROUPS) k_reduce_wnorms_set(const
     reduce_wnorms_block(devs[w.x], w.y);
 }
 
-// h (Eq. 7), the counter and the stop test, by the last block of a network's k_fin to finish (a
-// kernel of its own cost every iteration about 3 us at the smallest networks).
-__device__ __forceinline__ void tail_block(const Dev &d)
+// The history, the counter and the stop test, by one thread of a network's last k_fin block to
+// finish (a kernel of its own cost every iteration about 3 us at the smallest networks).
+__device__ __forceinline__ void tail(const Dev &d)
 {
     Ctl *ctl = d.ctl;
-    __shared__ double sh[256];
-    const int n = d.nbT * d.nwr;
-    double s = 0.0;
-    for (int q = threadIdx.x; q < n; q += blockDim.x)
-        s += d.hpart[q];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const double h = sh[0] / ((double)d.T * (double)d.G);
-        const int t = ctl->iters + 1;
-        if (t - 1 < HIST_CAP)
-            d.hist[t - 1] = h;
-        ctl->iters = t;
-        ctl->h_last = h;
-        ctl->converged = h < ctl->tol;
-        if (d.fp8) {  // the new state's norm maxima, and the scale of the next W' (Eq. 2)
-            for (int q = 0; q < 4; ++q) {
-                d.f8n[4 + q] = *(volatile unsigned *)&d.f8n[q];
-                d.f8n[q] = 0u;
-            }
-            d.f8[3] = e4m3_scale(fp8_bound_w(__uint_as_float(d.f8n[4]), __uint_as_float(d.f8n[5]),
-                                             __uint_as_float(d.f8n[6]), __uint_as_float(d.f8n[7])));
+    const double h = ctl->h_next;
+    const int t = ctl->iters + 1;
+    if (t - 1 < HIST_CAP)
+        d.hist[t - 1] = h;
+    ctl->iters = t;
+    ctl->h_last = h;
+    ctl->converged = h < ctl->tol;
+    if (d.fp8) {  // the new state's norm maxima, and the scale of the next W' (Eq. 2)
+        for (int q = 0; q < 4; ++q) {
+            d.f8n[4 + q] = *(volatile unsigned *)&d.f8n[q];
+            d.f8n[q] = 0u;
         }
-        ctl->fin_blocks = 0;
-        int status = *(volatile int *)&ctl->status;  // the other blocks' findings
-        if (!isfinite(h))
-            ctl->status = status |= ST_NONFINITE;
-        if (ctl->converged || t >= ctl->stop_at || status)
-            ctl->active = 0;
+        d.f8[3] = e4m3_scale(fp8_bound_w(__uint_as_float(d.f8n[4]), __uint_as_float(d.f8n[5]),
+                                         __uint_as_float(d.f8n[6]), __uint_as_float(d.f8n[7])));
     }
+    ctl->fin_blocks = 0;
+    int status = *(volatile int *)&ctl->status;  // the other blocks' findings
+    if (!isfinite(h))
+        ctl->status = status |= ST_NONFINITE;
+    if (ctl->converged || t >= ctl->stop_at || status)
+        ctl->active = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -174,13 +185,20 @@ __device__ __forceinline__ void fin_block(const Dev &d, int b)
     const Ctl *ctl = d.ctl;
     if (!ctl->active)  // (the network's last block clears it once every other block has passed here)
         return;
-    __shared__ int last;
+    if (b == ceil_div(d.T, RS_ROWS) + ceil_div(d.G, RS_ROWS))  // (h's block in a set's list: done)
+        return;
     __shared__ double sh[3][RS_GROUPS][RS_ROWS];
     const int bT = ceil_div(d.T, RS_ROWS);
     const bool isP = b < bT;
     const int i = ((isP ? b : b - bT) * RS_ROWS) + (threadIdx.x & (RS_ROWS - 1));
     const int n = isP ? d.T : d.G;       // network size
     const bool ok = i < n;
+    // what the end needs besides the sums is fetched with them
+    const double alpha = (double)ctl->alpha;
+    const int t = ctl->iters + 1;
+    const double growth = d.e2tab[t < HIST_CAP ? t : HIST_CAP];
+    double *dg = isP ? d.pd : d.cd;
+    const double old = threadIdx.x < RS_ROWS && ok ? dg[i] : 0.0;
     const int ld = isP ? d.Tp : d.Gp;
     const float *const src[3] = {isP ? d.ps_sum : d.cs_sum, isP ? d.ps_sq : d.cs_sq, isP ? d.ps_vsq : d.cs_vsq};
     double sums[3];
@@ -198,20 +216,16 @@ __device__ __forceinline__ void fin_block(const Dev &d, int b)
     }
     float nrm = 0.0f;  // the row's new squared norm (0 past the network)
     if (threadIdx.x < RS_ROWS && ok) {
-        const double s1 = sums[0], s2 = sums[1], sv = sums[2];
-        const double alpha = (double)ctl->alpha;
-        const int t = ctl->iters + 1;
-        const double growth = d.e2tab[t < HIST_CAP ? t : HIST_CAP];
+        const double s1 = sums[0], s2 = sums[1], sv = sums[2], inv = isP ? d.inv_n1P : d.inv_n1C;
         double sigma = 0.0;  // population std of the n - 1 off-diagonal entries (0 for one entry)
         if (n > 2) {
-            const double m = s1 / (double)(n - 1);
-            const double var = s2 / (double)(n - 1) - m * m;
+            const double m = s1 * inv;
+            const double var = s2 * inv - m * m;
             sigma = var > 0.0 ? sqrt(var) : 0.0;
         }
         const double gain = d.diag == 1 ? 1.0 : alpha;  // PANDA_DIAG_D0_LITERAL has no alpha
         const double mult = isP ? (double)d.G : (double)d.T;  // N_a with P, N_e with C
-        double *dg = isP ? d.pd : d.cd;
-        const double nd = (1.0 - alpha) * dg[i] + gain * mult * sigma * growth;
+        const double nd = (1.0 - alpha) * old + gain * mult * sigma * growth;
         dg[i] = nd;
         const float ndf = (float)nd;
         nrm = (float)(sv + nd * nd);
@@ -222,15 +236,14 @@ __device__ __forceinline__ void fin_block(const Dev &d, int b)
     }
     if (d.fp8 && threadIdx.x < RS_ROWS)  // the whole first warp, past the network too
         fp8_norm_max(&d.f8n[isP ? 0 : 1], nrm);
-    if (threadIdx.x < RS_ROWS)
+    if (threadIdx.x < RS_ROWS) {  // the first warp did the work
         __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0)
-        last = atomicAdd(&d.ctl->fin_blocks, 1u) + 1u == (unsigned)(bT + ceil_div(d.G, RS_ROWS));
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        tail_block(d);
+        __syncwarp();
+        if (threadIdx.x == 0 &&
+            atomicAdd(&d.ctl->fin_blocks, 1u) + 1u == (unsigned)(bT + ceil_div(d.G, RS_ROWS))) {
+            __threadfence();
+            tail(d);
+        }
     }
 }
 
@@ -249,7 +262,7 @@ __global__ void __launch_bounds__(RS_ROWS * RS_GROUPS) k_fin_set(const Dev *devs
 
 cudaError_t launch_reduce_wnorms(const Dev &d, cudaStream_t s)
 {
-    return launch(k_reduce_wnorms, set_norm_blocks(d.T, d.G), RS_ROWS * RS_GROUPS, 0, s, d);
+    return launch(k_reduce_wnorms, set_norm_blocks(d.T, d.G) + 1, RS_ROWS * RS_GROUPS, 0, s, d);
 }
 
 cudaError_t launch_reduce_wnorms_set(const Dev *devs, const int2 *blocks, int nblocks, cudaStream_t s)

@@ -2342,7 +2342,7 @@ cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out)
         const Dev &d = *ds[k];
         hd.push_back(d);
         hm.push_back(static_cast<const TcHost *>(d.tc_host)->maps);
-        for (int b = 0; b < set_norm_blocks(d.T, d.G); ++b)
+        for (int b = 0; b <= set_norm_blocks(d.T, d.G); ++b)
             bl.push_back(make_int2(k, b));
     }
     t->nblocks = (int)bl.size();

@@ -126,6 +126,8 @@ int plan_memory(panda_ctx *c)
     const size_t Tp = c->Tp, Gp = c->Gp;
     d.T = c->T; d.G = c->G; d.Tp = c->Tp; d.Gp = c->Gp; d.nbT = c->nbT; d.nbG = c->nbG;
     d.diag = c->diag;
+    d.inv_n1P = c->T > 1 ? 1.0 / (c->T - 1) : 0.0;
+    d.inv_n1C = c->G > 1 ? 1.0 / (c->G - 1) : 0.0;
     d.split_b = c->prec == PANDA_BF16X2 ? 0 : 1;  // the BF16 products of FP8MIX are BF16X3
     d.fp8 = c->prec == PANDA_FP8MIX ? 1 : 0;
     // BF16X3 and BF16X2 hold C as its split pair only (FP32 C is staged while the state is derived)

@@ -42,6 +42,7 @@ struct Ctl {
     unsigned fin_blocks;  // k_fin: blocks done in this iteration (the last one runs the tail)
     double tol;
     double h_last;
+    double h_next;  // h of the iteration under way (k_reduce_wnorms)
 };
 
 enum : int { ST_NONFINITE = 1, ST_TIMEOUT = 2 };
@@ -50,6 +51,7 @@ enum : int { ST_NONFINITE = 1, ST_TIMEOUT = 2 };
 struct Dev {
     int T, G, Tp, Gp, nbT, nbG;  // true sizes, padded sizes, 128-blocks
     int diag;                    // panda_diag
+    double inv_n1P, inv_n1C;     // 1 / (T - 1), 1 / (G - 1) (0 for one node)
     float *W[2], *Wt[2];         // Wt: FP32 and FP8MIX only (NULL under BF16X3 and BF16X2)
     float *Poff, *Coff;
     double *pd, *cd;
@@ -252,10 +254,10 @@ struct KernelEvents {
 // ---- after the products (k_norms.cu) ----------------------------------------
 // Diagonals, norms of P and C, h, counter, stop test
 cudaError_t launch_fin(const Dev &d, cudaStream_t s, KernelEvents &ke);
-// FP64 sums of the per-tile norm partials of W'
+// FP64 sums of the per-tile norm partials of W', and h
 cudaError_t launch_reduce_wnorms(const Dev &d, cudaStream_t s);
 // The same kernels over a set of networks (device arrays): blocks[b] = (network,
-// that network's block), set_norm_blocks(T, G) blocks per network.
+// that network's block), set_norm_blocks(T, G) + 1 blocks per network.
 cudaError_t launch_reduce_wnorms_set(const Dev *devs, const int2 *blocks, int nblocks, cudaStream_t s);
 cudaError_t launch_fin_set(const Dev *devs, const int2 *blocks, int nblocks, cudaStream_t s);
 int set_norm_blocks(int T, int G);

@@ -55,8 +55,7 @@ constexpr size_t STATIC_BYTES = 4 * SQ                  // W[2], Poff, Coff
                                 + 2 * VD + 6 * VF       // pd, cd; pdf, cdf, rsqP, csqC, rsqW, csqW
                                 + 8 * PART              // wrow, wcol, ps_sum/sq/vsq, cs_sum/sq/vsq
                                 + al256(sizeof(double) * 2 * SNB * SNB)  // hpart
-                                + al256(sizeof(Ctl)) + 2 * al256(2 * sizeof(double))  // ctl, hist, e2tab
-                                + al256(4 * sizeof(int))             // validation flags
+                                + al256(sizeof(Ctl) + 4 * sizeof(int)) + 2 * al256(2 * sizeof(double))  // ctl, hist, e2tab
                                 + al256(F32_STATIC_SLOT_BYTES) + al256(F32_STATIC_LIST_BYTES);
 
 __device__ __align__(256) unsigned char g_scratch[STATIC_BYTES];
@@ -125,6 +124,8 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     d.nwr = 2 * d.nbG;
     d.narrow = 1;
     d.diag = diag;
+    d.inv_n1P = T > 1 ? 1.0 / (T - 1) : 0.0;
+    d.inv_n1C = G > 1 ? 1.0 / (G - 1) : 0.0;
     unsigned char *p = base;
     auto take = [&p](size_t bytes) { unsigned char *q = p; p += bytes; return q; };
     auto part = [&take]() { return (__nv_bfloat16 *)take(BF); };
@@ -153,10 +154,10 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     d.cs_sq = (float *)take(PART);
     d.cs_vsq = (float *)take(PART);
     d.hpart = (double *)take(al256(sizeof(double) * 2 * SNB * SNB));
-    d.ctl = (Ctl *)take(al256(sizeof(Ctl)));
+    d.ctl = (Ctl *)take(al256(sizeof(Ctl) + 4 * sizeof(int)));
     d.hist = (double *)take(al256(2 * sizeof(double)));
     d.e2tab = (double *)take(al256(2 * sizeof(double)));
-    int *flags = (int *)take(al256(4 * sizeof(int)));
+    int *flags = (int *)(d.ctl + 1);  // read back with the control block
 
     d.p1_acc = (float *)take(al256(F32_STATIC_SLOT_BYTES));
     void *lists = take(al256(F32_STATIC_LIST_BYTES));
@@ -185,11 +186,11 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     SCU(launch_store(StateOut{T, G, d.Tp, d.Gp, d.W[1], d.Poff, d.Coff, nullptr, nullptr, d.pd, d.cd, dW, dP, dC, flags,
                               d.ctl},
                      s));
-    Ctl hc{};
-    int hflags[4] = {0, 0, 0, 0};
-    SCU(cudaMemcpyAsync(&hc, d.ctl, sizeof hc, cudaMemcpyDeviceToHost, s));
-    SCU(cudaMemcpyAsync(hflags, flags, sizeof hflags, cudaMemcpyDeviceToHost, s));
+    struct { Ctl ctl; int flags[4]; } back{};
+    SCU(cudaMemcpyAsync(&back, d.ctl, sizeof(Ctl) + 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
     SCU(cudaStreamSynchronize(s));
+    const Ctl &hc = back.ctl;
+    const int *hflags = back.flags;
     if (hflags[0])
         return fail(PANDA_ENONFINITE, "panda_step_static: a network has a non-finite entry");
     if (hflags[1])
