@@ -867,7 +867,6 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                     const float4 n4 = *reinterpret_cast<const float4 *>(colnrm + cc + ec);
                     const float nj[4] = {n4.x, n4.y, n4.z, n4.w};
                     const bool inner = k0 + 31 < j0 && j0 + 15 < nn;
-                    uint32_t vm = 0xffffu;  // bit 4 i + u: entry (row i, column u) counts
                     auto update = [&](int i, int u, bool valid) {
                         const float s = tanimoto_newton(x[i][u], nrow[i], nj[u]);
                         // (1 - a) X + a s without rounding 1 - a
@@ -889,8 +888,24 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
 #pragma unroll
                             for (int u = 0; u < 4; ++u)
                                 update(i, u, true);
+                        const size_t ro = xo + c * 16, r8 = (size_t)8 * ld;
+                        uint32_t p0[4][3], p1[4][3];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            split3(v[i][0], v[i][1], p0[i]);
+                            split3(v[i][2], v[i][3], p1[i]);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            *reinterpret_cast<float4 *>(X + ro + i * r8) =
+                                make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+#pragma unroll
+                        for (int p = 0; p < 3; ++p)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                *reinterpret_cast<uint2 *>(Xs[p] + ro + i * r8) = make_uint2(p0[i][p], p1[i][p]);
                     } else {
-                        vm = 0;
+                        uint32_t vm = 0;  // bit 4 i + u: entry (row i, column u) counts
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -899,29 +914,29 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                                 vm |= valid ? 1u << (4 * i + u) : 0u;
                                 update(i, u, valid);
                             }
-                    }
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const size_t ro = xo + (size_t)(8 * i) * ld + c * 16;
-                        const uint32_t m = vm >> (4 * i) & 15u;
-                        uint32_t p0[3], p1[3];
-                        split3(v[i][0], v[i][1], p0);
-                        split3(v[i][2], v[i][3], p1);
-                        if (m == 15u) {
-                            *reinterpret_cast<float4 *>(X + ro) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+                        for (int i = 0; i < 4; ++i) {
+                            const size_t ro = xo + (size_t)(8 * i) * ld + c * 16;
+                            const uint32_t m = vm >> (4 * i) & 15u;
+                            uint32_t p0[3], p1[3];
+                            split3(v[i][0], v[i][1], p0);
+                            split3(v[i][2], v[i][3], p1);
+                            if (m == 15u) {
+                                *reinterpret_cast<float4 *>(X + ro) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
 #pragma unroll
-                            for (int p = 0; p < 3; ++p)
-                                *reinterpret_cast<uint2 *>(Xs[p] + ro) = make_uint2(p0[p], p1[p]);
-                        } else if (m) {
+                                for (int p = 0; p < 3; ++p)
+                                    *reinterpret_cast<uint2 *>(Xs[p] + ro) = make_uint2(p0[p], p1[p]);
+                            } else if (m) {
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (m >> u & 1u) {
-                                    X[ro + u] = v[i][u];
+                                for (int u = 0; u < 4; ++u)
+                                    if (m >> u & 1u) {
+                                        X[ro + u] = v[i][u];
 #pragma unroll
-                                    for (int p = 0; p < 3; ++p)
-                                        reinterpret_cast<uint16_t *>(Xs[p])[ro + u] =
-                                            (uint16_t)((u < 2 ? p0[p] : p1[p]) >> (16 * (u & 1)));
-                                }
+                                        for (int p = 0; p < 3; ++p)
+                                            reinterpret_cast<uint16_t *>(Xs[p])[ro + u] =
+                                                (uint16_t)((u < 2 ? p0[p] : p1[p]) >> (16 * (u & 1)));
+                                    }
+                            }
                         }
                     }
                     // mirrored entries (j, k) through this warp's staging block, MR rows at a time: lane l

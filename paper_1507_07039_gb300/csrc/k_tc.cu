@@ -1570,7 +1570,6 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
                 const float4 n4 = *reinterpret_cast<const float4 *>(colnrm + cc + ec);
                 const float nj[4] = {n4.x, n4.y, n4.z, n4.w};
                 const bool inner = k0 + 31 < j0 && j0 + 15 < nn;  // the whole 32 x 16 block counts
-                uint32_t vm = 0xffffu;                            // bit 4 i + u: entry (row i, column u) counts
                 float cs[8], cv[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -1593,8 +1592,41 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
                             }
                             v[i][u] = w;
                         }
+                    // the new entries, row-major, from this lane's registers: the four lanes of a row
+                    // write 16 consecutive columns (32 bytes of each BF16 half, 64 of FP32)
+                    // (in one straight line; with the edge blocks' check of each row's mask the kernel took
+                    // 0.92 ms instead of 0.86 for 12 networks of 241-987 x 2238-7773, 0.74 instead of 0.72 at
+                    // 1000 x 17000 under BF16X3)
+                    const size_t r0 = xo + cc, r8 = (size_t)8 * ld;
+                    if (q8) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            *reinterpret_cast<uint32_t *>(d.C8 + r0 + i * r8) =
+                                e4m3x2(v[i][0], v[i][1], sC) | e4m3x2(v[i][2], v[i][3], sC) << 16;
+                    } else {
+                        uint32_t h2[4][2], l2[4][2];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            split_pair(v[i][0], v[i][1], h2[i][0], l2[i][0]);
+                            split_pair(v[i][2], v[i][3], h2[i][1], l2[i][1]);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            *reinterpret_cast<uint2 *>(Xh + r0 + i * r8) = make_uint2(h2[i][0], h2[i][1]);
+                        if (wlo) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                *reinterpret_cast<uint2 *>(Xl + r0 + i * r8) = make_uint2(l2[i][0], l2[i][1]);
+                        }
+                    }
+                    if (!sst) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            *reinterpret_cast<float4 *>(X + r0 + i * r8) =
+                                make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+                    }
                 } else {
-                    vm = 0;
+                    uint32_t vm = 0;  // bit 4 i + u: entry (row i, column u) counts
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -1615,54 +1647,52 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
                             v[i][u] = w;
                             vm |= valid ? 1u << (4 * i + u) : 0u;
                         }
-                }
-                // (a) the new entries, row-major, from this lane's registers: the four lanes of a row
-                // write 16 consecutive columns (32 bytes of each BF16 half, 64 of FP32)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const size_t ro = xo + (size_t)(8 * i) * ld + cc;
-                    const uint32_t m = vm >> (4 * i) & 15u;
-                    if (!q8) {
-                        uint32_t h2[2], l2[2];
-                        split_pair(v[i][0], v[i][1], h2[0], l2[0]);
-                        split_pair(v[i][2], v[i][3], h2[1], l2[1]);
-                        if (m == 15u) {
-                            *reinterpret_cast<uint2 *>(Xh + ro) = make_uint2(h2[0], h2[1]);
-                            if (wlo)
-                                *reinterpret_cast<uint2 *>(Xl + ro) = make_uint2(l2[0], l2[1]);
-                        } else if (m) {
+                    for (int i = 0; i < 4; ++i) {
+                        const size_t ro = xo + (size_t)(8 * i) * ld + cc;
+                        const uint32_t m = vm >> (4 * i) & 15u;
+                        if (!q8) {
+                            uint32_t h2[2], l2[2];
+                            split_pair(v[i][0], v[i][1], h2[0], l2[0]);
+                            split_pair(v[i][2], v[i][3], h2[1], l2[1]);
+                            if (m == 15u) {
+                                *reinterpret_cast<uint2 *>(Xh + ro) = make_uint2(h2[0], h2[1]);
+                                if (wlo)
+                                    *reinterpret_cast<uint2 *>(Xl + ro) = make_uint2(l2[0], l2[1]);
+                            } else if (m) {
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (m >> u & 1u) {
-                                    reinterpret_cast<uint16_t *>(Xh)[ro + u] = (uint16_t)(h2[u >> 1] >> (16 * (u & 1)));
-                                    if (wlo)
-                                        reinterpret_cast<uint16_t *>(Xl)[ro + u] =
-                                            (uint16_t)(l2[u >> 1] >> (16 * (u & 1)));
-                                }
+                                for (int u = 0; u < 4; ++u)
+                                    if (m >> u & 1u) {
+                                        reinterpret_cast<uint16_t *>(Xh)[ro + u] = (uint16_t)(h2[u >> 1] >> (16 * (u & 1)));
+                                        if (wlo)
+                                            reinterpret_cast<uint16_t *>(Xl)[ro + u] =
+                                                (uint16_t)(l2[u >> 1] >> (16 * (u & 1)));
+                                    }
+                            }
+                        } else {
+                            const uint32_t p8 = e4m3x2(v[i][0], v[i][1], sC) | e4m3x2(v[i][2], v[i][3], sC) << 16;
+                            if (m == 15u) {
+                                *reinterpret_cast<uint32_t *>(d.C8 + ro) = p8;
+                            } else if (m) {
+#pragma unroll
+                                for (int u = 0; u < 4; ++u)
+                                    if (m >> u & 1u)
+                                        d.C8[ro + u] = (uint8_t)(p8 >> (8 * u));
+                            }
                         }
-                    } else {
-                        const uint32_t p8 = e4m3x2(v[i][0], v[i][1], sC) | e4m3x2(v[i][2], v[i][3], sC) << 16;
-                        if (m == 15u) {
-                            *reinterpret_cast<uint32_t *>(d.C8 + ro) = p8;
-                        } else if (m) {
+                        if (!sst) {
+                            if (m == 15u) {
+                                *reinterpret_cast<float4 *>(X + ro) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+                            } else if (m) {
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (m >> u & 1u)
-                                    d.C8[ro + u] = (uint8_t)(p8 >> (8 * u));
-                        }
-                    }
-                    if (!sst) {
-                        if (m == 15u) {
-                            *reinterpret_cast<float4 *>(X + ro) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
-                        } else if (m) {
-#pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (m >> u & 1u)
-                                    X[ro + u] = v[i][u];
+                                for (int u = 0; u < 4; ++u)
+                                    if (m >> u & 1u)
+                                        X[ro + u] = v[i][u];
+                            }
                         }
                     }
                 }
-                // (b) the column sums over the warp's 32 rows: this lane's four rows are summed above,
+                // the column sums over the warp's 32 rows: this lane's four rows are summed above,
                 // the eight lanes of a column reduce-scatter their eight sums (7 shuffles)
                 {
                     const float t = lanes8_reduce_scatter8(cs);
@@ -1674,7 +1704,7 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
                             colred[(wq * NS + 2) * N2 + cc + ec + (lane >> 3 & 1) + 2 * (lane >> 4)] = tv;
                     }
                 }
-                // (c) mirrored entries (j, k), through this warp's staging block: lane l takes column
+                // mirrored entries (j, k), through this warp's staging block: lane l takes column
                 // (l & 15), rows 16 (l >> 4) + 0..15
                 if (mirror) {
 #pragma unroll
