@@ -230,108 +230,148 @@ __device__ __forceinline__ void load_w(const float *X, int rows, int cols, int l
 }
 
 // A symmetric n x n network (row stride ldi) as 64 x 64 blocks: each pair of
-// mirror blocks (bi, bj), (bj, bi), bi <= bj, is read once, along rows, into
-// shared memory.  flags[0] |= 1 on a non-finite entry, flags[1] |= 1 when
-// X[i][j] != X[j][i].  Written, padding (to out.ld) included: block (bi, bj) of
+// mirror blocks (bi, bj), (bj, bi), bi <= bj, is read once, along rows.
+// flags[0] |= 1 on a non-finite entry, flags[1] |= 1 when X[i][j] != X[j][i].
+// Written, padding (to out.ld, a multiple of 64) included: block (bi, bj) of
 // out.F and of the parts, block (bj, bi) too where the form holds it; the
 // diagonal goes to out.d and out.df and reads as zero in F and the parts.  X
 // may be out.F itself (each block pair is one block's alone).  256 threads.
+// Bound by memory.  A thread holds four entries of four rows of the upper block
+// in registers and only the lower block goes through shared memory; whole
+// blocks of 16-byte aligned rows load 16 bytes at a time without a bounds
+// check.  With both blocks in shared memory, scalar loads and a check per entry
+// the instructions took longer than the bytes: 545 us for the networks of
+// 1000 x 17000 under BF16X3 (2.07 GB), 355 us now.
 constexpr int LB = 64;
 __host__ __device__ inline int block_pairs(int ld) { return ceil_div(ld, LB) * (ceil_div(ld, LB) + 1) / 2; }
+// pair t of the upper triangle's blocks, numbered column by column; 8 t + 1 < 2^24 for n <= 46000, so
+// the FP32 square root is close; the loops correct it
+__device__ __forceinline__ void block_pair(int t, int &bi, int &bj)
+{
+    bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while (bj > 0 && bj * (bj + 1) / 2 > t)
+        --bj;
+    while ((bj + 1) * (bj + 2) / 2 <= t)
+        ++bj;
+    bi = t - bj * (bj + 1) / 2;
+}
 __device__ __forceinline__ void load_sym(const float *X, int n, int ldi, const double *stats, const SymOut &out, int *flags,
                                          int first, int step)
 {
     const int npairs = block_pairs(out.ld);
-    __shared__ float a[LB][LB + 1], b[LB][LB + 1];
-    const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // loads: 4 rows of 64
-    const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // stores: 16 rows of 16 x 4
-    int bad = 0, asym = 0;
+    __shared__ float lo[LB][LB + 1], up[LB][LB + 1];  // rows of 65: columns are read as well as rows
+    const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // rows tr, tr + 16, ..., four columns
+    const bool aligned = (ldi & 3) == 0 && ((uintptr_t)X & 15) == 0;
+    const float4 q = stats ? stats_pairs(stats) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float nf = 0.0f;  // NaN once an entry is not finite
+    bool asym = false;
     for (int t = first; t < npairs; t += step) {
-        // pairs are numbered column by column of the upper triangle; 8t + 1 < 2^24 for n <= 46000, so the
-        // FP32 square root is close; the loops correct it
-        int bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-        while (bj > 0 && bj * (bj + 1) / 2 > t)
-            --bj;
-        while ((bj + 1) * (bj + 2) / 2 <= t)
-            ++bj;
-        const int bi = t - bj * (bj + 1) / 2, i0 = bi * LB, j0 = bj * LB;
-        const bool diag = bi == bj;
+        int bi, bj;
+        block_pair(t, bi, bj);
+        const int i0 = bi * LB, j0 = bj * LB;
+        const bool whole = j0 + LB <= n;  // (i0 <= j0)
+        float a[4][4];
+        if (whole && aligned) {
+            float4 v[4], w[4];
 #pragma unroll
-        for (int k = 0; k < LB; k += 4) {
-            const int ra = i0 + k + ty, ca = j0 + tx;
-            a[k + ty][tx] = (ra < n && ca < n) ? X[(size_t)ra * ldi + ca] : 0.0f;
-        }
-        if (!diag) {
+            for (int k = 0; k < 4; ++k)
+                v[k] = __ldcs(reinterpret_cast<const float4 *>(X + (size_t)(i0 + 16 * k + tr) * ldi + j0 + c4));
 #pragma unroll
-            for (int k = 0; k < LB; k += 4) {
-                const int rb = j0 + k + ty, cb = i0 + tx;
-                b[k + ty][tx] = (rb < n && cb < n) ? X[(size_t)rb * ldi + cb] : 0.0f;
+            for (int k = 0; k < 4; ++k)
+                w[k] = __ldcs(reinterpret_cast<const float4 *>(X + (size_t)(j0 + 16 * k + tr) * ldi + i0 + c4));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                a[k][0] = v[k].x;
+                a[k][1] = v[k].y;
+                a[k][2] = v[k].z;
+                a[k][3] = v[k].w;
+                float *l = &lo[16 * k + tr][c4];
+                l[0] = w[k].x;
+                l[1] = w[k].y;
+                l[2] = w[k].z;
+                l[3] = w[k].w;
             }
-        }
-        __syncthreads();
-        const float(*m)[LB + 1] = diag ? a : b;
-        // rows of the upper block
+        } else {
 #pragma unroll
-        for (int k = 0; k < LB; k += 16) {
-            const int r = k + tr, gi = i0 + r;
-            float v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int gj = j0 + c4 + u;
-                v[u] = a[r][c4 + u];
-                bad |= !isfinite(v[u]) | !isfinite(m[r][c4 + u]);
-                asym |= v[u] != m[c4 + u][r];
-                if (stats && gi < n && gj < n)
-                    v[u] = zscore_one(v[u], stats_pairs(stats));
-                if (gi == gj && gi < n) {
-                    out.d[gi] = (double)v[u];
-                    out.df[gi] = v[u];
-                    v[u] = 0.0f;
-                }
-            }
-            if (gi < out.ld && j0 + c4 < out.ld) {
-                const size_t o = (size_t)gi * out.ld + j0 + c4;
-                if (out.F)
-                    *reinterpret_cast<float4 *>(out.F + o) = make_float4(v[0], v[1], v[2], v[3]);
-                put_parts(out.parts, o, v);
-            }
-        }
-        // rows of the lower block, from the upper one's columns
-        const bool lf = out.F && out.f_full, lp = out.parts.h && (out.p_full || i0 / out.p_block == j0 / out.p_block);
-        if (!diag && (lf || lp)) {
-#pragma unroll
-            for (int k = 0; k < LB; k += 16) {
-                const int r = k + tr, gj = j0 + r;
-                float v[4];
+            for (int k = 0; k < 4; ++k)
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    v[u] = a[c4 + u][r];
-                    if (stats && gj < n && i0 + c4 + u < n)
-                        v[u] = zscore_one(v[u], stats_pairs(stats));
+                    const int r = 16 * k + tr, c = c4 + u;
+                    a[k][u] = i0 + r < n && j0 + c < n ? X[(size_t)(i0 + r) * ldi + j0 + c] : 0.0f;
+                    lo[r][c] = j0 + r < n && i0 + c < n ? X[(size_t)(j0 + r) * ldi + i0 + c] : 0.0f;
                 }
-                if (gj < out.ld && i0 + c4 < out.ld) {
-                    const size_t o = (size_t)gj * out.ld + i0 + c4;
-                    if (lf)
-                        *reinterpret_cast<float4 *>(out.F + o) = make_float4(v[0], v[1], v[2], v[3]);
-                    if (lp)
-                        put_parts(out.parts, o, v);
-                }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float m = lo[c4 + u][16 * k + tr];
+                nf = fmaf(a[k][u], 0.0f, fmaf(m, 0.0f, nf));
+                asym |= a[k][u] != m;
+            }
+        if (stats) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (whole || (i0 + 16 * k + tr < n && j0 + c4 + u < n))
+                        a[k][u] = zscore_one(a[k][u], q);
+        }
+        if (bi == bj) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (16 * k + tr == c4 + u && i0 + c4 + u < n) {
+                        out.d[i0 + c4 + u] = (double)a[k][u];
+                        out.df[i0 + c4 + u] = a[k][u];
+                        a[k][u] = 0.0f;
+                    }
+        }
+        const bool lf = out.F && out.f_full, lp = out.parts.h && (out.p_full || i0 / out.p_block == j0 / out.p_block);
+        const bool lower = bi != bj && (lf || lp);
+        // rows of the upper block
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const size_t o = (size_t)(i0 + 16 * k + tr) * out.ld + j0 + c4;
+            if (out.F)
+                *reinterpret_cast<float4 *>(out.F + o) = make_float4(a[k][0], a[k][1], a[k][2], a[k][3]);
+            put_parts(out.parts, o, a[k]);
+            if (lower) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    up[16 * k + tr][c4 + u] = a[k][u];
             }
         }
         __syncthreads();
+        // rows of the lower block, from the upper one's columns (the next pair's writes to `up` are
+        // behind its own barrier)
+        if (lower) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int r = 16 * k + tr;
+                const float v[4] = {up[c4][r], up[c4 + 1][r], up[c4 + 2][r], up[c4 + 3][r]};
+                const size_t o = (size_t)(j0 + r) * out.ld + i0 + c4;
+                if (lf)
+                    *reinterpret_cast<float4 *>(out.F + o) = make_float4(v[0], v[1], v[2], v[3]);
+                if (lp)
+                    put_parts(out.parts, o, v);
+            }
+        }
     }
-    bad = __syncthreads_or(bad);
-    asym = __syncthreads_or(asym);
+    const int bad = __syncthreads_or(nf != nf);
+    const int ne = __syncthreads_or(asym);
     if (threadIdx.x == 0) {
         if (bad)
             atomicOr(&flags[0], 1);
-        if (asym)
+        if (ne)
             atomicOr(&flags[1], 1);
     }
 }
 
 // One launch: blocks [0, nc) C, [nc, nc + np) P, the rest W.
-__global__ void __launch_bounds__(256) k_load(const __grid_constant__ StateIn in, float *W, Parts wparts, int Gp,
+__global__ void __launch_bounds__(256, 4) k_load(const __grid_constant__ StateIn in, float *W, Parts wparts, int Gp,
                                               const __grid_constant__ SymOut P, const __grid_constant__ SymOut C, int nc,
                                               int np, int *flags)
 {
@@ -551,12 +591,9 @@ __device__ __forceinline__ void store_sym(const float *__restrict__ X, const __n
     const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // stores: 4 rows of 64
     const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // loads: 16 rows of 16 x 4
     for (int t = first; t < npairs; t += step) {
-        int bj = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);  // as in k_load_sym
-        while (bj > 0 && bj * (bj + 1) / 2 > t)
-            --bj;
-        while ((bj + 1) * (bj + 2) / 2 <= t)
-            ++bj;
-        const int bi = t - bj * (bj + 1) / 2, i0 = bi * LB, j0 = bj * LB;
+        int bi, bj;
+        block_pair(t, bi, bj);
+        const int i0 = bi * LB, j0 = bj * LB;
 #pragma unroll
         for (int k = 0; k < LB; k += 16) {
             const int r = k + tr, gi = i0 + r, gj = j0 + c4;
@@ -672,7 +709,7 @@ cudaError_t launch_stats(const float *X, int rows, int cols, int ld, double *sta
 cudaError_t launch_load(const StateIn &in, float *W, const Parts &wparts, int Tp, int Gp, const SymOut &P, const SymOut &C,
                         int *flags, cudaStream_t s)
 {
-    const int nc = std::min(block_pairs(C.ld), 152 * 6), np = std::min(block_pairs(P.ld), 152 * 2);
+    const int nc = std::min(block_pairs(C.ld), 152 * 4), np = std::min(block_pairs(P.ld), 152 * 2);
     k_load<<<nc + np + Tp * ceil_div(Gp, 1024), 256, 0, s>>>(in, W, wparts, Gp, P, C, nc, np, flags);
     return cudaGetLastError();
 }

@@ -140,6 +140,45 @@ __global__ void k_to_e4m3(const float *__restrict__ X, size_t n, uint8_t *__rest
         Q[q] = (uint8_t)e4m3x2(X[q], 0.0f, s);
 }
 
+// A symmetric matrix's E4M3 copy, both triangles, from the upper one (X and Q
+// Gp x Gp, Gp a multiple of 128): each 64 x 64 block above the diagonal is read
+// once and written twice, the second time turned through shared memory, four
+// entries to a word.  From both triangles the copy of C at 17000 genes took
+// 220 us and the load before it, which wrote them, 627 us; now 154 and 359.
+__global__ void __launch_bounds__(256) k_sym_to_e4m3(const float *__restrict__ X, int ld, uint8_t *__restrict__ Q,
+                                                     const float *scale)
+{
+    __shared__ float sh[64][65];
+    const int bi = blockIdx.x, bj = blockIdx.y, i0 = 64 * bi, j0 = 64 * bj;
+    if (bi > bj)
+        return;
+    const float s = *scale;
+    const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // rows tr, tr + 16, ..., four columns
+    float4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        v[k] = __ldcs(reinterpret_cast<const float4 *>(X + (size_t)(i0 + 16 * k + tr) * ld + j0 + c4));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = 16 * k + tr;
+        *reinterpret_cast<uint32_t *>(Q + (size_t)(i0 + r) * ld + j0 + c4) =
+            e4m3x2(v[k].x, v[k].y, s) | (e4m3x2(v[k].z, v[k].w, s) << 16);
+        sh[r][c4] = v[k].x;
+        sh[r][c4 + 1] = v[k].y;
+        sh[r][c4 + 2] = v[k].z;
+        sh[r][c4 + 3] = v[k].w;
+    }
+    if (bi == bj)  // holds both triangles
+        return;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = 16 * k + tr;
+        *reinterpret_cast<uint32_t *>(Q + (size_t)(j0 + r) * ld + i0 + c4) =
+            e4m3x2(sh[c4][r], sh[c4 + 1][r], s) | (e4m3x2(sh[c4 + 2][r], sh[c4 + 3][r], s) << 16);
+    }
+}
+
 // hi / lo of a whole array (padding stays zero because x is zero there); L may
 // be NULL (hi only).  Four values per thread from one 16-byte load, 8-byte
 // stores; a misaligned buffer takes the scalar loop.
@@ -2226,7 +2265,7 @@ cudaError_t tc_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
             k_fp8_init<<<1, 1024, 0, s>>>(d);
         k_to_e4m3<<<1024, 256, 0, s>>>(d.W[cur], TG, d.W8[cur], d.f8 + cur);
         k_to_e4m3<<<1024, 256, 0, s>>>(d.Wt[cur], TG, d.Wt8[cur], d.f8 + cur);
-        k_to_e4m3<<<2048, 256, 0, s>>>(d.Coff, (size_t)d.Gp * d.Gp, d.C8, d.f8 + 2);
+        k_sym_to_e4m3<<<dim3(d.Gp / 64, d.Gp / 64), 256, 0, s>>>(d.Coff, d.Gp, d.C8, d.f8 + 2);
     }
     if ((e = cudaGetLastError()))
         return e;

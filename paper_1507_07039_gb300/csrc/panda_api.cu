@@ -345,9 +345,9 @@ int load_state(panda_ctx *c, const float *W, const float *P, const float *C, int
     }
     const bool f32 = c->prec == PANDA_FP32;
     CU(cudaMemsetAsync(c->d_flags, 0, 4 * sizeof(int), c->stream));
-    // a network loaded in place keeps both triangles, for the norms below; FP8MIX's E4M3 copy of C is made from both
+    // a network loaded in place keeps both triangles, for the norms below
     const SymOut po{d.Poff, p.src == d.Poff, Parts{d.Ph, d.Pm, d.Pl}, 1, 256, c->Tp, d.pd, d.pdf};
-    const SymOut xo{d.c_split ? nullptr : d.Coff, d.fp8 || x.src == d.Coff,
+    const SymOut xo{d.c_split ? nullptr : d.Coff, x.src == d.Coff,
                     Parts{d.Ch, d.Cm, d.Cl}, 0, f32 ? f32_diag_block(d) : 256, c->Gp, d.cd, d.cdf};
     StateIn in{w.src, p.src, x.src, T, G, w.ld, p.ld, x.ld, st[0], st[1], st[2]};
     CU(launch_load(in, d.W[c->cur], Parts{d.Wh[c->cur], d.Wm[c->cur], d.Wl[c->cur]}, c->Tp, c->Gp, po, xo, c->d_flags,
