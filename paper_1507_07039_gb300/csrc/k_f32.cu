@@ -536,6 +536,43 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
             constexpr size_t FS = (size_t)(PAIR ? 2 : 1) * SLOT;
             if (cut)
                 rslot = fix;
+            // what the epilogue needs besides the sums comes in while the stages run (a pair's registers
+            // are taken by the sums: only the columns' vectors); read after them, its latency and a
+            // barrier were 1.5 us of a 34 us iteration at 125 x 125, 1 of 68 at 250 x 2100
+            for (int j = tt; j < N; j += 32 * EPI) {
+                const int gj = n0 + j;
+                const bool cj = gj < d.G;
+                colvec[j] = cj ? d.cdf[gj] : 0.0f;
+                colvec[N + j] = cj ? d.csqW[gj] : 0.0f;
+                colvec[2 * N + j] = cj ? d.csqC[gj] : 0.0f;
+            }
+            const int k0 = m0 + wq * 32;
+            const bool rows_in = m0 < d.Tp;
+            float pdi[4], rsp[4], rsw[4], rowsq[4];
+            auto fetch_rows = [&]() {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = k0 + er + 8 * i;
+                    const bool ri = r < d.T;
+                    pdi[i] = ri ? d.pdf[r] : 0.0f;
+                    rsp[i] = ri ? d.rsqP[r] : 0.0f;
+                    rsw[i] = ri ? d.rsqW[r] : 0.0f;
+                    rowsq[i] = 0.0f;
+                }
+            };
+            const size_t wo = (size_t)(k0 + er) * d.Gp + n0 + half * (N / 2) + ec;
+            uint4 wq0[4];
+            auto fetch_w = [&](int c) {
+                if (c < NCH && rows_in && n0 + half * (N / 2) + c * 16 < d.Gp) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        wq0[i] = *reinterpret_cast<const uint4 *>(W + wo + (size_t)(8 * i) * d.Gp + c * 16);
+                }
+            };
+            if (!PAIR) {
+                fetch_rows();
+                fetch_w(0);
+            }
             float acc[NCH][16];
             clear<NCH>(acc);
             bool live = sum_stages<PAIR>(sy, it, nR, g, tq, free_even, PAIR && !cut, ctl, acc, [&]() {
@@ -571,40 +608,18 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                 else
                     put_slot<NCH>(aslot, tt, acc);
             }
-            epi_bar();  // colvec of the item before is no longer read
-            for (int j = tt; j < N; j += 32 * EPI) {
-                const int gj = n0 + j;
-                const bool cj = gj < d.G;
-                colvec[j] = cj ? d.cdf[gj] : 0.0f;
-                colvec[N + j] = cj ? d.csqW[gj] : 0.0f;
-                colvec[2 * N + j] = cj ? d.csqC[gj] : 0.0f;
-            }
-            const int k0 = m0 + wq * 32;
-            const bool rows_in = m0 < d.Tp;
-            float pdi[4], rsp[4], rsw[4], rowsq[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = k0 + er + 8 * i;
-                const bool ri = r < d.T;
-                pdi[i] = ri ? d.pdf[r] : 0.0f;
-                rsp[i] = ri ? d.rsqP[r] : 0.0f;
-                rsw[i] = ri ? d.rsqW[r] : 0.0f;
-                rowsq[i] = 0.0f;
+            if (PAIR) {
+                fetch_rows();
+                fetch_w(0);
             }
             const float halfa = 0.5f * ctl->alpha;
-            const size_t wo = (size_t)(k0 + er) * d.Gp + n0 + half * (N / 2) + ec;
             float hsum = 0.0f;
-            epi_bar();
+            epi_bar();  // colvec is complete; colred and rowred of the item before are no longer read
             // W, R-num and the sums one chunk ahead
-            uint4 wq0[4];
             uint32_t rq0[16], ar[16];
-            auto fetch = [&](int c, uint4 (&wv)[4], uint32_t (&rv)[16]) {
-                if (c < NCH && live && rows_in && n0 + half * (N / 2) + c * 16 < d.Gp) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        wv[i] = *reinterpret_cast<const uint4 *>(W + wo + (size_t)(8 * i) * d.Gp + c * 16);
-                    get_slot16(rslot, c, tt, rv);
-                }
+            auto fetch_r = [&](int c) {
+                if (c < NCH && live && rows_in && n0 + half * (N / 2) + c * 16 < d.Gp)
+                    get_slot16(rslot, c, tt, rq0);
             };
             auto fetch_sums = [&](int c) {
                 if (in_tmem)
@@ -612,7 +627,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                 else
                     get_slot16(aslot, c, tt, ar);
             };
-            fetch(0, wq0, rq0);
+            fetch_r(0);
             if (live)
                 fetch_sums(0);
 #pragma unroll 1
@@ -633,7 +648,8 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                     w[i][2] = __uint_as_float(wq0[i].z);
                     w[i][3] = __uint_as_float(wq0[i].w);
                 }
-                fetch(c + 1, wq0, rq0);
+                fetch_w(c + 1);
+                fetch_r(c + 1);
                 if (rows_in && j0 < d.Gp) {
                     const float4 c4 = *reinterpret_cast<const float4 *>(colvec + cc + ec);
                     const float4 w4 = *reinterpret_cast<const float4 *>(colvec + N + cc + ec);
@@ -777,6 +793,37 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
             const int bm = (int)(it.a & 0x7fffu), bn = (int)(it.a >> 15 & 0x7fffu);
             constexpr size_t FS = (size_t)(PAIR ? 2 : 1) * SLOT;
             float *fix = d.p1_fix + (size_t)((PAIR ? 2 : 1) * it.slot) * SLOT + (size_t)rank * SLOT;
+            const int nn = isP ? d.T : d.G, ld = isP ? d.Tp : d.Gp;
+            const int m0 = bm * Tile<PAIR>::M + 128 * (int)rank, n0 = bn * N;
+            const float *nrm = isP ? d.rsqW : d.csqW;
+            float *X = isP ? d.Poff : d.Coff;
+            const bool rows_in = m0 < ld;
+            const int k0 = m0 + wq * 32;
+            // what the epilogue needs besides the sums comes in while the stages run (as in phase 1)
+            for (int j = tt; j < N; j += 32 * EPI)
+                colnrm[j] = n0 + j < nn ? nrm[n0 + j] : 0.0f;
+            float nrow[4], r1[4], r2[4], rv[4];
+            auto fetch_rows = [&]() {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    nrow[i] = k0 + er + 8 * i < nn ? nrm[k0 + er + 8 * i] : 0.0f;
+                    r1[i] = r2[i] = rv[i] = 0.0f;
+                }
+            };
+            const size_t xo = (size_t)(k0 + er) * ld + n0 + half * (N / 2) + ec;
+            // old values (and the sums below) one chunk ahead (three ahead measured the same)
+            uint4 o0[4];
+            auto fetch = [&](int c) {
+                if (c < NCH && rows_in && n0 + half * (N / 2) + c * 16 < ld) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        o0[i] = *reinterpret_cast<const uint4 *>(X + xo + (size_t)(8 * i) * ld + c * 16);
+                }
+            };
+            if (!PAIR) {
+                fetch_rows();
+                fetch(0);
+            }
             float acc[NCH][16];
             clear<NCH>(acc);
             const bool live = sum_stages<PAIR>(sy, it, -1, g, tq, free_even, PAIR && !cut, ctl, acc, []() {});
@@ -801,44 +848,22 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                 else
                     put_slot<NCH>(fix, tt, acc);
             }
-            const int nn = isP ? d.T : d.G, ld = isP ? d.Tp : d.Gp;
-            const int m0 = bm * Tile<PAIR>::M + 128 * (int)rank, n0 = bn * N;
-            const float *nrm = isP ? d.rsqW : d.csqW;
-            float *X = isP ? d.Poff : d.Coff;
             __nv_bfloat16 *Xs[3] = {isP ? d.Ph : d.Ch, isP ? d.Pm : d.Cm, isP ? d.Pl : d.Cl};
             // split copies of the lower triangle: all of P, of C only inside diagonal tiles
             const bool mirror = isP || (PAIR ? bm == bn : bm == bn >> 1);
-            const bool rows_in = m0 < ld;
             const float a = ctl->alpha;
-            epi_bar();  // colnrm, colred and rowred of the item before are no longer read
-            for (int j = tt; j < N; j += 32 * EPI)
-                colnrm[j] = n0 + j < nn ? nrm[n0 + j] : 0.0f;
-            const int k0 = m0 + wq * 32;
-            float nrow[4], r1[4], r2[4], rv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                nrow[i] = k0 + er + 8 * i < nn ? nrm[k0 + er + 8 * i] : 0.0f;
-                r1[i] = r2[i] = rv[i] = 0.0f;
+            if (PAIR) {
+                fetch_rows();
+                fetch(0);
             }
-            const size_t xo = (size_t)(k0 + er) * ld + n0 + half * (N / 2) + ec;
-            epi_bar();
-            // old values and sums one chunk ahead (three ahead measured the same)
-            uint4 o0[4];
+            epi_bar();  // colnrm is complete; colred and rowred of the item before are no longer read
             uint32_t ar[16];
-            auto fetch = [&](int c, uint4 (&v)[4]) {
-                if (c < NCH && live && rows_in && n0 + half * (N / 2) + c * 16 < ld) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        v[i] = *reinterpret_cast<const uint4 *>(X + xo + (size_t)(8 * i) * ld + c * 16);
-                }
-            };
             auto fetch_sums = [&](int c) {
                 if (in_tmem)
                     tmem_ld_frag16_nowait(tsum + c * 16, ar);
                 else
                     get_slot16(fix, c, tt, ar);
             };
-            fetch(0, o0);
             if (live)
                 fetch_sums(0);
 #pragma unroll 1
@@ -861,7 +886,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                     v[i][2] = __uint_as_float(o0[i].z);
                     v[i][3] = __uint_as_float(o0[i].w);
                 }
-                fetch(c + 1, o0);
+                fetch(c + 1);
                 // a block with no entry above the diagonal or inside the network has nothing to do
                 if (rows_in && j0 < ld && k0 < j0 + 15) {
                     const float4 n4 = *reinterpret_cast<const float4 *>(colnrm + cc + ec);
