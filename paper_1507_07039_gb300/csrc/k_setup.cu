@@ -581,7 +581,8 @@ __global__ void k_standardize_rows(const float *__restrict__ X, int G, int N, __
 // strict upper triangle, FP32 in X or a BF16 split pair H + L (exact in FP32;
 // row stride ldi, a multiple of 4), and its FP64 diagonal, in 64 x 64 blocks:
 // each block above the diagonal is read once and written twice, the second
-// time turned through shared memory.  256 threads.
+// time turned through shared memory, 16 bytes at a time where the rows allow it
+// (1000 x 17000: 335 us, 353 with 4-byte stores).  256 threads.
 __device__ __forceinline__ void store_sym(const float *__restrict__ X, const __nv_bfloat16 *__restrict__ H,
                                           const __nv_bfloat16 *__restrict__ L, int n, int ldi,
                                           const double *__restrict__ diag, float *__restrict__ out, int first, int step)
@@ -590,10 +591,12 @@ __device__ __forceinline__ void store_sym(const float *__restrict__ X, const __n
     __shared__ float a[LB][LB + 1];
     const int tx = threadIdx.x & (LB - 1), ty = threadIdx.x / LB;  // stores: 4 rows of 64
     const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // loads: 16 rows of 16 x 4
+    const bool aligned = (ldo & 3) == 0 && ((uintptr_t)out & 15) == 0;
     for (int t = first; t < npairs; t += step) {
         int bi, bj;
         block_pair(t, bi, bj);
         const int i0 = bi * LB, j0 = bj * LB;
+        const bool vec = aligned && bi < bj && j0 + LB <= n;  // 16 bytes at a time, no bounds, no diagonal
 #pragma unroll
         for (int k = 0; k < LB; k += 16) {
             const int r = k + tr, gi = i0 + r, gj = j0 + c4;
@@ -611,13 +614,23 @@ __device__ __forceinline__ void store_sym(const float *__restrict__ X, const __n
                     v[3] = __uint_as_float(h.y & 0xffff0000u) + __uint_as_float(l.y & 0xffff0000u);
                 }
             }
+            if (vec)
+                __stcs(reinterpret_cast<float4 *>(out + (size_t)gi * ldo + gj), make_float4(v[0], v[1], v[2], v[3]));
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 a[r][c4 + u] = v[u];
         }
         __syncthreads();
+        if (vec) {
+#pragma unroll
+            for (int k = 0; k < LB; k += 16) {
+                const int r = k + tr;
+                __stcs(reinterpret_cast<float4 *>(out + (size_t)(j0 + r) * ldo + i0 + c4),
+                       make_float4(a[c4][r], a[c4 + 1][r], a[c4 + 2][r], a[c4 + 3][r]));
+            }
+        }
 #pragma unroll 4
-        for (int k = 0; k < LB; k += 4) {
+        for (int k = 0; k < LB && !vec; k += 4) {
             const int r = k + ty;
             if (i0 + r < n && j0 + tx < n) {
                 const bool up = bi < bj || r < tx;
@@ -643,9 +656,15 @@ __global__ void __launch_bounds__(256) k_store(const __grid_constant__ StateOut 
         store_sym(o.P, nullptr, nullptr, o.T, o.Tp, o.pd, o.oP, b - nc, np);
     } else {
         const int r = b - nc - np;
+        const float *w = o.W + (size_t)r * o.Gp;
+        float *out = o.oW + (size_t)r * o.G;
+        const int g4 = (o.G & 3) == 0 && ((uintptr_t)o.oW & 15) == 0 ? o.G >> 2 : 0;
 #pragma unroll 4
-        for (int c = threadIdx.x; c < o.G; c += 256)
-            o.oW[(size_t)r * o.G + c] = o.W[(size_t)r * o.Gp + c];
+        for (int c = threadIdx.x; c < g4; c += 256)
+            __stcs(reinterpret_cast<float4 *>(out) + c, reinterpret_cast<const float4 *>(w)[c]);
+#pragma unroll 4
+        for (int c = 4 * g4 + threadIdx.x; c < o.G; c += 256)
+            out[c] = w[c];
     }
 }
 
