@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <cstring>
 #include <queue>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_fp8.h>
@@ -558,12 +559,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // The finished tile is taken as TMEM fragments, like phase 2's: values move
 // straight between registers and memory (8 x 64 bytes per row group), sums in
 // registers and by shuffles, everything a 16-column sub-chunk ahead; only
-// FP8MIX's transposed copy passes through shared memory.  The epilogue is not
-// overlapped with MMAs: 2.6 us per sub-chunk and 21 us per tile when each row
-// belonged to a lane and every block was staged.  Phase 1 at 250 x 2100 (one
-// tile per pair) 67 -> 58.5 us, 600 x 6000 130 -> 123.5 us, FP8MIX at 1000 x
-// 17000 421 -> 401 us, BF16X3 there 1.07 -> 1.06 ms (bound by its MMAs: 12 of
-// 128 cycles a stage of 1530 cycles, at the clock the power limit leaves).
+// FP8MIX's transposed copy passes through shared memory.  2.6 us per sub-chunk
+// and 21 us per tile when each row belonged to a lane and every block was
+// staged: phase 1 at 250 x 2100 (one tile per pair) 67 -> 58.5 us, 600 x 6000
+// 130 -> 123.5 us.  Where a pair has several tiles the epilogue runs beside
+// the next tile's MMAs (phase1_pair).  BF16X3 at 1000 x 17000, 1.02 ms, is
+// bound by its MMAs: 12 of 128 cycles a stage of 1530 cycles, at the clock the
+// power limit leaves.
 constexpr int ST1 = 3;
 constexpr uint32_t STAGE1 = 4 * A_BYTES;   // per CTA: A hi, A lo, B hi, B lo (128 rows each)
 constexpr int EPI1 = 8, THREADS1 = 64 + 32 * EPI1;
@@ -634,14 +636,16 @@ __device__ __forceinline__ bool flag_wait_bounded(int *f, int *abort, Ctl *ctl)
 
 struct Sync1 {
     uint64_t full[ST1], empty[ST1];
-    uint64_t accum;
-    uint64_t chunk_done[2];  // MMA -> epilogue: an A-num chunk in TMEM buffer b is complete
-    uint64_t buf_free[2];    // epilogue warps of both CTAs -> MMA issuer: buffer b has been drained
+    uint64_t done[2];   // MMA -> epilogue: the sums in TMEM buffer b are complete
+    uint64_t free_[2];  // epilogue warps of both CTAs -> MMA issuer: buffer b has been read
+    uint64_t fin;       // every MMA of the pair is complete
     uint32_t tmem;
     int abort, issued, consumed;
 };
 
 constexpr size_t P1_COLVEC = 3 * 256;   // c_j, |W_.j|^2, |C_.j|^2 of the tile's columns
+// p_i, |P_i.|^2, |W_i.|^2 of this CTA's rows (held in registers they cost spills, 2.5 us a tile)
+constexpr size_t P1_ROWVEC = 3 * 128;
 constexpr size_t P1_COLRED = 4 * 256;   // [quarter][column] sums of W'^2
 constexpr size_t P1_ROWRED = 2 * 128;   // [half][row] sums of W'^2
 constexpr size_t P1_BLK = 32 * 17;      // per epilogue warp: 32 x 16 staging block (padded)
@@ -649,7 +653,7 @@ constexpr size_t P1_BLK = 32 * 17;      // per epilogue warp: 32 x 16 staging bl
 constexpr size_t phase1_smem()
 {
     return 1024 + (size_t)ST1 * STAGE1 + ((sizeof(Sync1) + 15) & ~size_t(15)) +
-           (P1_COLVEC + P1_COLRED + P1_ROWRED + EPI1 * P1_BLK) * sizeof(float) + EPI1 * sizeof(double);
+           (P1_COLVEC + P1_ROWVEC + P1_COLRED + P1_ROWRED + EPI1 * P1_BLK) * sizeof(float) + EPI1 * sizeof(double);
 }
 
 __device__ __forceinline__ Sync1 &phase1_sync()
@@ -658,441 +662,534 @@ __device__ __forceinline__ Sync1 &phase1_sync()
     return *reinterpret_cast<Sync1 *>(align1024(smem_raw) + ST1 * STAGE1);
 }
 
-// Set-up of a phase-1 CTA, once per kernel: the pipeline barriers (their
-// phases then run on over every tile the CTA computes, counted by the stage
-// counter g and the tile counter of phase1_tile) and the pair's 512 TMEM
-// columns (a CTA gives up its allocation permit after the first allocation,
-// so a persistent CTA keeps them over all its tiles).  Released by
-// phase1_tmem_free.
-__device__ __forceinline__ void phase1_tmem_alloc()
-{
-    Sync1 &sy = phase1_sync();
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < ST1; ++q) {
-            mbar_init(&sy.full[q], 1);
-            mbar_init(&sy.empty[q], 1);
-        }
-        mbar_init(&sy.accum, 1);
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&sy.chunk_done[b], 1);
-            mbar_init(&sy.buf_free[b], 2 * EPI1);
-        }
-        sy.abort = 0;
-        fence_mbar_init();
+// Where phase 1 finds its pieces: one network given by value, or a set.
+struct P1Piece {
+    int net, mt, nt, c0, c1, cut;  // cut: the slot where a cut tile's two pieces meet (-1: whole)
+};
+struct P1One {
+    const TcMaps &m;
+    const Dev &d;
+    int c;
+    const int4 *items;  // (mt, nt, c0 | c1 << 16, cut)
+    const int *off;
+    __device__ const Dev &dev(int) const { return d; }
+    __device__ const TcMaps &maps(int) const { return m; }
+    __device__ int cur(int) const { return c; }
+    __device__ bool active(int) const { return true; }  // no piece runs otherwise
+    __device__ bool any() const { return d.ctl->active != 0; }
+    __device__ P1Piece piece(int q) const
+    {
+        const int4 w = items[q];
+        return P1Piece{0, w.x, w.y, w.z & 0xffff, w.z >> 16, w.w};
     }
-    if ((threadIdx.x >> 5) == 1)
-        tmem_alloc_pair(&sy.tmem, 512);
-    tc_fence_before();
-    cluster_sync();  // both CTAs' barriers and TMEM address are ready before any cross-CTA signal
-    tc_fence_after();
-}
-__device__ __forceinline__ void phase1_tmem_free()
-{
-    tc_fence_before();
-    cluster_sync();  // both CTAs release together (also when a pair had no tile to run)
-    if ((threadIdx.x >> 5) == 1) {
-        tc_fence_after();
-        tmem_dealloc_pair(phase1_sync().tmem, 512);
+    __device__ float *scratch() const { return d.p1_acc + (size_t)blockIdx.x * P1_SLOT; }
+};
+struct P1Set {
+    const SetArgs &a;
+    const int4 *items;  // (network, mt, nt, cost)
+    const int *off;
+    __device__ const Dev &dev(int k) const { return a.devs[k]; }
+    __device__ const TcMaps &maps(int k) const { return a.maps[k]; }
+    __device__ int cur(int k) const { return set_cur(a, k); }
+    __device__ bool active(int k) const { return a.devs[k].ctl->active != 0; }
+    __device__ bool any() const { return true; }
+    __device__ P1Piece piece(int q) const
+    {
+        const int4 w = items[q];
+        return P1Piece{w.x, w.y, w.z, 0, 1 << 15, -1};
     }
-}
+    __device__ float *scratch() const { return a.acc + (size_t)blockIdx.x * P1_SLOT; }
+};
 
-// The body of phase 1 for the A-num chunks c0 .. c1 - 1 of the tile (mt, nt)
-// of one network (c1 at or past the chunk count: through the last chunk, then
-// R-num and the epilogue): maps and d are that network's (kernel parameters
-// for one network, entries of arrays in global memory for a set), cur its
-// current W buffer, scr this CTA's slot of 128 x 256 floats for the running
-// A-num sum ([column][row]).  A piece that does not start at chunk 0 waits for
-// *flag before it touches scr; one that does not end the tile raises *flag
-// when its adds have landed (flag NULL: a whole tile).  g counts the pipeline
-// stages, tile the pieces and u[b] the drains of TMEM buffer b this CTA has
-// run before (barrier phases follow them); all advance here.  Both CTAs of
-// the pair run every call together and end it at a cluster barrier, after
-// which TMEM is free for the next piece.
-__device__ __forceinline__ void phase1_tile(const TcMaps &maps, const Dev &d, int cur, int mt, int nt, int c0,
-                                            int c1, int *flag, int &g, int &tile, int (&u)[2], float *scr)
+// The k-blocks of a piece: A-num chunks c0 .. c1 - 1 (c1 at or past the chunk
+// count: through the last one), then, if it ends its tile, R-num.  R-num runs
+// over TFs (nR k-blocks of 64 BF16 per row), A-num over genes (nA of 64 BF16,
+// or of 128 E4M3 under FP8MIX) in nc chunks of P1_CHUNK.
+struct P1Range {
+    int nR, nA, nc, c0, c1, a0, nAp, nk;
+    bool ends;
+    __device__ __forceinline__ P1Range(int Tp, int Gp, int fp8, const P1Piece &w)
+    {
+        nR = Tp / BK;
+        nA = Gp / (fp8 ? 2 * BK : BK);
+        nc = (nA + P1_CHUNK - 1) / P1_CHUNK;
+        c0 = w.c0;
+        c1 = w.c1 < nc ? w.c1 : nc;
+        ends = c1 == nc;
+        a0 = c0 * P1_CHUNK;
+        nAp = min(c1 * P1_CHUNK, nA) - a0;
+        nk = nAp + (ends ? nR : 0);
+    }
+};
+
+// The body of phase 1 for one CTA pair's list of pieces: tiles, or a tile's
+// head or tail (see build_p1).  Every role walks the list by itself and skips
+// the pieces of a stopped network alike, so the stage counter g and the TMEM
+// counter `use` (an A-num chunk or an R-num each; use q in buffer q & 1) stay
+// in step.  The pair's 512 TMEM columns are kept over all pieces.
+//
+// A piece's last chunk is drained into the running sum like the others when
+// another piece follows: its buffer is then free for the next tile's MMAs,
+// which run on while the epilogue works through R-num's buffer.  The pair's
+// last tile takes that chunk straight from TMEM (the drain and the way back
+// from L2 would only delay it).  When every role ended a tile at a cluster
+// barrier the tensor core stood still for each epilogue; phase 1 then and now:
+// 12 networks of 241-987 x 2238-7773 1.27 and 1.05 ms, 1000 x 17000 BF16X3 1.07
+// and 1.02 ms, FP8MIX 401 and 358 us, 1600 x 30000 5.62 and 5.36 ms; 250 x 2100
+// and 600 x 6000 (one tile per pair) 58.5 and 124 us both.
+//
+// A piece that does not start at chunk 0 waits for its flag before it touches
+// the slot where it meets its head; a head raises it when its adds have landed.
+template <class Src>
+__device__ __forceinline__ void phase1_pair(const Src &src, Ctl *ctl0)
 {
-    Ctl *ctl = d.ctl;
-    if (!ctl->active)  // both CTAs of a pair see the same value and leave together
-        return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *stages = align1024(smem_raw);
     Sync1 &sy = phase1_sync();
     float *colvec = reinterpret_cast<float *>(stages + ST1 * STAGE1 + ((sizeof(Sync1) + 15) & ~size_t(15)));
-    float *colred = colvec + P1_COLVEC;
+    float *rowvec = colvec + P1_COLVEC;
+    float *colred = rowvec + P1_ROWVEC;
     float *rowred = colred + P1_COLRED;
     float *blocks = rowred + P1_ROWRED;
     double *hred = reinterpret_cast<double *>(blocks + EPI1 * P1_BLK);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
-    const int m0 = mt * 256 + 128 * (int)rank;  // this CTA's 128 rows (TFs)
-    const int n0 = nt * 256;                    // the tile's 256 columns (genes)
-    // k-blocks kb: R-num over TFs (kb < nR, 64 BF16 per row) and A-num over genes (kb >= nR, 64 BF16,
-    // or 128 E4M3 under FP8MIX).  A-num runs in nc chunks of P1_CHUNK k-blocks (chunk c in TMEM
-    // buffer c & 1), R-num after the last chunk (buffer nc & 1).  This piece issues, in the order
-    // s = 0 .. nk - 1, the k-blocks of chunks c0 .. c1 - 1 and, if it ends the tile, R-num.
-    const int nR = d.Tp / BK, nA = d.Gp / (d.fp8 ? 2 * BK : BK);
-    const int nc = (nA + P1_CHUNK - 1) / P1_CHUNK, bR = nc & 1;
-    c1 = c1 < nc ? c1 : nc;
-    const bool ends = c1 == nc;                              // R-num and the epilogue are this piece's
-    const int a0 = c0 * P1_CHUNK, nAp = min(c1 * P1_CHUNK, nA) - a0;  // the piece's A-num k-blocks
-    const int nk = nAp + (ends ? nR : 0);
-    auto kb_of = [nR, a0, nAp](int s) { return s < nAp ? nR + a0 + s : s - nAp; };
-    const int cd = c1 < nc - 1 ? c1 : nc - 1;  // chunks c0 .. cd - 1 are drained into scr
-
-    const int g0 = g;      // stages run by this CTA before this piece
-    const uint32_t tpar = (uint32_t)tile & 1u;  // phase of the accumulator barrier for this piece
-    const int u0[2] = {u[0], u[1]};  // drains of each buffer before this piece
-    g += nk;
-    ++tile;
-    if (cd > c0) {  // the piece's i-th drain of a buffer is chunk c0 + 2 i or c0 + 1 + 2 i
-        u[c0 & 1] += (cd - c0 + 1) / 2;
-        u[(c0 & 1) ^ 1] += (cd - c0) / 2;
-    }
+    const int pair = blockIdx.x >> 1;
+    // the list is on its way while the barriers and TMEM are set up
+    const int first = src.off[pair], end = src.off[pair + 1];
+    const bool any = src.any();
     if (threadIdx.x == 0) {
-        sy.issued = 0;
-        sy.consumed = 0;
+        for (int q = 0; q < ST1; ++q) {
+            mbar_init(&sy.full[q], 1);
+            mbar_init(&sy.empty[q], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&sy.done[b], 1);
+            mbar_init(&sy.free_[b], 2 * EPI1);
+        }
+        mbar_init(&sy.fin, 1);
+        sy.abort = sy.issued = sy.consumed = 0;
+        fence_mbar_init();
     }
-    __syncthreads();
+    if (warp == 1)
+        tmem_alloc_pair(&sy.tmem, 512);
+    tc_fence_before();
+    cluster_sync();  // both CTAs' barriers and TMEM address are ready before any cross-CTA signal
+    tc_fence_after();
+    const int last = any ? end : first;
+    auto next = [&](int q) {  // the next piece of a network that runs
+        do
+            ++q;
+        while (q < last && !src.active(src.piece(q).net));
+        return q;
+    };
 
     if (warp == 0) {
         if (lane == 0) {  // ---- TMA producer (both CTAs; completion counted on the even CTA) ----
-            const int nb0 = n0 + 128 * (int)rank;  // this CTA's half of the B rows
-            int s = 0;
-            for (; s < nk; ++s) {
-                const int kb = kb_of(s), st = (g0 + s) % ST1;
-                if (!wait_bounded(&sy.empty[st], ((uint32_t)((g0 + s) / ST1) & 1u) ^ 1u, &sy.abort, ctl))
-                    break;
-                const uint32_t fb = mapa_shared(smem_u32(&sy.full[st]), 0);
-                if (rank == 0)  // both CTAs' tiles: 4 per CTA, 3 without B's lo half, 2 of E4M3
-                    mbar_arrive_expect_tx(&sy.full[st], (kb >= nR && d.fp8 ? 4 : (d.split_b ? 8 : 6)) * A_BYTES);
-                uint8_t *b = stages + (size_t)st * STAGE1;
-                if (kb < nR) {  // responsibility: P_off rows x W columns, K over TFs
-                    const int k = kb * BK;
-                    tma_load_2d_pair(b, &maps.Ph, fb, k, m0);
-                    tma_load_2d_pair(b + A_BYTES, &maps.Pl, fb, k, m0);
-                    for (int h = 0; h < 2; ++h) {  // W rows k.. k + 63, this CTA's 128 genes: MN-major
-                        tma_load_2d_pair(b + 2 * A_BYTES + h * (A_BYTES / 2), &maps.Whm[cur], fb, nb0 + 64 * h, k);
-                        if (d.split_b)
-                            tma_load_2d_pair(b + 3 * A_BYTES + h * (A_BYTES / 2), &maps.Wlm[cur], fb, nb0 + 64 * h,
-                                             k);
+            int g = 0;
+            bool ok = true;
+            for (int q = next(first - 1); q < last && ok; q = next(q)) {
+                const P1Piece w = src.piece(q);
+                const Dev &d = src.dev(w.net);
+                const TcMaps &maps = src.maps(w.net);
+                const int cur = src.cur(w.net), m0 = w.mt * 256 + 128 * (int)rank, n0 = w.nt * 256;
+                const P1Range p(d.Tp, d.Gp, d.fp8, w);
+                const int nR = p.nR;
+                const int nb0 = n0 + 128 * (int)rank;  // this CTA's half of the B rows
+                for (int s = 0; s < p.nk; ++s, ++g) {
+                    const int kb = s < p.nAp ? nR + p.a0 + s : s - p.nAp, st = g % ST1;
+                    if (!wait_bounded(&sy.empty[st], ((uint32_t)(g / ST1) & 1u) ^ 1u, &sy.abort, d.ctl)) {
+                        ok = false;
+                        break;
                     }
-                } else if (d.fp8) {  // availability on E4M3 copies (C8 holds both triangles)
-                    const int k = (kb - nR) * 2 * BK;
-                    tma_load_2d_pair(b, &maps.W8[cur], fb, k, m0);
-                    tma_load_2d_pair(b + A_BYTES, &maps.C8, fb, k, nb0);
-                } else {        // availability: W rows x C_off rows, K over genes
-                    const int k = (kb - nR) * BK;
-                    tma_load_2d_pair(b, &maps.Wh[cur], fb, k, m0);
-                    tma_load_2d_pair(b + A_BYTES, &maps.Wl[cur], fb, k, m0);
-                    if (k >= n0) {  // C_off[j][k], k at or past the tile's diagonal block: stored rows
-                        tma_load_2d_pair(b + 2 * A_BYTES, &maps.Ch, fb, k, nb0);
-                        if (d.split_b)
-                            tma_load_2d_pair(b + 3 * A_BYTES, &maps.Cl, fb, k, nb0);
-                    } else {        // k < j: C_off[j][k] = C_off[k][j], rows k of the upper triangle
-                        for (int h = 0; h < 2; ++h) {
-                            tma_load_2d_pair(b + 2 * A_BYTES + h * (A_BYTES / 2), &maps.Chm, fb, nb0 + 64 * h, k);
+                    const uint32_t fb = mapa_shared(smem_u32(&sy.full[st]), 0);
+                    if (rank == 0)  // both CTAs' tiles: 4 per CTA, 3 without B's lo half, 2 of E4M3
+                        mbar_arrive_expect_tx(&sy.full[st], (kb >= nR && d.fp8 ? 4 : (d.split_b ? 8 : 6)) * A_BYTES);
+                    uint8_t *b = stages + (size_t)st * STAGE1;
+                    if (kb < nR) {  // responsibility: P_off rows x W columns, K over TFs
+                        const int k = kb * BK;
+                        tma_load_2d_pair(b, &maps.Ph, fb, k, m0);
+                        tma_load_2d_pair(b + A_BYTES, &maps.Pl, fb, k, m0);
+                        for (int h = 0; h < 2; ++h) {  // W rows k.. k + 63, this CTA's 128 genes: MN-major
+                            tma_load_2d_pair(b + 2 * A_BYTES + h * (A_BYTES / 2), &maps.Whm[cur], fb, nb0 + 64 * h, k);
                             if (d.split_b)
-                                tma_load_2d_pair(b + 3 * A_BYTES + h * (A_BYTES / 2), &maps.Clm, fb, nb0 + 64 * h,
+                                tma_load_2d_pair(b + 3 * A_BYTES + h * (A_BYTES / 2), &maps.Wlm[cur], fb, nb0 + 64 * h,
                                                  k);
+                        }
+                    } else if (d.fp8) {  // availability on E4M3 copies (C8 holds both triangles)
+                        const int k = (kb - nR) * 2 * BK;
+                        tma_load_2d_pair(b, &maps.W8[cur], fb, k, m0);
+                        tma_load_2d_pair(b + A_BYTES, &maps.C8, fb, k, nb0);
+                    } else {        // availability: W rows x C_off rows, K over genes
+                        const int k = (kb - nR) * BK;
+                        tma_load_2d_pair(b, &maps.Wh[cur], fb, k, m0);
+                        tma_load_2d_pair(b + A_BYTES, &maps.Wl[cur], fb, k, m0);
+                        if (k >= n0) {  // C_off[j][k], k at or past the tile's diagonal block: stored rows
+                            tma_load_2d_pair(b + 2 * A_BYTES, &maps.Ch, fb, k, nb0);
+                            if (d.split_b)
+                                tma_load_2d_pair(b + 3 * A_BYTES, &maps.Cl, fb, k, nb0);
+                        } else {        // k < j: C_off[j][k] = C_off[k][j], rows k of the upper triangle
+                            for (int h = 0; h < 2; ++h) {
+                                tma_load_2d_pair(b + 2 * A_BYTES + h * (A_BYTES / 2), &maps.Chm, fb, nb0 + 64 * h, k);
+                                if (d.split_b)
+                                    tma_load_2d_pair(b + 3 * A_BYTES + h * (A_BYTES / 2), &maps.Clm, fb, nb0 + 64 * h,
+                                                     k);
+                            }
                         }
                     }
                 }
             }
-            sy.issued = s;
+            sy.issued = g;
         }
     } else if (warp == 1) {
         if (rank == 0) {  // ---- MMA issuer of the pair (a whole warp, see mma_bf16_warp) ----
             constexpr uint32_t idesc = idesc_bf16_f32(256, 256);
             const uint32_t leader = elect_one(), tmem = __shfl_sync(0xffffffffu, sy.tmem, 0);
-            const bool fp8 = __shfl_sync(0xffffffffu, d.fp8, 0) != 0, split_b = __shfl_sync(0xffffffffu, d.split_b, 0) != 0;
-            int s = 0, st = g0 % ST1;
-            uint32_t ph = (uint32_t)(g0 / ST1) & 1u;
-            for (; s < nk; ++s) {
-                const int kb = kb_of(s);
-                // this k-block's accumulator: A-num chunk c in buffer c & 1, R-num in buffer bR; a buffer
-                // is written again only once the epilogue has drained the chunk it held two chunks before
-                const int a = kb - nR, c = a / P1_CHUNK;
-                const int buf = kb >= nR ? (c & 1) : bR;
-                const bool fresh = kb >= nR ? a % P1_CHUNK == 0 : kb == 0;
-                const int prev = kb >= nR ? c - 2 : nc - 2;  // chunk that last used buf (< c0: none here)
-                bool ok = true;
-                if (fresh && prev >= c0)
-                    ok = wait_bounded(&sy.buf_free[buf], (uint32_t)(u0[buf] + ((prev - c0) >> 1)) & 1u, &sy.abort, ctl);
-                ok = ok && wait_bounded(&sy.full[st], ph, &sy.abort, ctl);
-                if (!__all_sync(0xffffffffu, ok))
-                    break;
-                tc_fence_after();
-                const uint32_t base = smem_u32(stages + (size_t)st * STAGE1);
-                const uint32_t dacc = tmem + (uint32_t)buf * 256u;
-                // a chunk other than the last ends: the epilogue drains it into the running sum
-                const bool chunk_end = kb >= nR && c < nc - 1 && (a % P1_CHUNK == P1_CHUNK - 1);
-                const bool e4 = kb >= nR && fp8;
-                const bool bmn = !e4 && (kb < nR || (kb - nR) * BK < n0);  // B block loaded MN-major
-                const uint64_t a0 = sdesc_k_sw128(base);
-                const uint64_t b0 = bmn ? sdesc_mn_sw128(base + 2 * A_BYTES, A_BYTES / 2) : sdesc_k_sw128(base + 2 * A_BYTES);
-                const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32), b_lo = (uint32_t)b0,
-                               b_hi = (uint32_t)(b0 >> 32);
-                const uint32_t bs = bmn ? 2048 >> 4 : 32 >> 4, id = bmn ? (idesc | IDESC_B_MN) : idesc;
-                constexpr uint32_t PART = A_BYTES >> 4;
-                if (e4) {  // one E4M3 tile of A, then one of B; K = 32 per MMA
+            int g = 0, st = 0, use = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int q = next(first - 1); q < last && ok; q = next(q)) {
+                P1Piece w = src.piece(q);
+                w.c0 = __shfl_sync(0xffffffffu, w.c0, 0);
+                w.c1 = __shfl_sync(0xffffffffu, w.c1, 0);
+                const Dev &d = src.dev(w.net);
+                const bool fp8 = __shfl_sync(0xffffffffu, d.fp8, 0) != 0;
+                const bool split_b = __shfl_sync(0xffffffffu, d.split_b, 0) != 0;
+                const int n0 = __shfl_sync(0xffffffffu, w.nt, 0) * 256;
+                const P1Range p(__shfl_sync(0xffffffffu, d.Tp, 0), __shfl_sync(0xffffffffu, d.Gp, 0), fp8, w);
+                const int nR = p.nR;
+                for (int s = 0; s < p.nk; ++s, ++g) {
+                    const int kb = s < p.nAp ? nR + p.a0 + s : s - p.nAp, a = kb - nR;
+                    // a chunk's or R-num's first and last k-block; a buffer is written again once the epilogue
+                    // warps of both CTAs have read the use before the last
+                    const bool fresh = kb >= nR ? a % P1_CHUNK == 0 : kb == 0;
+                    const bool ends = kb >= nR ? a % P1_CHUNK == P1_CHUNK - 1 || a == p.nA - 1 : kb == nR - 1;
+                    const int buf = use & 1;
+                    if (fresh)
+                        ok = wait_bounded(&sy.free_[buf], ((uint32_t)(use >> 1) & 1u) ^ 1u, &sy.abort, d.ctl);
+                    ok = ok && wait_bounded(&sy.full[st], ph, &sy.abort, d.ctl);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok)
+                        break;
+                    tc_fence_after();
+                    const uint32_t base = smem_u32(stages + (size_t)st * STAGE1);
+                    const uint32_t dacc = tmem + (uint32_t)buf * 256u;
+                    const bool e4 = kb >= nR && fp8;
+                    const bool bmn = !e4 && (kb < nR || (kb - nR) * BK < n0);  // B block loaded MN-major
+                    const uint64_t a0 = sdesc_k_sw128(base);
+                    const uint64_t b0 =
+                        bmn ? sdesc_mn_sw128(base + 2 * A_BYTES, A_BYTES / 2) : sdesc_k_sw128(base + 2 * A_BYTES);
+                    const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32), b_lo = (uint32_t)b0,
+                                   b_hi = (uint32_t)(b0 >> 32);
+                    const uint32_t bs = bmn ? 2048 >> 4 : 32 >> 4, id = bmn ? (idesc | IDESC_B_MN) : idesc;
+                    constexpr uint32_t PART = A_BYTES >> 4;
+                    if (e4) {  // one E4M3 tile of A, then one of B; K = 32 per MMA
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        mma_e4m3_warp(leader, dacc, a_lo + kk * 2, a_hi, a_lo + PART + kk * 2, a_hi,
-                                      idesc_e4m3_f32(256, 256), !(fresh && kk == 0));
-                } else {
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_e4m3_warp(leader, dacc, a_lo + kk * 2, a_hi, a_lo + PART + kk * 2, a_hi,
+                                          idesc_e4m3_f32(256, 256), !(fresh && kk == 0));
+                    } else {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        const uint32_t ah = a_lo + kk * 2, bh = b_lo + kk * bs;
-                        mma_bf16_warp<true>(leader, dacc, ah, a_hi, bh, b_hi, id, !(fresh && kk == 0));
-                        if (split_b)
-                            mma_bf16_warp<true>(leader, dacc, ah, a_hi, bh + PART, b_hi, id, true);
-                        mma_bf16_warp<true>(leader, dacc, ah + PART, a_hi, bh, b_hi, id, true);
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            const uint32_t ah = a_lo + kk * 2, bh = b_lo + kk * bs;
+                            mma_bf16_warp<true>(leader, dacc, ah, a_hi, bh, b_hi, id, !(fresh && kk == 0));
+                            if (split_b)
+                                mma_bf16_warp<true>(leader, dacc, ah, a_hi, bh + PART, b_hi, id, true);
+                            mma_bf16_warp<true>(leader, dacc, ah + PART, a_hi, bh, b_hi, id, true);
+                        }
+                    }
+                    mma_commit_warp<true>(leader, &sy.empty[st]);
+                    if (ends) {
+                        mma_commit_warp<true>(leader, &sy.done[buf]);
+                        ++use;
+                    }
+                    if (++st == ST1) {
+                        st = 0;
+                        ph ^= 1u;
                     }
                 }
-                mma_commit_warp<true>(leader, &sy.empty[st]);
-                if (chunk_end)
-                    mma_commit_warp<true>(leader, &sy.chunk_done[buf]);
-                if (++st == ST1) {
-                    st = 0;
-                    ph ^= 1u;
-                }
             }
-            sy.consumed = s;
-            mma_commit_warp<true>(leader, &sy.accum);  // also on abort, so the epilogues can drain
+            sy.consumed = g;
+            mma_commit_warp<true>(leader, &sy.fin);  // also on abort, for the teardown
         }
     } else {  // ---- epilogue: warps 2..9 of both CTAs ----
         const int e = warp - 2, wq = warp & 3, half = e >> 2;
         const int tt = threadIdx.x - 64;  // 0..255
         // finished columns are taken as fragments (see frag_to_rows): rows er + 8 i of the warp's 32, columns
         // ec .. ec + 3 of 16
-        const int k0 = m0 + wq * 32, er = lane >> 2, ec = 8 * (lane & 1) + 2 * (lane & 2);
+        const int er = lane >> 2, ec = 8 * (lane & 1) + 2 * (lane & 2);
         float *blk = blocks + (size_t)e * P1_BLK;
-        const int nx = cur ^ 1;
-        const float *W = d.W[cur];
-        float *Wn = d.W[nx];
-        __nv_bfloat16 *Wh = d.Wh[nx], *Wl = d.Wl[nx];
-        // FP8MIX: the A-num accumulator holds the scaled E4M3 products; W' gets E4M3 copies too
-        const bool q8 = d.fp8 != 0;
-        const float ainv = q8 ? 1.0f / (d.f8[cur] * d.f8[2]) : 1.0f, s8 = q8 ? d.f8[3] : 1.0f;
-        if (q8 && mt == 0 && nt == 0 && rank == 0 && threadIdx.x == 64)
-            d.f8[nx] = s8;  // the scale of W8[nx] and Wt8[nx] from here on
-        // what does not depend on the accumulators is fetched before waiting for them
-        {
-            const int j = n0 + tt;
-            const bool cj = j < d.G;
-            colvec[tt] = cj ? d.cdf[j] : 0.0f;
-            colvec[256 + tt] = cj ? d.csqW[j] : 0.0f;
-            colvec[512 + tt] = cj ? d.csqC[j] : 0.0f;
-        }
-        float pdi[4], rsp[4], rsw[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = k0 + er + 8 * i;
-            const bool ri = r < d.T;
-            pdi[i] = ri ? d.pdf[r] : 0.0f;
-            rsp[i] = ri ? d.rsqP[r] : 0.0f;
-            rsw[i] = ri ? d.rsqW[r] : 0.0f;
-        }
-        const size_t wo = (size_t)(k0 + er) * d.Gp + n0 + half * 128 + ec;
-        uint4 wnx[4];
-        ld_old_f32(W + wo, d.Gp, wnx);
-        epi_bar2();
         const uint32_t trow = sy.tmem + ((uint32_t)(wq * 32) << 16) + half * 128;  // this warp's lanes and columns
-        // while the MMAs run on: add each finished A-num chunk but the last into the running sum
-        // (fragment registers in fours at [4 chunk-of-16 + q][thread]: 16 bytes each, coalesced)
-        bool live = true;
-        if (c0 > 0) {  // the tile's head was added into scr by another pair: wait for its flag
-            if (threadIdx.x == 64 && !flag_wait_bounded(flag, &sy.abort, ctl))
-                sy.abort = 1;
+        const uint32_t free_even = mapa_shared(smem_u32(&sy.free_[0]), 0);
+        int use = 0;
+        for (int q = next(first - 1), q1; q < last; q = q1) {
+            q1 = next(q);
+            const P1Piece pc = src.piece(q);
+            const Dev &d = src.dev(pc.net);
+            Ctl *ctl = d.ctl;
+            const P1Range p(d.Tp, d.Gp, d.fp8, pc);
+            const int mt = pc.mt, nt = pc.nt, cur = src.cur(pc.net), c0 = p.c0, nc = p.nc;
+            const int m0 = mt * 256 + 128 * (int)rank;  // this CTA's 128 rows (TFs)
+            const int n0 = nt * 256;                    // the tile's 256 columns (genes)
+            const bool ends = p.ends;
+            const bool direct = ends && q1 >= last;     // the last chunk is read from TMEM
+            const int cd = direct ? nc - 1 : p.c1;      // chunks c0 .. cd - 1 are drained into scr
+            const bool cut = pc.cut >= 0;
+            float *scr = cut ? d.p1_fix + (size_t)(2 * pc.cut + (int)rank) * P1_SLOT : src.scratch();
+            int *flag = cut ? d.p1_flag + 2 * pc.cut + (int)rank : nullptr;
+            const int k0 = m0 + wq * 32;
+            const int nx = cur ^ 1;
+            const float *W = d.W[cur];
+            float *Wn = d.W[nx];
+            __nv_bfloat16 *Wh = d.Wh[nx], *Wl = d.Wl[nx];
+            // FP8MIX: the A-num accumulator holds the scaled E4M3 products; W' gets E4M3 copies too
+            const bool q8 = d.fp8 != 0;
+            const float ainv = q8 ? 1.0f / (d.f8[cur] * d.f8[2]) : 1.0f, s8 = q8 ? d.f8[3] : 1.0f;
+            if (q8 && mt == 0 && nt == 0 && rank == 0 && threadIdx.x == 64)
+                d.f8[nx] = s8;  // the scale of W8[nx] and Wt8[nx] from here on
+            // what does not depend on the accumulators is fetched before waiting for them
+            {
+                const int j = n0 + tt;
+                const bool cj = j < d.G;
+                colvec[tt] = cj ? d.cdf[j] : 0.0f;
+                colvec[256 + tt] = cj ? d.csqW[j] : 0.0f;
+                colvec[512 + tt] = cj ? d.csqC[j] : 0.0f;
+            }
+            if (tt < 128) {
+                const int i = m0 + tt;
+                const bool ri = i < d.T;
+                rowvec[tt] = ri ? d.pdf[i] : 0.0f;
+                rowvec[128 + tt] = ri ? d.rsqP[i] : 0.0f;
+                rowvec[256 + tt] = ri ? d.rsqW[i] : 0.0f;
+            }
+            const size_t wo = (size_t)(k0 + er) * d.Gp + n0 + half * 128 + ec;
+            uint4 wnx[4];
+            ld_old_f32(W + wo, d.Gp, wnx);
             epi_bar2();
-            live = !*(volatile int *)&sy.abort;
-        }
-        const uint32_t bfree_even = mapa_shared(smem_u32(&sy.buf_free[0]), 0);
-        for (int c = c0; c < cd && live; ++c) {
-            const int b = c & 1;
-            live = wait_bounded(&sy.chunk_done[b], (uint32_t)(u0[b] + ((c - c0) >> 1)) & 1u, &sy.abort, ctl) &&
-                   !*(volatile int *)&sy.abort;
-            tc_fence_after();
-            if (!live)
-                break;
-            float4 *sp = reinterpret_cast<float4 *>(scr) + tt;
-            uint32_t v[16];
-            tmem_ld_frag16_nowait(trow + (uint32_t)b * 256u, v);
-#pragma unroll 1
-            for (int j = 0; j < 8; ++j) {
-                tmem_wait16(v);
-                float f[16];
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    f[q] = __uint_as_float(v[q]);
-                if (j < 7)
-                    tmem_ld_frag16_nowait(trow + (uint32_t)b * 256u + (j + 1) * 16, v);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float4 *p = sp + (4 * j + q) * 256;
-                    if (c == 0)
-                        *p = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
-                    else
-                        red_add4(&p->x, f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
-                }
+            // while the MMAs run on: add each finished A-num chunk (but a direct tile's last) into the running sum
+            // (fragment registers in fours at [4 chunk-of-16 + q][thread]: 16 bytes each, coalesced)
+            bool live = true;
+            if (c0 > 0) {  // the tile's head was added into scr by another pair: wait for its flag
+                if (threadIdx.x == 64 && !flag_wait_bounded(flag, &sy.abort, ctl))
+                    sy.abort = 1;
+                epi_bar2();
+                live = !*(volatile int *)&sy.abort;
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0)  // this warp is done with the buffer: tell the even CTA's MMA issuer
-                mbar_arrive_cluster(bfree_even + (uint32_t)b * (uint32_t)sizeof(uint64_t));
-        }
-        if (!ends) {  // a head piece: its adds are done; the accumulator barrier's phase still completes
-            live = live && wait_bounded(&sy.accum, tpar, &sy.abort, ctl) && !*(volatile int *)&sy.abort;
-            epi_bar2();
-            if (threadIdx.x == 64 && live)
-                flag_raise(flag);
-        } else {
-        // the running sum's first sub-chunk, from L2 (where the adds landed), in flight while the
-        // last chunk and R-num finish; each later one, the next W and the accumulators are fetched a
-        // sub-chunk ahead
-        const float4 *sp = reinterpret_cast<const float4 *>(scr) + tt;
-        float4 snx[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            snx[q] = (live && nc > 1) ? __ldcg(sp + q * 256) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        live = live && wait_bounded(&sy.accum, tpar, &sy.abort, ctl) && !*(volatile int *)&sy.abort;
-        tc_fence_after();
-        const float a = ctl->alpha, keep = 1.0f - a, halfa = 0.5f * a;
-        float rowsq[4] = {0.0f, 0.0f, 0.0f, 0.0f}, hsum = 0.0f;
-        const uint32_t tR = trow + (uint32_t)bR * 256u, tA = trow + (uint32_t)(bR ^ 1) * 256u;  // A: the last chunk
-        uint32_t fr[16], fa[16];
-        if (live) {
-            tmem_ld_frag16_nowait(tR, fr);
-            tmem_ld_frag16_nowait(tA, fa);
-        }
-#pragma unroll 1
-        for (int c = 0; c < 8 && live; ++c) {
-            const int cc = half * 128 + c * 16, j0 = n0 + cc;
-            float x[4][4], y[4][4], w[4][4];
-            tmem_wait16(fr);
-            tmem_wait16(fa);
-            if (nc > 1) {
-                const float sv[16] = {snx[0].x, snx[0].y, snx[0].z, snx[0].w, snx[1].x, snx[1].y, snx[1].z, snx[1].w,
-                                      snx[2].x, snx[2].y, snx[2].z, snx[2].w, snx[3].x, snx[3].y, snx[3].z, snx[3].w};
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    fa[q] = __float_as_uint(sv[q] + __uint_as_float(fa[q]));
-            }
-            frag_to_rows(fr, x);
-            frag_to_rows(fa, y);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                unpack4(wnx[i], w[i]);
-            if (c < 7) {
-                tmem_ld_frag16_nowait(tR + (c + 1) * 16, fr);
-                tmem_ld_frag16_nowait(tA + (c + 1) * 16, fa);
-                ld_old_f32(W + wo + (c + 1) * 16, d.Gp, wnx);
-                if (nc > 1) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        snx[q] = __ldcg(sp + (4 * (c + 1) + q) * 256);
-                }
-            }
-            const float4 c4 = *reinterpret_cast<const float4 *>(colvec + cc + ec);
-            const float4 w4 = *reinterpret_cast<const float4 *>(colvec + 256 + cc + ec);
-            const float4 q4 = *reinterpret_cast<const float4 *>(colvec + 512 + cc + ec);
-            const float cdj[4] = {c4.x, c4.y, c4.z, c4.w}, nwj[4] = {w4.x, w4.y, w4.z, w4.w},
-                        ncj[4] = {q4.x, q4.y, q4.z, q4.w};
-            const bool inner = k0 + 31 < d.T && j0 + 15 < d.G;
-            float cs[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            // (a) W' and its split copies, row-major from this lane's registers
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float wv = w[i][u];
-                    const float rnum = x[i][u] + pdi[i] * wv;                // P_i. . W_.j
-                    const float anum = fmaf(y[i][u], ainv, wv * cdj[u]);     // W_i. . C_.j
-                    const float R = tanimoto_clamped(rnum, rsp[i], nwj[u]);
-                    const float A = tanimoto_clamped(anum, rsw[i], ncj[u]);
-                    float wn = fmaf(keep, wv, halfa * (A + R));
-                    if (!inner)  // padding stays zero
-                        wn = k0 + er + 8 * i < d.T && j0 + ec + u < d.G ? wn : 0.0f;
-                    hsum += fabsf(wn - wv);
-                    rowsq[i] = fmaf(wn, wn, rowsq[i]);
-                    cs[u] = fmaf(wn, wn, cs[u]);
-                    w[i][u] = wn;
-                }
-                const size_t ro = wo + (size_t)(8 * i) * d.Gp + c * 16;
-                uint32_t h2[2], l2[2];
-                split_pair(w[i][0], w[i][1], h2[0], l2[0]);
-                split_pair(w[i][2], w[i][3], h2[1], l2[1]);
-                *reinterpret_cast<float4 *>(Wn + ro) = make_float4(w[i][0], w[i][1], w[i][2], w[i][3]);
-                *reinterpret_cast<uint2 *>(Wh + ro) = make_uint2(h2[0], h2[1]);
-                *reinterpret_cast<uint2 *>(Wl + ro) = make_uint2(l2[0], l2[1]);
-                if (q8)
-                    *reinterpret_cast<uint32_t *>(d.W8[nx] + ro) = e4m3x2(w[i][0], w[i][1], s8) | e4m3x2(w[i][2], w[i][3], s8) << 16;
-            }
-            // (b) the column sums of W'^2 over the warp's 32 rows
-            const float t = lanes8_reduce_scatter4(cs);
-            if (!(lane & 4))
-                colred[wq * 256 + cc + ec + (lane >> 3 & 1) + 2 * (lane >> 4)] = t;
-            // (c) under FP8MIX the transposed E4M3 copy, through this warp's staging block: lane l takes
-            //     column (l & 15), rows 16 (l >> 4) + 0..15
-            if (q8) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        blk[(er + 8 * i) * 17 + ec + u] = w[i][u];
+            auto waits = [&](int u) {
+                return wait_bounded(&sy.done[u & 1], (uint32_t)(u >> 1) & 1u, &sy.abort, ctl) && !*(volatile int *)&sy.abort;
+            };
+            auto frees = [&](int u) {  // this warp is done with the use's buffer: tell the even CTA's MMA issuer
+                tc_fence_before();
                 __syncwarp();
-                const int col = lane & 15, h16 = 16 * (lane >> 4);
-                const size_t to = (size_t)(j0 + col) * d.Tp + k0 + h16;
-                uint32_t p8[4];
+                if (lane == 0)
+                    mbar_arrive_cluster(free_even + (uint32_t)(u & 1) * (uint32_t)sizeof(uint64_t));
+            };
+            for (int c = c0; c < cd && live; ++c, ++use) {
+                const int b = use & 1;
+                live = waits(use);
+                tc_fence_after();
+                if (!live)
+                    break;
+                float4 *sp = reinterpret_cast<float4 *>(scr) + tt;
+                uint32_t v[16];
+                tmem_ld_frag16_nowait(trow + (uint32_t)b * 256u, v);
+#pragma unroll 1
+                for (int j = 0; j < 8; ++j) {
+                    tmem_wait16(v);
+                    float f[16];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float *b = blk + (h16 + 4 * q) * 17 + col;
-                    p8[q] = e4m3x2(b[0], b[17], s8) | e4m3x2(b[34], b[51], s8) << 16;
+                    for (int q = 0; q < 16; ++q)
+                        f[q] = __uint_as_float(v[q]);
+                    if (j < 7)
+                        tmem_ld_frag16_nowait(trow + (uint32_t)b * 256u + (j + 1) * 16, v);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float4 *p = sp + (4 * j + q) * 256;
+                        if (c == 0)
+                            *p = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+                        else
+                            red_add4(&p->x, f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+                    }
                 }
-                *reinterpret_cast<uint4 *>(d.Wt8[nx] + to) = make_uint4(p8[0], p8[1], p8[2], p8[3]);
-                __syncwarp();
+                frees(use);
             }
-        }
+            if (!ends) {  // a head piece: its adds are done
+                epi_bar2();
+                if (threadIdx.x == 64 && live)
+                    flag_raise(flag);
+            } else {
+                // the running sum's first sub-chunk, from L2 (where the adds landed), in flight while the
+                // last chunk and R-num finish; each later one, the next W and the accumulators are fetched a
+                // sub-chunk ahead
+                const float4 *sp = reinterpret_cast<const float4 *>(scr) + tt;
+                float4 snx[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float rs = rowsq[i];
-            rs += __shfl_xor_sync(0xffffffffu, rs, 1);
-            rs += __shfl_xor_sync(0xffffffffu, rs, 2);
-            if ((lane & 3) == 0)
-                rowred[half * 128 + wq * 32 + er + 8 * i] = rs;
-        }
-        double hv = (double)hsum;
+                for (int q = 0; q < 4; ++q)
+                    snx[q] = (live && cd > 0) ? __ldcg(sp + q * 256) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                const int uA = use, uR = use + (direct ? 1 : 0);  // the uses read from TMEM: the last chunk, R-num
+                use = uR + 1;
+                if (direct)
+                    live = live && waits(uA);
+                live = live && waits(uR);
+                tc_fence_after();
+                const float a = ctl->alpha, keep = 1.0f - a, halfa = 0.5f * a;
+                float rowsq[4] = {0.0f, 0.0f, 0.0f, 0.0f}, hsum = 0.0f;
+                const uint32_t tR = trow + (uint32_t)(uR & 1) * 256u, tA = trow + (uint32_t)(uA & 1) * 256u;
+                uint32_t fr[16], fa[16];
+                // this warp's columns; DIRECT is `direct`, known to the compiler
+                auto columns = [&](auto kind) {
+                    constexpr bool DIRECT = decltype(kind)::value;
+                    if (live) {
+                        tmem_ld_frag16_nowait(tR, fr);
+                        if (DIRECT)
+                            tmem_ld_frag16_nowait(tA, fa);
+                    }
+#pragma unroll 1
+                    for (int c = 0; c < 8 && live; ++c) {
+                        const int cc = half * 128 + c * 16, j0 = n0 + cc;
+                        float x[4][4], y[4][4], w[4][4];
+                        tmem_wait16(fr);
+                        if (DIRECT)
+                            tmem_wait16(fa);
+                        if (!DIRECT || cd > 0) {
+                            const float *sv = reinterpret_cast<const float *>(snx);
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1)
-            hv += __shfl_xor_sync(0xffffffffu, hv, off);
-        if (lane == 0)
-            hred[e] = hv;
-        epi_bar2();
-        if (live) {
-            const int slot = m0 / 128;  // this CTA's 128-row block
-            if (n0 + tt < d.Gp)
-                d.wcol_part[(size_t)slot * d.Gp + n0 + tt] =
-                    ((colred[tt] + colred[256 + tt]) + colred[512 + tt]) + colred[768 + tt];
-            if (tt < 128)
-                d.wrow_part[(size_t)nt * d.Tp + m0 + tt] = rowred[tt] + rowred[128 + tt];
-            if (tt == 0) {
-                double hs = 0.0;
-                for (int q = 0; q < EPI1; ++q)
-                    hs += hred[q];
-                d.hpart[(size_t)nt * d.nbT + slot] = hs;
+                            for (int q = 0; q < 16; ++q)
+                                fa[q] = __float_as_uint(DIRECT ? sv[q] + __uint_as_float(fa[q]) : sv[q]);
+                        }
+                        frag_to_rows(fr, x);
+                        frag_to_rows(fa, y);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            unpack4(wnx[i], w[i]);
+                        if (c == 7)
+                            frees(uR);
+                        if (c < 7) {
+                            tmem_ld_frag16_nowait(tR + (c + 1) * 16, fr);
+                            if (DIRECT)
+                                tmem_ld_frag16_nowait(tA + (c + 1) * 16, fa);
+                            ld_old_f32(W + wo + (c + 1) * 16, d.Gp, wnx);
+                            if (!DIRECT || cd > 0) {
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    snx[q] = __ldcg(sp + (4 * (c + 1) + q) * 256);
+                            }
+                        }
+                        const float4 c4 = *reinterpret_cast<const float4 *>(colvec + cc + ec);
+                        const float4 w4 = *reinterpret_cast<const float4 *>(colvec + 256 + cc + ec);
+                        const float4 q4 = *reinterpret_cast<const float4 *>(colvec + 512 + cc + ec);
+                        const float cdj[4] = {c4.x, c4.y, c4.z, c4.w}, nwj[4] = {w4.x, w4.y, w4.z, w4.w},
+                                    ncj[4] = {q4.x, q4.y, q4.z, q4.w};
+                        const bool inner = k0 + 31 < d.T && j0 + 15 < d.G;
+                        float cs[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                        // (a) W' and its split copies, row-major from this lane's registers
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float *rv = rowvec + wq * 32 + er + 8 * i;
+                            const float pdi = rv[0], rsp = rv[128], rsw = rv[256];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const float wv = w[i][u];
+                                const float rnum = x[i][u] + pdi * wv;                // P_i. . W_.j
+                                const float anum = fmaf(y[i][u], ainv, wv * cdj[u]);     // W_i. . C_.j
+                                const float R = tanimoto_clamped(rnum, rsp, nwj[u]);
+                                const float A = tanimoto_clamped(anum, rsw, ncj[u]);
+                                float wn = fmaf(keep, wv, halfa * (A + R));
+                                if (!inner)  // padding stays zero
+                                    wn = k0 + er + 8 * i < d.T && j0 + ec + u < d.G ? wn : 0.0f;
+                                hsum += fabsf(wn - wv);
+                                rowsq[i] = fmaf(wn, wn, rowsq[i]);
+                                cs[u] = fmaf(wn, wn, cs[u]);
+                                w[i][u] = wn;
+                            }
+                            const size_t ro = wo + (size_t)(8 * i) * d.Gp + c * 16;
+                            uint32_t h2[2], l2[2];
+                            split_pair(w[i][0], w[i][1], h2[0], l2[0]);
+                            split_pair(w[i][2], w[i][3], h2[1], l2[1]);
+                            *reinterpret_cast<float4 *>(Wn + ro) = make_float4(w[i][0], w[i][1], w[i][2], w[i][3]);
+                            *reinterpret_cast<uint2 *>(Wh + ro) = make_uint2(h2[0], h2[1]);
+                            *reinterpret_cast<uint2 *>(Wl + ro) = make_uint2(l2[0], l2[1]);
+                            if (q8)
+                                *reinterpret_cast<uint32_t *>(d.W8[nx] + ro) =
+                                    e4m3x2(w[i][0], w[i][1], s8) | e4m3x2(w[i][2], w[i][3], s8) << 16;
+                        }
+                        // (b) the column sums of W'^2 over the warp's 32 rows
+                        const float t = lanes8_reduce_scatter4(cs);
+                        if (!(lane & 4))
+                            colred[wq * 256 + cc + ec + (lane >> 3 & 1) + 2 * (lane >> 4)] = t;
+                        // (c) under FP8MIX the transposed E4M3 copy, through this warp's staging block: lane l takes
+                        //     column (l & 15), rows 16 (l >> 4) + 0..15
+                        if (q8) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                                for (int u = 0; u < 4; ++u)
+                                    blk[(er + 8 * i) * 17 + ec + u] = w[i][u];
+                            __syncwarp();
+                            const int col = lane & 15, h16 = 16 * (lane >> 4);
+                            const size_t to = (size_t)(j0 + col) * d.Tp + k0 + h16;
+                            uint32_t p8[4];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const float *b = blk + (h16 + 4 * q) * 17 + col;
+                                p8[q] = e4m3x2(b[0], b[17], s8) | e4m3x2(b[34], b[51], s8) << 16;
+                            }
+                            *reinterpret_cast<uint4 *>(d.Wt8[nx] + to) = make_uint4(p8[0], p8[1], p8[2], p8[3]);
+                            __syncwarp();
+                        }
+                    }
+                };
+                if (direct)
+                    columns(std::true_type{});
+                else
+                    columns(std::false_type{});
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float rs = rowsq[i];
+                    rs += __shfl_xor_sync(0xffffffffu, rs, 1);
+                    rs += __shfl_xor_sync(0xffffffffu, rs, 2);
+                    if ((lane & 3) == 0)
+                        rowred[half * 128 + wq * 32 + er + 8 * i] = rs;
+                }
+                double hv = (double)hsum;
+#pragma unroll
+                for (int off = 16; off >= 1; off >>= 1)
+                    hv += __shfl_xor_sync(0xffffffffu, hv, off);
+                if (lane == 0)
+                    hred[e] = hv;
+                epi_bar2();
+                if (live) {
+                    const int slot = m0 / 128;  // this CTA's 128-row block
+                    if (n0 + tt < d.Gp)
+                        d.wcol_part[(size_t)slot * d.Gp + n0 + tt] =
+                            ((colred[tt] + colred[256 + tt]) + colred[512 + tt]) + colred[768 + tt];
+                    if (tt < 128)
+                        d.wrow_part[(size_t)nt * d.Tp + m0 + tt] = rowred[tt] + rowred[128 + tt];
+                    if (tt == 0) {
+                        double hs = 0.0;
+                        for (int q = 0; q < EPI1; ++q)
+                            hs += hred[q];
+                        d.hpart[(size_t)nt * d.nbT + slot] = hs;
+                    }
+                }
             }
-        }
         }
     }
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && rank == 0)  // loads counted here but not consumed (abort only)
-        for (int s = sy.consumed; s < sy.consumed + ST1 && s < sy.issued; ++s)
-            wait_bounded(&sy.full[(g0 + s) % ST1], (uint32_t)((g0 + s) / ST1) & 1u, &sy.abort, ctl, true);
-    cluster_sync();  // neither CTA goes on while the pair may still signal it
+        for (int g = sy.consumed; g < sy.consumed + ST1 && g < sy.issued; ++g)
+            wait_bounded(&sy.full[g % ST1], (uint32_t)(g / ST1) & 1u, &sy.abort, ctl0, true);
+    if (threadIdx.x == 0)
+        wait_bounded(&sy.fin, 0, &sy.abort, ctl0, true);  // no MMA is left in flight
+    __syncthreads();
+    cluster_sync();  // both CTAs release together: neither leaves while the pair may still signal it
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(sy.tmem, 512);
+    }
 }
-
 
 // One network: persistent CTA pairs (at most one per SM pair), pair p over
 // its host-built list items[off[p] .. off[p + 1]) of pieces (mt, nt, chunks
@@ -1103,18 +1200,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS1, 1)
     k_tc_phase1(const __grid_constant__ TcMaps maps, const __grid_constant__ Dev d, int cur, const int4 *items,
                 const int *off)
 {
-    phase1_tmem_alloc();
-    int g = 0, tile = 0, u[2] = {0, 0};
-    const int pair = blockIdx.x >> 1, rank = (int)cluster_ctarank();
-    const bool active = d.ctl->active;  // both CTAs of a pair see the same value
-    for (int q = off[pair]; active && q < off[pair + 1]; ++q) {
-        const int4 w = items[q];
-        const bool cut = w.w >= 0;
-        float *scr = cut ? d.p1_fix + (size_t)(2 * w.w + rank) * P1_SLOT : d.p1_acc + (size_t)blockIdx.x * P1_SLOT;
-        phase1_tile(maps, d, cur, w.x, w.y, w.z & 0xffff, w.z >> 16, cut ? d.p1_flag + 2 * w.w + rank : nullptr, g,
-                    tile, u, scr);
-    }
-    phase1_tmem_free();
+    phase1_pair(P1One{maps, d, cur, items, off}, d.ctl);
 }
 
 // A set of networks: persistent CTA pairs, each over its host-built list of
@@ -1122,15 +1208,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS1, 1)
 // both CTAs alike.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS1, 1) k_tc_phase1_set(const SetArgs a)
 {
-    const int pair = blockIdx.x >> 1;
-    phase1_tmem_alloc();
-    int g = 0, tile = 0, u[2] = {0, 0};
-    float *scr = a.acc + (size_t)blockIdx.x * P1_SLOT;
-    for (int q = a.p1_off[pair]; q < a.p1_off[pair + 1]; ++q) {
-        const int4 w = a.items1[q];  // (network, mt, nt, cost)
-        phase1_tile(a.maps[w.x], a.devs[w.x], set_cur(a, w.x), w.y, w.z, 0, 1 << 15, nullptr, g, tile, u, scr);
-    }
-    phase1_tmem_free();
+    phase1_pair(P1Set{a, a.items1, a.p1_off}, a.devs[0].ctl);
 }
 
 // ---------------------------------------------------------------------------
@@ -1263,7 +1341,7 @@ struct P2Set {
     __device__ int net(int n) const { return a.sched_net[n]; }
     __device__ const Dev &dev(int k) const { return a.devs[k]; }
     __device__ const TcMaps &maps(int k) const { return a.maps[k]; }
-    // phase 2 works on W' (the other buffer: the count moves on only in k_tail)
+    // phase 2 works on W' (the other buffer: the count moves on only in k_fin)
     __device__ int cur(int k) const { return set_cur(a, k) ^ 1; }
     __device__ bool active(int k) const { return a.devs[k].ctl->active != 0; }
     __device__ bool any() const { return true; }
