@@ -21,8 +21,8 @@
 // the accumulator is still 2^-8 of its final size, the four h.h MMAs last, and
 // the stages are added up in FP32 registers, rounding to nearest.  Four
 // truncations and one rounding per 64 products, where FFMA rounded 64 times:
-// W after 3 iterations at 1000 x 17000 is 1.1e-7 from FP64 (2-norm), FFMA
-// 5.1e-7.  The two TMEM buffers alternate between stages, so the epilogue
+// W after 3 iterations at 1000 x 17000 is 6e-8 from FP64 (2-norm), FFMA
+// 5.0e-7.  The two TMEM buffers alternate between stages, so the epilogue
 // warps drain one (and add it up) while the tensor core fills the other.
 //
 // Bound: the tensor pipe, 6 x the algorithmic flops (FFMA: 78 TFLOP/s
@@ -35,10 +35,20 @@
 // tile's epilogue is a quarter as long, and a third operand stage fits).
 // Against 128 x 128 on one CTA the narrow tile took phases 1 + 2 from 94 to
 // 85 us at 1000 x 1000, 97 to 78 us at 250 x 2100 and 44 to 38 us at 125 x 125
-// (with the timing events' own 5 us each).  Tiles that would leave workers idle are cut along K (f32_plan):
-// every part but the last to arrive leaves its sums in slots in L2; the last
-// one adds all parts in part order, so the result does not depend on who that
-// is, and nobody waits.
+// (with the timing events' own 5 us each).
+//
+// Tiles that would leave workers idle are cut along K (f32_plan): every part
+// but the last to arrive leaves its sums in slots in L2; the last one adds all
+// parts in part order, so the result does not depend on who that is, and
+// nobody waits.
+//
+// On pairs phase 2 (1.51 ms at 1000 x 17000, 1.07 of it MMAs at the rate of
+// phase 1) waits for a tile's epilogue, 13 us beside 16 stages of 1.9 us, but
+// for the two stages that the buffers hold.  Slower or no faster: the sums
+// handed to four epilogue warps of their own through L2 (1.45-1.47 ms here, 215
+// instead of 174 us at 1000 x 5200), the epilogue a chunk at a time between the
+// next tile's stages (1.66 ms: too few registers beside the sums), the sums
+// through L2 instead of TMEM so that both buffers are free (1.64 ms).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

@@ -5,9 +5,8 @@
 // need bounds checks in their main loops; the epilogues mask by the true T
 // and G):
 //   W[2]   Tp x Gp  fp32   regulatory network, ping-pong (current / next)
-//   Wt[2]  Gp x Tp  fp32   its transpose: written by the FP32 path's epilogue;
-//                          on the tensor-core path made at create and load only
-//                          (column norms, FP8MIX's E4M3 copy)
+//   Wt[2]  Gp x Tp  fp32   its transpose, FP8MIX only: the source of the E4M3
+//                          copy at create, set_state and load
 //   Poff   Tp x Tp  fp32   P with a zero diagonal (diagonal kept in pd)
 //   Coff   Gp x Gp  fp32   C with a zero diagonal (diagonal kept in cd); in the
 //                          BF16X3 and BF16X2 modes only while a create or
@@ -52,7 +51,7 @@ struct Dev {
     int T, G, Tp, Gp, nbT, nbG;  // true sizes, padded sizes, 128-blocks
     int diag;                    // panda_diag
     double inv_n1P, inv_n1C;     // 1 / (T - 1), 1 / (G - 1) (0 for one node)
-    float *W[2], *Wt[2];         // Wt: FP32 and FP8MIX only (NULL under BF16X3 and BF16X2)
+    float *W[2], *Wt[2];         // Wt: FP8MIX only (else NULL)
     float *Poff, *Coff;
     double *pd, *cd;
     float *pdf, *cdf;            // FP32 copies of the diagonals for epilogues
@@ -90,11 +89,12 @@ struct Dev {
     unsigned *f8n;               // squared-norm maxima (float bits): [0..3] this iteration's
                                  // (rsqP, csqC, rsqW, csqW), [4..7] the state's, latched
     void *tc_host;               // host-side tensor maps of the split copies (tensor-core path)
-    float *p1_acc;               // tensor-core phase 1: per CTA of its grid, a 128 x 256 slot for the
-                                 // running sum of the availability numerator's chunks
-    float *p1_fix;               // per tile cut between two CTA pairs (at most one per pair), a
-                                 // 128 x 256 slot per CTA rank where its two pieces meet
-    int *p1_flag;                // per cut tile and CTA rank: its head's adds have landed
+    float *p1_acc;               // phase 1: per CTA of its grid, a tile's slot: the running sum of the
+                                 // availability numerator's chunks; FP32: an uncut tile's R-num
+    float *p1_fix;               // slots where a cut tile's parts meet: per tile cut between two CTA
+                                 // pairs one per CTA rank; FP32: one per part and rank
+    int *p1_flag;                // per cut tile and CTA rank: its head's adds have landed (FP32: the
+                                 // parts that have arrived)
     int p1_cuts;                 // cut tiles (slots and flag pairs above)
 };
 
