@@ -393,19 +393,6 @@ __global__ void k_diag_to_float(const double *d, float *df, int n)
         df[i] = (float)d[i];
 }
 
-// Y (cols_p x rows_p) = X^T (X is rows_p x cols_p); both multiples of 32.
-__global__ void k_transpose(const float *__restrict__ X, int rows_p, int cols_p, float *__restrict__ Y)
-{
-    __shared__ float tile[32][33];
-    int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-    int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-    for (int k = ty; k < 32; k += 8)
-        tile[k][tx] = X[(size_t)(by + k) * cols_p + bx + tx];
-    __syncthreads();
-    for (int k = ty; k < 32; k += 8)
-        Y[(size_t)(bx + k) * rows_p + by + tx] = tile[tx][k];
-}
-
 // x^2 into a compensated FP32 pair: x^2 = p + pe exactly, p through TwoSum
 __device__ __forceinline__ void sq_add(float x, float &acc, float &cmp)
 {
@@ -742,13 +729,6 @@ cudaError_t launch_norms(const StateNorms &n, cudaStream_t s)
 cudaError_t launch_diag_to_float(const double *d, float *df, int n, cudaStream_t s)
 {
     k_diag_to_float<<<ceil_div(n, 256), 256, 0, s>>>(d, df, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_transpose(const float *X, int rows_p, int cols_p, float *Y, cudaStream_t s)
-{
-    dim3 grid(cols_p / 32, rows_p / 32), block(32, 8);
-    k_transpose<<<grid, block, 0, s>>>(X, rows_p, cols_p, Y);
     return cudaGetLastError();
 }
 

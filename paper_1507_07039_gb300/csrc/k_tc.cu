@@ -141,6 +141,37 @@ __global__ void k_to_e4m3(const float *__restrict__ X, size_t n, uint8_t *__rest
         Q[q] = (uint8_t)e4m3x2(X[q], 0.0f, s);
 }
 
+// W's E4M3 copies, W8 as it lies (Tp x Gp, both multiples of 64) and Wt8
+// transposed: each 64 x 64 block read once, turned through shared memory.  A
+// transposed FP32 copy and a conversion of each took 74 us at 1000 x 17000 (19
+// now) and 141 MB.
+__global__ void __launch_bounds__(256) k_w_to_e4m3(const float *__restrict__ X, int Tp, int Gp, uint8_t *__restrict__ W8,
+                                                   uint8_t *__restrict__ Wt8, const float *scale)
+{
+    __shared__ float sh[64][65];
+    const int i0 = 64 * blockIdx.y, j0 = 64 * blockIdx.x;
+    const float s = *scale;
+    const int c4 = 4 * (threadIdx.x & 15), tr = threadIdx.x >> 4;  // rows tr, tr + 16, ..., four columns
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = 16 * k + tr;
+        const size_t o = (size_t)(i0 + r) * Gp + j0 + c4;
+        const float4 v = *reinterpret_cast<const float4 *>(X + o);
+        *reinterpret_cast<uint32_t *>(W8 + o) = e4m3x2(v.x, v.y, s) | (e4m3x2(v.z, v.w, s) << 16);
+        sh[r][c4] = v.x;
+        sh[r][c4 + 1] = v.y;
+        sh[r][c4 + 2] = v.z;
+        sh[r][c4 + 3] = v.w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = 16 * k + tr;
+        *reinterpret_cast<uint32_t *>(Wt8 + (size_t)(j0 + r) * Tp + i0 + c4) =
+            e4m3x2(sh[c4][r], sh[c4 + 1][r], s) | (e4m3x2(sh[c4 + 2][r], sh[c4 + 3][r], s) << 16);
+    }
+}
+
 // A symmetric matrix's E4M3 copy, both triangles, from the upper one (X and Q
 // Gp x Gp, Gp a multiple of 128): each 64 x 64 block above the diagonal is read
 // once and written twice, the second time turned through shared memory, four
@@ -2341,8 +2372,7 @@ cudaError_t tc_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
     if (d.fp8) {  // scales from the state's norms (or as restored), then the E4M3 copies
         if (!restored)
             k_fp8_init<<<1, 1024, 0, s>>>(d);
-        k_to_e4m3<<<1024, 256, 0, s>>>(d.W[cur], TG, d.W8[cur], d.f8 + cur);
-        k_to_e4m3<<<1024, 256, 0, s>>>(d.Wt[cur], TG, d.Wt8[cur], d.f8 + cur);
+        k_w_to_e4m3<<<dim3(d.Gp / 64, d.Tp / 64), 256, 0, s>>>(d.W[cur], d.Tp, d.Gp, d.W8[cur], d.Wt8[cur], d.f8 + cur);
         k_sym_to_e4m3<<<dim3(d.Gp / 64, d.Gp / 64), 256, 0, s>>>(d.Coff, d.Gp, d.C8, d.f8 + 2);
     }
     if ((e = cudaGetLastError()))

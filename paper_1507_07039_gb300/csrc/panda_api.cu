@@ -132,11 +132,8 @@ int plan_memory(panda_ctx *c)
     d.fp8 = c->prec == PANDA_FP8MIX ? 1 : 0;
     // BF16X3 and BF16X2 hold C as its split pair only (FP32 C is staged while the state is derived)
     d.c_split = (c->prec == PANDA_BF16X3 || c->prec == PANDA_BF16X2) ? 1 : 0;
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < 2; ++b)
         DALLOC(d.W[b], Tp * Gp);
-        if (d.fp8)  // the source of the E4M3 transposes
-            DALLOC(d.Wt[b], Gp * Tp);
-    }
     DALLOC(d.Poff, Tp * Tp);
     if (!d.c_split)
         DALLOC(d.Coff, Gp * Gp);
@@ -352,8 +349,6 @@ int load_state(panda_ctx *c, const float *W, const float *P, const float *C, int
     StateIn in{w.src, p.src, x.src, T, G, w.ld, p.ld, x.ld, st[0], st[1], st[2]};
     CU(launch_load(in, d.W[c->cur], Parts{d.Wh[c->cur], d.Wm[c->cur], d.Wl[c->cur]}, c->Tp, c->Gp, po, xo, c->d_flags,
                    c->stream));
-    if (d.Wt[c->cur])
-        CU(launch_transpose(d.W[c->cur], c->Tp, c->Gp, d.Wt[c->cur], c->stream));
     // norms of the same entries as loaded: those loaded in place are Z-scored by now
     in.W = d.W[c->cur];
     in.ldw = c->Gp;
@@ -1037,8 +1032,6 @@ int panda_load(panda_ctx *c, const void *buf, long long bytes)
         p += it.bytes;
     }
     Dev &d = c->d;
-    if (d.Wt[c->cur])
-        CU(launch_transpose(d.W[c->cur], c->Tp, c->Gp, d.Wt[c->cur], c->stream));
     CU(launch_diag_to_float(d.pd, d.pdf, c->T, c->stream));
     CU(launch_diag_to_float(d.cd, d.cdf, c->G, c->stream));
     if (tensor_prec(c->prec))

@@ -5,8 +5,6 @@
 // need bounds checks in their main loops; the epilogues mask by the true T
 // and G):
 //   W[2]   Tp x Gp  fp32   regulatory network, ping-pong (current / next)
-//   Wt[2]  Gp x Tp  fp32   its transpose, FP8MIX only: the source of the E4M3
-//                          copy at create, set_state and load
 //   Poff   Tp x Tp  fp32   P with a zero diagonal (diagonal kept in pd)
 //   Coff   Gp x Gp  fp32   C with a zero diagonal (diagonal kept in cd); in the
 //                          BF16X3 and BF16X2 modes only while a create or
@@ -51,7 +49,7 @@ struct Dev {
     int T, G, Tp, Gp, nbT, nbG;  // true sizes, padded sizes, 128-blocks
     int diag;                    // panda_diag
     double inv_n1P, inv_n1C;     // 1 / (T - 1), 1 / (G - 1) (0 for one node)
-    float *W[2], *Wt[2];         // Wt: FP8MIX only (else NULL)
+    float *W[2];
     float *Poff, *Coff;
     double *pd, *cd;
     float *pdf, *cdf;            // FP32 copies of the diagonals for epilogues
@@ -207,7 +205,6 @@ struct StateIn {
 // those forms, the padding up to Tp x Gp, Tp x Tp and Gp x Gp as zeros
 cudaError_t launch_load(const StateIn &in, float *W, const Parts &wparts, int Tp, int Gp, const SymOut &P, const SymOut &C,
                         int *flags, cudaStream_t s);
-cudaError_t launch_transpose(const float *X, int rows_p, int cols_p, float *Y, cudaStream_t s);
 // Squared norms: rows and columns of W (as loaded, row stride Gp), rows of P and C from where
 // they lie, the diagonal entry left out and pd, cd added; P and C Z-scored by their stats
 struct StateNorms {
