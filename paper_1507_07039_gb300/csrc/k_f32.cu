@@ -1412,12 +1412,15 @@ __global__ void k_f32_static_lists(const __grid_constant__ StaticArgs a, uint8_t
     }
 }
 
+// On the stream of the kernels that read it, which does not wait for the default stream: a plain
+// cudaMemcpy from pageable memory may return with its last bytes still on the way.  v lives until the
+// caller has waited for s.
 template <class T>
-cudaError_t to_device(T **dst, const std::vector<T> &v)
+cudaError_t to_device(T **dst, const std::vector<T> &v, cudaStream_t s)
 {
     cudaError_t e = cudaMalloc(dst, std::max<size_t>(1, v.size()) * sizeof(T));
     if (!e && !v.empty())
-        e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, s);
     return e;
 }
 
@@ -1473,8 +1476,8 @@ cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
     if ((e = make_maps(d, h->maps)) || (e = all_smem_limits()))
         return e;
     const F32Plan &p = h->plan;
-    if ((e = to_device(&h->off[0], p.p1.off)) || (e = to_device(&h->items[0], p.p1.items)) ||
-        (e = to_device(&h->off[1], p.p2.off)) || (e = to_device(&h->items[1], p.p2.items)))
+    if ((e = to_device(&h->off[0], p.p1.off, s)) || (e = to_device(&h->items[0], p.p1.items, s)) ||
+        (e = to_device(&h->off[1], p.p2.off, s)) || (e = to_device(&h->items[1], p.p2.items, s)))
         return e;
     h->ready = true;
     return cudaSuccess;

@@ -2023,7 +2023,21 @@ struct TcHost {
     int clusters = 0;          // two-CTA clusters of phase 1 resident at once (occupancy calculator)
     int grid1 = 0, grid2 = 0;  // CTAs of the persistent phase-1 and phase-2 launches
     int epi2 = 12;             // epilogue warps of the phase-2 kernel (p2_epi)
+    std::vector<int> off1, off2, tiles;  // the lists above, on their way to the device until a caller has waited
+    std::vector<int4> items1;
 };
+
+// v into a new device array, on the stream of the kernels that read it: that stream does not wait for
+// the default one, and a plain cudaMemcpy from pageable memory may return with its last bytes still
+// on the way.  v lives until the caller has waited for s.
+template <class T>
+cudaError_t upload(T **dst, const std::vector<T> &v, cudaStream_t s)
+{
+    cudaError_t e = cudaMalloc(dst, std::max<size_t>(1, v.size()) * sizeof(T));
+    if (!e && !v.empty())
+        e = cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, s);
+    return e;
+}
 
 // Cost of a phase-2 tile in MMA issue slots (a BF16 MMA of K = 16 and an E4M3
 // MMA of K = 32 take the same time) plus a fixed epilogue share.
@@ -2407,27 +2421,18 @@ cudaError_t tc_prepare(Dev &d, int cur, cudaStream_t s, bool restored)
         int dev = 0, nsm = 0;
         if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)))
             return e;
-        std::vector<int> off, tiles;
-        build_schedule(d, nsm / 2, off, tiles);  // one list per CTA pair
-        h->grid2 = 2 * ((int)off.size() - 1);
+        build_schedule(d, nsm / 2, h->off2, h->tiles);  // one list per CTA pair
+        h->grid2 = 2 * ((int)h->off2.size() - 1);
         h->epi2 = p2_epi(tile_cost(d, false, 0));
         int pairs = 0;
         bool resident = false;
-        std::vector<int> off1;
-        std::vector<int4> items1;
         if ((e = phase1_pairs(pairs, resident, &h->clusters)))
             return e;
-        if (build_p1(d, pairs, resident, off1, items1) > d.p1_cuts)
+        if (build_p1(d, pairs, resident, h->off1, h->items1) > d.p1_cuts)
             return cudaErrorInvalidValue;  // the memory plan made fewer cut slots (cannot happen)
-        h->grid1 = 2 * ((int)off1.size() - 1);
-        if ((e = cudaMalloc(&h->sched_off, off.size() * sizeof(int))) ||
-            (e = cudaMalloc(&h->sched, tiles.size() * sizeof(int))) ||
-            (e = cudaMemcpy(h->sched_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice)) ||
-            (e = cudaMemcpy(h->sched, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyHostToDevice)) ||
-            (e = cudaMalloc(&h->p1_off, off1.size() * sizeof(int))) ||
-            (e = cudaMalloc(&h->p1_items, items1.size() * sizeof(int4))) ||
-            (e = cudaMemcpy(h->p1_off, off1.data(), off1.size() * sizeof(int), cudaMemcpyHostToDevice)) ||
-            (e = cudaMemcpy(h->p1_items, items1.data(), items1.size() * sizeof(int4), cudaMemcpyHostToDevice)))
+        h->grid1 = 2 * ((int)h->off1.size() - 1);
+        if ((e = upload(&h->sched_off, h->off2, s)) || (e = upload(&h->sched, h->tiles, s)) ||
+            (e = upload(&h->p1_off, h->off1, s)) || (e = upload(&h->p1_items, h->items1, s)))
             return e;
     }
     return cudaSuccess;
@@ -2491,19 +2496,7 @@ struct TcSet {
     std::vector<P2> p2;
 };
 
-namespace {
-template <class T>
-cudaError_t upload(T **dst, const std::vector<T> &v)
-{
-    cudaError_t e = cudaMalloc(dst, std::max<size_t>(1, v.size()) * sizeof(T));
-    if (!e && !v.empty())
-        e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
-    return e;
-}
-
-}  // namespace
-
-cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out)
+cudaError_t tc_set_create(const std::vector<const Dev *> &ds, cudaStream_t s, TcSet **out)
 {
     *out = nullptr;
     cudaError_t e = set_smem_limits();
@@ -2515,6 +2508,11 @@ cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out)
     std::vector<Dev> hd;
     std::vector<TcMaps> hm;
     std::vector<int2> bl;
+    // an array of the set: uploaded on s and waited for, so the vectors below may go out of scope
+    auto put = [s](auto **dst, const auto &v) {
+        const cudaError_t e = upload(dst, v, s);
+        return e ? e : cudaStreamSynchronize(s);
+    };
     for (int k = 0; k < t->n; ++k) {
         const Dev &d = *ds[k];
         hd.push_back(d);
@@ -2525,8 +2523,8 @@ cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out)
     t->nblocks = (int)bl.size();
     int dev = 0, nsm = 0;
     if (!(e = cudaGetDevice(&dev)) && !(e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) &&
-        !(e = upload(&t->devs, hd)) && !(e = upload(&t->maps, hm)) && !(e = upload(&t->blocks, bl)) &&
-        !(e = cudaMalloc(&t->parity, t->n * sizeof(int))) && !(e = cudaMemset(t->parity, 0, t->n * sizeof(int))) &&
+        !(e = put(&t->devs, hd)) && !(e = put(&t->maps, hm)) && !(e = put(&t->blocks, bl)) &&
+        !(e = cudaMalloc(&t->parity, t->n * sizeof(int))) && !(e = cudaMemsetAsync(t->parity, 0, t->n * sizeof(int), s)) &&
         !(e = cudaMalloc(&t->gather, t->n * sizeof(Ctl))) &&
         !(e = cudaMalloc(&t->acc, sizeof(float) * P1_SLOT * (size_t)(nsm & ~1)))) {
         t->pairs = nsm / 2;
@@ -2544,8 +2542,8 @@ cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out)
             lpt_lists(all, std::min<int>(t->pairs, (int)all.size()), false, off, items);
             off.resize(t->pairs + 1, off.back());  // pairs beyond the items get empty lists
             TcSet::P1 c;
-            if (!(e = upload(&c.items, items)))
-                e = upload(&c.off, off);
+            if (!(e = put(&c.items, items)))
+                e = put(&c.off, off);
             t->p1.push_back(c);
         }
         long long slots = 0;  // the longest C' tile decides the set's phase-2 configuration
@@ -2557,8 +2555,8 @@ cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out)
             build_p2(ds, t->pairs, TC_P2_SPEC[q], off, tiles, nets);
             c.epi2 = (p2_epi(slots) == 8) != (TC_P2_SPEC[q].other != 0) ? 8 : 12;
             c.pairs = (int)off.size() - 1;
-            if (!(e = upload(&c.off, off)) && !(e = upload(&c.tiles, tiles)))
-                e = upload(&c.nets, nets);
+            if (!(e = put(&c.off, off)) && !(e = put(&c.tiles, tiles)))
+                e = put(&c.nets, nets);
             t->p2.push_back(c);
         }
     }

@@ -1408,9 +1408,9 @@ int panda_batch_create(panda_batch **out, int n, const int *T, const int *G, con
         for (panda_ctx *c : b->nets)
             ds.push_back(&c->d);
         b->graph_iters = b->nets[0]->graph_iters > 0 ? b->nets[0]->graph_iters : 2;
-        cudaError_t e = tc_set_create(ds, &b->set);
+        cudaError_t e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
         if (!e)
-            e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
+            e = tc_set_create(ds, b->stream, &b->set);
         if (!e)
             e = cudaMallocHost(&b->h_ctls, n * sizeof(Ctl));
         for (int q = 0; q < 3 && !e; ++q)

@@ -330,7 +330,8 @@ struct TcSet;
 constexpr int TC_P1_CANDS = 2, TC_P2_CANDS = 6;
 extern const char *const TC_P1_NAMES[TC_P1_CANDS];
 extern const char *const TC_P2_NAMES[TC_P2_CANDS];
-cudaError_t tc_set_create(const std::vector<const Dev *> &ds, TcSet **out);
+// s: the stream that every other call of the set is given
+cudaError_t tc_set_create(const std::vector<const Dev *> &ds, cudaStream_t s, TcSet **out);
 cudaError_t tc_set_parity(TcSet *t, const std::vector<int> &parity, cudaStream_t s);
 // one iteration of every active network with phase-1 schedule p1 and phase-2
 // schedule p2; events (each may be NULL) before phase 1, before phase 2, after phase 2
