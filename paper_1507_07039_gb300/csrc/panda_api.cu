@@ -291,22 +291,14 @@ int download(panda_ctx *c, float *dst, const float *src, int ld, int rows, int c
     return 0;
 }
 
-// Whether p is device (or managed) memory.
-bool device_pointer(const void *p)
-{
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
-}
+// Whether the context's kernels can work on p where it lies.
+bool in_place(const panda_ctx *c, const void *p) { return where_is(p, c->device) == Where::HERE; }
 
 // The state in W[c->cur], P and C from the three networks (each host or device
 // memory; C's row stride ldc, 0: G): validated, Z-scored if `normalize`, every
-// derived vector and copy made.  A device network is read where it lies; a
-// host one is first copied to where its FP32 matrix lives (or, for a C held as
-// its split pair, into a staging buffer).  One wait at the end tells what the
+// derived vector and copy made.  A network on this device is read where it
+// lies; any other is first copied to where its FP32 matrix lives (or, for a C
+// held as its split pair, into a staging buffer).  One wait at the end tells what the
 // checks found.
 int load_state(panda_ctx *c, const float *W, const float *P, const float *C, int ldc, bool normalize)
 {
@@ -314,17 +306,17 @@ int load_state(panda_ctx *c, const float *W, const float *P, const float *C, int
     const int T = c->T, G = c->G;
     int rc;
     struct { const float *src; int ld; } w{W, G}, p{P, T}, x{C, ldc > 0 ? ldc : G};
-    if (!device_pointer(W)) {
+    if (!in_place(c, W)) {
         if ((rc = upload(c, d.W[c->cur], c->Gp, W, T, G)))
             return rc;
         w = {d.W[c->cur], c->Gp};
     }
-    if (!device_pointer(P)) {
+    if (!in_place(c, P)) {
         if ((rc = upload(c, d.Poff, c->Tp, P, T, T)))
             return rc;
         p = {d.Poff, c->Tp};
     }
-    if (!device_pointer(C)) {
+    if (!in_place(c, C)) {
         if ((rc = stage_c(c)) || (rc = upload(c, d.Coff, c->Gp, C, G, G, x.ld)))
             return rc;
         x = {d.Coff, c->Gp};
@@ -835,11 +827,12 @@ static int full_matrices(panda_ctx *c)
     return 0;
 }
 
-// The networks into dense arrays (each may be NULL).  Those in device memory: one
+// The networks into dense arrays (each may be NULL).  Those on this device: one
 // launch mirrors the upper triangles, puts the diagonals in and writes them all.
-// Host memory: W is copied; a C held as its split pair is written so into a
+// Elsewhere: W is copied; a C held as its split pair is written so into a
 // temporary device buffer and copied; an FP32 matrix is mirrored where it is
-// and copied, its diagonal put in on the host.
+// and copied, its diagonal put in on the host (or, in another GPU's memory, by
+// a strided copy).
 static int get_impl(panda_ctx *c, float *W, float *P, float *C)
 {
     if (int rc = check_state(c))
@@ -847,12 +840,12 @@ static int get_impl(panda_ctx *c, float *W, float *P, float *C)
     Dev &d = c->d;
     StateOut o{c->T, c->G, c->Tp, c->Gp, d.W[c->cur], d.Poff, d.c_split ? nullptr : d.Coff, d.Ch, d.Cl, d.pd, d.cd,
                nullptr, nullptr, nullptr, nullptr, nullptr};
-    if (W && device_pointer(W))
+    if (W && in_place(c, W))
         o.oW = W, W = nullptr;
-    if (P && device_pointer(P))
+    if (P && in_place(c, P))
         o.oP = P, P = nullptr;
     float *tmp = nullptr;
-    if (C && device_pointer(C)) {
+    if (C && in_place(c, C)) {
         o.oC = C, C = nullptr;
     } else if (C && d.c_split) {
         CU(cudaMalloc(&tmp, sizeof(float) * (size_t)c->G * c->G));
@@ -865,7 +858,7 @@ static int get_impl(panda_ctx *c, float *W, float *P, float *C)
             if (int rc = download(c, W, d.W[c->cur], c->Gp, c->T, c->G))
                 return rc;
         if (tmp)
-            CU(cudaMemcpyAsync(C, tmp, sizeof(float) * (size_t)c->G * c->G, cudaMemcpyDeviceToHost, c->stream));
+            CU(cudaMemcpyAsync(C, tmp, sizeof(float) * (size_t)c->G * c->G, cudaMemcpyDefault, c->stream));
         struct { float *dst, *X; const double *diag; int n, ld; } sym[2] = {{P, d.Poff, d.pd, c->T, c->Tp},
                                                                              {tmp ? nullptr : C, d.Coff, d.cd, c->G, c->Gp}};
         for (int q = 0; q < 2; ++q) {
@@ -878,9 +871,20 @@ static int get_impl(panda_ctx *c, float *W, float *P, float *C)
             CU(cudaMemcpyAsync(dg[q].data(), sym[q].diag, sym[q].n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         }
         CU(cudaStreamSynchronize(c->stream));
-        for (int q = 0; q < 2; ++q)
-            for (size_t i = 0; i < dg[q].size(); ++i)
-                sym[q].dst[i * (sym[q].n + 1)] = (float)dg[q][i];
+        for (int q = 0; q < 2; ++q) {
+            if (dg[q].empty())
+                continue;
+            const size_t n = dg[q].size(), step = n + 1;
+            if (where_is(sym[q].dst, c->device) == Where::ELSEWHERE) {
+                const std::vector<float> f(dg[q].begin(), dg[q].end());
+                CU(cudaMemcpy2DAsync(sym[q].dst, step * sizeof(float), f.data(), sizeof(float), sizeof(float), n,
+                                     cudaMemcpyDefault, c->stream));
+                CU(cudaStreamSynchronize(c->stream));
+                continue;
+            }
+            for (size_t i = 0; i < n; ++i)
+                sym[q].dst[i * step] = (float)dg[q][i];
+        }
         return 0;
     };
     const int rc = rest();

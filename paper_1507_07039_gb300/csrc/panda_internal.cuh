@@ -132,6 +132,21 @@ inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
     return cudaGetLastError();
 }
 
+// Where a caller's array lies: in memory that kernels on `device` may read and write (HERE), in
+// another GPU's (ELSEWHERE: only copies reach it, whether or not peer access is on), or on the host.
+enum class Where { HOST, HERE, ELSEWHERE };
+inline Where where_is(const void *p, int device)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return Where::HOST;
+    }
+    if (a.type == cudaMemoryTypeManaged)
+        return Where::HERE;
+    return a.type != cudaMemoryTypeDevice ? Where::HOST : a.device == device ? Where::HERE : Where::ELSEWHERE;
+}
+
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline int round_up(int a, int b) { return ceil_div(a, b) * b; }
 

@@ -50,6 +50,7 @@ constexpr size_t VF = al256(sizeof(float) * SMAX);
 constexpr size_t VD = al256(sizeof(double) * SMAX);
 constexpr size_t PART = al256(sizeof(float) * 3 * SNB * SMAX);  // partial-sum slots
 constexpr size_t BF = al256(sizeof(__nv_bfloat16) * SMAX * SMAX);  // one part of a padded square matrix
+static_assert(2 * BF >= SQ, "two neighbouring parts hold a dense matrix");
 constexpr size_t STATIC_BYTES = 4 * SQ                  // W[2], Poff, Coff
                                 + 12 * BF               // three parts of W[2], P, C
                                 + 2 * VD + 6 * VF       // pd, cd; pdf, cdf, rsqP, csqC, rsqW, csqW
@@ -171,10 +172,22 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
 
     // one iteration at index t: counter 0, growth factor e^{2 alpha t} in slot 1
     SCU(f32_static_lists(d, alpha, std::exp(2.0 * (double)alpha * (double)t), lists, flags, s));
-    // the state, exactly as a context builds it
-    const SymOut po{d.Poff, 0, Parts{d.Ph, d.Pm, d.Pl}, 1, 64, d.Tp, d.pd, d.pdf};
-    const SymOut xo{d.Coff, 0, Parts{d.Ch, d.Cm, d.Cl}, 0, 64, d.Gp, d.cd, d.cdf};
-    StateIn in{dW, dP, dC, T, G, G, T, G, nullptr, nullptr, nullptr};
+    // the state, exactly as a context builds it; a network that is not on this device is copied to
+    // where its matrix lives, and back from the room that its old values or its parts took
+    const bool hW = where_is(dW, dev) == Where::HERE, hP = where_is(dP, dev) == Where::HERE,
+               hC = where_is(dC, dev) == Where::HERE;
+    SymOut po{d.Poff, !hP, Parts{d.Ph, d.Pm, d.Pl}, 1, 64, d.Tp, d.pd, d.pdf};
+    SymOut xo{d.Coff, !hC, Parts{d.Ch, d.Cm, d.Cl}, 0, 64, d.Gp, d.cd, d.cdf};
+    StateIn in{hW ? dW : d.W[0], hP ? dP : d.Poff, hC ? dC : d.Coff, T, G, hW ? G : d.Gp, hP ? T : d.Tp, hC ? G : d.Gp,
+               nullptr, nullptr, nullptr};
+    struct Moved { bool here; float *user, *in; int rows, cols, ld; float *out; };
+    const Moved moved[3] = {{hW, dW, d.W[0], T, G, d.Gp, d.W[0]},
+                            {hP, dP, d.Poff, T, T, d.Tp, reinterpret_cast<float *>(d.Ph)},   // Ph and Pm: 4 bytes an entry
+                            {hC, dC, d.Coff, G, G, d.Gp, reinterpret_cast<float *>(d.Ch)}};  // Ch and Cm
+    for (const Moved &m : moved)
+        if (!m.here)
+            SCU(cudaMemcpy2DAsync(m.in, (size_t)m.ld * 4, m.user, (size_t)m.cols * 4, (size_t)m.cols * 4, m.rows,
+                                  cudaMemcpyDeviceToDevice, s));
     SCU(launch_load(in, d.W[0], Parts{d.Wh[0], d.Wm[0], d.Wl[0]}, d.Tp, d.Gp, po, xo, flags, s));
     in.W = d.W[0];
     in.ldw = d.Gp;
@@ -183,8 +196,8 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     SCU(launch_iteration_f32(d, 0, s, ke));
     // results back into the caller's buffers, diagonals from the FP64 vectors; a failed call leaves
     // the caller's networks as they were
-    SCU(launch_store(StateOut{T, G, d.Tp, d.Gp, d.W[1], d.Poff, d.Coff, nullptr, nullptr, d.pd, d.cd, dW, dP, dC, flags,
-                              d.ctl},
+    SCU(launch_store(StateOut{T, G, d.Tp, d.Gp, d.W[1], d.Poff, d.Coff, nullptr, nullptr, d.pd, d.cd,
+                              hW ? dW : moved[0].out, hP ? dP : moved[1].out, hC ? dC : moved[2].out, flags, d.ctl},
                      s));
     struct { Ctl ctl; int flags[4]; } back{};
     SCU(cudaMemcpyAsync(&back, d.ctl, sizeof(Ctl) + 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -199,6 +212,11 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
         return fail(PANDA_ETIMEOUT, "panda_step_static: a bounded device wait expired");
     if (hc.status & ST_NONFINITE)
         return fail(PANDA_ENONFINITE, "panda_step_static: the networks became non-finite (left unchanged)");
+    for (const Moved &m : moved)
+        if (!m.here)
+            SCU(cudaMemcpyAsync(m.user, m.out, (size_t)m.rows * m.cols * 4, cudaMemcpyDeviceToDevice, s));
+    if (!hW || !hP || !hC)
+        SCU(cudaStreamSynchronize(s));
     if (h_out)
         *h_out = hc.h_last;
     return PANDA_OK;

@@ -64,10 +64,10 @@ char *at(const void *p)  // where the CPU finds p's contents
 }  // namespace
 
 struct Record {
-    char what[64];           // "copy", "set", "sync", or a kernel's name
+    char what[128];          // "copy", "set", "sync", or a kernel's name
     unsigned long long dst, src, bytes, stream;
     int async, grid;
-    unsigned long long arg[32];  // a launch: the first words of its first argument
+    unsigned long long arg[16];  // a launch: the first words at its first argument (and what follows it)
 };
 static std::vector<Record> records;
 static Record &record(const char *what, const void *dst, const void *src, size_t bytes, const void *stream, int async)

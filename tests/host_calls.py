@@ -26,8 +26,8 @@ class Opts(ctypes.Structure):
 
 
 class Record(ctypes.Structure):
-    _fields_ = [("what", ctypes.c_char * 64)] + [(n, ctypes.c_uint64) for n in ("dst", "src", "bytes", "stream")] + [
-        ("async_", ctypes.c_int), ("grid", ctypes.c_int), ("arg", ctypes.c_uint64 * 32)]
+    _fields_ = [("what", ctypes.c_char * 128)] + [(n, ctypes.c_uint64) for n in ("dst", "src", "bytes", "stream")] + [
+        ("async_", ctypes.c_int), ("grid", ctypes.c_int), ("arg", ctypes.c_uint64 * 16)]
 
 
 def link() -> str:
@@ -105,6 +105,62 @@ def check_stream_order():
             if r.what in (b"copy", b"set"):
                 assert r.async_ and r.stream, (prec, r.what, r.bytes)
         lib.panda_batch_destroy(batch)
+
+
+def check_another_gpu():
+    """Arrays in another GPU's memory are copied, never handed to a kernel and
+    never touched by the CPU: create, set_state, get and the static step."""
+    lib = load()
+    T, G = 40, 300
+
+    def foreign():
+        out = []
+        for x in networks(T, G):
+            a = lib.fake_alloc(1, x.nbytes)
+            ctypes.memmove(lib.fake_shadow(a), x.ctypes.data, x.nbytes)
+            out.append(a)
+        return out
+
+    def no_kernel_sees(arrays, what):
+        for r in records(lib):
+            if r.what not in (b"copy", b"set", b"sync"):  # StateIn, StateOut, or a pointer comes first
+                words = 9 if b"k_load" in r.what or b"k_norms" in r.what else 14 if b"k_store" in r.what else 1
+                assert not set(arrays) & set(r.arg[:words]), (what, r.what)
+
+    def copied(arrays, field, what):
+        sizes = [4 * T * G, 4 * T * T, 4 * G * G]
+        for a, n in zip(arrays, sizes):
+            assert sum(r.bytes for r in records(lib) if r.what == b"copy" and getattr(r, field) == a) >= n, what
+
+    for prec in range(4):
+        nets, out = foreign(), foreign()
+        ctx, o = ctypes.c_void_p(), Opts(prec, 0, 0, 0, 8)
+        lib.fake_clear()
+        rc = lib.panda_create_device(ctypes.byref(ctx), T, G, *(p(a) for a in nets), ctypes.byref(o), p(0x5550))
+        assert rc == 0, lib.panda_last_error(None)
+        copied(nets, "src", "create")
+        no_kernel_sees(nets, "create")
+        lib.fake_clear()
+        assert lib.panda_set_state(ctx, *(p(a) for a in nets), 3) == 0, lib.panda_last_error(ctx)
+        copied(nets, "src", "set_state")
+        no_kernel_sees(nets, "set_state")
+        lib.fake_clear()
+        assert lib.panda_get_device(ctx, *(p(a) for a in out)) == 0, lib.panda_last_error(ctx)
+        copied(out, "dst", "get")
+        no_kernel_sees(out, "get")
+        lib.panda_destroy(ctx)
+    nets = foreign()
+    lib.fake_clear()
+    rc = lib.panda_step_static(T, G, *(p(a) for a in nets), ctypes.c_float(0.1), 1, 0, None, None)
+    assert rc == 0, lib.panda_last_error(None)
+    copied(nets, "src", "static")
+    copied(nets, "dst", "static")
+    no_kernel_sees(nets, "static")
+    # on this device they are read and written where they lie
+    here = [lib.fake_alloc(0, x.nbytes) for x in networks(T, G)]
+    lib.fake_clear()
+    assert lib.panda_step_static(T, G, *(p(a) for a in here), ctypes.c_float(0.1), 1, 0, None, None) == 0
+    assert not any(r.what == b"copy" and (r.src in here or r.dst in here) for r in records(lib))
 
 
 if __name__ == "__main__":
