@@ -602,8 +602,12 @@ int create_common(panda_ctx **out, int T, int G, const float *W0, const float *P
         return set_err(nullptr, PANDA_EUNSUPPORTED, "unknown precision mode");
     if (opts.diag < 0 || opts.diag > 2 || opts.t0 < 0 || opts.t0 >= HIST_CAP || opts.graph_iters < 0)
         return set_err(nullptr, PANDA_EINVAL, "bad option value");
-    if (tensor_prec(opts.prec) && !tc_supported())
-        return set_err(nullptr, PANDA_EUNSUPPORTED, "the tensor-core modes need an sm_103 device");
+    int dev = 0;
+    const cudaError_t dev_err = cudaGetDevice(&dev);
+    if (dev_err && opts.prec == PANDA_FP32)
+        return set_err(nullptr, PANDA_ECUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(dev_err));
+    if (!tc_supported())  // every mode's products run on tcgen05
+        return set_err(nullptr, PANDA_EUNSUPPORTED, "the library needs an sm_103 device");
 
     panda_ctx *c = new panda_ctx();
     c->T = T; c->G = G;
@@ -622,11 +626,8 @@ int create_common(panda_ctx **out, int T, int G, const float *W0, const float *P
         g_create_error = msg;
         return code;
     };
-    cudaError_t e = cudaGetDevice(&c->device);
-    if (e != cudaSuccess) {
-        c->err = std::string("cudaGetDevice: ") + cudaGetErrorString(e);
-        return fail(PANDA_ECUDA);
-    }
+    c->device = dev;
+    cudaError_t e;
     if (device_ptrs) {
         c->stream = static_cast<cudaStream_t>(stream);
     } else {
@@ -666,13 +667,7 @@ extern "C" {
 
 int panda_precision_supported(int prec)
 {
-    if (prec == PANDA_FP32) {
-        int n = 0;
-        return cudaGetDeviceCount(&n) == cudaSuccess && n > 0;
-    }
-    if (tensor_prec(prec))
-        return tc_supported() ? 1 : 0;
-    return 0;
+    return (prec == PANDA_FP32 || tensor_prec(prec)) && tc_supported() ? 1 : 0;
 }
 
 void panda_default_opts(panda_opts *o)

@@ -114,6 +114,8 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     SCU(cudaGetDevice(&dev));
     if (dev < 0 || dev >= MAX_DEVICES)
         return fail(PANDA_EUNSUPPORTED, "panda_step_static: device index out of range");
+    if (!tc_supported())
+        return fail(PANDA_EUNSUPPORTED, "panda_step_static: needs an sm_103 device");
     unsigned char *base = nullptr;
     SCU(scratch_address(dev, &base));
 

@@ -163,6 +163,25 @@ def check_another_gpu():
     assert not any(r.what == b"copy" and (r.src in here or r.dst in here) for r in records(lib))
 
 
+def check_other_device():
+    """On a GPU without tcgen05 every mode, the default one and the static step
+    included, is refused before it touches the device."""
+    lib = load()
+    assert [lib.panda_precision_supported(k) for k in range(-1, 5)] == [0, 1, 1, 1, 1, 0]
+    lib.fake_capability(9, 0)
+    assert [lib.panda_precision_supported(k) for k in range(4)] == [0, 0, 0, 0]
+    nets = networks(8, 20)
+    for prec in range(4):
+        ctx, o = ctypes.c_void_p(), Opts(prec, 0, 0, 0, 8)
+        lib.fake_clear()
+        rc = lib.panda_create(ctypes.byref(ctx), 8, 20, *(p(x) for x in nets), ctypes.byref(o))
+        assert (rc, ctx.value, lib.fake_count()) == (-8, None, 0), (prec, rc)
+    here = [lib.fake_alloc(0, x.nbytes) for x in nets]
+    lib.fake_clear()
+    rc = lib.panda_step_static(8, 20, *(p(a) for a in here), ctypes.c_float(0.1), 1, 0, None, None)
+    assert (rc, lib.fake_count()) == (-8, 0), rc
+
+
 if __name__ == "__main__":
     globals()["check_" + sys.argv[1]]()
     print("ok")

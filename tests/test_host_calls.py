@@ -11,7 +11,7 @@ import pytest
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 
-@pytest.mark.parametrize("check", ["stream_order", "another_gpu"])
+@pytest.mark.parametrize("check", ["stream_order", "another_gpu", "other_device"])
 def test_host_calls(check):
     r = subprocess.run([sys.executable, os.path.join(HERE, "host_calls.py"), check], capture_output=True, text=True,
                        timeout=600)
