@@ -93,20 +93,14 @@ __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 &hi, __nv_bflo
 
 // Eq. 1 from the numerator and the two squared norms with the hardware
 // reciprocal square root (rsqrtf, within 2 ulp): the tensor-core path's
-// epilogues, whose products carry BF16X3 error far above that; 0 when the
-// denominator is 0 (both vectors zero).
+// epilogues, whose products carry BF16X3 error far above that.  The denominator
+// is at least (|x|^2 + |y|^2) / 2, so only two zero vectors meet the clamp at
+// the smallest positive float, and their numerator is 0 too.  (Eq. 1 scales
+// with its vectors: a larger clamp, 1e-30 once, gave norms below 1e-15 too
+// small a result.)
 __device__ __forceinline__ float tanimoto_fast(float num, float nx, float ny)
 {
-    const float den = (nx + ny) - fabsf(num);
-    return den > 0.0f ? num * rsqrtf(den) : 0.0f;
-}
-
-// As tanimoto_fast without the branch: the denominator is at least
-// (|x|^2 + |y|^2)/2 > 0 unless both vectors are zero, in which case the
-// numerator is 0 too and the clamp keeps the result 0.
-__device__ __forceinline__ float tanimoto_clamped(float num, float nx, float ny)
-{
-    return num * rsqrtf(fmaxf((nx + ny) - fabsf(num), 1e-30f));
+    return num * rsqrtf(fmaxf((nx + ny) - fabsf(num), 1.401298464e-45f));
 }
 
 // hi / lo of two values at once, packed as BF16 pairs (first value in the low half)
@@ -1124,8 +1118,8 @@ __device__ __forceinline__ void phase1_pair(const Src &src, Ctl *ctl0)
                                 const float wv = w[i][u];
                                 const float rnum = x[i][u] + pdi * wv;                // P_i. . W_.j
                                 const float anum = fmaf(y[i][u], ainv, wv * cdj[u]);     // W_i. . C_.j
-                                const float R = tanimoto_clamped(rnum, rsp, nwj[u]);
-                                const float A = tanimoto_clamped(anum, rsw, ncj[u]);
+                                const float R = tanimoto_fast(rnum, rsp, nwj[u]);
+                                const float A = tanimoto_fast(anum, rsw, ncj[u]);
                                 float wn = fmaf(keep, wv, halfa * (A + R));
                                 if (!inner)  // padding stays zero
                                     wn = k0 + er + 8 * i < d.T && j0 + ec + u < d.G ? wn : 0.0f;
@@ -1727,7 +1721,7 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            const float s = tanimoto_clamped(x[i][u], nrow[i], nj[u]);
+                            const float s = tanimoto_fast(x[i][u], nrow[i], nj[u]);
                             const float w = fmaf(a, s, keep * v[i][u]);
                             const float y = SIM_SIGMA ? s : w;
                             r1[i] += y;
