@@ -161,18 +161,19 @@ __device__ __forceinline__ void split3(float x0, float x1, uint32_t (&p)[3])
     }
 }
 
-// Eq. 1 from the numerator and the squared norms: the hardware reciprocal
-// square root with one Newton step (about 1 ulp).  The denominator is at least
-// (|x|^2 + |y|^2) / 2, so its clamp only meets vectors that are zero (numerator
-// 0, result 0) or below 1e-19 in norm; the upper clamp keeps the Newton step
-// finite where a norm has overflowed (y = 0, result 0).
+// Eq. 1 from the numerator and the squared norms: rsqrtf with one Newton step
+// (about 1 ulp) over the whole range of floats.  The denominator is at least
+// (|x|^2 + |y|^2) / 2, so only two zero vectors meet the lower clamp (numerator
+// 0, result 0); the upper one keeps the Newton step finite where a norm has
+// overflowed (y = 0, result 0).  (With the denominator clamped at the smallest
+// normal float, entries of 2^-66 gave W off by 4e-2 of its largest one; rsqrtf's
+// care of subnormal arguments costs 0.5% to 2%: 125 x 125 to h < 1e-3 784 -> 801
+// us, 1000 x 17000, three iterations, 11.63 -> 11.70 ms.)
 __device__ __forceinline__ float tanimoto_newton(float num, float nx, float ny)
 {
-    const float den = fmaxf((nx + ny) - fabsf(num), 1.17549435e-38f);
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(den));
-    const float s = num * y;
-    return fmaf(0.5f * s, fmaf(-fminf(den, 3.0e38f) * y, y, 1.0f), s);
+    const float den = fmaxf((nx + ny) - fabsf(num), 1.401298464e-45f);
+    const float y = rsqrtf(den), s = num * y;
+    return fmaf(0.5f * s, fmaf(-fminf(den, 3.402823466e38f) * y, y, 1.0f), s);
 }
 
 // ---- one CTA or a CTA pair ----------------------------------------------------------
