@@ -176,6 +176,23 @@ __device__ __forceinline__ float tanimoto_newton(float num, float nx, float ny)
     return fmaf(0.5f * s, fmaf(-fminf(den, 3.402823466e38f) * y, y, 1.0f), s);
 }
 
+// Eqs. 2 and 5: (1 - alpha) x + alpha y, y the mean of n similarities given as their sum.  Below
+// alpha = 1/2 as x + alpha (y - x), which does not round 1 - alpha; from there on, where 1 - alpha is
+// exact, as it stands: alpha = 1 gives y, where the first form would leave a rounding of x's size in
+// it (2-norm of one update's error at alpha = 0.1, 0.5, 0.9, 1, first form and second: 2.6e-8, 3.9e-8,
+// 4.6e-8, 4.0e-8 and 4.3e-8, 2.8e-8, 2.5e-8, 0).
+struct Damp {
+    float a, keep, minus;
+    __device__ __forceinline__ Damp(float alpha, float n)
+        : a(alpha / n), keep(alpha < 0.5f ? 1.0f : 1.0f - alpha), minus(alpha < 0.5f ? -n : 0.0f)
+    {
+    }
+    __device__ __forceinline__ float operator()(float x, float sum) const
+    {
+        return fmaf(a, fmaf(minus, x, sum), keep * x);
+    }
+};
+
 // ---- one CTA or a CTA pair ----------------------------------------------------------
 template <bool PAIR>
 __device__ __forceinline__ void load_box(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y)
@@ -623,7 +640,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                 fetch_rows();
                 fetch_w(0);
             }
-            const float halfa = 0.5f * ctl->alpha;
+            const Damp damp(ctl->alpha, 2.0f);
             float hsum = 0.0f;
             epi_bar();  // colvec is complete; colred and rowred of the item before are no longer read
             // W, R-num and the sums one chunk ahead
@@ -677,8 +694,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                             const float anum = y[i][u] + w[i][u] * cd[u];    // W_i. . C_.j
                             const float R = tanimoto_newton(rnum, rsp[i], nw[u]);
                             const float A = tanimoto_newton(anum, rsw[i], nc[u]);
-                            // (1 - a) W + a/2 (A + R) without rounding 1 - a
-                            const float v = fmaf(halfa, fmaf(-2.0f, w[i][u], A + R), w[i][u]);
+                            const float v = damp(w[i][u], A + R);
                             wn[u] = ri && j0 + ec + u < d.G ? v : 0.0f;
                             hsum += fabsf(wn[u] - w[i][u]);  // (padding holds zeros)
                             rowsq[i] = fmaf(wn[u], wn[u], rowsq[i]);
@@ -862,7 +878,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
             __nv_bfloat16 *Xs[3] = {isP ? d.Ph : d.Ch, isP ? d.Pm : d.Cm, isP ? d.Pl : d.Cl};
             // split copies of the lower triangle: all of P, of C only inside diagonal tiles
             const bool mirror = isP || (PAIR ? bm == bn : bm == bn >> 1);
-            const float a = ctl->alpha;
+            const Damp damp(ctl->alpha, 1.0f);
             if (PAIR) {
                 fetch_rows();
                 fetch(0);
@@ -905,8 +921,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                     const bool inner = k0 + 31 < j0 && j0 + 15 < nn;
                     auto update = [&](int i, int u, bool valid) {
                         const float s = tanimoto_newton(x[i][u], nrow[i], nj[u]);
-                        // (1 - a) X + a s without rounding 1 - a
-                        const float w = valid ? fmaf(a, s - v[i][u], v[i][u]) : 0.0f;
+                        const float w = valid ? damp(v[i][u], s) : 0.0f;
                         const float y = SIM ? (valid ? s : 0.0f) : w;
                         r1[i] += y;
                         r2[i] = fmaf(y, y, r2[i]);
