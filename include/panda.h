@@ -330,6 +330,15 @@ int panda_phase1_plan(int T, int G, int prec, int pairs, int all_resident, int *
  * NULL.  Returns 0, or PANDA_EINVAL for NULL c or an FP32 context. */
 int panda_phase1_layout(const panda_ctx *c, int *pairs, int *clusters, int *cuts);
 
+/* How the two tile phases of an FP32 iteration of one network of T TFs and G
+ * genes are spread over `sms` SMs (a host computation: no device is needed).
+ * *pair: 1 for 256 x 256 tiles on CTA pairs, 0 for 128 x 64 tiles on single
+ * CTAs.  ctas, items and cuts receive two ints each, phase 1 (W') and phase 2
+ * (P' and C'): the CTAs launched, the work items (tiles, or parts of tiles
+ * along their sum) and the tiles cut into parts.  Returns 0, or PANDA_EINVAL
+ * (a size or sms out of range, a NULL pointer). */
+int panda_fp32_plan(int T, int G, int sms, int *pair, int *ctas, int *items, int *cuts);
+
 const char *panda_batch_last_error(const panda_batch *b);
 void panda_batch_destroy(panda_batch *b);
 

@@ -1349,6 +1349,19 @@ F32Plan f32_plan_for(const Dev &d, int nsm)
     return best;
 }
 
+// CTAs of a phase: the workers up to the last that has an item.  A CTA takes an SM to itself (217 KB
+// of shared memory, all of TMEM), so one that finds nothing to do keeps another network of a set
+// waiting: with 152 CTAs whatever the work, 64 networks of 125 x 125 took 286 us an iteration (81
+// now), 64 of 60 x 300 382 (154), 16 of 250 x 600 184 (144).
+int grid_of(const F32Plan &p, int phase)
+{
+    const Phase &ph = phase ? p.p2 : p.p1;
+    int n = (int)ph.off.size() - 1;
+    while (n > 1 && ph.off[n - 1] == ph.off[n])
+        --n;
+    return (p.pair ? 2 : 1) * n;
+}
+
 struct F32Host {
     F32Maps maps;
     F32Plan plan;  // its lists are on the device once `ready`
@@ -1463,14 +1476,27 @@ void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fix
     if (!h) {
         d.f32_host = h = new F32Host;
         h->plan = f32_plan_for(d, nsm);
-        h->grid[0] = h->grid[1] = h->plan.pair ? nsm & ~1 : nsm;
+        for (int q = 0; q < 2; ++q)
+            h->grid[q] = grid_of(h->plan, q);
     }
     const F32Plan &p = h->plan;
     const size_t slot = p.pair ? Tile<true>::SLOT : Tile<false>::SLOT, ranks = p.pair ? 2 : 1;
-    *slot_floats = slot * (size_t)h->grid[0];
+    *slot_floats = slot * (size_t)h->grid[0];  // (phase 1's alone)
     *fix_floats = slot * ranks * (size_t)std::max(p.p1.slots, p.p2.slots);
     *fixes = std::max(p.p1.fixes, p.p2.fixes);
     *pair = p.pair;
+}
+
+void f32_plan_info(const Dev &d, int nsm, bool *pair, int *ctas, int *items, int *cuts)
+{
+    const F32Plan p = f32_plan_for(d, nsm);
+    *pair = p.pair;
+    for (int q = 0; q < 2; ++q) {
+        const Phase &ph = q ? p.p2 : p.p1;
+        ctas[q] = grid_of(p, q);
+        items[q] = (int)ph.items.size();
+        cuts[q] = ph.fixes;
+    }
 }
 
 int f32_diag_block(const Dev &d) { return static_cast<const F32Host *>(d.f32_host)->plan.pair ? 256 : 64; }

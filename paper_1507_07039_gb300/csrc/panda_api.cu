@@ -1574,6 +1574,19 @@ int panda_phase1_plan(int T, int G, int prec, int pairs, int all_resident, int *
     return cuts;
 }
 
+int panda_fp32_plan(int T, int G, int sms, int *pair, int *ctas, int *items, int *cuts)
+{
+    if (T < 1 || G < 1 || T > 46000 || G > 46000 || sms < 2 || !pair || !ctas || !items || !cuts)
+        return set_err(nullptr, PANDA_EINVAL, "panda_fp32_plan: bad argument");
+    Dev d{};
+    d.T = T; d.G = G;
+    d.Tp = round_up(T, TILE); d.Gp = round_up(G, TILE);
+    bool p = false;
+    f32_plan_info(d, sms, &p, ctas, items, cuts);
+    *pair = p;
+    return 0;
+}
+
 const char *panda_batch_last_error(const panda_batch *b) { return b ? b->err.c_str() : g_create_error.c_str(); }
 
 void panda_batch_destroy(panda_batch *b)

@@ -321,6 +321,8 @@ extern const char *const F32_KERNEL_NAMES[F32_KERNELS];
 // scratch they need: floats of the per-CTA slots and of the cut tiles' slots,
 // cut tiles (two counters each), the tile shape.
 void f32_plan(Dev &d, int nsm, size_t *slot_floats, size_t *fix_floats, int *fixes, bool *pair);
+// That plan's tile shape, and per phase its CTAs, items and cut tiles.  Host only.
+void f32_plan_info(const Dev &d, int nsm, bool *pair, int *ctas, int *items, int *cuts);
 // Tensor maps and device lists at the first call; restored: also the split copies of W[cur], Poff, Coff.
 cudaError_t f32_prepare(Dev &d, int cur, cudaStream_t s, bool restored);
 // Edge of the diagonal blocks inside which phase 2 keeps both triangles of C's split copy.

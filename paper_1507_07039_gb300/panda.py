@@ -81,6 +81,7 @@ def _load() -> ctypes.CDLL:
         "panda_batch_schedule_name": (ctypes.c_char_p, [i, i]),
         "panda_phase1_plan": (i, [i, i, i, i, i, pi, i, pi]),
         "panda_phase1_layout": (i, [vp, pi, pi, pi]),
+        "panda_fp32_plan": (i, [i, i, i, pi, pi, pi, pi]),
         "panda_batch_destroy": (None, [vp]),
         "panda_destroy": (None, [vp]),
     }
@@ -310,6 +311,14 @@ def panda_phase1_plan(T: int, G: int, prec: int, pairs: int, all_resident: bool 
     cuts = _check(lib.panda_phase1_plan(int(T), int(G), int(prec), int(pairs), int(bool(all_resident)),
                                         out.ctypes.data_as(ctypes.POINTER(ctypes.c_int)), n.value, ctypes.byref(n)))
     return cuts, out
+
+
+def panda_fp32_plan(T: int, G: int, sms: int = 152) -> dict:
+    """The FP32 iteration's tile shape and, per phase, its CTAs, items and cut tiles."""
+    pair, two = ctypes.c_int(0), ctypes.c_int * 2
+    ctas, items, cuts = two(), two(), two()
+    _check(lib.panda_fp32_plan(T, G, sms, ctypes.byref(pair), ctas, items, cuts))
+    return dict(pair=bool(pair.value), ctas=list(ctas), items=list(items), cuts=list(cuts))
 
 
 def panda_phase1_layout(ctx) -> dict:
