@@ -641,6 +641,9 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                 fetch_w(0);
             }
             const Damp damp(ctl->alpha, 2.0f);
+            // a row's squares and |W' - W| are added four columns at a time, these over the chunks: no chain
+            // of additions is longer than 8 (32 and 128 in one left 15% to 20% more error than FFMA's
+            // slots of 128 columns)
             float hsum = 0.0f;
             epi_bar();  // colvec is complete; colred and rowred of the item before are no longer read
             // W, R-num and the sums one chunk ahead
@@ -684,10 +687,11 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                     const float4 q4 = *reinterpret_cast<const float4 *>(colvec + 2 * N + cc + ec);
                     const float cd[4] = {c4.x, c4.y, c4.z, c4.w}, nw[4] = {w4.x, w4.y, w4.z, w4.w},
                                 nc[4] = {q4.x, q4.y, q4.z, q4.w};
+                    float hc = 0.0f;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const bool ri = k0 + er + 8 * i < d.T;
-                        float wn[4];
+                        float wn[4], r4 = 0.0f, h4 = 0.0f;
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             const float rnum = x[i][u] + pdi[i] * w[i][u];   // P_i. . W_.j
@@ -696,10 +700,12 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                             const float A = tanimoto_newton(anum, rsw[i], nc[u]);
                             const float v = damp(w[i][u], A + R);
                             wn[u] = ri && j0 + ec + u < d.G ? v : 0.0f;
-                            hsum += fabsf(wn[u] - w[i][u]);  // (padding holds zeros)
-                            rowsq[i] = fmaf(wn[u], wn[u], rowsq[i]);
+                            h4 += fabsf(wn[u] - w[i][u]);  // (padding holds zeros)
+                            r4 = fmaf(wn[u], wn[u], r4);
                             cs[u] = fmaf(wn[u], wn[u], cs[u]);
                         }
+                        hc += h4;
+                        rowsq[i] += r4;
                         const size_t o = wo + (size_t)(8 * i) * d.Gp + c * 16;
                         *reinterpret_cast<float4 *>(Wn + o) = make_float4(wn[0], wn[1], wn[2], wn[3]);
                         uint32_t p0[3], p1[3];
@@ -709,6 +715,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                         for (int p = 0; p < 3; ++p)
                             *reinterpret_cast<uint2 *>(Ws[p] + o) = make_uint2(p0[p], p1[p]);
                     }
+                    hsum += hc;
                 }
                 const float t = lanes8_reduce_scatter4(cs);
                 if (!(lane & 4))
@@ -919,17 +926,25 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(NTHREADS,
                     const float4 n4 = *reinterpret_cast<const float4 *>(colnrm + cc + ec);
                     const float nj[4] = {n4.x, n4.y, n4.z, n4.w};
                     const bool inner = k0 + 31 < j0 && j0 + 15 < nn;
+                    float l1 = 0.0f, l2 = 0.0f, lv = 0.0f;
                     auto update = [&](int i, int u, bool valid) {
                         const float s = tanimoto_newton(x[i][u], nrow[i], nj[u]);
                         const float w = valid ? damp(v[i][u], s) : 0.0f;
                         const float y = SIM ? (valid ? s : 0.0f) : w;
-                        r1[i] += y;
-                        r2[i] = fmaf(y, y, r2[i]);
+                        // a row's four columns first, then the chunks (as in phase 1)
+                        l1 = u ? l1 + y : y;
+                        l2 = u ? fmaf(y, y, l2) : y * y;
                         cs[u] += y;
                         cs[4 + u] = fmaf(y, y, cs[4 + u]);
                         if (SIM) {
-                            rv[i] = fmaf(w, w, rv[i]);
+                            lv = u ? fmaf(w, w, lv) : w * w;
                             cv[u] = fmaf(w, w, cv[u]);
+                        }
+                        if (u == 3) {
+                            r1[i] += l1;
+                            r2[i] += l2;
+                            if (SIM)
+                                rv[i] += lv;
                         }
                         v[i][u] = w;
                     };
