@@ -150,14 +150,6 @@ inline Where where_is(const void *p, int device)
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline int round_up(int a, int b) { return ceil_div(a, b) * b; }
 
-// Eq. 1 from a numerator and the two squared norms (FP32, IEEE sqrt and
-// division); 0 when the denominator is 0 (both vectors zero).
-__device__ __forceinline__ float tanimoto_f(float num, float nx, float ny)
-{
-    float den = sqrtf((nx + ny) - fabsf(num));
-    return den > 0.0f ? num / den : 0.0f;
-}
-
 // ---- FP32 error-free transforms --------------------------------------------
 // This GPU's FP64 pipe issues about two operations per clock per SM, the FP32
 // pipe 128, so sums and products that want more than FP32 accuracy run as

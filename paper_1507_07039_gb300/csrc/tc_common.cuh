@@ -1,11 +1,14 @@
 // Blackwell (sm_103a) building blocks of the tensor-core path: mbarriers,
 // TMA tile loads, tcgen05 MMA issue / commit, TMEM allocation and loads, and
-// a warp-specialised pipeline shared by every tcgen05 kernel here:
+// the roles that every tcgen05 kernel here is split into:
 //
-//   warp 0, one lane   TMA producer: fills a ring of shared-memory stages
-//   warp 1, one lane   MMA issuer:   BF16 x BF16 -> FP32 tcgen05.mma into TMEM
-//   warps 2-5          epilogue:     tcgen05.ld of the accumulators (one row
-//                                    of the 128-row tile per thread)
+//   TMA producer   one lane of a warp: fills a ring of shared-memory stages
+//   MMA issuer     a whole converged warp, whose elected lane issues the
+//                  tcgen05.mma (in the self-test and Pearson kernels, whose
+//                  pipeline stands at the end of this file, one lane)
+//   epilogue       tcgen05.ld of the accumulators: as fragments of 16 rows
+//                  (frag_to_rows), or (self-test and Pearson) one row of the
+//                  128-row tile per thread
 //
 // Operands are K-major BF16 tiles of 64 elements (128 bytes) per row, loaded
 // by TMA with the 128-byte swizzle, which is the canonical K-major SW128
@@ -370,20 +373,8 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t *bar)
         : "memory");
 }
 
-// Start a 16-column TMEM load without waiting (the registers are valid after tmem_wait()).
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// The wait for a tmem_ld16_nowait into r: r is an in-out operand, so no use of
-// it can be scheduled before the loaded values have arrived.
+// The wait for a tmem_ld_frag16_nowait into r (below): r is an in-out operand,
+// so no use of it can be scheduled before the loaded values have arrived.
 __device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
