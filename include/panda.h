@@ -23,7 +23,8 @@
  * All matrices crossing this interface are dense, row-major, FP32, with no
  * padding: W has T*G entries, P has T*T, C has G*G (P and C include their
  * diagonals).  Host pointers are plain host memory (pageable or pinned);
- * device pointers are CUDA device memory of the current device.
+ * device pointers are CUDA device memory of the current device (worked on in
+ * place; an array in another GPU's memory is copied through this one).
  *
  * Return codes: 0 success; 1 PANDA_NOT_CONVERGED (max_iter reached, outputs
  * valid); negative values are errors and leave a message readable with
@@ -57,8 +58,8 @@ extern "C" {
  * carry 16 significant bits instead of 24; panda_get and panda_get_state
  * return hi + lo (exact in FP32) with the diagonal from its FP64 vector. */
 typedef enum {
-    PANDA_FP32 = 0,   /* FP32 products on the tensor cores: x = h + m + l in BF16 exactly, the six part
-                         products down to 2^-16, summed in FP32 registers every 64 terms */
+    PANDA_FP32 = 0,   /* FP32 products on the tensor cores: x = h + m + l in BF16 (exactly for |x| > 2^-110),
+                         the six part products down to 2^-16, summed in FP32 registers every 64 terms */
     PANDA_BF16X3 = 1, /* tensor cores: x = hi + lo in BF16, hi*hi + hi*lo + lo*hi, FP32 accumulation */
     PANDA_BF16X2 = 2, /* tensor cores: A operands split hi + lo, B operands BF16 hi only: hi*hi + lo*hi
                          (about 2^-9 relative error on each B entry; 2/3 of BF16X3's tensor work) */
@@ -181,7 +182,12 @@ int panda_get_history(panda_ctx *ctx, double *h, int cap, int *n);
 /* Shape, mode and counters of a context. */
 int panda_info(const panda_ctx *ctx, int *T, int *G, int *prec, int *t);
 
-/* Bytes of device memory the context holds between calls. */
+/* Bytes of device memory the context holds between calls: about 20 per entry
+ * of W and 10 per entry of P and C under PANDA_FP32 (the FP32 networks and
+ * their three BF16 parts), 16, 8 and 4 under PANDA_BF16X3 and PANDA_BF16X2,
+ * 20, 8 and 5 under PANDA_FP8MIX, sizes padded to multiples of 128 (FP32) or
+ * 256, and some tens of MB of work space: 3.3, 1.55 and 1.9 GB at 1000 x
+ * 17000. */
 long long panda_device_bytes(const panda_ctx *ctx);
 
 /* The most device memory the context has held at once: under PANDA_BF16X3

@@ -11,9 +11,10 @@
 //
 // Every FP32 operand is held beside its value as three BF16 parts, h = bf16(x),
 // m = bf16(x - h), l = x - h - m: 3 x 8 significant bits, so h + m + l = x
-// exactly.  A product takes the six part products of weight down to 2^-16
-// (h.h, h.m, m.h, m.m, h.l, l.h; what is left out is below 2^-23 of |a||b|, of
-// either sign), so nothing is lost in the operands.  What the tensor core does
+// exactly for |x| above 2^-110 (below, l leaves BF16's range and x keeps fewer
+// bits, to a spacing of 2^-133).  A product takes the six part products of
+// weight down to 2^-16 (h.h, h.m, m.h, m.m, h.l, l.h; the three left out are
+// below 2^-23 of |a||b| together, of either sign).  What the tensor core does
 // lose is its accumulation: FP32, but truncated toward zero at every MMA
 // (measured: -1.9e-8 of the running sum per MMA), where the former FFMA kernel
 // rounded to nearest at every product.  So no chain is long: each K = 64
@@ -27,7 +28,7 @@
 //
 // Bound: the tensor pipe, 6 x the algorithmic flops (FFMA: 78 TFLOP/s
 // measured, 49 reached).  A stage's operands are 96 KB per CTA for 24 MMAs,
-// two thirds of BF16X3's bytes per MMA.
+// three quarters of BF16X3's bytes per MMA (64 KB for 12).
 //
 // Two tile shapes, the same code: 256 x 256 on a CTA pair (cta_group::2), and
 // 128 x 64 on one CTA for networks with too few tiles to fill the chip with
@@ -1344,8 +1345,8 @@ struct F32Plan {
 };
 
 // The tile shape whose busiest worker is done first by the stage times; one
-// CTA per tile only where pairs would have few tiles each (it reads twice the
-// operand bytes per flop).
+// CTA per tile only where pairs would have few tiles each (it reads three times
+// the operand bytes per flop).
 F32Plan f32_plan_for(const Dev &d, int nsm)
 {
     F32Plan best{};

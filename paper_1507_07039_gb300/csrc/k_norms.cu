@@ -86,8 +86,6 @@ __device__ __forceinline__ void fp8_norm_max(unsigned *slot, float v)
         atomicMax(slot, u);
 }
 
-// rsqW[i] = sum_b wrow_part[b][i], csqW[j] = sum_b wcol_part[b][j] (FP64).
-// Blocks [0, ceil(T/32)) take rows of W, the rest its columns.
 // h (Eq. 7) of the iteration under way from phase 1's partial sums, in FP64 in a fixed order.
 __device__ __forceinline__ void sum_h(const Dev &d)
 {
@@ -109,7 +107,8 @@ __device__ __forceinline__ void sum_h(const Dev &d)
     }
 }
 
-// block b of one network's launch: b < ceil(T/32) rows of W, then its columns, the last one h
+// rsqW[i] = sum_b wrow_part[b][i], csqW[j] = sum_b wcol_part[b][j] (FP64): block b of one network's
+// launch, b < ceil(T/32) rows of W, then its columns, the last one h
 __device__ __forceinline__ void reduce_wnorms_block(const Dev &d, int b)
 {
     if (!d.ctl->active)

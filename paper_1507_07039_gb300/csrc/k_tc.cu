@@ -589,8 +589,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // staged: phase 1 at 250 x 2100 (one tile per pair) 67 -> 58.5 us, 600 x 6000
 // 130 -> 123.5 us.  Where a pair has several tiles the epilogue runs beside
 // the next tile's MMAs (phase1_pair).  BF16X3 at 1000 x 17000, 1.02 ms, is
-// bound by its MMAs: 12 of 128 cycles a stage of 1530 cycles, at the clock the
-// power limit leaves.
+// bound by its MMAs: a stage's 12 of 128 cycles each are the 1.53 thousand cycles
+// that it takes, at the clock the power limit leaves.
 constexpr int ST1 = 3;
 constexpr uint32_t STAGE1 = 4 * A_BYTES;   // per CTA: A hi, A lo, B hi, B lo (128 rows each)
 constexpr int EPI1 = 8, THREADS1 = 64 + 32 * EPI1;
@@ -2242,9 +2242,11 @@ cudaError_t phase2_smem_limits()
 // issue slots each (the largest over a set): twelve (two operand stages) only
 // where a tile is almost all epilogue, eight (three stages) otherwise.
 // Measured, twelve against eight: FP8MIX at 1000 x 17000 (32 slots) 0.633 and
-// 0.675 ms; BF16X3 at 250 x 2100 (48) even; at 600 x 6000 (120) 131 and 134 us,
-// at 1000 x 17000 (192) 0.734 and 0.715 ms, a set of twelve networks (48 to
-// 192) 1.12 and 0.97 ms; 1600 x 30000 (336) 3.7 and 2.9 ms.
+// 0.675 ms; BF16X3 at 250 x 2100 (48) even; at 350 x 6000 (72) 112.6 and 110.7
+// us, 500 x 6000 (96) 114.4 and 111.7, 600 x 6000 (120) 129.4 and 130.3, 600 x
+// 12000 330 and 324, 880 x 6000 (168) 133.1 and 134.9; BF16X2 at 600 x 6000 (80)
+// 122 and 109; BF16X3 at 1000 x 17000 (192) 0.734 and 0.715 ms, a set of twelve
+// networks (48 to 192) 1.12 and 0.97 ms; 1600 x 30000 (336) 3.7 and 2.9 ms.
 int p2_epi(long long mma_slots) { return mma_slots > 64 ? 8 : 12; }
 
 // One phase-2 launch of EPI epilogue warps
