@@ -189,7 +189,7 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
     for (const Moved &m : moved)
         if (!m.here)
             SCU(cudaMemcpy2DAsync(m.in, (size_t)m.ld * 4, m.user, (size_t)m.cols * 4, (size_t)m.cols * 4, m.rows,
-                                  cudaMemcpyDeviceToDevice, s));
+                                  cudaMemcpyDefault, s));
     SCU(launch_load(in, d.W[0], Parts{d.Wh[0], d.Wm[0], d.Wl[0]}, d.Tp, d.Gp, po, xo, flags, s));
     in.W = d.W[0];
     in.ldw = d.Gp;
@@ -216,7 +216,7 @@ extern "C" int panda_step_static(int T, int G, float *dW, float *dP, float *dC, 
         return fail(PANDA_ENONFINITE, "panda_step_static: the networks became non-finite (left unchanged)");
     for (const Moved &m : moved)
         if (!m.here)
-            SCU(cudaMemcpyAsync(m.user, m.out, (size_t)m.rows * m.cols * 4, cudaMemcpyDeviceToDevice, s));
+            SCU(cudaMemcpyAsync(m.user, m.out, (size_t)m.rows * m.cols * 4, cudaMemcpyDefault, s));
     if (!hW || !hP || !hC)
         SCU(cudaStreamSynchronize(s));
     if (h_out)

@@ -120,26 +120,32 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p)
     a->device = r ? r->device : -2;
     return cudaSuccess;
 }
-static cudaError_t copy(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, void *st, int async)
+static cudaError_t copy(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind kind, void *st,
+                        int async)
 {
+    char *base;
+    const bool dd = find(d, &base), sd = find(s, &base);  // the kind, where one is given, fits the pointers
+    if (kind != cudaMemcpyDefault && kind != (sd ? (dd ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost)
+                                                 : (dd ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost)))
+        return cudaErrorInvalidValue;
     for (size_t r = 0; r < h; ++r)
         std::memcpy(at((char *)d + r * dp), at((const char *)s + r * sp), w);
     record("copy", d, s, w * h, st, async);
     return cudaSuccess;
 }
-cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { return copy(d, n, s, n, n, 1, nullptr, 0); }
-cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t st)
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind k) { return copy(d, n, s, n, n, 1, k, nullptr, 0); }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind k, cudaStream_t st)
 {
-    return copy(d, n, s, n, n, 1, st, 1);
+    return copy(d, n, s, n, n, 1, k, st, 1);
 }
-cudaError_t cudaMemcpy2D(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind)
+cudaError_t cudaMemcpy2D(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind k)
 {
-    return copy(d, dp, s, sp, w, h, nullptr, 0);
+    return copy(d, dp, s, sp, w, h, k, nullptr, 0);
 }
-cudaError_t cudaMemcpy2DAsync(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind,
+cudaError_t cudaMemcpy2DAsync(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind k,
                               cudaStream_t st)
 {
-    return copy(d, dp, s, sp, w, h, st, 1);
+    return copy(d, dp, s, sp, w, h, k, st, 1);
 }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t st)
 {

@@ -156,6 +156,11 @@ def check_another_gpu():
     copied(nets, "src", "static")
     copied(nets, "dst", "static")
     no_kernel_sees(nets, "static")
+    # in host memory too (kernels read it only on machines that share their page tables)
+    nets = networks(T, G)
+    rc = lib.panda_step_static(T, G, *(p(a) for a in nets), ctypes.c_float(0.1), 1, 0, None, None)
+    assert rc == 0, lib.panda_last_error(None)
+    no_kernel_sees([a.ctypes.data for a in nets], "static, host")
     # on this device they are read and written where they lie
     here = [lib.fake_alloc(0, x.nbytes) for x in networks(T, G)]
     lib.fake_clear()
