@@ -1140,37 +1140,85 @@ __global__ void k_split3(const float *__restrict__ X, size_t n4, __nv_bfloat16 *
 // host side
 // ---------------------------------------------------------------------------
 struct Phase {
-    std::vector<int> off;      // per worker, its range of items
+    std::vector<int> off;      // per worker, its range of items (once finished)
     std::vector<Item> items;
+    std::vector<int> who, order;  // while it is made: each item's worker; the order they are given out in
     int fixes = 0, slots = 0;  // cut tiles; slots per CTA rank that they meet in
     double cost = 0;           // of the busiest worker, in stages
 };
 
-// Longest first to the least loaded list; the largest load added.
-double assign(std::vector<std::pair<double, Item>> &all, std::vector<std::vector<Item>> &list)
+// The items from `from` on, whose costs are given: longest first (equals in the order they stand
+// in) to the least loaded worker (the first of equals); the largest load.  There are few different
+// costs, so the order takes one pass.
+double assign(Phase &ph, int from, const std::vector<double> &cost, int workers)
 {
-    std::stable_sort(all.begin(), all.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-    using L = std::pair<double, int>;
-    std::priority_queue<L, std::vector<L>, std::greater<L>> heap;
-    for (int w = 0; w < (int)list.size(); ++w)
-        heap.push({0.0, w});
+    std::vector<double> kinds;
+    std::vector<uint16_t> kind(cost.size());
+    size_t k = 0;
+    for (size_t q = 0; q < cost.size(); ++q) {
+        if (k >= kinds.size() || kinds[k] != cost[q])
+            k = std::find(kinds.begin(), kinds.end(), cost[q]) - kinds.begin();
+        if (k == kinds.size())
+            kinds.push_back(cost[q]);
+        kind[q] = (uint16_t)k;
+    }
+    std::vector<int> rank(kinds.size());
+    for (size_t q = 0; q < rank.size(); ++q)
+        rank[q] = (int)q;
+    std::sort(rank.begin(), rank.end(), [&kinds](int x, int y) { return kinds[x] > kinds[y]; });
+    std::vector<int> at(kinds.size());  // where each kind's items go in the order
+    for (uint16_t q : kind)
+        ++at[q];
+    int n = from;
+    for (int r : rank) {
+        const int c = at[r];
+        at[r] = n;
+        n += c;
+    }
+    ph.order.resize(ph.items.size());
+    for (int q = 0; q < from; ++q)
+        ph.order[q] = q;
+    for (size_t q = 0; q < kind.size(); ++q)
+        ph.order[at[kind[q]]++] = from + (int)q;
+    // a heap of (load, worker), the least at the root
+    std::vector<std::pair<double, int>> heap(workers);
+    for (int w = 0; w < workers; ++w)
+        heap[w] = {0.0, w};
     double most = 0.0;
-    for (const auto &x : all) {
-        L top = heap.top();
-        heap.pop();
-        list[top.second].push_back(x.second);
-        heap.push({top.first + x.first, top.second});
-        most = std::max(most, top.first + x.first);
+    ph.who.resize(ph.items.size());
+    for (size_t q = from; q < ph.items.size(); ++q) {
+        std::pair<double, int> x = heap[0];
+        ph.who[ph.order[q]] = x.second;
+        x.first += cost[ph.order[q] - from];
+        most = std::max(most, x.first);
+        int h = 0;
+        for (int c = 1; c < workers; c = 2 * h + 1) {
+            c += c + 1 < workers && heap[c + 1] < heap[c];
+            if (!(heap[c] < x))
+                break;
+            heap[h] = heap[c];
+            h = c;
+        }
+        heap[h] = x;
     }
     return most;
 }
-void finish(const std::vector<std::vector<Item>> &list, Phase &ph)
+// The lists, worker by worker, each in the order in which its items were given out
+void finish(Phase &ph, int workers)
 {
-    ph.off.assign(1, 0);
-    for (const auto &l : list) {
-        ph.items.insert(ph.items.end(), l.begin(), l.end());
-        ph.off.push_back((int)ph.items.size());
+    ph.off.assign(workers + 1, 0);
+    for (int w : ph.who)
+        ++ph.off[w + 1];
+    for (int w = 0; w < workers; ++w)
+        ph.off[w + 1] += ph.off[w];
+    std::vector<int> next(ph.off.begin(), ph.off.end() - 1);
+    std::vector<Item> lists(ph.items.size());
+    for (size_t q = 0; q < lists.size(); ++q) {
+        const int n = ph.order.empty() ? (int)q : ph.order[q];
+        lists[next[ph.who[n]]++] = ph.items[n];
     }
+    ph.items = std::move(lists);
+    ph.who = ph.order = std::vector<int>();
 }
 
 // Costs in stages of K = 64 (measured: 1.9 us on a pair, 0.8 us on one CTA): a
@@ -1193,26 +1241,31 @@ Phase plan_phase1_cut(const Dev &d, int workers, bool pair, int whole, int np)
     const int nR = ceil_div(d.Tp, BK), K = nR + ceil_div(d.Gp, BK), rest = ntile - whole;
     const double E = EPILOGUE[pair];
     Phase ph;
-    std::vector<std::vector<Item>> list(workers);
-    std::vector<double> load(workers, 0.0);
-    std::vector<std::pair<double, Item>> parts;
+    std::vector<double> load(workers, 0.0), parts;  // of the workers; costs of the parts to give out
+    ph.items.reserve(whole + 2 * (size_t)std::max(rest, np * rest));
+    ph.who.reserve(ph.items.capacity());
+    auto give = [&ph](const Item &it, int w) {
+        ph.items.push_back(it);
+        ph.who.push_back(w);
+    };
     for (int t = 0; t < whole; ++t) {
         Item it{};
         it.a = (uint32_t)(t % nmt) | (uint32_t)(t / nmt) << 16;
         it.s1 = (uint16_t)K;
         it.nparts = 1;
-        list[t % workers].push_back(it);
+        give(it, t % workers);
         load[t % workers] += K + E;
     }
     const double share = rest > 0 ? rest * (K + E) / workers : 1.0;
-    std::vector<int> order;  // equal shares go TF-block-major, so that the workers on one gene block's
-    for (int t = whole; t < ntile; ++t)  // TF blocks run side by side
-        order.push_back(t);
-    if (np == 0)
-        std::stable_sort(order.begin(), order.end(), [nmt](int x, int y) { return x % nmt < y % nmt; });
+    std::vector<int> order, cut;
+    if (np == 0) {  // equal shares go TF-block-major, so that the workers on one gene block's TF blocks
+        for (int m = 0; m < nmt; ++m)  // run side by side
+            for (int t = whole + ((m - whole) % nmt + nmt) % nmt; t < ntile; t += nmt)
+                order.push_back(t);
+    }
     for (int q = 0; q < rest; ++q) {
-        const int t = order[q];
-        std::vector<int> cut{0};  // part p: stages [cut[p], cut[p + 1])
+        const int t = np == 0 ? order[q] : whole + q;
+        cut.assign(1, 0);  // part p: stages [cut[p], cut[p + 1])
         const double x0 = q * (K + E);
         if (np > 0) {
             const int e0 = std::max(K / np, nR);
@@ -1241,10 +1294,11 @@ Phase plan_phase1_cut(const Dev &d, int workers, bool pair, int whole, int np)
             const double c = it.s1 - it.s0 + (n > 1 ? CUT[pair] : 0.0) +
                              (p == n - 1 ? E + (n > 1 ? CUT_LAST[pair] : 0.0) : 0.0);
             if (np > 0) {
-                parts.push_back({c, it});
+                ph.items.push_back(it);
+                parts.push_back(c);
             } else {
                 const int w = std::min(workers - 1, (int)((x0 + 0.5 * (cut[p] + cut[p + 1])) / share));
-                list[w].push_back(it);
+                give(it, w);
                 load[w] += c;
             }
         }
@@ -1254,10 +1308,9 @@ Phase plan_phase1_cut(const Dev &d, int workers, bool pair, int whole, int np)
         }
     }
     if (np > 0)
-        ph.cost = ceil_div(whole, workers) * (K + E) + assign(parts, list);
+        ph.cost = ceil_div(whole, workers) * (K + E) + assign(ph, whole, parts, workers);
     else
         ph.cost = *std::max_element(load.begin(), load.end());
-    finish(list, ph);
     return ph;
 }
 
@@ -1270,8 +1323,10 @@ Phase plan_phase1(const Dev &d, int workers, bool pair)
     const int ntile = ceil_div(d.Tp, tile_m(pair)) * ceil_div(d.Gp, tile_n(pair));
     const int nR = ceil_div(d.Tp, BK), K = nR + ceil_div(d.Gp, BK);
     Phase best = plan_phase1_cut(d, workers, pair, ntile, 1);
-    if ((double)ceil_div(ntile, workers) * workers <= 1.05 * ntile)
+    if ((double)ceil_div(ntile, workers) * workers <= 1.05 * ntile) {
+        finish(best, workers);
         return best;
+    }
     const int whole = std::max(0, ntile / workers - 1) * workers;
     for (int np : {0, 2, 3, 4, 6, 8, 12}) {
         if (np > 0 && ((ntile - whole) * np > 4 * workers || K - std::max(K / np, nR) < (np - 1) * MIN_PART))
@@ -1280,6 +1335,7 @@ Phase plan_phase1(const Dev &d, int workers, bool pair)
         if (ph.cost < best.cost)
             best = std::move(ph);
     }
+    finish(best, workers);
     return best;
 }
 
@@ -1290,10 +1346,13 @@ Phase plan_phase2_cap(const Dev &d, int workers, bool pair, int cap)
     const int M = tile_m(pair), N = tile_n(pair);
     const double E = EPILOGUE[pair];
     Phase ph;
-    std::vector<std::pair<double, Item>> all;
+    std::vector<double> cost;
     for (int isP = 1; isP >= 0; --isP) {
         const int ld = isP ? d.Tp : d.Gp, nbm = ceil_div(ld, M), nbn = ceil_div(ld, N), K = ceil_div(isP ? d.Gp : d.Tp, BK);
         const int np = std::min(ceil_div(K, cap), 64);
+        const size_t most = ph.items.size() + (size_t)nbm * (nbn + M / N) / 2 * np;
+        ph.items.reserve(most);
+        cost.reserve(most);
         for (int bm = 0; bm < nbm; ++bm)
             for (int bn = bm * (M / N); bn < nbn; ++bn) {
                 for (int p = 0; p < np; ++p) {
@@ -1307,9 +1366,9 @@ Phase plan_phase2_cap(const Dev &d, int workers, bool pair, int cap)
                     }
                     // (a mirrored tile's epilogue takes almost twice as long)
                     const double e = isP || bn < (bm + 1) * (M / N) ? 1.8 * E : E;
-                    all.push_back({it.s1 - it.s0 + (np > 1 ? CUT[pair] : 0.0) +
-                                       (p == np - 1 ? e + (np > 1 ? CUT_LAST[pair] : 0.0) : 0.0),
-                                   it});
+                    ph.items.push_back(it);
+                    cost.push_back(it.s1 - it.s0 + (np > 1 ? CUT[pair] : 0.0) +
+                                   (p == np - 1 ? e + (np > 1 ? CUT_LAST[pair] : 0.0) : 0.0));
                 }
                 if (np > 1) {
                     ph.fixes += 1;
@@ -1317,9 +1376,7 @@ Phase plan_phase2_cap(const Dev &d, int workers, bool pair, int cap)
                 }
             }
     }
-    std::vector<std::vector<Item>> list(workers);
-    ph.cost = assign(all, list);
-    finish(list, ph);
+    ph.cost = assign(ph, 0, cost, workers);
     return ph;
 }
 
@@ -1333,9 +1390,10 @@ Phase plan_phase2(const Dev &d, int workers, bool pair)
         if (cap < (1 << 20) && parts > 8LL * workers)  // enough items to balance without cutting more
             break;
         Phase ph = plan_phase2_cap(d, workers, pair, cap);
-        if (best.off.empty() || ph.cost < best.cost)
+        if (best.items.empty() || ph.cost < best.cost)
             best = std::move(ph);
     }
+    finish(best, workers);
     return best;
 }
 
@@ -1343,6 +1401,20 @@ struct F32Plan {
     bool pair;
     Phase p1, p2;
 };
+
+// What both phases' busiest workers cost at least: every tile whole, all workers equally busy
+double least_cost(const Dev &d, int workers, bool pair)
+{
+    const int M = tile_m(pair), N = tile_n(pair), kT = ceil_div(d.Tp, BK), kG = ceil_div(d.Gp, BK);
+    const double E = EPILOGUE[pair];
+    double c = (double)ceil_div(d.Tp, M) * ceil_div(d.Gp, N) * (kT + kG + E);
+    for (int isP = 0; isP < 2; ++isP) {
+        const int ld = isP ? d.Tp : d.Gp, nbm = ceil_div(ld, M), nbn = ceil_div(ld, N);
+        for (int bm = 0; bm < nbm; ++bm)
+            c += (nbn - bm * (M / N)) * ((isP ? kG : kT) + E);
+    }
+    return c / workers;
+}
 
 // The tile shape whose busiest worker is done first by the stage times; one
 // CTA per tile only where pairs would have few tiles each (it reads three times
@@ -1355,6 +1427,8 @@ F32Plan f32_plan_for(const Dev &d, int nsm)
         if (!pair && (long long)ceil_div(d.Gp, 256) * ceil_div(d.Tp, 256) > 2LL * nsm)
             continue;
         const int workers = pair ? nsm / 2 : nsm;
+        if (!best.p1.off.empty() && STAGE_US[pair] * least_cost(d, workers, pair != 0) > t_best * (1.0 + 1e-9))
+            continue;  // not even with its work spread evenly
         F32Plan p{pair != 0, plan_phase1(d, workers, pair != 0), plan_phase2(d, workers, pair != 0)};
         const double t = STAGE_US[pair] * (p.p1.cost + p.p2.cost);
         if (best.p1.off.empty() || t < t_best) {
