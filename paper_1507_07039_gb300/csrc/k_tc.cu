@@ -970,7 +970,8 @@ __device__ __forceinline__ void phase1_pair(const Src &src, Ctl *ctl0)
             __nv_bfloat16 *Wh = d.Wh[nx], *Wl = d.Wl[nx];
             // FP8MIX: the A-num accumulator holds the scaled E4M3 products; W' gets E4M3 copies too
             const bool q8 = d.fp8 != 0;
-            const float ainv = q8 ? 1.0f / (d.f8[cur] * d.f8[2]) : 1.0f, s8 = q8 ? d.f8[3] : 1.0f;
+            // (powers of two, inverted one by one: the product of two scales overflows for norms below 2^-57)
+            const float ainv = q8 ? (1.0f / d.f8[cur]) * (1.0f / d.f8[2]) : 1.0f, s8 = q8 ? d.f8[3] : 1.0f;
             if (q8 && mt == 0 && nt == 0 && rank == 0 && threadIdx.x == 64)
                 d.f8[nx] = s8;  // the scale of W8[nx] and Wt8[nx] from here on
             // what does not depend on the accumulators is fetched before waiting for them
@@ -1586,7 +1587,7 @@ __device__ __forceinline__ void phase2_pair(const Src &src, Ctl *ctl)
             const float a = d.ctl->alpha, keep = 1.0f - a;
             // FP8MIX: C-tile accumulators hold products of W'^T scaled by f8[cur] on both sides; C' gets
             // an E4M3 copy scaled so that no entry saturates (bound from |C_k.| and |W'_.k|)
-            const float sw = d.fp8 ? d.f8[cur] : 1.0f, ainv2 = 1.0f / (sw * sw);
+            const float sw = d.fp8 ? d.f8[cur] : 1.0f, ainv2 = (1.0f / sw) * (1.0f / sw);
             const float sC =
                 d.fp8 ? e4m3_scale(fp8_bound_c(__uint_as_float(d.f8n[5]), __uint_as_float(d.f8n[3]))) : 1.0f;
             if (d.fp8 && threadIdx.x == 64)

@@ -35,6 +35,28 @@ def test_small_networks_scale(T, G, prec):
             assert np.array_equal(got[n], one[n] * c), (n, k)
 
 
+def close(got, one, c):
+    """Each network within 1e-3 of its largest entry, P's and C's diagonals apart."""
+    for n in ("W", "P", "C"):
+        x, y = got[n].astype(np.float64) / float(c), one[n].astype(np.float64)
+        if n != "W":
+            d = np.diag(y)
+            assert np.max(np.abs(np.diag(x) - d)) <= 1e-3 * np.max(np.abs(d)), n
+            x, y = x - np.diag(np.diag(x)), y - np.diag(d)
+        assert np.max(np.abs(x - y)) <= 1e-3 * np.max(np.abs(y)), n
+
+
+def test_fp8mix_scales_whose_product_overflows():
+    """Entries of about 2^-60: the E4M3 copies are scaled by 2^65 each, whose product
+    is no float.  The scaled entries are the same bytes; what is lost is the BF16
+    products' and squares' part below 2^-149, 2^-20 of them.  (With the product
+    of the scales inverted, A and the new C were 0: 1e-1 of the largest entry.)"""
+    nets = networks(40, 70)
+    one = gh.gpu_run(*nets, 3, 0.1, 0.0, 2, normalize=False)
+    c = np.float32(2.0) ** -58
+    close(gh.gpu_run(*(x * c for x in nets), 3, 0.1, 0.0, 2, normalize=False), one, c)
+
+
 @pytest.mark.parametrize("T,G", [(40, 70), (1024, 2048)])  # one CTA a tile; CTA pairs
 def test_fp32_scales(T, G):
     """Where no part product leaves the normal range the bits are the same."""
@@ -57,14 +79,7 @@ def test_fp32_squared_norms_below_the_normal_range(k):
     nets = networks(40, 70)
     one = gh.gpu_run(*nets, 0, 0.1, 0.0, 1, normalize=False)
     c = np.float32(2.0) ** k
-    got = gh.gpu_run(*(x * c for x in nets), 0, 0.1, 0.0, 1, normalize=False)
-    for n in ("W", "P", "C"):
-        x, y = got[n].astype(np.float64) / float(c), one[n].astype(np.float64)
-        if n != "W":
-            d = np.diag(y)
-            assert np.max(np.abs(np.diag(x) - d)) <= 1e-3 * np.max(np.abs(d)), n
-            x, y = x - np.diag(np.diag(x)), y - np.diag(d)
-        assert np.max(np.abs(x - y)) <= 1e-3 * np.max(np.abs(y)), n
+    close(gh.gpu_run(*(x * c for x in nets), 0, 0.1, 0.0, 1, normalize=False), one, c)
 
 
 def test_fp32_squared_norms_near_the_largest_float():
